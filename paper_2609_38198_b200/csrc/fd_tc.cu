@@ -110,6 +110,12 @@ __device__ __forceinline__ ItemGeometry item_geometry(const TcParams& p, int w, 
     return g;
 }
 
+// The thread of an issuing warp that issues.  Row-sum modes keep a lane test: their tensor pipe is mostly idle and the slower
+// issue it compiles to is part of the pacing of their Gram MMAs (with elect.sync both degree passes at N = 2^18 took 26.7 ms
+// instead of 26.3).
+template <int MODE>
+__device__ __forceinline__ bool issuing_thread(int lane) { return is_rowsum(MODE) ? lane == 0 : elect_one(); }
+
 // ------------------------------------------------------------------------------------------------ the kernel
 // Tiles of one work item are numbered n = 2 j + t (column tile j, row tile t) and flow through a ring of NBUF
 // S buffers in TMEM (3 in block mode, 4 in row-sum mode), so the tensor core runs up to NBUF tiles ahead of the
@@ -130,7 +136,7 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
     Barriers* bars = (Barriers*)(xi_base + 2 * K16 * SM::kXChunk);
     volatile int* abort_flag = &bars->abort_flag;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = is_rowsum(MODE) ? threadIdx.x >> 5 : warp_index(), lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
         // a column stage is released by the Gram issuer alone (row-sum mode) or by both product issuers (block mode)
@@ -185,7 +191,7 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
       asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(40));
       if (warp == 8) {
         // =============================================================== TMA producer (one thread)
-        if (lane == 0) {
+        if (issuing_thread<MODE>(lane)) {
             prefetch_tmap(&map_xrow); prefetch_tmap(&map_xcol);
             if (!is_rowsum(MODE)) prefetch_tmap(&map_whi);
             uint32_t it = 0;
@@ -230,7 +236,7 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
       } else if (warp == 11) {
         // =============================================================== Gram MMA issuer (one thread)
         // Issues S(n) = A_t B_j^T for every tile as soon as its ring buffer is free again; runs up to NBUF tiles ahead.
-        if (lane == 0) {
+        if (issuing_thread<MODE>(lane)) {
           if constexpr (is_rowsum(MODE)) {
             // Row-sum mode: the MUFU binds and the tensor pipe is mostly idle; descriptors are rebuilt per MMA, which paces
             // the Gram MMAs between the warpgroups' TMEM loads (issuing them in tight bursts measured 5 % slower).
@@ -351,7 +357,7 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
       } else if (!is_rowsum(MODE)) {
         // =============================================================== product MMA issuers: warp 9 -> row tile 0, warp 10 -> row tile 1
         // Two issuing threads so that the per-tile bookkeeping of one overlaps the MMAs of the other.
-        if (lane == 0) {
+        if (issuing_thread<MODE>(lane)) {
             constexpr uint32_t idesc_y = idesc_f16(BT);
             const int t = warp - 9;
             // W stage descriptor as (low, high) words: 128 B rows (SWIZZLE_128B), 1024 B between 8-row groups

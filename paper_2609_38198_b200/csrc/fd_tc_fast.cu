@@ -79,7 +79,7 @@ k_bp(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
     BarriersP* bars = (BarriersP*)(xi_base + K16 * SM::kXChunk);
     volatile int* abort_flag = &bars->abort_flag;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) { mbar_init(&bars->full[s], 1); mbar_init(&bars->empty[s], 1); }
@@ -121,7 +121,7 @@ k_bp(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
       asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsUtil));
       if (warp == 20) {
         // =============================================================== TMA producer (one thread)
-        if (lane == 0) {
+        if (elect_one()) {
             prefetch_tmap(&map_xrow); prefetch_tmap(&map_xcol); prefetch_tmap(&map_whi);
             uint32_t it = 0;
             bool ok = true;
@@ -159,7 +159,7 @@ k_bp(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
         // =============================================================== Gram MMA issuer (one thread)
         // S(gt) = A_I B_J^T as soon as its buffer is free again (the product MMAs of tile gt - 3 have completed); runs up to
         // three tiles ahead of the product.
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc_g = idesc_f16(128);
             // descriptors as (low, high) words: 64 B rows (SWIZZLE_64B), 512 B between 8-row groups
             const uint64_t xd = smem_desc(smem_u32(xi_base), 512, 4);
@@ -210,7 +210,7 @@ k_bp(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
         }
       } else if (warp == 21) {
         // =============================================================== product MMA issuer (one thread)
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc_y = idesc_f16(BT);
             const uint32_t y_addr = tmem + kYCol;
             // W stage descriptor as (low, high) words: 128 B rows (SWIZZLE_128B), 1024 B between 8-row groups
