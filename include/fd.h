@@ -86,15 +86,14 @@ fd_status fd_create(fd_ctx** out, const float* X_dev, int64_t N, int32_t D, int6
 fd_status fd_destroy(fd_ctx* ctx);
 
 /* Tuning / test knobs by name: "path" (FD_PATH_*), "splits" (0 = auto), "flush" (column tiles
- * between accumulator flushes of the tensor-core kernels; 0 = default: 1 in the fp32-grade mode, whose eigenvalue budget
- * the tensor core's round-toward-zero accumulation would otherwise eat, 8 in the reduced-precision mode), "tc_max_mag" (largest beta * log2(e) *
+ * between accumulator flushes of the tensor-core kernels; 0 = default: 2 (up to 32 columns) or 1 in the fp32-grade mode, whose
+ * eigenvalue budget the tensor core's round-toward-zero accumulation would otherwise eat, 8 in the reduced-precision mode), "tc_max_mag" (largest beta * log2(e) *
  * max|x - mu|^2 for which the Gram-form tensor-core kernel serves the fp32 mode), "jt_chunk" (column
  * tiles per L2-resident chunk of the tensor-core block product), "sym" (1, default: the degree passes on the Gram-form
  * kernels use K = K^T and evaluate only the tiles on or above the diagonal -- each off-diagonal tile gives the row sums
  * of its rows and, transposed, of its columns, N (N + 128) / 2 exponentials instead of N^2; 0: every tile; row-sharded
- * contexts always evaluate every tile of their rows), "tail_split" (1, default: in a block product with a single column
- * chunk the row pairs of the last, partly filled round of CTAs -- all pairs when there are fewer than CTAs -- are
- * shared by two CTAs each, half the columns per CTA, partial results added atomically; 0: off), "wait_selftest"
+ * contexts always evaluate every tile of their rows), "tail_split" (0 or 1: accepted, without effect: the block
+ * product cuts its work into equal ranges for every size), "wait_selftest"
  * (value = limit in SM cycles: enqueues
  * a one-thread kernel whose bounded wait on a barrier that nothing completes must expire; the next
  * fd_synchronize then returns FD_ERR_TIMEOUT and the context stays usable).  fd_get_option also reports "last_path" (the

@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(128, 1) k_probe_mma(long long* __restrict__ cy
     uint8_t* base = (uint8_t*)(((uintptr_t)raw + 1023) & ~(uintptr_t)1023);
     __shared__ uint64_t bar;
     __shared__ uint32_t tbase;
-    const int warp = warp_index(), lane = threadIdx.x & 31;
+    const int warp = warp_index();
     if (threadIdx.x == 0) { mbar_init(&bar, 1); asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
     for (int i = threadIdx.x; i < 48 * 1024 / 4; i += blockDim.x) ((uint32_t*)base)[i] = 0u;
     if (warp == 0) {

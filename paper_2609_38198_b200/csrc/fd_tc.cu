@@ -1,4 +1,5 @@
-// Gram-form kernel on the 5th-generation tensor cores (tcgen05 + TMEM), Eqs. 4-6.
+// Gram-form row sums on the 5th-generation tensor cores (tcgen05 + TMEM), Eqs. 4-6, the operand packing and the host side of every
+// Gram-form pass.  (The block products' kernels: fd_tc_block.cu, fp32-grade; fd_tc_fast.cu, reduced precision.)
 //
 // Per (row tile I, column tile J) of 128 x 128 pairs:
 //   1. Gram MMA (fp16 hi/lo split, three products per 16-wide K slab, fp32 accumulation in TMEM)
@@ -6,27 +7,18 @@
 //        S_ij = 2 b' x_i.x_j - b' r_i - b' r_j + bias            (b' = beta log2 e, Eq. 4)
 //      the norms ride along as extra K columns ([.., e_i, 1] . [.., 1, e_j]), each norm carried by
 //      two hi/lo pairs so it is exact to fp32.
-//   2. Two warpgroups (one per row tile; thread = row) read S from TMEM, take 2^S on the MUFU,
-//      split P = 2^S into fp16 hi + lo (mask / subtract), and write both halves back IN PLACE over
-//      the S columns as the TMEM A operand.
-//   3. Product MMA  Y_I += P_hi W_hi + P_lo W_hi + P_hi W_lo  with W = diag(right) V pre-split into
-//      fp16 hi / lo (per-column power-of-two scaling), fp32 accumulation in TMEM (Eq. 6).
-//   4. Every `flush` column tiles the TMEM accumulator is added into fp32 registers and restarted,
-//      so tensor-core accumulation error does not grow with N.
-// S tiles flow through a ring of TMEM buffers shared by both row tiles, so the tensor core runs ahead of
-// the warpgroups and the product MMA of a tile overlaps the exponentials of the next ones.
-// Row-sum mode (rectangular and row-sharded passes): no product MMA; the warpgroups add P (and P^2) on the FMA pipe,
+//   2. Two warpgroups (one per row tile; thread = row) read S from TMEM, take 2^S on the MUFU and add P (and P^2).
+// S tiles flow through a ring of TMEM buffers shared by both row tiles, so the tensor core runs ahead of the warpgroups.
+// Row-sum mode (rectangular and row-sharded passes): the warpgroups add P (and P^2) on the FMA pipe,
 // fp32 within a column tile and fp64 across tiles; a positive right vector enters through e_j.
 // Symmetric row-sum mode (the degree passes of a whole data set, K = K^T): only the tiles on or above the diagonal are
 // evaluated; the S tile is built with the streamed points on the TMEM lanes, so one thread adds up both what a tile gives
 // its streamed point (one fixed-point atomic per tile) and, in 128 per-thread accumulators reduced across lanes every
 // 64 tiles, what it gives the resident points.
 //
-// One persistent CTA per SM: warps 0-3 / 4-7 = the two exponential warpgroups (raised to 232 registers);
-// warp 8 = TMA producer, warps 9 / 10 = product-MMA issuers for row tile 0 / 1, warp 11 = Gram-MMA issuer
-// (lowered to 40 registers).  Three issuing threads because the per-tile bookkeeping of a lone issuer
-// (waits, commits, descriptors) cost about as much as its MMAs and left the tensor pipe idle.  Column tiles are staged by TMA (every CTA loads its own copy) through a 4-deep ring.
-// Every mbarrier wait is bounded; on expiry the CTA raises a status word, drains and exits.
+// One persistent CTA per SM: warps 0-3 / 4-7 = the two exponential warpgroups (raised to 232 registers); warp 8 = TMA producer,
+// warp 11 = Gram-MMA issuer (lowered to 40 registers).  Column tiles are staged by TMA (every CTA loads its own copy) through
+// a 4-deep ring.  Every mbarrier wait is bounded; on expiry the CTA raises a status word, drains and exits.
 #include <cuda.h>
 
 #include <algorithm>
@@ -44,11 +36,9 @@ using namespace tc;
 template <int BT, int MODE>
 struct Smem {
     static constexpr int kXChunk = 128 * 64;                       // one K slab (hi|lo) of 128 points: 8 KB
-    static constexpr int kWHalf = is_rowsum(MODE) ? 0 : BT * 128;   // 64 j x BT columns fp16
-    static constexpr int kWBytes = is_rowsum(MODE) ? 0 : 4 * kWHalf;   // [W_hi j-half 0][W_hi j-half 1][W_lo 0][W_lo 1]
     // symmetric row-sum mode: per-warp column partial sums, [row tile][parity][warp quarter][128 columns] floats
     static constexpr int kColPartBytes = (MODE == kModeRowsumSym) ? 2 * 2 * 4 * 128 * 4 + 64 : 0;   // + four mbarriers (col_ready[row tile][parity])
-    static __host__ __device__ constexpr int stage_bytes(int K16) { return K16 * kXChunk + kWBytes; }
+    static __host__ __device__ constexpr int stage_bytes(int K16) { return K16 * kXChunk; }
     static __host__ __device__ constexpr int total(int K16) {
         return 1024 /*align slack*/ + kStages * stage_bytes(K16) + 2 * K16 * kXChunk + 1024 /*barriers*/ + kColPartBytes;
     }
@@ -64,22 +54,18 @@ struct Barriers {
     // the previous phase complete; a barrier per buffer alone, shared by both row tiles, lets a waiter that skips
     // alternate phases pass one phase early.)
     uint64_t s_full[kMaxBuf][2];            // S tile ready in ring buffer (Gram issuer -> warpgroup)
-    uint64_t s_done[kMaxBuf][2];            // block mode: P written in place; row-sum mode: S consumed (warpgroup -> issuer)
-    uint64_t p_half[kMaxBuf][2];            // block mode: first 64 columns of P written (lets the product MMA start early)
-    uint64_t kw_done[kMaxBuf][2];           // block mode: product MMAs that read P from this buffer have completed
-    uint64_t y_full[2], y_empty[2];         // accumulator flush hand-off (per row tile)
+    uint64_t s_done[kMaxBuf][2];            // S consumed (warpgroup -> issuer)
     uint32_t tmem_base;
     int abort_flag;
 };
 
 // ------------------------------------------------------------------------------------------------ work items
 // Work item w of a CTA -> (row pair, first column tile, number of column tiles, column chunk).
-//   block / row-sum modes: (column chunk c, row pair r) with c outermost, r = blockIdx.x + k * gridDim.x;
-//   block mode with tail split: full rounds first, then one half-range item of a tail pair (see TcParams);
+//   row-sum mode: (column chunk c, row pair r) with c outermost, r = blockIdx.x + k * gridDim.x;
 //   symmetric row-sum mode: only tiles on or above the diagonal.  Row pair r needs column tiles 2 r .. num_jt - 1; pairing r
 //     with num_work - 1 - r gives work units of equal length (num_jt + 2 tiles): unit u = blockIdx.x + k * gridDim.x is the
 //     two items {u, num_work - 1 - u} (the middle pair of an odd count stands alone: its second item is empty).
-struct ItemGeometry { int item, j0, num_jt, cch; bool tail_item; };
+struct ItemGeometry { int item, j0, num_jt, cch; };
 
 template <int MODE>
 __device__ __forceinline__ ItemGeometry item_geometry(const TcParams& p, int w, int my_rows) {
@@ -90,45 +76,25 @@ __device__ __forceinline__ ItemGeometry item_geometry(const TcParams& p, int w, 
         g.item = (w & 1) ? p.num_work - 1 - unit : unit;
         g.j0 = 2 * g.item;
         g.num_jt = ((w & 1) && g.item == unit) ? 0 : p.num_jt - g.j0;
-        g.tail_item = false;
-    } else if constexpr (MODE == kModeBlockTail) {
-        const int full_rounds = p.tail_first / (int)gridDim.x;
-        const int half = (p.num_jt + 1) / 2;
-        g.cch = 0;
-        g.tail_item = w >= full_rounds;
-        const int part = g.tail_item ? (int)blockIdx.x / p.tail_pairs : 0;
-        g.item = g.tail_item ? p.tail_first + (int)blockIdx.x % p.tail_pairs : (int)blockIdx.x + w * (int)gridDim.x;
-        g.j0 = g.tail_item ? part * half : 0;
-        g.num_jt = g.tail_item ? (part == 0 ? half : p.num_jt - half) : p.num_jt;
     } else {
         g.cch = w / my_rows;
         g.item = (int)blockIdx.x + (w % my_rows) * (int)gridDim.x;
         g.j0 = g.cch * p.jt_chunk;
         g.num_jt = (p.num_jt - g.j0 < p.jt_chunk) ? p.num_jt - g.j0 : p.jt_chunk;
-        g.tail_item = false;
     }
     return g;
 }
 
-// The thread of an issuing warp that issues.  Row-sum modes keep a lane test: their tensor pipe is mostly idle and the slower
-// issue it compiles to is part of the pacing of their Gram MMAs (with elect.sync both degree passes at N = 2^18 took 26.7 ms
-// instead of 26.3).
-template <int MODE>
-__device__ __forceinline__ bool issuing_thread(int lane) { return is_rowsum(MODE) ? lane == 0 : elect_one(); }
-
 // ------------------------------------------------------------------------------------------------ the kernel
-// Tiles of one work item are numbered n = 2 j + t (column tile j, row tile t) and flow through a ring of NBUF
-// S buffers in TMEM (3 in block mode, 4 in row-sum mode), so the tensor core runs up to NBUF tiles ahead of the
-// warpgroups and neither warpgroup waits for the product MMA of its previous tile.
+// Tiles of one work item are numbered n = 2 j + t (column tile j, row tile t) and flow through a ring of four S buffers in
+// TMEM, so the tensor core runs up to four tiles ahead of the warpgroups.  BT = 16: with the sum of squares, 32: without.
 template <int BT, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
-k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUtensorMap map_xcol,
-     const __grid_constant__ CUtensorMap map_whi, const TcParams p) {
+k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUtensorMap map_xcol, const TcParams p) {
     extern __shared__ uint8_t smem_raw[];
     using SM = Smem<BT, MODE>;
-    constexpr int NBUF = is_rowsum(MODE) ? 4 : 3;
-    constexpr uint32_t kRingPeriod = (NBUF & 1) ? 2 * NBUF : NBUF;   // tiles between two uses of a buffer by the same row tile
-    constexpr uint32_t kYCol = 384;                    // block mode: Y_t at columns 384 + 64 t
+    constexpr int NBUF = 4;
+    constexpr uint32_t kRingPeriod = NBUF;             // tiles between two uses of a buffer by the same row tile
     const int K16 = p.K16;
     uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* stage_base = base;
@@ -136,18 +102,15 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
     Barriers* bars = (Barriers*)(xi_base + 2 * K16 * SM::kXChunk);
     volatile int* abort_flag = &bars->abort_flag;
 
-    const int warp = is_rowsum(MODE) ? threadIdx.x >> 5 : warp_index(), lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
-        // a column stage is released by the Gram issuer alone (row-sum mode) or by both product issuers (block mode)
-        for (int s = 0; s < kStages; ++s) { mbar_init(&bars->full[s], 1); mbar_init(&bars->empty[s], is_rowsum(MODE) ? 1 : 2); }
+        for (int s = 0; s < kStages; ++s) { mbar_init(&bars->full[s], 1); mbar_init(&bars->empty[s], 1); }
         mbar_init(&bars->xfull, 1); mbar_init(&bars->xempty, 1);
         for (int u = 0; u < kMaxBuf; ++u)
             for (int t = 0; t < 2; ++t) {
                 mbar_init(&bars->s_full[u][t], 1); mbar_init(&bars->s_done[u][t], 4);
-                mbar_init(&bars->kw_done[u][t], 1); mbar_init(&bars->p_half[u][t], 4);
             }
-        for (int t = 0; t < 2; ++t) { mbar_init(&bars->y_full[t], 1); mbar_init(&bars->y_empty[t], 4); }
         if constexpr (MODE == kModeRowsumSym) {
             uint64_t* col_ready = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(bars) + 1024 + 2 * 2 * 4 * 128 * 4);
             for (int u = 0; u < 4; ++u) mbar_init(&col_ready[u], 4);          // the four warps' column partials of a tile are written
@@ -170,30 +133,24 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
     // column operands at about the same time; a row's partial results always come from the same threads, in order.
     // (item_geometry above has the other modes' orders.)
     constexpr bool kSym = MODE == kModeRowsumSym;
-    constexpr bool kTail = MODE == kModeBlockTail;
     const int my_rows = kSym ? ((p.num_work + 1) / 2 - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x
                              : (p.num_work - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-    const int my_items = kSym ? 2 * my_rows
-                       : kTail ? p.tail_first / (int)gridDim.x + ((int)blockIdx.x < 2 * p.tail_pairs ? 1 : 0) : my_rows * p.num_chunks;
+    const int my_items = kSym ? 2 * my_rows : my_rows * p.num_chunks;
 #define FD_ITEM_GEOMETRY(w)                                                                         \
     const ItemGeometry geo_ = item_geometry<MODE>(p, (w), my_rows);                                 \
     const int cch = geo_.cch;                                                                       \
     const int item = geo_.item;                                                                     \
     const int j0 = geo_.j0;                                                                         \
     const int num_jt = geo_.num_jt;                                                                 \
-    const bool tail_item = geo_.tail_item;                                                          \
     const int tiles_per_item = 2 * num_jt;                                                          \
-    (void)tail_item;                                                                                \
-    (void)item; (void)tiles_per_item; (void)cch
-    const int flush = p.flush;
+    (void)item; (void)tiles_per_item; (void)cch; (void)j0
 
     if (warp >= 8) {
       asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(40));
       if (warp == 8) {
         // =============================================================== TMA producer (one thread)
-        if (issuing_thread<MODE>(lane)) {
+        if (lane == 0) {
             prefetch_tmap(&map_xrow); prefetch_tmap(&map_xcol);
-            if (!is_rowsum(MODE)) prefetch_tmap(&map_whi);
             uint32_t it = 0;
             bool ok = true;
             for (int w = 0; w < my_items && ok; ++w) {
@@ -213,15 +170,6 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
                     mbar_expect_tx(&bars->full[s], SM::stage_bytes(K16));
                     for (int c = 0; c < K16; ++c)
                         tma_load_2d(st + c * SM::kXChunk, &map_xcol, 0, (int)(c * p.np_cols + (int64_t)(j0 + j) * 128), &bars->full[s]);
-                    if (!is_rowsum(MODE)) {
-                        uint8_t* wst = st + K16 * SM::kXChunk;
-                        tma_load_2d(wst, &map_whi, (j0 + j) * 128, 0, &bars->full[s]);
-                        tma_load_2d(wst + SM::kWHalf, &map_whi, (j0 + j) * 128 + 64, 0, &bars->full[s]);
-                        // (W_hi and W_lo are rows 0.. and lo_row.. of one array: one tensor map, and a parameter block that
-                        // stays below 640 bytes -- above it the kernel measured 2.5 % more SM cycles)
-                        tma_load_2d(wst + 2 * SM::kWHalf, &map_whi, (j0 + j) * 128, p.lo_row, &bars->full[s]);
-                        tma_load_2d(wst + 3 * SM::kWHalf, &map_whi, (j0 + j) * 128 + 64, p.lo_row, &bars->full[s]);
-                    }
                 }
             }
             if (!ok) {
@@ -236,10 +184,10 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
       } else if (warp == 11) {
         // =============================================================== Gram MMA issuer (one thread)
         // Issues S(n) = A_t B_j^T for every tile as soon as its ring buffer is free again; runs up to NBUF tiles ahead.
-        if (issuing_thread<MODE>(lane)) {
-          if constexpr (is_rowsum(MODE)) {
-            // Row-sum mode: the MUFU binds and the tensor pipe is mostly idle; descriptors are rebuilt per MMA, which paces
-            // the Gram MMAs between the warpgroups' TMEM loads (issuing them in tight bursts measured 5 % slower).
+        if (lane == 0) {
+            // The MUFU binds and the tensor pipe is mostly idle; descriptors are rebuilt per MMA under a plain lane test, which paces
+            // the Gram MMAs between the warpgroups' TMEM loads (issuing them in tight bursts measured 5 % slower, electing
+            // the thread with elect.sync 2 %).
             constexpr uint32_t idesc_g = idesc_f16(128);
             uint32_t it0 = 0, gn0 = 0;
             bool ok = true;
@@ -256,7 +204,7 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
                     if (g >= (uint32_t)NBUF) {
                         // the tile that used this buffer last (NBUF tiles ago, possibly of the other row tile) must be finished
                         const uint32_t gp = g - NBUF;
-                        uint64_t* fb = is_rowsum(MODE) ? &bars->s_done[buf][gp & 1] : &bars->kw_done[buf][gp & 1];
+                        uint64_t* fb = &bars->s_done[buf][gp & 1];
                         ok = mbar_wait(fb, (gp / kRingPeriod) & 1, abort_flag, p.status, 5);
                         if (!ok) break;
                     }
@@ -285,131 +233,11 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
                         mma_ss(s_addr, a, b, idesc_g, 1);
                     }
                     tc_commit(&bars->s_full[buf][n & 1]);
-                    if (is_rowsum(MODE) && (n & 1)) tc_commit(&bars->empty[s]);   // both Gram MMAs of this column tile issued
+                    if (n & 1) tc_commit(&bars->empty[s]);   // both Gram MMAs of this column tile issued
                 }
                 if (ok) tc_commit(&bars->xempty);                  // the row operand tiles may be replaced
                 it0 += (uint32_t)num_jt;
                 gn0 += (uint32_t)tiles_per_item;
-            }
-          } else {
-            constexpr uint32_t idesc_g = idesc_f16(128);
-            // Operand descriptors as (low, high) words and ring positions as counters: this thread shares its scheduler
-            // with busy warps, so every instruction it does not issue shortens the gap between two MMAs.
-            const uint64_t xd = smem_desc(smem_u32(xi_base), 512, 4);      // 64 B rows (SWIZZLE_64B), 512 B between 8-row groups
-            const uint32_t xi_lo = (uint32_t)xd, xdesc_hi = (uint32_t)(xd >> 32);
-            const uint32_t stage_lo = (uint32_t)smem_desc(smem_u32(stage_base), 512, 4);
-            const uint32_t stage_step = (uint32_t)(SM::stage_bytes(K16) >> 4);
-            constexpr uint32_t kSlab = SM::kXChunk >> 4;
-            uint32_t itj = 0, buf = 0, gr = 0, ph = 0;              // column-tile counter; tile index mod NBUF, mod kRingPeriod, ring phase
-            bool first_round = true;                                // no buffer has been used yet
-            bool ok = true;
-            for (int w = 0; w < my_items && ok; ++w) {
-                FD_ITEM_GEOMETRY(w);
-                ok = mbar_wait(&bars->xfull, w & 1, abort_flag, p.status, 3);
-                if (!ok) break;
-                tc_fence_after();
-                for (int n = 0; n < tiles_per_item && ok; ++n) {
-                    const int t = n & 1;
-                    const int s = itj % kStages;
-                    if (!first_round) {
-                        // the tile that used this buffer last (NBUF tiles ago, possibly of the other row tile) must be finished
-                        const int tp = (NBUF & 1) ? (t ^ 1) : t;
-                        const uint32_t php = gr >= (uint32_t)NBUF ? ph : ph ^ 1u;
-                        uint64_t* fb = is_rowsum(MODE) ? &bars->s_done[buf][tp] : &bars->kw_done[buf][tp];
-                        ok = mbar_wait(fb, php, abort_flag, p.status, 5);
-                        if (!ok) break;
-                    }
-                    if (t == 0) {
-                        ok = mbar_wait(&bars->full[s], (itj / kStages) & 1, abort_flag, p.status, 4);
-                        if (!ok) break;
-                    }
-                    tc_fence_after();
-                    // The two small cross terms (hi x lo) go first and the large hi x hi term last: each MMA rounds its
-                    // result at the magnitude of its largest addend, so only the final one rounds at full magnitude.
-                    const uint32_t s_addr = tmem + 128u * buf;
-                    const uint32_t a0 = xi_lo + (uint32_t)(t * K16) * kSlab, b0 = stage_lo + (uint32_t)s * stage_step;
-                    if (K16 == 1) {
-                        mma_ss2<0>(s_addr, a0, xdesc_hi, b0 + 2, xdesc_hi, idesc_g);          // + 2: the lo half starts 32 B into the row
-                        mma_ss2<1>(s_addr, a0 + 2, xdesc_hi, b0, xdesc_hi, idesc_g);
-                        mma_ss2<1>(s_addr, a0, xdesc_hi, b0, xdesc_hi, idesc_g);
-                    } else {
-                        for (int c = 0; c < K16; ++c) {
-                            const uint32_t a = a0 + (uint32_t)c * kSlab, b = b0 + (uint32_t)c * kSlab;
-                            if (c == 0) mma_ss2<0>(s_addr, a, xdesc_hi, b + 2, xdesc_hi, idesc_g);
-                            else mma_ss2<1>(s_addr, a, xdesc_hi, b + 2, xdesc_hi, idesc_g);
-                            mma_ss2<1>(s_addr, a + 2, xdesc_hi, b, xdesc_hi, idesc_g);
-                        }
-                        for (int c = 0; c < K16; ++c)
-                            mma_ss2<1>(s_addr, a0 + (uint32_t)c * kSlab, xdesc_hi, b0 + (uint32_t)c * kSlab, xdesc_hi, idesc_g);
-                    }
-                    tc_commit(&bars->s_full[buf][t]);
-                    if (t == 1) {
-                        if (is_rowsum(MODE)) tc_commit(&bars->empty[s]);   // both Gram MMAs of this column tile issued
-                        ++itj;
-                    }
-                    if (++buf == (uint32_t)NBUF) { buf = 0; first_round = false; }
-                    if (++gr == kRingPeriod) { gr = 0; ph ^= 1u; }
-                }
-                if (ok) tc_commit(&bars->xempty);                  // the row operand tiles may be replaced
-            }
-          }
-        }
-      } else if (!is_rowsum(MODE)) {
-        // =============================================================== product MMA issuers: warp 9 -> row tile 0, warp 10 -> row tile 1
-        // Two issuing threads so that the per-tile bookkeeping of one overlaps the MMAs of the other.
-        if (issuing_thread<MODE>(lane)) {
-            constexpr uint32_t idesc_y = idesc_f16(BT);
-            const int t = warp - 9;
-            // W stage descriptor as (low, high) words: 128 B rows (SWIZZLE_128B), 1024 B between 8-row groups
-            const uint64_t wd = smem_desc(smem_u32(stage_base + K16 * SM::kXChunk), 1024, 2);
-            const uint32_t wbase_lo = (uint32_t)wd, wdesc_hi = (uint32_t)(wd >> 32);
-            const uint32_t stage_step = (uint32_t)(SM::stage_bytes(K16) >> 4);
-            constexpr uint32_t kLoOff = (uint32_t)((2 * SM::kWHalf) >> 4);          // W_lo tiles follow the two W_hi tiles of a stage
-            uint32_t itj = 0, n_grp = 0;
-            uint32_t buf = (uint32_t)t % NBUF, gr = (uint32_t)t, ph = 0;            // this row tile's tile index mod NBUF, mod kRingPeriod, ring phase
-            bool ok = true;
-            const uint32_t y_addr = tmem + kYCol + 64 * t;
-            for (int w = 0; w < my_items && ok; ++w) {
-                FD_ITEM_GEOMETRY(w);
-                int in_group = 0;                                  // tiles accumulated in the current group (no division in the hot loop)
-                for (int j = 0; j < num_jt && ok; ++j, ++itj) {
-                    const int s = itj % kStages;
-                    ok = mbar_wait(&bars->p_half[buf][t], ph, abort_flag, p.status, 7);
-                    if (!ok) break;
-                    const bool group_start = in_group == 0;
-                    const bool group_end = in_group + 1 == flush || j + 1 == num_jt;
-                    in_group = group_end ? 0 : in_group + 1;
-                    if (group_start && n_grp > 0) {
-                        ok = mbar_wait(&bars->y_empty[t], (n_grp - 1) & 1, abort_flag, p.status, 6);
-                        if (!ok) break;
-                    }
-                    tc_fence_after();
-                    // Y_t += P W : 8 K steps of 16 columns j; K step ks reads P_hi at S-buffer columns [16 ks, 16 ks + 8)
-                    // and P_lo at [16 ks + 8, 16 ks + 16) (the warpgroup wrote them in place over S).  The first four K steps
-                    // start as soon as the first half of P is written, the rest once the tile is complete.
-                    const uint32_t w_lo = wbase_lo + (uint32_t)s * stage_step;
-                    const uint32_t p_addr = tmem + 128u * buf;
-#pragma unroll
-                    for (int ks = 0; ks < 8; ++ks) {
-                        if (ks == 4) {
-                            ok = mbar_wait(&bars->s_done[buf][t], ph, abort_flag, p.status, 7);
-                            if (!ok) break;
-                            tc_fence_after();
-                        }
-                        const uint32_t off = (uint32_t)(((ks >> 2) * SM::kWHalf + (ks & 3) * 32) >> 4);
-                        const uint32_t a_hi = p_addr + 16 * ks;
-                        if (ks == 0 && group_start) mma_ts2<0>(y_addr, a_hi, w_lo + off, wdesc_hi, idesc_y);
-                        else mma_ts2<1>(y_addr, a_hi, w_lo + off, wdesc_hi, idesc_y);
-                        mma_ts2<1>(y_addr, a_hi + 8, w_lo + off, wdesc_hi, idesc_y);
-                        mma_ts2<1>(y_addr, a_hi, w_lo + kLoOff + off, wdesc_hi, idesc_y);
-                    }
-                    if (!ok) break;
-                    tc_commit(&bars->kw_done[buf][t]);
-                    if (group_end) { tc_commit(&bars->y_full[t]); ++n_grp; }
-                    tc_commit(&bars->empty[s]);
-                    buf += 2; if (buf >= (uint32_t)NBUF) buf -= NBUF;
-                    gr += 2; if (gr >= kRingPeriod) { gr -= kRingPeriod; ph ^= 1u; }
-                }
             }
         }
       }
@@ -420,7 +248,7 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
         const int wq = warp & 3;                       // TMEM lane quarter this warp may access
         const uint32_t lane_addr = (uint32_t)(wq * 32) << 16;
         const int row_in_tile = wq * 32 + lane;
-        uint32_t gn0 = 0, n_grp = 0;
+        uint32_t gn0 = 0;
         uint32_t ncol = 0;                             // symmetric row-sum mode: off-diagonal tiles this row tile has finished
         bool ok = true;
 
@@ -524,7 +352,7 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
                     // this thread's share of sum_ij K_ij^2: only the total over all threads is meaningful.  (A thread whose
                     // slot It * 128 + r lies beyond N has only seen streamed points J * 128 + r >= N, i.e. zeros.)
                     p.rowsq[row] = dsq * (1.0 / ((double)(1 << kBias) * (double)(1 << kBias)));
-            } else if (MODE == kModeRowsum) {
+            } else {
                 double dsum = 0.0, dsq = 0.0;
                 for (int j = 0; j < num_jt && ok; ++j) {
                     const uint32_t g = gn0 + 2u * j + t;
@@ -562,100 +390,6 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
                     const double l = (p.left ? (double)p.left[row] : 1.0) * (1.0 / (double)(1 << kBias));
                     p.q[row] = (float)(dsum * l);
                     if (p.rowsq) p.rowsq[row] = dsq * (1.0 / ((double)(1 << kBias) * (double)(1 << kBias)));
-                }
-            } else {
-                float acc[BT];
-#pragma unroll
-                for (int c = 0; c < BT; ++c) acc[c] = 0.f;
-                bool pending = false;
-                // Adds the finished TMEM accumulator of this row tile into the registers and hands it back.
-                // The tensor core adds each K step into the TMEM accumulator with round-toward-zero.  For a sum whose partial
-                // sums keep one sign, n additions lose n / 4 ulp of the result on average (half an ulp each, at a running
-                // magnitude that averages half the final one): measured 2.85e-8 per addition against 2^-25 = 2.98e-8.  The
-                // flush adds that expected loss back (one FMA instead of one add), which removes the common scale error of
-                // M V that would otherwise shift every eigenvalue by ~7e-7 per column tile in the group.
-                auto do_flush = [&](int tiles_in_group) -> bool {
-                    const float corr = 1.0f + (float)(tiles_in_group * 8 * 3) * 2.98023224e-8f;
-                    if (!mbar_wait(&bars->y_full[t], n_grp & 1, abort_flag, p.status, 10)) return false;
-                    ++n_grp;
-                    tc_fence_after();
-                    const uint32_t yaddr = tmem + lane_addr + kYCol + 64 * t;
-                    // all loads first, one wait (the S registers are free between tiles), and the accumulator is handed
-                    // back before the additions
-                    uint32_t v[BT / 16][16];
-#pragma unroll
-                    for (int c0 = 0; c0 < BT / 16; ++c0) tmem_ld16(yaddr + 16 * c0, v[c0]);
-                    tmem_wait_ld();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&bars->y_empty[t]);
-#pragma unroll
-                    for (int c0 = 0; c0 < BT / 16; ++c0)
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) acc[16 * c0 + i] = fmaf(__uint_as_float(v[c0][i]), corr, acc[16 * c0 + i]);
-                    return true;
-                };
-                int in_group = 0;
-                for (int j = 0; j < num_jt && ok; ++j) {
-                    const uint32_t g = gn0 + 2u * j + t;
-                    const int buf = g % NBUF;
-                    ok = mbar_wait(&bars->s_full[buf][t], (g / kRingPeriod) & 1, abort_flag, p.status, 9);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint32_t addr = tmem + lane_addr + 128u * buf;
-                    // whole S row into registers first (the four loads overlap), then exponentials and in-place stores
-                    uint32_t sv[4][32];
-#pragma unroll
-                    for (int qd = 0; qd < 4; ++qd) tmem_ld32(addr + 32 * qd, sv[qd]);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int ch = 0; ch < 8; ++ch) {
-                        uint32_t hi[8], lo[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const float p0 = ex2f(__uint_as_float(sv[ch >> 1][16 * (ch & 1) + 2 * i]));
-                            const float p1 = ex2f(__uint_as_float(sv[ch >> 1][16 * (ch & 1) + 2 * i + 1]));
-                            const float h0 = __uint_as_float(__float_as_uint(p0) & 0xFFFFE000u);
-                            const float h1 = __uint_as_float(__float_as_uint(p1) & 0xFFFFE000u);
-                            hi[i] = pack_f16x2(h0, h1);
-                            lo[i] = pack_f16x2(p0 - h0, p1 - h1);
-                        }
-                        tmem_st8(addr + 16 * ch, hi);
-                        tmem_st8(addr + 16 * ch + 8, lo);
-                        if (ch == 3) {
-                            tmem_wait_st();
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(&bars->p_half[buf][t]);
-                        }
-                    }
-                    tmem_wait_st();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&bars->s_done[buf][t]);
-                    // flush of the accumulator group that ended with the PREVIOUS tile of this row tile (its product
-                    // MMA has had a whole tile of time to finish); the last group of the work item is flushed at once
-                    if (pending) { ok = do_flush(flush); pending = false; if (!ok) break; }
-                    ++in_group;
-                    if (in_group == flush || j + 1 == num_jt) {
-                        if (j + 1 == num_jt) { ok = do_flush(in_group); if (!ok) break; }
-                        else pending = true;
-                        in_group = 0;
-                    }
-                }
-                if (ok && row < p.Nrow) {
-                    const float l = p.left ? p.left[row] : 1.0f;
-#pragma unroll
-                    for (int c = 0; c < BT; ++c)
-                        if (c < p.b) {
-                            float* o = p.Y + row + (int64_t)c * p.ldy;
-                            const float v = acc[c] * l * p.colscale_inv[c];
-                            if (kTail && tail_item) atomicAdd(o, v);   // the other half of the column range arrives from another CTA
-                            // later column chunks add to the partial result of the same thread; streaming loads and stores:
-                            // the partial results are touched once per chunk round and should not push the fp16 operands,
-                            // which every CTA re-reads, out of L2
-                            else __stcs(o, cch == 0 ? v : __ldcs(o) + v);
-                        }
                 }
             }
             gn0 += (uint32_t)tiles_per_item;
@@ -827,12 +561,12 @@ bool make_map_2d(CUtensorMap* m, void* base, uint64_t inner, uint64_t outer, uin
 }
 
 template <int BT, int MODE>
-fd_status launch_tc(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, const CUtensorMap& mh, const TcParams& p, int grid) {
+fd_status launch_tc(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, const TcParams& p, int grid) {
     const int smem = Smem<BT, MODE>::total(p.K16);
     if (smem > 227 * 1024) return fail(c, FD_ERR_UNSUPPORTED, "tensor-core kernel needs %d B of shared memory", smem);
     // the attribute is per device: set it on every launch (cheap) rather than remembering one device
     FD_CUDA(c, cudaFuncSetAttribute(k_tc<BT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-    k_tc<BT, MODE><<<grid, kThreads, smem, c->stream>>>(mr, mc, mh, p);
+    k_tc<BT, MODE><<<grid, kThreads, smem, c->stream>>>(mr, mc, p);
     FD_LAUNCH_CHECK(c, "k_tc");
     return FD_OK;
 }
@@ -899,7 +633,6 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
     p.num_chunks = (int)ceil_div(p.num_jt, p.jt_chunk);
     p.np_rows = NP; p.np_cols = NP; p.K16 = K16;
     p.left = a.left; p.status = status;
-    p.flush = c->opt_flush > 0 ? c->opt_flush : 1;
     const int grid = std::min(p.num_work, c->sm_count);
 
     if (rowsum && sym) {
@@ -914,28 +647,25 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
         p.sym_shift = 61 - kBias - lg;
         FD_CUDA(c, cudaMemsetAsync(p.symsum, 0, (size_t)N * 8, c->stream));
         const int sym_grid = std::min((p.num_work + 1) / 2, c->sm_count);
-        if (p.rowsq) FD_TRY((launch_tc<16, kModeRowsumSym>(c, mr, mc, mc, p, sym_grid)));
-        else FD_TRY((launch_tc<32, kModeRowsumSym>(c, mr, mc, mc, p, sym_grid)));
+        if (p.rowsq) FD_TRY((launch_tc<16, kModeRowsumSym>(c, mr, mc, p, sym_grid)));
+        else FD_TRY((launch_tc<32, kModeRowsumSym>(c, mr, mc, p, sym_grid)));
         k_sym_finish<<<(unsigned)ceil_div(N, 256), 256, 0, c->stream>>>(p.symsum, N, std::ldexp(1.0, -(kBias + (int)p.sym_shift)), a.Y);
         FD_LAUNCH_CHECK(c, "k_sym_finish");
     } else if (rowsum) {
         p.q = a.Y; p.rowsq = a.rowsq; p.b = 1;
-        if (p.rowsq) FD_TRY((launch_tc<16, kModeRowsum>(c, mr, mc, mc, p, grid)));
-        else FD_TRY((launch_tc<32, kModeRowsum>(c, mr, mc, mc, p, grid)));
+        if (p.rowsq) FD_TRY((launch_tc<16, kModeRowsum>(c, mr, mc, p, grid)));
+        else FD_TRY((launch_tc<32, kModeRowsum>(c, mr, mc, p, grid)));
     } else {
         __half* wt_hi = c->at<__half>(L.wt_hi);
-        __half* wt_lo = c->at<__half>(L.wt_lo);
         float* scale = c->at<float>(L.colscale);
         float* inv = scale + L.BP + 8;
         float* part = c->at<float>(L.part);
         const bool fast = a.prec == FD_PREC_FAST;
-        // widest column chunk whose stages fit in shared memory: 64 columns up to D = 28, 32 up to D = 44, 16 beyond (the
-        // fp32-grade kernel stages W_hi and W_lo; the reduced-precision kernel stages one of them and always fits 64)
-        const int limit = 227 * 1024;
-        const int cw = fast || Smem<64, kModeBlock>::total(K16) <= limit ? 64 : Smem<32, kModeBlock>::total(K16) <= limit ? 32 : 16;
+        // column chunks of at most 64, of about equal width (multiples of 16)
+        const int cw = fast ? 64 : (int)round_up(ceil_div(a.b, ceil_div(a.b, 64)), 16);
         for (int c0 = 0; c0 < a.b; c0 += cw) {
             const int bc = std::min(cw, a.b - c0);
-            const int BT = bc <= 16 ? 16 : bc <= 32 ? 32 : 64;
+            const int BT = bc <= 16 ? 16 : bc <= 32 ? 32 : bc <= 48 && !fast ? 48 : 64;
             if (BT > L.BP) return fail(c, FD_ERR_WORKSPACE, "column tile %d wider than the provisioned block buffers (%d)", BT, L.BP);
             const int cm_blocks = (int)std::min<int64_t>(256, ceil_div(N, 1024));
             k_colmax_partial<<<dim3(cm_blocks, bc), 256, 0, c->stream>>>(a.V, a.ldv, a.right, N, c0, bc, part);
@@ -943,12 +673,10 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
             k_colscale<<<1, 64, 0, c->stream>>>(part, cm_blocks, bc, BT, scale, inv);
             FD_LAUNCH_CHECK(c, "k_colscale");
             k_pack_wt<<<dim3((unsigned)std::min<int64_t>(1024, ceil_div(NP, 256)), BT), 256, 0, c->stream>>>(
-                a.V, a.ldv, a.right, N, NP, c0, bc, scale, wt_hi, fast ? nullptr : wt_lo);
+                a.V, a.ldv, a.right, N, NP, c0, bc, scale, wt_hi, fast ? nullptr : wt_hi + (size_t)BT * NP);
             FD_LAUNCH_CHECK(c, "k_pack_wt");
-            // one map over W_hi (rows 0 .. BT) and, in the fp32-grade mode, W_lo behind it (rows BP .. BP + BT of the same array)
-            if (wt_lo != wt_hi + (size_t)L.BP * NP) return fail(c, FD_ERR_INVALID, "W_hi and W_lo are not adjacent in the workspace");
-            p.lo_row = L.BP;
-            if (!make_map_2d(&mh, wt_hi, (uint64_t)NP, (uint64_t)(fast ? BT : L.BP + BT), (uint64_t)NP * 2, 64, BT, CU_TENSOR_MAP_SWIZZLE_128B))
+            // one map over W_hi (rows 0 .. BT) and, in the fp32-grade mode, W_lo behind it (rows BT .. 2 BT of the same array)
+            if (!make_map_2d(&mh, wt_hi, (uint64_t)NP, (uint64_t)(fast ? BT : 2 * BT), (uint64_t)NP * 2, 64, fast ? BT : 2 * BT, CU_TENSOR_MAP_SWIZZLE_128B))
                 return fail(c, FD_ERR_CUDA, "cuTensorMapEncodeTiled failed for the block operands");
             p.b = bc; p.colscale_inv = inv; p.Y = a.Y + (int64_t)c0 * a.ldy; p.ldy = a.ldy;
             if (fast) {
@@ -957,39 +685,14 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
                 pb.num_work = (int)ceil_div(a.Nrow, 128);
                 // the accumulator is flushed every 8 column tiles here: the round-toward-zero loss of the longer groups
                 // (a few 1e-6) is far below this mode's own error (3e-4), and the flushes cost 4 %
-                if (c->opt_flush <= 0) pb.flush = 8;
+                pb.flush = c->opt_flush > 0 ? c->opt_flush : 8;
                 FD_TRY(launch_fast_product(c, BT, mr, mc, mh, pb, std::min(pb.num_work, c->sm_count)));
                 continue;
             }
-            // Tail split: with a single column chunk (N up to about 2^17) the row pairs of the last, partly filled round --
-            // or all pairs when there are fewer than CTAs -- are each shared by two CTAs (half the column range each).
-            int bgrid = grid;
-            p.tail_split = 0;
-            if (p.num_chunks == 1 && p.num_jt >= 2 && c->opt_tail_split != 0) {
-                const int tail = p.num_work % grid;                  // pairs in the last round (grid = min(pairs, SMs))
-                const int tail_pairs = p.num_work < c->sm_count ? p.num_work : tail;
-                if (tail_pairs > 0 && 2 * tail_pairs <= c->sm_count) {
-                    p.tail_split = 2;
-                    p.tail_pairs = tail_pairs;
-                    p.tail_first = p.num_work - tail_pairs;
-                    bgrid = std::max(grid, 2 * tail_pairs);
-                    const int64_t r0t = (int64_t)p.tail_first * 256;
-                    FD_CUDA(c, cudaMemset2DAsync(p.Y + r0t, (size_t)p.ldy * 4, 0, (size_t)(a.Nrow - r0t) * 4, (size_t)bc, c->stream));
-                }
-            }
-            if (p.tail_split == 2) {
-                switch (BT) {
-                    case 16: FD_TRY((launch_tc<16, kModeBlockTail>(c, mr, mc, mh, p, bgrid))); break;
-                    case 32: FD_TRY((launch_tc<32, kModeBlockTail>(c, mr, mc, mh, p, bgrid))); break;
-                    default: FD_TRY((launch_tc<64, kModeBlockTail>(c, mr, mc, mh, p, bgrid))); break;
-                }
-                continue;
-            }
-            switch (BT) {
-                case 16: FD_TRY((launch_tc<16, kModeBlock>(c, mr, mc, mh, p, grid))); break;
-                case 32: FD_TRY((launch_tc<32, kModeBlock>(c, mr, mc, mh, p, grid))); break;
-                default: FD_TRY((launch_tc<64, kModeBlock>(c, mr, mc, mh, p, grid))); break;
-            }
+            // Accumulator flush: after two column tiles where the small terms have columns of their own (16 additions at the
+            // magnitude of the sum), after every tile where the three terms share them (24); see fd_tc_block.cu.
+            p.flush = c->opt_flush > 0 ? c->opt_flush : (BT <= 32 ? 2 : 1);
+            FD_TRY(launch_block_product(c, BT, mr, mc, mh, p));
         }
     }
     return FD_OK;

@@ -9,17 +9,15 @@ namespace fd {
 namespace tc {
 
 constexpr int kStages = 4;
-constexpr int kThreads = 384;                // warps 0-3 / 4-7: exponential warpgroups; warps 8-11: TMA, MMA, 2 idle
+constexpr int kThreads = 384;                // row-sum kernel: warps 0-3 / 4-7 exponential warpgroups; warps 8-11: TMA, 2 idle, MMA
 constexpr int kBias = 15;                    // P' = 2^15 P keeps fp16 hi/lo of P out of the denormal range
 constexpr uint32_t kTmemCols = 512;
 constexpr long long kWaitCycles = 4000000000ll;   // ~2 s: far beyond any legitimate wait
 
-// kModeRowsumSym: row sums of a SYMMETRIC weighted kernel matrix from its upper triangle of tiles alone (K = K^T, Sec.
-// 2.1): every off-diagonal tile also yields the column sums that the mirrored tile's rows would have computed.
-// kModeBlockTail: the block product with the tail split of TcParams (an instantiation of its own, so that the kernel of the
-// large, multi-chunk products carries none of its geometry).
-enum Mode { kModeBlock = 0, kModeBlockTail = 1, kModeRowsum = 2, kModeRowsumSym = 3 };
-__host__ __device__ constexpr bool is_rowsum(int mode) { return mode == kModeRowsum || mode == kModeRowsumSym; }
+// Row-sum kernel: kModeRowsum evaluates every tile of its rows; kModeRowsumSym the row sums of a SYMMETRIC weighted kernel matrix
+// from its upper triangle of tiles alone (K = K^T, Sec. 2.1): every off-diagonal tile also yields the column sums that
+// the mirrored tile's rows would have computed.
+enum Mode { kModeRowsum = 2, kModeRowsumSym = 3 };
 
 struct TcParams {
     int64_t Nrow, N;             // valid rows / columns
@@ -31,30 +29,17 @@ struct TcParams {
     int K16;
     int b;                       // real block columns to store
     int flush;                   // column tiles per accumulator flush
-    int lo_row;                  // block modes: first row of W_lo inside the W operand array (W_hi starts at row 0)
     const float* left;           // may be null
     const float* colscale_inv;   // per column: 2^-bias / colscale
-    // The parameter block keeps the size it had with the block and row-sum outputs alone (the block product's kernel
-    // measured 2.5 % more SM cycles with a larger one): the modes added later borrow the fields their mode does not use.
     union {
-        struct { float* Y; int64_t ldy; };                       // block modes: output block
+        struct { float* Y; int64_t ldy; };                       // block products: output block
         struct { unsigned long long* symsum; int64_t sym_shift; };   // symmetric row-sum mode: fixed-point row + column sums, one
                                                                  // 64-bit integer per point, in units of 2^-sym_shift of the
                                                                  // (2^bias-scaled) kernel values
     };
-    union {
-        struct { float* q; double* rowsq; };                     // row-sum modes: outputs
-        // Tail split (block mode with a single column chunk): the row pairs left over after the full rounds -- all of them
-        // when there are fewer pairs than CTAs -- are each served by TWO CTAs, one per half of the column range, whose
-        // partial results meet in Y by atomic addition (Y zeroed beforehand; a sum of two terms does not depend on order).
-        struct { int tail_split;                                 // 0 = off, 2 = on
-                 int tail_first;                                 // first row pair of the tail
-                 int tail_pairs;                                 // number of row pairs in the tail
-                 int tail_pad_; };
-    };
+    float* q; double* rowsq;     // row-sum modes: outputs
     unsigned int* status;
 };
-static_assert(sizeof(TcParams) == 120, "the kernels' parameter block has a measured size");
 
 // ------------------------------------------------------------------------------------------------ PTX
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -236,6 +221,9 @@ __host__ __device__ constexpr uint32_t idesc_f16(int n) {
 // Reduced-precision block product (fd_tc_fast.cu): one row tile per CTA, work items of 128 rows.
 fd_status launch_fast_product(fd_ctx* c, int BT, const CUtensorMap& mr, const CUtensorMap& mc, const CUtensorMap& mh,
                               const TcParams& p, int grid);
+// fp32-grade block product of BT = 16, 32, 48 or 64 columns (fd_tc_block.cu).
+fd_status launch_block_product(fd_ctx* c, int BT, const CUtensorMap& mr, const CUtensorMap& mc, const CUtensorMap& mw,
+                               const TcParams& tp);
 
 }  // namespace tc
 }  // namespace fd

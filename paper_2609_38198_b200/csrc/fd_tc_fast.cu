@@ -25,9 +25,7 @@
 // that the decreases do not cover would block for ever), and the host checks the compiled count before launching.
 // Every mbarrier wait is bounded; on expiry the CTA raises a status word, drains and exits.
 //
-// The fp32-grade product (fp16 hi + lo pieces of P and W, three MMA terms) stays on the two-row-tile kernel of
-// fd_tc.cu: with three times the tensor work per tile the GPU runs at its power limit, and sharing each staged column
-// tile between two row tiles costs less energy per pair than this layout (measured at N = 2^20: 537 ms against 582 ms).
+// (The fp32-grade product, with fp16 hi + lo pieces of P and W: fd_tc_block.cu.)
 #include <algorithm>
 
 #include "fd_tc_common.h"
