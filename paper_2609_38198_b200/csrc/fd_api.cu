@@ -64,6 +64,7 @@ Layout make_layout(int64_t N, int32_t D, int32_t b_max, int32_t m_max) {
     L.colscale = carve(cur, (size_t)(L.BP + 8) * 4 * 2);
     L.status = carve(cur, 256);
     L.symsum = carve(cur, (size_t)N * 8);
+    L.weights = carve(cur, (size_t)L.NP * 4);
     if (m_max > 0) {
         L.eig_q = carve(cur, (size_t)N * m_max * 4);
         L.eig_w = carve(cur, (size_t)N * m_max * 4);

@@ -30,6 +30,7 @@ struct Layout {
     size_t wp = 0, part = 0, part_floats = 0;
     size_t xp_col = 0, xp_row = 0, wt_hi = 0, wt_lo = 0, colscale = 0, status = 0;
     size_t yacc = 0;
+    size_t weights = 0;              // NP right weights of a Gram-form row sum
     size_t symsum = 0;               // N 64-bit fixed-point sums of the symmetric row-sum mode
     size_t eig_q = 0, eig_w = 0, eig_x = 0, eig_r = 0, eig_t = 0, eig_small = 0, eig_small_doubles = 0;
     size_t total = 0;
@@ -51,7 +52,10 @@ struct fd_ctx {
     // current operator state (set by fd_degree)
     bool have_s = false;
     double beta = 0.0, alpha = 0.0;
-    double packed_beta = -1.0;       // bandwidth the tensor-core column operand is packed for
+    // what the tensor-core operands hold: bandwidth of the unweighted column operand, of the unweighted row operand and its rows
+    // (-1: something else)
+    double packed_beta = -1.0, packed_row_beta = -1.0;
+    int64_t packed_row0 = 0, packed_rows = 0;
     // options
     int opt_path = FD_PATH_AUTO;
     int opt_splits = 0;

@@ -9,12 +9,9 @@
 //      two hi/lo pairs so it is exact to fp32.
 //   2. Two warpgroups (one per row tile; thread = row) read S from TMEM, take 2^S on the MUFU and add P (and P^2).
 // S tiles flow through a ring of TMEM buffers shared by both row tiles, so the tensor core runs ahead of the warpgroups.
-// Row-sum mode (rectangular and row-sharded passes): the warpgroups add P (and P^2) on the FMA pipe,
-// fp32 within a column tile and fp64 across tiles; a positive right vector enters through e_j.
-// Symmetric row-sum mode (the degree passes of a whole data set, K = K^T): only the tiles on or above the diagonal are
-// evaluated; the S tile is built with the streamed points on the TMEM lanes, so one thread adds up both what a tile gives
-// its streamed point (one fixed-point atomic per tile) and, in 128 per-thread accumulators reduced across lanes every
-// 64 tiles, what it gives the resident points.
+// Rectangular and row-sharded passes: the warpgroups add P (and P^2) on the FMA pipe,
+// fp32 within a column tile and fp64 across tiles; a right vector multiplies P.
+// (The degree passes of a whole data set use K = K^T: fd_tc_sym.cu.)
 //
 // One persistent CTA per SM: warps 0-3 / 4-7 = the two exponential warpgroups (raised to 232 registers); warp 8 = TMA producer,
 // warp 11 = Gram-MMA issuer (lowered to 40 registers).  Column tiles are staged by TMA (every CTA loads its own copy) through
@@ -33,14 +30,11 @@ namespace {
 using namespace tc;
 
 // ------------------------------------------------------------------------------------------------ shared memory map
-template <int BT, int MODE>
 struct Smem {
     static constexpr int kXChunk = 128 * 64;                       // one K slab (hi|lo) of 128 points: 8 KB
-    // symmetric row-sum mode: per-warp column partial sums, [row tile][parity][warp quarter][128 columns] floats
-    static constexpr int kColPartBytes = (MODE == kModeRowsumSym) ? 2 * 2 * 4 * 128 * 4 + 64 : 0;   // + four mbarriers (col_ready[row tile][parity])
     static __host__ __device__ constexpr int stage_bytes(int K16) { return K16 * kXChunk; }
     static __host__ __device__ constexpr int total(int K16) {
-        return 1024 /*align slack*/ + kStages * stage_bytes(K16) + 2 * K16 * kXChunk + 1024 /*barriers*/ + kColPartBytes;
+        return 1024 /*align slack*/ + kStages * stage_bytes(K16) + 2 * K16 * kXChunk + 1024 /*barriers*/;
     }
 };
 
@@ -60,39 +54,16 @@ struct Barriers {
 };
 
 // ------------------------------------------------------------------------------------------------ work items
-// Work item w of a CTA -> (row pair, first column tile, number of column tiles, column chunk).
-//   row-sum mode: (column chunk c, row pair r) with c outermost, r = blockIdx.x + k * gridDim.x;
-//   symmetric row-sum mode: only tiles on or above the diagonal.  Row pair r needs column tiles 2 r .. num_jt - 1; pairing r
-//     with num_work - 1 - r gives work units of equal length (num_jt + 2 tiles): unit u = blockIdx.x + k * gridDim.x is the
-//     two items {u, num_work - 1 - u} (the middle pair of an odd count stands alone: its second item is empty).
-struct ItemGeometry { int item, j0, num_jt, cch; };
-
-template <int MODE>
-__device__ __forceinline__ ItemGeometry item_geometry(const TcParams& p, int w, int my_rows) {
-    ItemGeometry g;
-    if constexpr (MODE == kModeRowsumSym) {
-        const int unit = (int)blockIdx.x + (w >> 1) * (int)gridDim.x;
-        g.cch = 0;
-        g.item = (w & 1) ? p.num_work - 1 - unit : unit;
-        g.j0 = 2 * g.item;
-        g.num_jt = ((w & 1) && g.item == unit) ? 0 : p.num_jt - g.j0;
-    } else {
-        g.cch = w / my_rows;
-        g.item = (int)blockIdx.x + (w % my_rows) * (int)gridDim.x;
-        g.j0 = g.cch * p.jt_chunk;
-        g.num_jt = (p.num_jt - g.j0 < p.jt_chunk) ? p.num_jt - g.j0 : p.jt_chunk;
-    }
-    return g;
-}
+// Work item w of a CTA: row pair blockIdx.x + w * gridDim.x, all column tiles.
 
 // ------------------------------------------------------------------------------------------------ the kernel
 // Tiles of one work item are numbered n = 2 j + t (column tile j, row tile t) and flow through a ring of four S buffers in
-// TMEM, so the tensor core runs up to four tiles ahead of the warpgroups.  BT = 16: with the sum of squares, 32: without.
-template <int BT, int MODE>
+// TMEM, so the tensor core runs up to four tiles ahead of the warpgroups.  BT = 16: with the sum of squares, 32: with weights.
+template <int BT>
 __global__ void __launch_bounds__(kThreads, 1)
 k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUtensorMap map_xcol, const TcParams p) {
     extern __shared__ uint8_t smem_raw[];
-    using SM = Smem<BT, MODE>;
+    using SM = Smem;
     constexpr int NBUF = 4;
     constexpr uint32_t kRingPeriod = NBUF;             // tiles between two uses of a buffer by the same row tile
     const int K16 = p.K16;
@@ -111,10 +82,6 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
             for (int t = 0; t < 2; ++t) {
                 mbar_init(&bars->s_full[u][t], 1); mbar_init(&bars->s_done[u][t], 4);
             }
-        if constexpr (MODE == kModeRowsumSym) {
-            uint64_t* col_ready = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(bars) + 1024 + 2 * 2 * 4 * 128 * 4);
-            for (int u = 0; u < 4; ++u) mbar_init(&col_ready[u], 4);          // the four warps' column partials of a tile are written
-        }
         bars->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -128,22 +95,8 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
     const uint32_t tmem = bars->tmem_base;
     const long long t_begin = clock64();
 
-    // Work items of this CTA: (column chunk c, row-pair tile r) with c outermost, r = blockIdx.x + k * gridDim.x.  Every CTA
-    // sweeps chunk c for all of its rows before chunk c + 1, so the whole grid reads the same L2-sized slice of the
-    // column operands at about the same time; a row's partial results always come from the same threads, in order.
-    // (item_geometry above has the other modes' orders.)
-    constexpr bool kSym = MODE == kModeRowsumSym;
-    const int my_rows = kSym ? ((p.num_work + 1) / 2 - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x
-                             : (p.num_work - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-    const int my_items = kSym ? 2 * my_rows : my_rows * p.num_chunks;
-#define FD_ITEM_GEOMETRY(w)                                                                         \
-    const ItemGeometry geo_ = item_geometry<MODE>(p, (w), my_rows);                                 \
-    const int cch = geo_.cch;                                                                       \
-    const int item = geo_.item;                                                                     \
-    const int j0 = geo_.j0;                                                                         \
-    const int num_jt = geo_.num_jt;                                                                 \
-    const int tiles_per_item = 2 * num_jt;                                                          \
-    (void)item; (void)tiles_per_item; (void)cch; (void)j0
+    const int num_jt = p.num_jt, tiles_per_item = 2 * num_jt;
+    const int my_items = (p.num_work - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
 
     if (warp >= 8) {
       asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(40));
@@ -154,7 +107,7 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
             uint32_t it = 0;
             bool ok = true;
             for (int w = 0; w < my_items && ok; ++w) {
-                FD_ITEM_GEOMETRY(w);
+                const int item = (int)blockIdx.x + w * (int)gridDim.x;
                 ok = mbar_wait(&bars->xempty, (w & 1) ^ 1, abort_flag, p.status, 1);
                 if (!ok) break;
                 mbar_expect_tx(&bars->xfull, 2 * K16 * SM::kXChunk);
@@ -169,7 +122,7 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
                     uint8_t* st = stage_base + s * SM::stage_bytes(K16);
                     mbar_expect_tx(&bars->full[s], SM::stage_bytes(K16));
                     for (int c = 0; c < K16; ++c)
-                        tma_load_2d(st + c * SM::kXChunk, &map_xcol, 0, (int)(c * p.np_cols + (int64_t)(j0 + j) * 128), &bars->full[s]);
+                        tma_load_2d(st + c * SM::kXChunk, &map_xcol, 0, (int)(c * p.np_cols + (int64_t)j * 128), &bars->full[s]);
                 }
             }
             if (!ok) {
@@ -192,7 +145,6 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
             uint32_t it0 = 0, gn0 = 0;
             bool ok = true;
             for (int w = 0; w < my_items && ok; ++w) {
-                FD_ITEM_GEOMETRY(w);
                 ok = mbar_wait(&bars->xfull, w & 1, abort_flag, p.status, 3);
                 if (!ok) break;
                 tc_fence_after();
@@ -218,18 +170,15 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
                     const uint32_t s_addr = tmem + 128u * buf;
                     const int t = n & 1;
                     uint8_t* st = stage_base + s * SM::stage_bytes(K16);
-                    // (symmetric mode: the streamed tile is the M operand, so TMEM lanes = streamed points)
                     for (int c = 0; c < K16; ++c) {
                         uint64_t a = smem_desc(smem_u32(xi_base + (t * K16 + c) * SM::kXChunk), 512, 4);
                         uint64_t b = smem_desc(smem_u32(st + c * SM::kXChunk), 512, 4);
-                        if (MODE == kModeRowsumSym) { const uint64_t x = a; a = b; b = x; }
                         mma_ss(s_addr, a, b + 2, idesc_g, c > 0);          // + 2: the lo half starts 32 B into the row
                         mma_ss(s_addr, a + 2, b, idesc_g, 1);
                     }
                     for (int c = 0; c < K16; ++c) {
                         uint64_t a = smem_desc(smem_u32(xi_base + (t * K16 + c) * SM::kXChunk), 512, 4);
                         uint64_t b = smem_desc(smem_u32(st + c * SM::kXChunk), 512, 4);
-                        if (MODE == kModeRowsumSym) { const uint64_t x = a; a = b; b = x; }
                         mma_ss(s_addr, a, b, idesc_g, 1);
                     }
                     tc_commit(&bars->s_full[buf][n & 1]);
@@ -249,110 +198,12 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
         const uint32_t lane_addr = (uint32_t)(wq * 32) << 16;
         const int row_in_tile = wq * 32 + lane;
         uint32_t gn0 = 0;
-        uint32_t ncol = 0;                             // symmetric row-sum mode: off-diagonal tiles this row tile has finished
         bool ok = true;
 
         for (int w = 0; w < my_items && ok; ++w) {
-            FD_ITEM_GEOMETRY(w);
+            const int item = (int)blockIdx.x + w * (int)gridDim.x;
             const int64_t row = (int64_t)item * 256 + t * 128 + row_in_tile;
-            if constexpr (MODE == kModeRowsumSym) {
-                // Symmetric half-work row sums.  The S tile is built the other way round here (lanes = points of the
-                // STREAMED tile J, columns = points of the CTA's resident tile It), so a thread owns one streamed point:
-                //   * its sum over the 128 columns is that point's share of tile (J, It): one fixed-point atomic per tile;
-                //   * acc[c] += P[., c] collects, over the whole sweep, the resident point c's sum over the streamed
-                //     points that fall on this lane; the 128 lanes are reduced (butterfly of shuffles, the four warps
-                //     through shared memory) only every kSymFlush tiles, which also bounds the fp32 accumulation length.
-                // J < It is the mirror of a tile another resident tile evaluates (skipped: only J = 2 item for the second
-                // resident tile); J == It counts once (resident side only); J > It counts for both sides.  Sums go to one
-                // 64-bit fixed-point integer per point: integer additions commute, so the result does not depend on the
-                // order in which CTAs arrive.
-                constexpr int kSymFlush = 64;
-                constexpr bool kWantSq = BT == 16;             // the sum of squares rides along in the first degree pass only (BT = 32: without)
-                float* colpart = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 1024);
-                uint64_t* col_ready = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(bars) + 1024 + 2 * 2 * 4 * 128 * 4);
-                const double fix = (double)(1ull << p.sym_shift);
-                const int It = 2 * item + t;
-                float acc[128];
-#pragma unroll
-                for (int c = 0; c < 128; ++c) acc[c] = 0.f;
-                double dsq = 0.0;
-                int pending = 0;                               // tiles accumulated in acc since the last reduction
-                // reduces acc over the 128 lanes of the resident tile and adds the sums to the resident points
-                auto reduce_acc = [&]() -> bool {
-                    const uint32_t slot = ncol & 1u;
-                    float* mine = colpart + (((t * 2 + (int)slot) * 4 + wq) * 128);
-#pragma unroll
-                    for (int ch = 0; ch < 4; ++ch) {
-#pragma unroll
-                        for (int m = 16; m >= 1; m >>= 1) {
-                            const bool up = (lane & m) != 0;
-#pragma unroll
-                            for (int k = 0; k < m; ++k) {
-                                const float send = up ? acc[32 * ch + k] : acc[32 * ch + k + m];
-                                const float keep = up ? acc[32 * ch + k + m] : acc[32 * ch + k];
-                                acc[32 * ch + k] = keep + __shfl_xor_sync(0xffffffffu, send, m);
-                            }
-                        }
-                        mine[ch * 32 + lane] = acc[32 * ch];
-                    }
-#pragma unroll
-                    for (int c = 0; c < 128; ++c) acc[c] = 0.f;
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&col_ready[t * 2 + slot]);
-                    if (!mbar_wait(&col_ready[t * 2 + slot], (ncol >> 1) & 1u, abort_flag, p.status, 11)) return false;
-                    const float* all = colpart + ((t * 2 + (int)slot) * 4) * 128;
-                    const int cidx = wq * 32 + lane;
-                    const float csum = (all[cidx] + all[128 + cidx]) + (all[256 + cidx] + all[384 + cidx]);
-                    const int64_t pt = (int64_t)It * 128 + cidx;
-                    if (pt < p.N) atomicAdd(p.symsum + pt, (unsigned long long)__double2ll_rn((double)csum * fix));
-                    ++ncol;
-                    return true;
-                };
-                for (int j = 0; j < num_jt && ok; ++j) {
-                    const uint32_t g = gn0 + 2u * j + t;
-                    const int buf = g % NBUF;
-                    ok = mbar_wait(&bars->s_full[buf][t], (g / kRingPeriod) & 1, abort_flag, p.status, 8);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint32_t addr = tmem + lane_addr + 128u * buf;
-                    const int J = j0 + j;
-                    const bool use = J >= It;
-                    float r0 = 0.f, r1 = 0.f, q0 = 0.f, q1 = 0.f;
-                    uint32_t sv[2][32];
-                    tmem_ld32(addr, sv[0]);
-#pragma unroll
-                    for (int ch = 0; ch < 4; ++ch) {
-                        tmem_wait_ld();
-                        if (ch < 3) tmem_ld32(addr + 32 * (ch + 1), sv[(ch + 1) & 1]);
-                        if (use) {
-#pragma unroll
-                            for (int i = 0; i < 32; i += 2) {
-                                const float p0 = ex2f(__uint_as_float(sv[ch & 1][i])), p1 = ex2f(__uint_as_float(sv[ch & 1][i + 1]));
-                                acc[32 * ch + i] += p0; acc[32 * ch + i + 1] += p1;
-                                r0 += p0; r1 += p1;
-                                if (kWantSq) { q0 = fmaf(p0, p0, q0); q1 = fmaf(p1, p1, q1); }
-                            }
-                        }
-                    }
-                    // the buffer can be refilled: its values are in registers or consumed
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&bars->s_done[buf][t]);
-                    if (!use) continue;                            // mirrored tile: evaluated by the other resident tile
-                    const bool offdiag = J > It;
-                    dsq += (double)(q0 + q1) * (offdiag ? 2.0 : 1.0);
-                    if (offdiag) {
-                        const int64_t pt = (int64_t)J * 128 + row_in_tile;
-                        if (pt < p.N) atomicAdd(p.symsum + pt, (unsigned long long)__double2ll_rn((double)(r0 + r1) * fix));
-                    }
-                    if (++pending == kSymFlush) { ok = reduce_acc(); pending = 0; if (!ok) break; }
-                }
-                if (ok && pending > 0) ok = reduce_acc();
-                if (ok && num_jt > 0 && row < p.Nrow && p.rowsq)
-                    // this thread's share of sum_ij K_ij^2: only the total over all threads is meaningful.  (A thread whose
-                    // slot It * 128 + r lies beyond N has only seen streamed points J * 128 + r >= N, i.e. zeros.)
-                    p.rowsq[row] = dsq * (1.0 / ((double)(1 << kBias) * (double)(1 << kBias)));
-            } else {
+            {
                 double dsum = 0.0, dsq = 0.0;
                 for (int j = 0; j < num_jt && ok; ++j) {
                     const uint32_t g = gn0 + 2u * j + t;
@@ -361,6 +212,7 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t addr = tmem + lane_addr + 128u * buf;
+                    const float4* wcol = reinterpret_cast<const float4*>(p.weights) + (int64_t)j * 32;
                     float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f, q0 = 0.f, q1 = 0.f;
                     uint32_t sv[4][32];
 #pragma unroll
@@ -376,8 +228,11 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
                         for (int i = 0; i < 32; i += 4) {
                             const float p0 = ex2f(__uint_as_float(sv[ch][i])), p1 = ex2f(__uint_as_float(sv[ch][i + 1]));
                             const float p2 = ex2f(__uint_as_float(sv[ch][i + 2])), p3 = ex2f(__uint_as_float(sv[ch][i + 3]));
-                            a0 += p0; a1 += p1; a2 += p2; a3 += p3;
-                            if (BT == 16) {                // (BT = 32: the instantiation without the sum of squares)
+                            if (BT == 32) {                // weights instead of the sum of squares (broadcast reads)
+                                const float4 w4 = __ldg(wcol + 8 * ch + i / 4);
+                                a0 = fmaf(p0, w4.x, a0); a1 = fmaf(p1, w4.y, a1); a2 = fmaf(p2, w4.z, a2); a3 = fmaf(p3, w4.w, a3);
+                            } else {
+                                a0 += p0; a1 += p1; a2 += p2; a3 += p3;
                                 q0 = fmaf(p0, p0, q0); q1 = fmaf(p1, p1, q1); q0 = fmaf(p2, p2, q0); q1 = fmaf(p3, p3, q1);
                             }
                         }
@@ -387,9 +242,9 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
                 }
                 if (ok && row < p.Nrow) {
                     // undo the 2^bias scaling of P (exact powers of two)
-                    const double l = (p.left ? (double)p.left[row] : 1.0) * (1.0 / (double)(1 << kBias));
-                    p.q[row] = (float)(dsum * l);
-                    if (p.rowsq) p.rowsq[row] = dsq * (1.0 / ((double)(1 << kBias) * (double)(1 << kBias)));
+                    constexpr double scale = 1.0 / (double)(1 << kBias);
+                    p.q[row] = (float)(p.left ? dsum * (scale * (double)p.left[row]) : dsum * scale);
+                    if (p.rowsq) p.rowsq[row] = dsq * (scale * scale);
                 }
             }
             gn0 += (uint32_t)tiles_per_item;
@@ -419,114 +274,133 @@ __global__ void k_wait_selftest(unsigned int* status, long long limit_cycles) {
 
 // ------------------------------------------------------------------------------------------------ operand packing
 // Augmented fp16 hi|lo operand rows.  role 0 (rows of the product): [c x, e, 1]; role 1 (columns): [c x, 1, e] with
-// c = sqrt(2 b'), e = -b' |x - mu|^2 (+ the bias for role 1, + log2 of a positive weight vector when one is given).
+// c = sqrt(2 b'), e = -b' |x - mu|^2 (+ the bias for role 1).
 // Layout: slab s (16 augmented columns) of point p at out[(s * np + p) * 32 ..]: 16 hi then 16 lo halves.
-__global__ void k_pack_points(const float* __restrict__ xs, int DP, int D, int64_t n, int64_t np, const double* __restrict__ mu,
-                              double bprime, int role, double bias, const float* __restrict__ logw_src, int K16,
-                              __half* __restrict__ out) {
-    int64_t pidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Where as many slabs of 12 coordinates suffice (slab_norms), every slab carries the norm of its own coordinates in its last
+// four columns: the partial sum over the slabs is then -b' |difference|^2 of the coordinates so far (plus bias), never larger than the
+// final exponent, instead of a dot product of the size of the norms that the last slab takes back.  The tensor core
+// rounds each MMA at the magnitude of its sum, so this removes most of the exponent's error for far-out points (R^30, exponents
+// up to 60: worst eigenvalue error of 33 pairs 9.7e-7 -> 6.6e-7).  Else coordinates first, the four norm columns after the last one.
+// One thread per (point, slab, role): the 64 bytes it writes are contiguous.
+struct PackRole { const float* xs; __half* out; int64_t n; };   // n: valid points of this role
+__global__ void __launch_bounds__(256)
+k_pack_points(const PackRole rows, const PackRole cols, int first_role, int DP, int D, int64_t np, const double* __restrict__ mu, double bprime,
+              double cs, int slab_norms) {
+    const int64_t pidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (pidx >= np) return;
-    const bool valid = pidx < n;
-    const double cs = sqrt(2.0 * bprime);
-    double r = 0.0;
-    if (valid)
-        for (int k = 0; k < D; ++k) { double v = (double)xs[pidx * DP + k] - mu[k]; r += v * v; }
-    double e = -bprime * r;
-    if (logw_src && valid) e += log2((double)logw_src[pidx]);     // a positive weight rides in the exponent
-    if (role == 1) e += bias;
-    if (!valid) e = -30000.0;                           // padded point: 2^e = 0 (its row / column contributes nothing)
-    // norm pieces: two hi/lo pairs carry e to beyond fp32 precision
-    const __half e_h1 = __double2half(e);
-    const double r1 = e - (double)__half2float(e_h1);
-    const __half e_l1 = __double2half(r1);
-    const double r2 = r1 - (double)__half2float(e_l1);
-    const __half e_h2 = __double2half(r2);
-    const __half e_l2 = __double2half(r2 - (double)__half2float(e_h2));
-    const __half one = __float2half(1.0f), zero = __float2half(0.0f);
-    for (int s = 0; s < K16; ++s) {
-        __half* o = out + ((int64_t)s * np + pidx) * 32;
-        for (int kk = 0; kk < 16; ++kk) {
-            const int col = s * 16 + kk;
-            __half h = zero, l = zero;
-            if (col < D) {
-                if (valid) {
-                    const double v = cs * ((double)xs[pidx * DP + col] - mu[col]);
-                    h = __double2half(v);
-                    l = __double2half(v - (double)__half2float(h));
-                }
-            } else if (col == D || col == D + 1) {          // row-norm slots: role 0 carries e, role 1 carries 1
-                if (role == 0) { h = col == D ? e_h1 : e_h2; l = col == D ? e_l1 : e_l2; }
-                else h = one;
-            } else if (col == D + 2 || col == D + 3) {      // column-norm slots
-                if (role == 1) { h = col == D + 2 ? e_h1 : e_h2; l = col == D + 2 ? e_l1 : e_l2; }
-                else h = one;
-            }
-            o[kk] = h;
-            o[16 + kk] = l;
+    const int s = blockIdx.y, role = first_role + (int)blockIdx.z;
+    const PackRole pr = role == 0 ? rows : cols;
+    const bool valid = pidx < pr.n;
+    const float* x = pr.xs + pidx * DP;
+    const int c0 = slab_norms ? 12 * s : 16 * s;                  // first coordinate of this slab
+    const int norm0 = slab_norms ? 12 : D - c0;                   // first norm column inside the slab (may lie outside it)
+    __half hi[16], lo[16];
+    double r = 0.0;                                               // norm of this slab's coordinates
+#pragma unroll
+    for (int kk = 0; kk < 16; ++kk) {
+        hi[kk] = lo[kk] = __float2half(0.0f);
+        if (valid && c0 + kk < D && kk < norm0) {
+            const double d = (double)x[c0 + kk] - mu[c0 + kk], v = cs * d;
+            r += d * d;
+            hi[kk] = __double2half(v);
+            lo[kk] = __double2half(v - (double)__half2float(hi[kk]));
         }
+    }
+    if (norm0 < 16 && norm0 > -4) {
+        if (!slab_norms) {
+            r = 0.0;
+            if (valid)
+                for (int k = 0; k < D; ++k) { const double d = (double)x[k] - mu[k]; r += d * d; }
+        }
+        double e = -bprime * r;
+        if (role == 1 && (s == 0 || !slab_norms)) e += (double)kBias;
+        if (!valid && (s == 0 || !slab_norms)) e = -30000.0;      // padded point: 2^e = 0 (its row / column contributes nothing)
+        // norm pieces: two hi/lo pairs carry e to beyond fp32 precision
+        const __half e_h1 = __double2half(e);
+        const double r1 = e - (double)__half2float(e_h1);
+        const __half e_l1 = __double2half(r1);
+        const double r2 = r1 - (double)__half2float(e_l1);
+        const __half e_h2 = __double2half(r2);
+        const __half e_l2 = __double2half(r2 - (double)__half2float(e_h2));
+#pragma unroll
+        for (int kk = 0; kk < 16; ++kk) {
+            const int q = kk - norm0;                             // 0, 1: row-norm columns (role 0 carries e, role 1 carries 1); 2, 3: column-norm
+            if (q < 0 || q > 3) continue;
+            if ((q >> 1) == role) { hi[kk] = (q & 1) ? e_h2 : e_h1; lo[kk] = (q & 1) ? e_l2 : e_l1; }
+            else { hi[kk] = __float2half(1.0f); lo[kk] = __float2half(0.0f); }
+        }
+    }
+    uint4* o = reinterpret_cast<uint4*>(pr.out + ((int64_t)s * np + pidx) * 32);
+    auto two = [](__half a, __half b) { return (uint32_t)__half_as_ushort(a) | ((uint32_t)__half_as_ushort(b) << 16); };
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        o[q] = make_uint4(two(hi[8 * q], hi[8 * q + 1]), two(hi[8 * q + 2], hi[8 * q + 3]), two(hi[8 * q + 4], hi[8 * q + 5]), two(hi[8 * q + 6], hi[8 * q + 7]));
+        o[2 + q] = make_uint4(two(lo[8 * q], lo[8 * q + 1]), two(lo[8 * q + 2], lo[8 * q + 3]), two(lo[8 * q + 4], lo[8 * q + 5]), two(lo[8 * q + 6], lo[8 * q + 7]));
     }
 }
 
-// Stage 1: per-block maxima of |right_j V_jc| for each column c.
-__global__ void k_colmax_partial(const float* __restrict__ V, int64_t ldv, const float* __restrict__ right, int64_t N, int c0,
-                                 int bc, float* __restrict__ part) {
-    __shared__ float sm[256];
-    const int c = blockIdx.y;
-    float m = 0.f;
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < N; j += (int64_t)gridDim.x * blockDim.x) {
-        float v = V[j + (int64_t)(c0 + c) * ldv];
-        if (right) v *= right[j];
-        m = fmaxf(m, fabsf(v));
-    }
-    sm[threadIdx.x] = m;
-    __syncthreads();
-    for (int off = 128; off > 0; off >>= 1) {
-        if (threadIdx.x < off) sm[threadIdx.x] = fmaxf(sm[threadIdx.x], sm[threadIdx.x + off]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) part[(size_t)c * gridDim.x + blockIdx.x] = sm[0];
-    (void)bc;
+// out[j] = w[j] (1 without w) for j < n, 0 up to np: the weights of a row sum, padded to whole column tiles.
+__global__ void k_pad_weights(const float* __restrict__ w, int64_t n, int64_t np, float* __restrict__ out) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < np) out[j] = j < n ? (w ? w[j] : 1.f) : 0.f;
 }
-// Stage 2: column scale = power of two that puts the column maximum in [2^12, 2^13); stores the scale and the
-// epilogue factor 2^-bias / scale.
-__global__ void k_colscale(const float* __restrict__ part, int blocks, int bc, int BT, float* __restrict__ scale,
-                           float* __restrict__ inv) {
-    const int c = threadIdx.x;
-    if (c >= BT) return;
+
+// Per-block maxima of |right_j V_jc| for each column c.
+__global__ void __launch_bounds__(256)
+k_colmax_partial(const float* __restrict__ V, int64_t ldv, const float* __restrict__ right, int64_t N, int c0, float* __restrict__ part) {
+    __shared__ float sm[8];
+    const float* v = V + (int64_t)(c0 + blockIdx.y) * ldv;
     float m = 0.f;
-    if (c < bc)
-        for (int b = 0; b < blocks; ++b) m = fmaxf(m, part[(size_t)c * blocks + b]);
+    for (int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x; j < N; j += (int64_t)gridDim.x * 256) m = fmaxf(m, fabsf(right ? v[j] * right[j] : v[j]));
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        m = sm[threadIdx.x];
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffu, m, off));
+        if (threadIdx.x == 0) part[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = m;
+    }
+}
+// wt [c * np + j] = fp16 hi piece of scale_c * right_j * V[j, c0 + c], and the lo piece BT rows below when `with_lo`; zero padding for
+// j >= N and c >= bc.  scale_c = the power of two that puts the column maximum in [2^12, 2^13): every block reduces the
+// partial maxima of its column itself (they are at most 256 values); the first one stores the epilogue factor 2^-bias / scale.
+__global__ void __launch_bounds__(256)
+k_pack_wt(const float* __restrict__ V, int64_t ldv, const float* __restrict__ right, int64_t N, int64_t np, int c0, int bc,
+          const float* __restrict__ part, int parts, float* __restrict__ inv, __half* __restrict__ wt, int with_lo) {
+    __shared__ float sm[8];
+    const int c = blockIdx.y;
+    float m = c < bc && (int)threadIdx.x < parts ? part[(size_t)c * parts + threadIdx.x] : 0.f;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
+    __syncthreads();
+    m = sm[0];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) m = fmaxf(m, sm[w]);
     float sc = 1.0f;
     if (m > 0.f && isfinite(m)) {
         int e;
         frexpf(m, &e);                               // m = f * 2^e, f in [0.5, 1)
         sc = ldexpf(1.0f, 13 - e);
     }
-    scale[c] = sc;
-    inv[c] = ldexpf(1.0f, -kBias) / sc;
-}
-// wt_hi / wt_lo [c * np + j] = fp16 split of scale_c * right_j * V[j, c0 + c]; zero padding for j >= N and c >= bc.
-__global__ void k_pack_wt(const float* __restrict__ V, int64_t ldv, const float* __restrict__ right, int64_t N, int64_t np,
-                          int c0, int bc, const float* __restrict__ scale, __half* __restrict__ hi, __half* __restrict__ lo) {
-    const int c = blockIdx.y;
-    const float sc = scale[c];
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < np; j += (int64_t)gridDim.x * blockDim.x) {
-        float v = 0.f;
-        if (c < bc && j < N) {
-            v = V[j + (int64_t)(c0 + c) * ldv];
-            if (right) v *= right[j];
-            v *= sc;
+    if (blockIdx.x == 0 && threadIdx.x == 0) inv[c] = ldexpf(1.0f, -kBias) / sc;
+    const float* v = V + (int64_t)(c0 + (c < bc ? c : 0)) * ldv;
+    __half2* hi = reinterpret_cast<__half2*>(wt + (int64_t)c * np);
+    __half2* lo = reinterpret_cast<__half2*>(wt + (int64_t)(gridDim.y + c) * np);
+    for (int64_t j2 = (int64_t)blockIdx.x * 256 + threadIdx.x; j2 < np / 2; j2 += (int64_t)gridDim.x * 256) {
+        float x[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int64_t j = 2 * j2 + u;
+            x[u] = 0.f;
+            if (c < bc && j < N) x[u] = (right ? v[j] * right[j] : v[j]) * sc;
         }
-        const __half h = __float2half_rn(v);
-        hi[(int64_t)c * np + j] = h;
-        if (lo) lo[(int64_t)c * np + j] = __float2half_rn(v - __half2float(h));
+        const __half2 h = __floats2half2_rn(x[0], x[1]);
+        hi[j2] = h;
+        if (with_lo) lo[j2] = __floats2half2_rn(x[0] - __low2float(h), x[1] - __high2float(h));
     }
-}
-
-// Symmetric row-sum mode: fixed-point sums -> q.
-__global__ void k_sym_finish(const unsigned long long* __restrict__ sums, int64_t n, double scale, float* __restrict__ q) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) q[i] = (float)((double)(long long)sums[i] * scale);
 }
 
 // ------------------------------------------------------------------------------------------------ host side
@@ -560,13 +434,13 @@ bool make_map_2d(CUtensorMap* m, void* base, uint64_t inner, uint64_t outer, uin
               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BT, int MODE>
+template <int BT>
 fd_status launch_tc(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, const TcParams& p, int grid) {
-    const int smem = Smem<BT, MODE>::total(p.K16);
+    const int smem = Smem::total(p.K16);
     if (smem > 227 * 1024) return fail(c, FD_ERR_UNSUPPORTED, "tensor-core kernel needs %d B of shared memory", smem);
     // the attribute is per device: set it on every launch (cheap) rather than remembering one device
-    FD_CUDA(c, cudaFuncSetAttribute(k_tc<BT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-    k_tc<BT, MODE><<<grid, kThreads, smem, c->stream>>>(mr, mc, p);
+    FD_CUDA(c, cudaFuncSetAttribute(k_tc<BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    k_tc<BT><<<grid, kThreads, smem, c->stream>>>(mr, mc, p);
     FD_LAUNCH_CHECK(c, "k_tc");
     return FD_OK;
 }
@@ -588,7 +462,7 @@ bool tc_supported(const fd_ctx* c, const ApplyArgs& a) {
     // exponent magnitude the fp16 hi/lo norm pieces and the fp32 Gram accumulation can carry accurately
     const double mag = bprime * (a.rows_are_ctx ? c->max_sq : std::max(c->max_sq, c->row_max_sq));
     if (!(mag < (a.prec == FD_PREC_FAST ? 2000.0 : c->opt_tc_max_mag))) return false;
-    if (a.V == nullptr && a.right != nullptr && !a.right_pos) return false;   // row-sum mode folds a POSITIVE right vector into e_j
+    if (a.V == nullptr && a.right != nullptr && (!a.right_pos || a.rowsq)) return false;   // (row sums with squares carry no weights)
     return true;
 }
 
@@ -603,20 +477,26 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
     __half* xp_row = c->at<__half>(L.xp_row);
     unsigned int* status = c->at<unsigned int>(L.status);
     const int K16 = L.K16;
-    const int pk_blocks = (int)ceil_div(NP, 256);
-    // operands: columns (role 1) always from the context's points, rows (role 0) from a.xrow
-    // the same bias in both modes: the S tiles of the degree pass and of the block product are then bit-identical, so
-    // any rounding bias of the Gram accumulation is common to q and to K and cancels in diag(s) K diag(s)
-    k_pack_points<<<pk_blocks, 256, 0, c->stream>>>(c->xs(), L.DP, L.D, N, NP, mu, bprime, 1, (double)kBias,
-                                                   rowsum ? a.right : nullptr, K16, xp_col);
-    FD_LAUNCH_CHECK(c, "k_pack_points(col)");
     // Symmetric row sums (K = K^T): a square pass over the context's own points whose left and right weights are the same
-    // vector (the degree passes) evaluates only the tiles on or above the diagonal; the weight is folded into both exponents.
+    // vector (the degree passes) evaluates only the tiles on or above the diagonal.
     const bool sym = rowsum && a.sym_ok && c->opt_sym != 0 && a.rows_are_ctx && a.xrow == c->xs() && a.Nrow == N &&
                      a.left == a.right && L.symsum != 0;
-    k_pack_points<<<pk_blocks, 256, 0, c->stream>>>(a.xrow, L.DP, L.D, a.Nrow, NP, mu, bprime, 0, 0.0, sym ? a.right : nullptr, K16,
-                                                   xp_row);
-    FD_LAUNCH_CHECK(c, "k_pack_points(row)");
+    // operands: columns (role 1) always from the context's points, rows (role 0) from a.xrow.  They are the same for every kind of
+    // pass: the S tiles of the degree passes and of the block product are bit-identical, so any rounding bias of the Gram
+    // accumulation is common to q, d and K and cancels in diag(s) K diag(s).  The operands of the context's own points stay
+    // packed for the bandwidth: the products of a solve reuse them.
+    const PackRole rows{a.xrow, xp_row, a.Nrow}, cols{c->xs(), xp_col, N};
+    const int64_t row0 = a.rows_are_ctx ? (a.xrow - c->xs()) / L.DP : -1;
+    const bool have_rows = a.rows_are_ctx && c->packed_row_beta == a.beta && c->packed_row0 == row0 && c->packed_rows == a.Nrow;
+    const bool have_cols = c->packed_beta == a.beta;
+    if (!have_rows || !have_cols) {
+        const int first = have_rows ? 1 : 0, roles = (have_rows ? 0 : 1) + (have_cols ? 0 : 1);
+        k_pack_points<<<dim3((unsigned)ceil_div(NP, 256), (unsigned)K16, (unsigned)roles), 256, 0, c->stream>>>(
+            rows, cols, first, L.DP, L.D, NP, mu, bprime, std::sqrt(2.0 * bprime), L.D <= 12 * K16);
+        FD_LAUNCH_CHECK(c, "k_pack_points");
+        if (!have_rows) { c->packed_row_beta = a.rows_are_ctx ? a.beta : -1.0; c->packed_row0 = row0; c->packed_rows = a.Nrow; }
+        c->packed_beta = a.beta;
+    }
 
     CUtensorMap mr, mc, mh;
     if (!make_map_2d(&mr, xp_row, 32, (uint64_t)K16 * NP, 64, 32, 128, CU_TENSOR_MAP_SWIZZLE_64B) ||
@@ -635,30 +515,21 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
     p.left = a.left; p.status = status;
     const int grid = std::min(p.num_work, c->sm_count);
 
+    if (rowsum && !a.rowsq) {
+        float* w = c->at<float>(L.weights);
+        k_pad_weights<<<(unsigned)ceil_div(NP, 256), 256, 0, c->stream>>>(a.right, N, NP, w);
+        FD_LAUNCH_CHECK(c, "k_pad_weights");
+        p.weights = w;
+    }
     if (rowsum && sym) {
-        p.num_jt = (int)(NP / 128);                      // even: every row pair's two diagonal tiles exist (padding gives 2^e = 0)
-        p.jt_chunk = p.num_jt; p.num_chunks = 1;
-        p.left = nullptr;
-        p.q = a.Y; p.rowsq = a.rowsq; p.b = 1;
-        p.symsum = c->at<unsigned long long>(L.symsum);
-        // sums are at most NP * 2^bias in the kernel's scaled units: the fixed-point unit keeps them below 2^61
-        int lg = 0;
-        while (((int64_t)1 << lg) < NP) ++lg;
-        p.sym_shift = 61 - kBias - lg;
-        FD_CUDA(c, cudaMemsetAsync(p.symsum, 0, (size_t)N * 8, c->stream));
-        const int sym_grid = std::min((p.num_work + 1) / 2, c->sm_count);
-        if (p.rowsq) FD_TRY((launch_tc<16, kModeRowsumSym>(c, mr, mc, p, sym_grid)));
-        else FD_TRY((launch_tc<32, kModeRowsumSym>(c, mr, mc, p, sym_grid)));
-        k_sym_finish<<<(unsigned)ceil_div(N, 256), 256, 0, c->stream>>>(p.symsum, N, std::ldexp(1.0, -(kBias + (int)p.sym_shift)), a.Y);
-        FD_LAUNCH_CHECK(c, "k_sym_finish");
+        FD_TRY(launch_sym_rowsum(c, mr, mc, p.weights, a.left, a.Y, a.rowsq));
     } else if (rowsum) {
         p.q = a.Y; p.rowsq = a.rowsq; p.b = 1;
-        if (p.rowsq) FD_TRY((launch_tc<16, kModeRowsum>(c, mr, mc, p, grid)));
-        else FD_TRY((launch_tc<32, kModeRowsum>(c, mr, mc, p, grid)));
+        if (p.rowsq) FD_TRY((launch_tc<16>(c, mr, mc, p, grid)));
+        else FD_TRY((launch_tc<32>(c, mr, mc, p, grid)));
     } else {
         __half* wt_hi = c->at<__half>(L.wt_hi);
-        float* scale = c->at<float>(L.colscale);
-        float* inv = scale + L.BP + 8;
+        float* inv = c->at<float>(L.colscale);
         float* part = c->at<float>(L.part);
         const bool fast = a.prec == FD_PREC_FAST;
         // column chunks of at most 64, of about equal width (multiples of 16)
@@ -668,12 +539,10 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
             const int BT = bc <= 16 ? 16 : bc <= 32 ? 32 : bc <= 48 && !fast ? 48 : 64;
             if (BT > L.BP) return fail(c, FD_ERR_WORKSPACE, "column tile %d wider than the provisioned block buffers (%d)", BT, L.BP);
             const int cm_blocks = (int)std::min<int64_t>(256, ceil_div(N, 1024));
-            k_colmax_partial<<<dim3(cm_blocks, bc), 256, 0, c->stream>>>(a.V, a.ldv, a.right, N, c0, bc, part);
+            k_colmax_partial<<<dim3(cm_blocks, bc), 256, 0, c->stream>>>(a.V, a.ldv, a.right, N, c0, part);
             FD_LAUNCH_CHECK(c, "k_colmax_partial");
-            k_colscale<<<1, 64, 0, c->stream>>>(part, cm_blocks, bc, BT, scale, inv);
-            FD_LAUNCH_CHECK(c, "k_colscale");
-            k_pack_wt<<<dim3((unsigned)std::min<int64_t>(1024, ceil_div(NP, 256)), BT), 256, 0, c->stream>>>(
-                a.V, a.ldv, a.right, N, NP, c0, bc, scale, wt_hi, fast ? nullptr : wt_hi + (size_t)BT * NP);
+            k_pack_wt<<<dim3((unsigned)std::min<int64_t>(1024, ceil_div(NP, 512)), BT), 256, 0, c->stream>>>(
+                a.V, a.ldv, a.right, N, NP, c0, bc, part, cm_blocks, inv, wt_hi, fast ? 0 : 1);
             FD_LAUNCH_CHECK(c, "k_pack_wt");
             // one map over W_hi (rows 0 .. BT) and, in the fp32-grade mode, W_lo behind it (rows BT .. 2 BT of the same array)
             if (!make_map_2d(&mh, wt_hi, (uint64_t)NP, (uint64_t)(fast ? BT : 2 * BT), (uint64_t)NP * 2, 64, fast ? BT : 2 * BT, CU_TENSOR_MAP_SWIZZLE_128B))

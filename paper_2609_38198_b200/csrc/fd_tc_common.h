@@ -10,14 +10,10 @@ namespace tc {
 
 constexpr int kStages = 4;
 constexpr int kThreads = 384;                // row-sum kernel: warps 0-3 / 4-7 exponential warpgroups; warps 8-11: TMA, 2 idle, MMA
-constexpr int kBias = 15;                    // P' = 2^15 P keeps fp16 hi/lo of P out of the denormal range
+constexpr int kBias = 15;                    // P' = 2^15 P keeps fp16 hi/lo of P out of the denormal range (added to the exponent by the Gram MMAs:
+                                             // a multiplication after the exponential cost the product at N = 2^20 3 %)
 constexpr uint32_t kTmemCols = 512;
 constexpr long long kWaitCycles = 4000000000ll;   // ~2 s: far beyond any legitimate wait
-
-// Row-sum kernel: kModeRowsum evaluates every tile of its rows; kModeRowsumSym the row sums of a SYMMETRIC weighted kernel matrix
-// from its upper triangle of tiles alone (K = K^T, Sec. 2.1): every off-diagonal tile also yields the column sums that
-// the mirrored tile's rows would have computed.
-enum Mode { kModeRowsum = 2, kModeRowsumSym = 3 };
 
 struct TcParams {
     int64_t Nrow, N;             // valid rows / columns
@@ -31,13 +27,9 @@ struct TcParams {
     int flush;                   // column tiles per accumulator flush
     const float* left;           // may be null
     const float* colscale_inv;   // per column: 2^-bias / colscale
-    union {
-        struct { float* Y; int64_t ldy; };                       // block products: output block
-        struct { unsigned long long* symsum; int64_t sym_shift; };   // symmetric row-sum mode: fixed-point row + column sums, one
-                                                                 // 64-bit integer per point, in units of 2^-sym_shift of the
-                                                                 // (2^bias-scaled) kernel values
-    };
+    float* Y; int64_t ldy;       // block products: output block
     float* q; double* rowsq;     // row-sum modes: outputs
+    const float* weights;        // row-sum modes without squares: right weights, padded with zeros to whole tiles
     unsigned int* status;
 };
 
@@ -221,6 +213,10 @@ __host__ __device__ constexpr uint32_t idesc_f16(int n) {
 // Reduced-precision block product (fd_tc_fast.cu): one row tile per CTA, work items of 128 rows.
 fd_status launch_fast_product(fd_ctx* c, int BT, const CUtensorMap& mr, const CUtensorMap& mc, const CUtensorMap& mh,
                               const TcParams& p, int grid);
+// Row sums of the context's whole point set from the tiles on or above the diagonal (fd_tc_sym.cu): q = left * sum_j weights_j K_ij (no
+// weights: 1, and the total of rowsq's N entries is sum_ij K_ij^2).
+fd_status launch_sym_rowsum(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, const float* weights, const float* left, float* q,
+                            double* rowsq);
 // fp32-grade block product of BT = 16, 32, 48 or 64 columns (fd_tc_block.cu).
 fd_status launch_block_product(fd_ctx* c, int BT, const CUtensorMap& mr, const CUtensorMap& mc, const CUtensorMap& mw,
                                const TcParams& tp);

@@ -41,3 +41,27 @@ def test_block_product_edges(N, D, b, opts):
     Yo = dense.apply(X, beta, 1.0, V)
     assert np.linalg.norm(Y.cpu().numpy().astype(np.float64) - Yo) <= 1e-5 * np.linalg.norm(Yo)
     ctx.close()
+
+
+@pytest.mark.parametrize("N,D,beta", [(33, 3, 1.0), (385, 12, 2.0), (6401, 30, 1.0), (6401, 60, 0.3), (40003, 12, 2.0)])
+def test_symmetric_row_sums_against_every_tile(N, D, beta):
+    """The half-work degree passes against the passes that evaluate every tile (sym = 0): sizes with fewer steps than CTAs, ranges that
+    start inside a resident pair, more than 64 streamed tiles (a reduction inside an item), one to four K slabs (norms per slab and
+    norms after the last coordinate).  Both add the same fp32 kernel values: 64-term fp32 sums (2^-24 sqrt(64) each, random) then
+    fp64 / fixed point, so 1e-6 relative holds with a margin."""
+    import __graft_entry__ as g
+    g.build()
+    import paper_2609_38198_b200 as fd
+    dev = torch.device("cuda:0")
+    X = workloads.latent_torus(N, seed=N, D=D) if D > 12 else workloads.torus6(N, seed=N)[:, :D].copy()
+    ctx = fd.Context(torch.from_numpy(X).to(dev), b_max=8)
+    ctx.set_option("path", fd.FD_PATH_TC)
+    q1, d1, s1, so1, sq1 = ctx.degree(beta, 1.0)
+    q3, d3, s3, so3, sq3 = ctx.degree(beta, 1.0)
+    assert torch.equal(q1, q3) and torch.equal(d1, d3) and torch.equal(s1, s3) and (so1, sq1) == (so3, sq3)
+    ctx.set_option("sym", 0)
+    q0, d0, s0, so0, sq0 = ctx.degree(beta, 1.0)
+    for a, b in ((q1, q0), (d1, d0), (s1, s0)):
+        assert ((a - b).abs() / b).max().item() <= 1e-6
+    assert abs(so1 - so0) <= 1e-6 * (so0 + N) and abs(sq1 - sq0) <= 1e-6 * (sq0 + N)
+    ctx.close()
