@@ -1,6 +1,9 @@
-// Tall-skinny dense kernels for the eigensolver (HBM-bound O(N m b) work around the quadratic
-// apply): A^T B with fp64 accumulation and a deterministic two-stage reduction, C = A S updates,
-// column copies and conversions.  All blocks are column-major with N rows.
+// Tall-skinny dense kernels for the eigensolver (O(N m b) work around the quadratic apply): A^T B with fp64 accumulation and a
+// deterministic two-stage reduction, C = A S updates, column copies.  All blocks are column-major with N rows; a left
+// (right) factor may consist of two column ranges that lie in different arrays.
+//
+// What bounds them: FMA issue at N = 2^17 and up (one N x 200 x 32 product is 0.84 G FMAs = 24 us at the measured 124 FFMA per clock
+// per SM, its panel 105 MB = 16 us of HBM), launch and memory latency at N = 2^14.
 #include <algorithm>
 
 #include "fd_dense.h"
@@ -9,122 +12,202 @@ namespace fd {
 
 namespace {
 
-constexpr int kTnI = 64;          // output tile of the A^T B kernel: 64 (columns of A) x 32 (columns of B)
-constexpr int kTnJ = 32;
-constexpr int kTnRows = 64;       // rows staged per step; one step is summed in fp32, steps are added in fp64
+constexpr int kTnRows = 32;       // rows per pipeline stage
+constexpr int kTnPitch = 36;      // floats between two columns of a stage: 16-byte reads of 8 neighbouring columns hit all 32 banks
+constexpr int kTnStages = 3;
+constexpr int kTnFlush = 2;       // stages summed in fp32 (64 terms) before the sums are added in fp64
 
-// part[chunk][i + j * m1] = sum over this chunk's rows of A[r, i] * B[r, j].
-// 128 threads, each a 4 x 4 register tile.  Products of 64 consecutive rows are accumulated in fp32 (entries of
-// orthonormal columns are ~N^-1/2, so a 64-term partial sum loses ~1e-10 absolute) and every such partial sum is
-// added to an fp64 accumulator, which keeps the long sum over N rows at fp64 accuracy at fp32 FMA speed.
+__device__ __forceinline__ const float* panel_col(const Panel& a, int c) {
+    return c < a.m1 ? a.p1 + (int64_t)c * a.ld : a.p2 + (int64_t)(c - a.m1) * a.ld;
+}
+// Copies 4 consecutive rows of a column into shared memory; rows at or beyond `valid` (0..4) read as zero.
+template <bool ALIGNED>
+__device__ __forceinline__ void copy4(uint32_t dst, const float* src, int valid) {
+    if (ALIGNED) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(4 * valid) : "memory");
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 4 * i), "l"(src + (i < valid ? i : 0)), "r"(i < valid ? 4 : 0) : "memory");
+    }
+}
+
+// part[chunk][i + j * m] = sum over this chunk's rows of A[r, i] * B[r, j] for a tile of 16 UI x 8 UJ outputs.
+// 128 threads; thread (ti, tj) owns columns ti + 16 u of A and tj + 8 v of B.  Stages keep the columns contiguous (no transpose: a
+// stage is filled by asynchronous copies), a thread reads four rows of a column at once, so 4 UI UJ FMAs follow UI + UJ
+// 16-byte reads.  Products of 64 consecutive rows are accumulated in fp32 (entries of orthonormal columns are ~N^-1/2, so a
+// 64-term partial sum loses ~1e-10 absolute) and every such partial sum is added to an fp64 accumulator, which keeps the
+// long sum over N rows at fp64 accuracy at fp32 FMA speed.
+// N = 2^17, 200 x 32: 55 us against 106 for 4 x 4 outputs a thread from transposed stages without copies in flight.
+template <int UI, int UJ, bool ALIGNED>
 __global__ void __launch_bounds__(128)
-k_tn_partial(const float* __restrict__ A, int64_t lda, int m1, const float* __restrict__ B, int64_t ldb, int m2,
-             int64_t N, int64_t rows_per_chunk, double* __restrict__ part) {
-    constexpr int PA = kTnI + 4, PB = kTnJ + 4;                 // padded pitches (keep float4 alignment)
-    __shared__ __align__(16) float sa[kTnRows * PA];
-    __shared__ __align__(16) float sb[kTnRows * PB];
-    const int ti0 = blockIdx.x * kTnI, tj0 = blockIdx.y * kTnJ;
+k_tn_partial(const Panel A, const Panel B, int64_t N, int64_t rows_per_chunk, double* __restrict__ part) {
+    extern __shared__ __align__(16) float sm[];
+    constexpr int TI = 16 * UI, TJ = 8 * UJ, kStage = (TI + TJ) * kTnPitch;
+    const int m = A.m1 + A.m2, n = B.m1 + B.m2;
+    const int ti0 = blockIdx.x * TI, tj0 = blockIdx.y * TJ;
     const int64_t r_beg = (int64_t)blockIdx.z * rows_per_chunk;
     const int64_t r_end = r_beg + rows_per_chunk < N ? r_beg + rows_per_chunk : N;
-    const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;     // i0 = 4 ti, j0 = 4 tj
-    double acc[4][4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = 0.0;
-    for (int64_t r0 = r_beg; r0 < r_end; r0 += kTnRows) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < kTnRows * kTnI; t += 128) {
-            const int rr = t % kTnRows, cc = t / kTnRows;       // rows fastest: coalesced along a column
-            const int64_t r = r0 + rr;
-            sa[rr * PA + cc] = (r < r_end && ti0 + cc < m1) ? A[r + (int64_t)(ti0 + cc) * lda] : 0.f;
-        }
-        for (int t = threadIdx.x; t < kTnRows * kTnJ; t += 128) {
-            const int rr = t % kTnRows, cc = t / kTnRows;
-            const int64_t r = r0 + rr;
-            sb[rr * PB + cc] = (r < r_end && tj0 + cc < m2) ? B[r + (int64_t)(tj0 + cc) * ldb] : 0.f;
-        }
-        __syncthreads();
-        float f[4][4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) f[u][v] = 0.f;
-#pragma unroll 8
-        for (int rr = 0; rr < kTnRows; ++rr) {
-            const float4 a = *reinterpret_cast<const float4*>(&sa[rr * PA + 4 * ti]);
-            const float4 b = *reinterpret_cast<const float4*>(&sb[rr * PB + 4 * tj]);
-            const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) f[u][v] = fmaf(av[u], bv[v], f[u][v]);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] += (double)f[u][v];
-    }
-    double* o = part + (size_t)blockIdx.z * m1 * m2;
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int i = ti0 + 4 * ti + u, j = tj0 + 4 * tj + v;
-            if (i < m1 && j < m2) o[i + (size_t)j * m1] = acc[u][v];
-        }
-}
+    const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
+    const int steps = (int)((r_end - r_beg + kTnRows - 1) / kTnRows);
+    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(sm);
 
-__global__ void k_tn_reduce(const double* __restrict__ part, int chunks, int64_t mm, double* __restrict__ out) {
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= mm) return;
-    double acc = 0.0;
-    for (int c = 0; c < chunks; ++c) acc += part[(size_t)c * mm + e];
-    out[e] = acc;
-}
-
-// C[i, c] = alpha * sum_k A[i, k] S[k, c] + beta * C[i, c] for a strip of PT columns; one thread per row.
-template <int PT>
-__global__ void __launch_bounds__(128)
-k_nn(const float* __restrict__ A, int64_t lda, int m, const float* __restrict__ S, int lds, int p,
-     float* __restrict__ C, int64_t ldc, float alpha, float beta, int64_t N) {
-    __shared__ __align__(16) float ss[64 * PT];
-    const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
-    const int c0 = blockIdx.y * PT;
-    float acc[PT];
-#pragma unroll
-    for (int c = 0; c < PT; ++c) acc[c] = 0.f;
-    for (int k0 = 0; k0 < m; k0 += 64) {
-        const int kn = m - k0 < 64 ? m - k0 : 64;
-        __syncthreads();
-        for (int t = threadIdx.x; t < kn * PT; t += 128) {
-            int kk = t / PT, cc = t % PT;
-            ss[kk * PT + cc] = (c0 + cc < p) ? S[(k0 + kk) + (size_t)(c0 + cc) * lds] : 0.f;
-        }
-        __syncthreads();
-        if (i < N) {
-#pragma unroll 4
-            for (int kk = 0; kk < kn; ++kk) {
-                const float a = A[i + (int64_t)(k0 + kk) * lda];
-#pragma unroll
-                for (int c4 = 0; c4 < PT / 4; ++c4) {
-                    const float4 s4 = *reinterpret_cast<const float4*>(&ss[kk * PT + 4 * c4]);
-                    acc[4 * c4 + 0] = fmaf(a, s4.x, acc[4 * c4 + 0]);
-                    acc[4 * c4 + 1] = fmaf(a, s4.y, acc[4 * c4 + 1]);
-                    acc[4 * c4 + 2] = fmaf(a, s4.z, acc[4 * c4 + 2]);
-                    acc[4 * c4 + 3] = fmaf(a, s4.w, acc[4 * c4 + 3]);
-                }
+    auto load = [&](int s) {
+        if (s < steps) {
+            const int64_t r0 = r_beg + (int64_t)s * kTnRows;
+            const uint32_t st = sbase + 4u * (uint32_t)((s % kTnStages) * kStage);
+            // eight threads copy the 32 rows of a column
+            for (int t = threadIdx.x; t < (TI + TJ) * (kTnRows / 4); t += 128) {
+                const int cc = t >> 3, rr = (t & 7) * 4;
+                const bool left = cc < TI;
+                const int col = left ? ti0 + cc : tj0 + cc - TI;
+                int64_t valid = r_end - (r0 + rr);
+                valid = valid < 0 ? 0 : valid > 4 ? 4 : valid;
+                if (col >= (left ? m : n)) valid = 0;
+                const float* src = left ? panel_col(A, col < m ? col : 0) : panel_col(B, col < n ? col : 0);
+                copy4<ALIGNED>(st + 4u * (uint32_t)(cc * kTnPitch + rr), src + (valid > 0 ? r0 + rr : 0), (int)valid);
             }
         }
-    }
-    if (i >= N) return;
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+
+    double acc[UI][UJ];
+    float f[UI][UJ];
 #pragma unroll
-    for (int c = 0; c < PT; ++c) {
-        if (c0 + c < p) {
-            float* o = C + i + (int64_t)(c0 + c) * ldc;
-            *o = beta == 0.f ? alpha * acc[c] : fmaf(alpha, acc[c], beta * *o);
+    for (int u = 0; u < UI; ++u)
+#pragma unroll
+        for (int v = 0; v < UJ; ++v) { acc[u][v] = 0.0; f[u][v] = 0.f; }
+#pragma unroll
+    for (int s = 0; s < kTnStages - 1; ++s) load(s);
+    for (int s = 0; s < steps; ++s) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kTnStages - 2) : "memory");
+        __syncthreads();                               // stage s has landed; everybody is done with the stage that load() refills
+        load(s + kTnStages - 1);
+        const float* st = sm + (s % kTnStages) * kStage;
+        const float* sa = st + ti * kTnPitch;
+        const float* sb = st + (TI + tj) * kTnPitch;
+#pragma unroll 4
+        for (int rr = 0; rr < kTnRows; rr += 4) {
+            float4 a[UI], b[UJ];
+#pragma unroll
+            for (int u = 0; u < UI; ++u) a[u] = *reinterpret_cast<const float4*>(sa + 16 * u * kTnPitch + rr);
+#pragma unroll
+            for (int v = 0; v < UJ; ++v) b[v] = *reinterpret_cast<const float4*>(sb + 8 * v * kTnPitch + rr);
+#pragma unroll
+            for (int u = 0; u < UI; ++u)
+#pragma unroll
+                for (int v = 0; v < UJ; ++v) {
+                    float x = fmaf(a[u].x, b[v].x, f[u][v]);
+                    x = fmaf(a[u].y, b[v].y, x);
+                    x = fmaf(a[u].z, b[v].z, x);
+                    f[u][v] = fmaf(a[u].w, b[v].w, x);
+                }
+        }
+        if (s % kTnFlush == kTnFlush - 1 || s + 1 == steps) {
+#pragma unroll
+            for (int u = 0; u < UI; ++u)
+#pragma unroll
+                for (int v = 0; v < UJ; ++v) { acc[u][v] += (double)f[u][v]; f[u][v] = 0.f; }
         }
     }
+    double* o = part + (size_t)blockIdx.z * m * n;
+#pragma unroll
+    for (int u = 0; u < UI; ++u)
+#pragma unroll
+        for (int v = 0; v < UJ; ++v) {
+            const int i = ti0 + ti + 16 * u, j = tj0 + tj + 8 * v;
+            if (i < m && j < n) o[i + (size_t)j * m] = acc[u][v];
+        }
+}
+
+// out[e] = sum of the chunks' partials in a fixed order: 32 outputs x 8 partial sums per block, so that the chunks are read in
+// parallel.  `out` may be page-locked host memory: the values are stored there directly, no copy follows.
+__global__ void __launch_bounds__(256)
+k_tn_reduce(const double* __restrict__ part, int chunks, int64_t mm, double* __restrict__ out) {
+    __shared__ double sm[8][33];
+    const int64_t e = (int64_t)blockIdx.x * 32 + threadIdx.x;
+    double a0 = 0.0, a1 = 0.0;
+    if (e < mm) {
+        int c = threadIdx.y;
+        for (; c + 8 < chunks; c += 16) { a0 += part[(size_t)c * mm + e]; a1 += part[(size_t)(c + 8) * mm + e]; }
+        if (c < chunks) a0 += part[(size_t)c * mm + e];
+    }
+    sm[threadIdx.y][threadIdx.x] = a0 + a1;
+    __syncthreads();
+    if (threadIdx.y == 0 && e < mm) {
+        double acc = 0.0;
+#pragma unroll
+        for (int y = 0; y < 8; ++y) acc += sm[y][threadIdx.x];
+        out[e] = acc;
+    }
+}
+
+// C[i, c] = sum_k A[i, k] S[k, c] for a strip of PT columns; RPT rows per thread (two where there are enough rows: half the
+// shared-memory reads per FMA).  S is staged 32 rows at a time; the rows of A are read straight from memory, eight columns in flight.
+// N = 2^17, m = 200, p = 32: 48 us against 91 with one row per thread and four loads in flight.
+template <int PT, int RPT>
+__global__ void __launch_bounds__(128)
+k_nn(const Panel A, const float* __restrict__ S, int lds, int p, float* __restrict__ C, int64_t ldc, int64_t N) {
+    __shared__ __align__(16) float ss[32 * PT];
+    const int m = A.m1 + A.m2;
+    const int64_t i0 = (int64_t)blockIdx.x * (128 * RPT) + threadIdx.x;
+    const int c0 = blockIdx.y * PT;
+    int64_t row[RPT];
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) row[r] = i0 + 128 * r < N ? i0 + 128 * r : N - 1;
+    float acc[RPT][PT];
+#pragma unroll
+    for (int r = 0; r < RPT; ++r)
+#pragma unroll
+        for (int c = 0; c < PT; ++c) acc[r][c] = 0.f;
+    for (int k0 = 0; k0 < m; k0 += 32) {
+        __syncthreads();
+        for (int t = threadIdx.x; t < 32 * PT; t += 128) {
+            const int kk = t % 32, cc = t / 32;
+            ss[kk * PT + cc] = (k0 + kk < m && c0 + cc < p) ? S[(k0 + kk) + (size_t)(c0 + cc) * lds] : 0.f;
+        }
+        __syncthreads();
+        const int kn = m - k0 < 32 ? m - k0 : 32;
+        for (int kb = 0; kb < kn; kb += 8) {
+            float a[8][RPT];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int k = k0 + kb + u < m ? k0 + kb + u : m - 1;       // (padding columns meet zeros in S)
+                const float* col = panel_col(A, k);
+#pragma unroll
+                for (int r = 0; r < RPT; ++r) a[u][r] = col[row[r]];
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+#pragma unroll
+                for (int c4 = 0; c4 < PT / 4; ++c4) {
+                    const float4 s4 = *reinterpret_cast<const float4*>(&ss[(kb + u) * PT + 4 * c4]);
+#pragma unroll
+                    for (int r = 0; r < RPT; ++r) {
+                        acc[r][4 * c4 + 0] = fmaf(a[u][r], s4.x, acc[r][4 * c4 + 0]);
+                        acc[r][4 * c4 + 1] = fmaf(a[u][r], s4.y, acc[r][4 * c4 + 1]);
+                        acc[r][4 * c4 + 2] = fmaf(a[u][r], s4.z, acc[r][4 * c4 + 2]);
+                        acc[r][4 * c4 + 3] = fmaf(a[u][r], s4.w, acc[r][4 * c4 + 3]);
+                    }
+                }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < RPT; ++r)
+        if (i0 + 128 * r < N) {
+#pragma unroll
+            for (int c = 0; c < PT; ++c)
+                if (c0 + c < p) C[i0 + 128 * r + (int64_t)(c0 + c) * ldc] = acc[r][c];
+        }
+}
+
+// dst[:, c] = src[:, idx[c]]
+struct ColumnList { int n; uint16_t idx[256]; };
+__global__ void k_gather_cols(const float* __restrict__ src, float* __restrict__ dst, int64_t ld, const ColumnList list, int64_t N) {
+    const int c = blockIdx.y;
+    const float* s = src + (int64_t)list.idx[c] * ld;
+    float* d = dst + (int64_t)c * ld;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) d[i] = s[i];
 }
 
 // out[c] = sum_i A[i, c]^2 in fp64; one block per column, fixed summation order (bit-reproducible).
@@ -151,17 +234,6 @@ k_col_sqnorms(const float* __restrict__ A, int64_t lda, int64_t N, double* __res
     if (threadIdx.x == 0) out[blockIdx.x] = sm[0];
 }
 
-__global__ void k_d2f(const double* __restrict__ in, float* __restrict__ out, int64_t n, double scale) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = (float)(in[i] * scale);
-}
-
-__global__ void k_scale_cols(float* __restrict__ A, int64_t lda, int p, const float* __restrict__ f, int64_t N) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    for (int c = 0; c < p; ++c) A[i + (int64_t)c * lda] *= f[c];
-}
-
 // Counter-based uniform(-1, 1) fill for cold-start blocks (hash of (seed, element index)).
 __global__ void k_random_fill(float* __restrict__ A, int64_t lda, int p, int64_t N, int64_t row0, uint32_t seed) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -180,67 +252,86 @@ __global__ void k_sqrt_vec(const float* __restrict__ d, float* __restrict__ out,
 
 }  // namespace
 
-fd_status tn_product(fd_ctx* c, const float* A, int64_t lda, int m1, const float* B, int64_t ldb, int m2, int64_t N,
-                     double* out_dev, double* scratch, size_t scratch_doubles) {
-    if (m1 < 1 || m2 < 1) return FD_OK;
-    const size_t mm = (size_t)m1 * m2;
-    if (N < 1) {                                                  // a rank that owns no rows contributes zeros
-        FD_CUDA(c, cudaMemsetAsync(out_dev, 0, mm * sizeof(double), c->stream));
-        return FD_OK;
-    }
-    // Row chunks: at least 4096 rows each for large outputs, but enough chunks to put a few blocks on every SM when the
-    // output is small (a 32 x 32 Gram matrix is a single output tile: with 4096-row chunks it would run on 32 blocks).
-    const int64_t out_tiles = ceil_div(m1, kTnI) * ceil_div(m2, kTnJ);
-    int64_t chunks = std::max<int64_t>(ceil_div(N, 4096), ceil_div((int64_t)c->sm_count * 4, out_tiles));
-    if (chunks > 256) chunks = 256;
-    if (chunks > ceil_div(N, kTnRows)) chunks = ceil_div(N, kTnRows);
-    if ((size_t)chunks * mm > scratch_doubles) chunks = (int64_t)(scratch_doubles / mm);
-    if (chunks < 1) return fail(c, FD_ERR_WORKSPACE, "projection scratch too small for %d x %d", m1, m2);
-    int64_t rpc = round_up(ceil_div(N, chunks), kTnRows);
+namespace {
+
+bool panel_aligned(const Panel& a) {
+    return a.ld % 4 == 0 && (reinterpret_cast<uintptr_t>(a.p1) & 15) == 0 && (a.m2 == 0 || (reinterpret_cast<uintptr_t>(a.p2) & 15) == 0);
+}
+
+template <int UI, int UJ, bool ALIGNED>
+fd_status launch_tn(fd_ctx* c, const Panel& A, const Panel& B, int64_t N, int64_t max_chunks, double* scratch, int* chunks_out) {
+    constexpr int TI = 16 * UI, TJ = 8 * UJ, smem = kTnStages * (TI + TJ) * kTnPitch * 4;
+    const int m = A.m1 + A.m2, n = B.m1 + B.m2;
+    // row chunks: two blocks per SM, at least two pipeline fills of rows each
+    const int64_t tiles = ceil_div(m, TI) * ceil_div(n, TJ);
+    int64_t chunks = std::max<int64_t>(1, (int64_t)c->sm_count * 2 / tiles);
+    chunks = std::min(chunks, std::min(max_chunks, ceil_div(N, 2 * kTnRows)));
+    const int64_t rpc = round_up(ceil_div(N, chunks), 2 * kTnRows);
     chunks = ceil_div(N, rpc);
-    dim3 grid((unsigned)ceil_div(m1, kTnI), (unsigned)ceil_div(m2, kTnJ), (unsigned)chunks);
-    k_tn_partial<<<grid, 128, 0, c->stream>>>(A, lda, m1, B, ldb, m2, N, rpc, scratch);
+    FD_CUDA(c, cudaFuncSetAttribute(k_tn_partial<UI, UJ, ALIGNED>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    const dim3 grid((unsigned)ceil_div(m, TI), (unsigned)ceil_div(n, TJ), (unsigned)chunks);
+    k_tn_partial<UI, UJ, ALIGNED><<<grid, 128, smem, c->stream>>>(A, B, N, rpc, scratch);
     FD_LAUNCH_CHECK(c, "k_tn_partial");
-    k_tn_reduce<<<(unsigned)ceil_div((int64_t)mm, 256), 256, 0, c->stream>>>(scratch, (int)chunks, (int64_t)mm, out_dev);
+    *chunks_out = (int)chunks;
+    return FD_OK;
+}
+
+}  // namespace
+
+fd_status tn_product(fd_ctx* c, const Panel& A, const Panel& B, int64_t N, double* out, double* scratch, size_t scratch_doubles) {
+    const int m = A.m1 + A.m2, n = B.m1 + B.m2;
+    if (m < 1 || n < 1) return FD_OK;
+    const size_t mm = (size_t)m * n;
+    int chunks = 0;                                               // a rank that owns no rows contributes zeros
+    if (N >= 1) {
+        const int64_t max_chunks = (int64_t)std::min<size_t>(scratch_doubles / mm, 65535);
+        if (max_chunks < 1) return fail(c, FD_ERR_WORKSPACE, "projection scratch too small for %d x %d", m, n);
+        const bool al = panel_aligned(A) && panel_aligned(B);
+        // tile heights 128 / 64 by the number of left columns, widths 32 / 16 by the number of right columns: padding columns cost
+        // as much as real ones
+#define FD_TN(UI, UJ) FD_TRY((al ? launch_tn<UI, UJ, true>(c, A, B, N, max_chunks, scratch, &chunks)                  \
+                                 : launch_tn<UI, UJ, false>(c, A, B, N, max_chunks, scratch, &chunks)))
+        if (m > 64) { if (n > 16) FD_TN(8, 4); else FD_TN(8, 2); }
+        else { if (n > 16) FD_TN(4, 4); else FD_TN(4, 2); }
+#undef FD_TN
+    }
+    k_tn_reduce<<<(unsigned)ceil_div((int64_t)mm, 32), dim3(32, 8), 0, c->stream>>>(scratch, chunks, (int64_t)mm, out);
     FD_LAUNCH_CHECK(c, "k_tn_reduce");
     return FD_OK;
 }
 
-fd_status nn_product(fd_ctx* c, const float* A, int64_t lda, int m, const float* S_dev, int lds, int p, float* C,
-                     int64_t ldc, float alpha, float beta, int64_t N) {
+fd_status nn_product(fd_ctx* c, const Panel& A, const float* S_dev, int lds, int p, float* C, int64_t ldc, int64_t N) {
     if (p < 1 || N < 1) return FD_OK;
-    if (m < 1) return fail(c, FD_ERR_INVALID, "nn_product: m < 1");
-    if (p <= 8) {
-        dim3 grid((unsigned)ceil_div(N, 128), (unsigned)ceil_div(p, 8));
-        k_nn<8><<<grid, 128, 0, c->stream>>>(A, lda, m, S_dev, lds, p, C, ldc, alpha, beta, N);
-    } else {
-        dim3 grid((unsigned)ceil_div(N, 128), (unsigned)ceil_div(p, 32));
-        k_nn<32><<<grid, 128, 0, c->stream>>>(A, lda, m, S_dev, lds, p, C, ldc, alpha, beta, N);
-    }
+    if (A.m1 + A.m2 < 1) return fail(c, FD_ERR_INVALID, "nn_product: no columns");
+    // strips of 32 columns and two rows per thread where that still gives every SM a few blocks, else narrower strips
+    const int64_t blocks2 = ceil_div(N, 256) * ceil_div(p, 32), blocks1 = ceil_div(N, 128) * ceil_div(p, 32);
+    if (p > 16 && blocks2 >= 3 * c->sm_count)
+        k_nn<32, 2><<<dim3((unsigned)ceil_div(N, 256), (unsigned)ceil_div(p, 32)), 128, 0, c->stream>>>(A, S_dev, lds, p, C, ldc, N);
+    else if (p > 16 && blocks1 >= 2 * c->sm_count)
+        k_nn<32, 1><<<dim3((unsigned)ceil_div(N, 128), (unsigned)ceil_div(p, 32)), 128, 0, c->stream>>>(A, S_dev, lds, p, C, ldc, N);
+    else if (p > 8 && ceil_div(N, 128) * ceil_div(p, 16) >= 2 * c->sm_count)
+        k_nn<16, 1><<<dim3((unsigned)ceil_div(N, 128), (unsigned)ceil_div(p, 16)), 128, 0, c->stream>>>(A, S_dev, lds, p, C, ldc, N);
+    else
+        k_nn<8, 1><<<dim3((unsigned)ceil_div(N, 128), (unsigned)ceil_div(p, 8)), 128, 0, c->stream>>>(A, S_dev, lds, p, C, ldc, N);
     FD_LAUNCH_CHECK(c, "k_nn");
     return FD_OK;
 }
 
-fd_status col_sqnorms(fd_ctx* c, const float* A, int64_t lda, int p, int64_t N, double* out_dev) {
+fd_status gather_cols(fd_ctx* c, const float* src, float* dst, int64_t ld, const int* idx, int p, int64_t N) {
+    if (p < 1 || N < 1) return FD_OK;
+    if (p > 256) return fail(c, FD_ERR_INVALID, "gather_cols: more than 256 columns");
+    ColumnList list;
+    list.n = p;
+    for (int i = 0; i < p; ++i) list.idx[i] = (uint16_t)idx[i];
+    k_gather_cols<<<dim3((unsigned)std::min<int64_t>(64, ceil_div(N, 256)), (unsigned)p), 256, 0, c->stream>>>(src, dst, ld, list, N);
+    FD_LAUNCH_CHECK(c, "k_gather_cols");
+    return FD_OK;
+}
+
+fd_status col_sqnorms(fd_ctx* c, const float* A, int64_t lda, int p, int64_t N, double* out) {
     if (p < 1) return FD_OK;
-    if (N < 1) {
-        FD_CUDA(c, cudaMemsetAsync(out_dev, 0, (size_t)p * sizeof(double), c->stream));
-        return FD_OK;
-    }
-    k_col_sqnorms<<<(unsigned)p, 1024, 0, c->stream>>>(A, lda, N, out_dev);
+    k_col_sqnorms<<<(unsigned)p, 1024, 0, c->stream>>>(A, lda, N, out);
     FD_LAUNCH_CHECK(c, "k_col_sqnorms");
-    return FD_OK;
-}
-
-fd_status d2f(fd_ctx* c, const double* in, float* out, int64_t n, double scale) {
-    k_d2f<<<(unsigned)ceil_div(n, 256), 256, 0, c->stream>>>(in, out, n, scale);
-    FD_LAUNCH_CHECK(c, "k_d2f");
-    return FD_OK;
-}
-
-fd_status scale_cols(fd_ctx* c, float* A, int64_t lda, int p, const float* f_dev, int64_t N) {
-    k_scale_cols<<<(unsigned)ceil_div(N, 256), 256, 0, c->stream>>>(A, lda, p, f_dev, N);
-    FD_LAUNCH_CHECK(c, "k_scale_cols");
     return FD_OK;
 }
 

@@ -6,17 +6,20 @@
 
 namespace fd {
 
-// out_dev[m1 x m2] (column-major doubles, device) = A^T B over N rows, fp64 accumulation.
+// Columns of a tall matrix: m1 columns at p1 followed by m2 columns at p2 (m2 may be 0), column pitch ld.
+struct Panel { const float* p1; int m1; const float* p2; int m2; int64_t ld; };
+inline Panel panel(const float* p, int m, int64_t ld) { return Panel{p, m, nullptr, 0, ld}; }
+inline Panel panel(const float* p1, int m1, const float* p2, int m2, int64_t ld) { return Panel{p1, m1, p2, m2, ld}; }
+
+// out[(A columns) x (B columns)] (column-major doubles; device or page-locked host memory) = A^T B over N rows, fp64 accumulation.
 // scratch: device doubles for the per-chunk partials.
-fd_status tn_product(fd_ctx* c, const float* A, int64_t lda, int m1, const float* B, int64_t ldb, int m2, int64_t N,
-                     double* out_dev, double* scratch, size_t scratch_doubles);
-// C[N x p] = alpha * A[N x m] S[m x p] + beta * C; S_dev column-major floats with pitch lds.  C must not alias A.
-fd_status nn_product(fd_ctx* c, const float* A, int64_t lda, int m, const float* S_dev, int lds, int p, float* C,
-                     int64_t ldc, float alpha, float beta, int64_t N);
-// out_dev[c] = |A[:, c]|^2 (fp64) for the first p columns.
-fd_status col_sqnorms(fd_ctx* c, const float* A, int64_t lda, int p, int64_t N, double* out_dev);
-fd_status d2f(fd_ctx* c, const double* in, float* out, int64_t n, double scale);
-fd_status scale_cols(fd_ctx* c, float* A, int64_t lda, int p, const float* f_dev, int64_t N);
+fd_status tn_product(fd_ctx* c, const Panel& A, const Panel& B, int64_t N, double* out, double* scratch, size_t scratch_doubles);
+// C[N x p] = A[N x m] S[m x p]; S_dev column-major floats with pitch lds.  C must not alias A.
+fd_status nn_product(fd_ctx* c, const Panel& A, const float* S_dev, int lds, int p, float* C, int64_t ldc, int64_t N);
+// dst[:, i] = src[:, idx[i]] for p <= 256 columns, both with column pitch ld.
+fd_status gather_cols(fd_ctx* c, const float* src, float* dst, int64_t ld, const int* idx, int p, int64_t N);
+// out[c] = |A[:, c]|^2 (fp64; device or page-locked host memory) for the first p columns.
+fd_status col_sqnorms(fd_ctx* c, const float* A, int64_t lda, int p, int64_t N, double* out);
 // Counter-based uniform(-1, 1) fill of N rows x p columns; row i of A is row row0 + i of the stream, so a row range of
 // a larger block gets the values the whole block would.
 fd_status random_fill(fd_ctx* c, float* A, int64_t lda, int p, int64_t N, int64_t row0, uint32_t seed);

@@ -3,21 +3,29 @@
 //
 // The paper names "block implicitly restarted Lanczos" (Sec. 2.3) and gives no detail, so the
 // scheme is fixed here.  An orthonormal basis Q (N x m) is kept together with its image
-// W = M Q.  Each step: projected matrix T = Q^T W (fp64), Ritz pairs, explicit residuals
-// R_i = W x_i - theta_i Q x_i for the leading k + 1 + buffer pairs, the b residuals of largest
-// norm are orthogonalised against Q (classical Gram-Schmidt twice) and among themselves
-// (eigen-based orthogonalisation that drops dependent directions), appended, and M is applied
-// to the new block only.  For a cold one-block start this spans the same block Krylov space as
-// block Lanczos; unlike the three-term recurrence it accepts an arbitrary warm-start basis.
+// W = M Q and the projections T = Q^T W, G = Q^T Q (fp64).  A Rayleigh-Ritz step gives Ritz pairs, explicit residuals
+// R_i = W x_i - theta_i Q x_i for the leading k + 1 + buffer pairs, and the b residuals of largest
+// norm as the next block.  A block is orthogonalised against Q and within itself (eigen-based, drops dependent directions),
+// appended, and M is applied to it only.  The blocks after it continue the Krylov space of the newest one (M times the last
+// block, block Lanczos with full orthogonalisation) until the next Rayleigh-Ritz step: in exact arithmetic the residuals of all
+// Ritz vectors lie in the span of that continuation, so the space grows the same way (measured: the same number of products
+// within one or two), while the projected eigenproblem (host) and the residual passes (O(N m k)) are paid once in about four products.
+// For a cold one-block start this spans the block Krylov space of block Lanczos; unlike the three-term
+// recurrence it accepts an arbitrary warm-start basis.
 // When the basis is full it is compressed onto the leading Ritz vectors (thick restart).
 // The Perron vector sqrt(d) / |sqrt(d)| is known in closed form and always seeds the basis.
 // Vectors are fp32; every inner product and the small eigenproblem are fp64, and the measured
 // Gram matrix Q^T Q corrects the projected problem to first order, so fp32 loss of
 // orthogonality does not reach the Ritz values.
 //
+// What bounds it: the products with M at N >= 2^17; below, the host waits of a step (two: the projections of the new block
+// and of its first orthogonalisation) and the launches between them.  A step costs two A^T B passes, two A S passes and one product.
+// N = 16384 (R^4, k = 32, b = 16): 87 -> 45 ms; N = 65536 (R^30, k = 32, b = 32): 64 -> 45 ms; N = 2^17 (R^12, k = 64, b = 32): 457 -> 355 ms
+// against a Rayleigh-Ritz step per product with separate passes for every projection.
+//
 // Row-sharded contexts: every rank keeps rows [r0, r0 + n) of Q, W and the work blocks (pitch N, same addresses as
-// the unsharded layout), all tall-skinny products run on those rows, every reduced quantity that reaches the host
-// is summed over the ranks there (so all ranks take the same decisions), and the rows of a new block are gathered
+// the unsharded layout), all tall-skinny products run on those rows, every reduced quantity
+// is summed over the ranks on the host (so all ranks take the same decisions), and the rows of a new block are gathered
 // from their owners before M is applied to it.
 #include <algorithm>
 #include <chrono>
@@ -40,44 +48,62 @@ struct Solver {
     int64_t N;                      // pitch of every tall matrix = number of points
     int64_t r0, n;                  // rows this rank owns (0, N unless the context is row-sharded)
     int m_cap, BP;
-    float *Q, *W, *X;               // N x m_cap each (X = spare for out-of-place updates)
-    float *R, *R2;                  // N x BP each
-    double* d_out;                  // device: m_cap x BP doubles (projection results)
-    float* d_S;                     // device: m_cap x m_cap floats (small right factors)
+    float *Q, *W, *X;               // N x m_cap each (X = spare for out-of-place updates and the residuals)
+    float* R;                       // N x BP
+    float* d_S;                     // device: small right factors
     double* d_scr; size_t scr_n;    // device: partials of the projections
+    size_t S_floats;                // capacity of d_S and of a staging slot
     std::vector<double> T, G;       // host, column-major, pitch m_cap
-    std::vector<double> h_out;      // host staging
-    int stage_next = 0;             // next slot of the context's pinned staging ring
+    double* h = nullptr;            // page-locked result of the latest projection
+    int stage_next = 0;             // next slot of the context's staging ring
     int m = 0;
     int applies = 0, restarts = 0;
     double t_apply = 0.0;
 
-    fd_status to_host(int cnt) {
-        FD_CUDA(c, cudaMemcpyAsync(h_out.data(), d_out, sizeof(double) * (size_t)cnt, cudaMemcpyDeviceToHost, c->stream));
-        FD_CUDA(c, cudaStreamSynchronize(c->stream));
-        return allreduce_host(c, h_out.data(), cnt);
-    }
-    // The staging ring lives in the context (pinned HOST memory, allocated once): an upload never waits for the stream
-    // unless its slot is still in flight.
-    fd_status init_staging(size_t floats) {
-        if (c->stage_floats >= floats) return FD_OK;
-        for (int i = 0; i < fd_ctx::kStageSlots; ++i) {
-            if (c->stage[i]) { FD_CUDA(c, cudaFreeHost(c->stage[i])); c->stage[i] = nullptr; }
-            FD_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->stage[i]), sizeof(float) * floats));
-            if (!c->stage_ev[i]) FD_CUDA(c, cudaEventCreateWithFlags(&c->stage_ev[i], cudaEventDisableTiming));
+    Panel own(const float* p, int cols) const { return panel(p + r0, cols, N); }
+    Panel own(const float* p1, int c1, const float* p2, int c2) const { return panel(p1 + r0, c1, p2 + r0, c2, N); }
+
+    // The page-locked buffers live in the context (allocated once): an upload never waits for the stream unless its slot is
+    // still in flight.
+    fd_status init_staging(size_t out_doubles) {
+        if (c->stage_floats < S_floats || c->h_out_doubles < out_doubles) {
+            FD_CUDA(c, cudaStreamSynchronize(c->stream));
+            if (c->stage) { FD_CUDA(c, cudaFreeHost(c->stage)); c->stage = nullptr; c->stage_floats = 0; c->h_out_doubles = 0; }
+            const size_t slot = (size_t)round_up((int64_t)S_floats, 64);
+            FD_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->stage), sizeof(float) * slot * fd_ctx::kStageSlots + sizeof(double) * out_doubles));
+            c->stage_floats = slot;
+            c->h_out = reinterpret_cast<double*>(c->stage + slot * fd_ctx::kStageSlots);
+            c->h_out_doubles = out_doubles;
+            for (int i = 0; i < fd_ctx::kStageSlots; ++i)
+                if (!c->stage_ev[i]) FD_CUDA(c, cudaEventCreateWithFlags(&c->stage_ev[i], cudaEventDisableTiming));
         }
-        c->stage_floats = floats;
+        h = c->h_out;
         return FD_OK;
     }
-    fd_status upload_S(const std::vector<float>& S) {
-        if (S.size() > c->stage_floats) return fail(c, FD_ERR_WORKSPACE, "staging buffer too small for a right factor");
-        const int k = stage_next;
-        stage_next = (stage_next + 1) % fd_ctx::kStageSlots;
-        FD_CUDA(c, cudaEventSynchronize(c->stage_ev[k]));  // the copy that used this slot last (four uploads ago) has finished
-        std::copy(S.begin(), S.end(), c->stage[k]);
-        FD_CUDA(c, cudaMemcpyAsync(d_S, c->stage[k], sizeof(float) * S.size(), cudaMemcpyHostToDevice, c->stream));
-        FD_CUDA(c, cudaEventRecord(c->stage_ev[k], c->stream));
+    // Slot for a right factor of `floats` entries: the caller fills it and sends it.
+    fd_status stage_slot(size_t floats, float** p) {
+        if (floats > S_floats) return fail(c, FD_ERR_WORKSPACE, "staging buffer too small for a right factor");
+        FD_CUDA(c, cudaEventSynchronize(c->stage_ev[stage_next]));     // the copy that used this slot last (four uploads ago) has finished
+        *p = c->stage + c->stage_floats * stage_next;
         return FD_OK;
+    }
+    fd_status send_slot(size_t floats) {
+        FD_CUDA(c, cudaMemcpyAsync(d_S, c->stage + c->stage_floats * stage_next, sizeof(float) * floats, cudaMemcpyHostToDevice, c->stream));
+        FD_CUDA(c, cudaEventRecord(c->stage_ev[stage_next], c->stream));
+        stage_next = (stage_next + 1) % fd_ctx::kStageSlots;
+        return FD_OK;
+    }
+    // Waits for the projection written to h (cnt doubles) and sums it over the ranks.
+    fd_status fetch(int64_t cnt) {
+        FD_CUDA(c, cudaStreamSynchronize(c->stream));
+        return allreduce_host(c, h, cnt);
+    }
+    // h = A^T B (column-major, pitch = columns of A)
+    fd_status project(const Panel& A, const Panel& B) {
+        const int64_t cnt = (int64_t)(A.m1 + A.m2) * (B.m1 + B.m2);
+        if ((size_t)cnt > c->h_out_doubles) return fail(c, FD_ERR_WORKSPACE, "projection larger than its buffer");
+        FD_TRY(tn_product(c, A, B, n, h, d_scr, scr_n));
+        return fetch(cnt);
     }
 
     // W[:, c0 : c0 + n) = M Q[:, c0 : c0 + n), in blocks of at most bw columns
@@ -95,102 +121,162 @@ struct Solver {
         return FD_OK;
     }
 
-    // out(m1 x m2) -> host h_out, column-major pitch m1; right factor chunked to BP columns
-    fd_status project(const float* A, int m1, const float* B, int m2, std::vector<double>& dst) {
-        dst.assign((size_t)m1 * m2, 0.0);
-        for (int c0 = 0; c0 < m2; c0 += BP) {
-            int w = std::min(BP, m2 - c0);
-            FD_TRY(tn_product(c, A + r0, N, m1, B + (int64_t)c0 * N + r0, N, w, n, d_out, d_scr, scr_n));
-            FD_TRY(to_host(m1 * w));
-            std::copy(h_out.begin(), h_out.begin() + (size_t)m1 * w, dst.begin() + (size_t)c0 * m1);
+    // Recompute T = Q^T W and G = Q^T Q for the first m columns.
+    fd_status full_projection() {
+        const int step = std::max(1, (int)std::min<size_t>((size_t)m, scr_n / (size_t)m));
+        for (int pass = 0; pass < 2; ++pass) {
+            std::vector<double>& D = pass ? G : T;
+            for (int j0 = 0; j0 < m; j0 += step) {
+                const int w = std::min(step, m - j0);
+                FD_TRY(project(own(Q, m), own((pass ? Q : W) + (int64_t)j0 * N, w)));
+                for (int j = 0; j < w; ++j)
+                    for (int i = 0; i < m; ++i) D[i + (size_t)(j0 + j) * m_cap] = h[i + (size_t)j * m];
+            }
+            for (int j = 0; j < m; ++j)
+                for (int i = 0; i < j; ++i) {
+                    const double v = 0.5 * (D[i + (size_t)j * m_cap] + D[j + (size_t)i * m_cap]);
+                    D[i + (size_t)j * m_cap] = D[j + (size_t)i * m_cap] = v;
+                }
         }
         return FD_OK;
     }
 
-    // Recompute T = Q^T W and G = Q^T Q for the first m columns.
-    fd_status full_projection() {
-        std::vector<double> tmp;
-        FD_TRY(project(Q, m, W, m, tmp));
-        for (int j = 0; j < m; ++j)
-            for (int i = 0; i < m; ++i) T[i + (size_t)j * m_cap] = 0.5 * (tmp[i + (size_t)j * m] + tmp[j + (size_t)i * m]);
-        FD_TRY(project(Q, m, Q, m, tmp));
-        for (int j = 0; j < m; ++j)
-            for (int i = 0; i < m; ++i) G[i + (size_t)j * m_cap] = 0.5 * (tmp[i + (size_t)j * m] + tmp[j + (size_t)i * m]);
-        return FD_OK;
-    }
-
-    // After appending nb columns at position m: fill the new rows / columns of T and G.
-    fd_status extend_projection(int nb) {
-        const int mt = m + nb;
-        std::vector<double> tmp;
-        FD_TRY(project(Q, mt, W + (int64_t)m * N, nb, tmp));
-        for (int j = 0; j < nb; ++j)
-            for (int i = 0; i < mt; ++i) {
-                double v = tmp[i + (size_t)j * mt];
-                if (i >= m) v = 0.5 * (v + tmp[(m + j) + (size_t)(i - m) * mt]);
-                T[i + (size_t)(m + j) * m_cap] = v;
-                T[(m + j) + (size_t)i * m_cap] = v;
-            }
-        FD_TRY(project(Q, mt, Q + (int64_t)m * N, nb, tmp));
-        for (int j = 0; j < nb; ++j)
-            for (int i = 0; i < mt; ++i) {
-                double v = tmp[i + (size_t)j * mt];
-                if (i >= m) v = 0.5 * (v + tmp[(m + j) + (size_t)(i - m) * mt]);
-                G[i + (size_t)(m + j) * m_cap] = v;
-                G[(m + j) + (size_t)i * m_cap] = v;
-            }
+    // After p columns were appended at position m (their images in W): fills the new rows / columns of T and G.  On return
+    // h holds [Q W_new]^T [Q_new W_new] with Q including the new columns (m + p rows) -- the projection that the block
+    // W_new needs when it becomes the next expansion.
+    fd_status extend_projection(int p) {
+        const int mt = m + p, rows = mt + p;
+        const float *Qn = Q + (int64_t)m * N, *Wn = W + (int64_t)m * N;
+        FD_TRY(project(own(Q, mt, Wn, p), own(Qn, p, Wn, p)));
+        for (int pass = 0; pass < 2; ++pass) {
+            std::vector<double>& D = pass ? G : T;
+            const double* z = h + (size_t)(pass ? 0 : p) * rows;
+            for (int j = 0; j < p; ++j)
+                for (int i = 0; i < mt; ++i) {
+                    double v = z[i + (size_t)j * rows];
+                    if (i >= m) v = 0.5 * (v + z[(m + j) + (size_t)(i - m) * rows]);
+                    D[i + (size_t)(m + j) * m_cap] = v;
+                    D[(m + j) + (size_t)i * m_cap] = v;
+                }
+        }
         m = mt;
         return FD_OK;
     }
 
-    // Orthonormalise the p columns of B (N x p, pitch N) among themselves; dependent directions
-    // (eigenvalue of the unit-diagonal Gram matrix below drop_tol) are dropped.  Result in B, p updated.
-    fd_status orthonormalise(float*& B, float*& spare, int& p, double drop_tol) {
-        if (p == 0) return FD_OK;
-        FD_TRY(tn_product(c, B + r0, N, p, B + r0, N, p, n, d_out, d_scr, scr_n));
-        FD_TRY(to_host(p * p));
-        std::vector<double> g((size_t)p * p), dinv(p);
+    // Eigen-decomposition of the p x p Gram matrix g (column-major, overwritten) scaled to a unit diagonal.  On return F
+    // (p x rank, column-major) turns the columns whose Gram matrix g is into orthonormal ones; directions with an
+    // eigenvalue at or below drop_tol are left out.  lam_min: the smallest eigenvalue kept.
+    fd_status orthonormal_factor(double* g, int p, double drop_tol, std::vector<double>& F, int& rank, double& lam_min) {
+        std::vector<double> dinv(p);
         for (int j = 0; j < p; ++j) {
-            double dj = h_out[j + (size_t)j * p];
+            const double dj = g[j + (size_t)j * p];
             dinv[j] = dj > 1e-60 ? 1.0 / std::sqrt(dj) : 0.0;
         }
         for (int j = 0; j < p; ++j)
-            for (int i = 0; i < p; ++i)
-                g[i + (size_t)j * p] = 0.5 * (h_out[i + (size_t)j * p] + h_out[j + (size_t)i * p]) * dinv[i] * dinv[j];
+            for (int i = 0; i <= j; ++i) {
+                const double v = 0.5 * (g[i + (size_t)j * p] + g[j + (size_t)i * p]) * dinv[i] * dinv[j];
+                g[i + (size_t)j * p] = g[j + (size_t)i * p] = v;
+            }
         std::vector<double> lam, U;
-        if (!sym_eig(g.data(), p, lam, U)) return fail(c, FD_ERR_NOT_CONVERGED, "small eigenproblem (orthonormalise) failed");
-        std::vector<int> keep;
-        for (int j = p - 1; j >= 0; --j)
-            if (lam[j] > drop_tol) keep.push_back(j);
-        const int pk = (int)keep.size();
-        if (pk == 0) { p = 0; return FD_OK; }
-        std::vector<float> S((size_t)p * pk);
-        for (int jj = 0; jj < pk; ++jj) {
-            const int j = keep[jj];
+        if (!sym_eig(g, p, lam, U)) return fail(c, FD_ERR_NOT_CONVERGED, "small eigenproblem (orthonormalise) failed");
+        rank = 0;
+        lam_min = 1.0;
+        F.clear();
+        for (int j = p - 1; j >= 0; --j) {
+            if (!(lam[j] > drop_tol)) continue;
             const double f = 1.0 / std::sqrt(lam[j]);
-            for (int i = 0; i < p; ++i) S[i + (size_t)jj * p] = (float)(dinv[i] * U[i + (size_t)j * p] * f);
+            for (int i = 0; i < p; ++i) F.push_back(dinv[i] * U[i + (size_t)j * p] * f);
+            lam_min = lam[j];
+            ++rank;
         }
-        FD_TRY(upload_S(S));
-        FD_TRY(nn_product(c, B + r0, N, p, d_S, p, pk, spare + r0, N, 1.f, 0.f, n));
-        std::swap(B, spare);
-        p = pk;
         return FD_OK;
     }
 
-    // B <- B - Q[:, 0:mq) (Q^T B), once.
-    fd_status project_out(float* B, int p, int mq) {
-        if (p == 0 || mq == 0) return FD_OK;
-        FD_TRY(tn_product(c, Q + r0, N, mq, B + r0, N, p, n, d_out, d_scr, scr_n));
-        if (c->sh.on) {
-            // the coefficients are sums over the ranks: through the host, like every other projection
-            FD_TRY(to_host(mq * p));
-            std::vector<float> S((size_t)mq * p);
-            for (size_t i = 0; i < S.size(); ++i) S[i] = (float)(-h_out[i]);
-            FD_TRY(upload_S(S));
-        } else {
-            FD_TRY(d2f(c, d_out, d_S, (int64_t)mq * p, -1.0));
+    // Orthonormalise the p columns of B (pitch N) among themselves.  Result in B, p updated.
+    fd_status orthonormalise(float*& B, float*& spare, int& p, double drop_tol) {
+        if (p == 0) return FD_OK;
+        FD_TRY(project(own(B, p), own(B, p)));
+        std::vector<double> g(h, h + (size_t)p * p), F;
+        int rank; double lam_min;
+        FD_TRY(orthonormal_factor(g.data(), p, drop_tol, F, rank, lam_min));
+        if (rank == 0) { p = 0; return FD_OK; }
+        float* S = nullptr;
+        FD_TRY(stage_slot(F.size(), &S));
+        for (size_t i = 0; i < F.size(); ++i) S[i] = (float)F[i];
+        FD_TRY(send_slot(F.size()));
+        FD_TRY(nn_product(c, own(B, p), d_S, p, rank, spare + r0, N, n));
+        std::swap(B, spare);
+        p = rank;
+        return FD_OK;
+    }
+
+    // dst = (B - Q C) F for p columns B and the basis Q[:, 0 : m): z = [Q B]^T B holds C (rows 0 .. m, pitch ldz); F is p x pk.
+    fd_status subtract_and_mix(const float* B, int p, const double* z, int ldz, const double* F, int pk, float* dst) {
+        float* S = nullptr;
+        const size_t cnt = (size_t)(m + p) * pk;
+        FD_TRY(stage_slot(cnt, &S));
+        std::vector<double> col(m);
+        for (int j = 0; j < pk; ++j) {
+            const double* f = F + (size_t)j * p;
+            std::fill(col.begin(), col.end(), 0.0);
+            for (int l = 0; l < p; ++l) {
+                const double fl = f[l];
+                if (fl == 0.0) continue;
+                const double* zl = z + (size_t)l * ldz;
+                for (int i = 0; i < m; ++i) col[i] -= zl[i] * fl;
+            }
+            for (int i = 0; i < m; ++i) S[i + (size_t)j * (m + p)] = (float)col[i];
+            for (int l = 0; l < p; ++l) S[m + l + (size_t)j * (m + p)] = (float)f[l];
         }
-        FD_TRY(nn_product(c, Q + r0, N, mq, d_S, mq, p, B + r0, N, 1.f, 1.f, n));
+        FD_TRY(send_slot(cnt));
+        return nn_product(c, own(Q, m, B, p), d_S, m + p, pk, dst + r0, N, n);
+    }
+
+    // Orthonormalises the block B (p <= BP columns, not inside Q's first m columns) against the basis and within itself; the
+    // result goes to Q[:, m ..) and p is updated (0: nothing new).  z: [Q B]^T B of pitch ldz if the caller has it, else null.
+    //   1. R = (B - Q C) scaled to unit columns: removes the basis to fp32 rounding of B's own size;
+    //   2. Q_new = (R - Q C') F with C' = Q^T R (small now) and F from R^T R - C'^T C', which is accurate because C' is small;
+    //   3. once more if the block was nearly dependent, so that step 2's rounding was magnified.
+    fd_status expand(const float* B, int& p, const double* z, int ldz) {
+        if (p == 0) return FD_OK;
+        std::vector<double> F;
+        if (!z) {
+            FD_TRY(project(own(Q, m, B, p), own(B, p)));
+            z = h; ldz = m + p;
+        }
+        F.assign((size_t)p * p, 0.0);
+        for (int j = 0; j < p; ++j) {
+            const double* zj = z + (size_t)j * ldz;
+            double d = zj[m + j], cc = 0.0;
+            for (int i = 0; i < m; ++i) cc += zj[i] * zj[i];
+            const double left = std::max(d - cc, 1e-12 * d);      // |column|^2 after the projection (floor: cancellation)
+            F[j + (size_t)j * p] = left > 1e-60 ? 1.0 / std::sqrt(left) : 0.0;
+        }
+        float* dst = B == R ? Q + (int64_t)m * N : R;
+        FD_TRY(subtract_and_mix(B, p, z, ldz, F.data(), p, dst));
+        for (int pass = 0; pass < 2; ++pass) {
+            const float* src = dst;
+            FD_TRY(project(own(Q, m, src, p), own(src, p)));
+            const int ld = m + p;
+            std::vector<double> g((size_t)p * p);
+            double cmax = 0.0;
+            for (int j = 0; j < p; ++j)
+                for (int i = 0; i < p; ++i) {
+                    const double *ci = h + (size_t)i * ld, *cj = h + (size_t)j * ld;
+                    double v = cj[m + i];
+                    for (int l = 0; l < m; ++l) v -= ci[l] * cj[l];
+                    g[i + (size_t)j * p] = v;
+                    if (i == 0) for (int l = 0; l < m; ++l) cmax = std::max(cmax, std::fabs(cj[l]) / std::sqrt(std::max(cj[m + j], 1e-60)));
+                }
+            int rank; double lam_min;
+            FD_TRY(orthonormal_factor(g.data(), p, pass == 0 ? 1e-5 : 1e-3, F, rank, lam_min));
+            if (rank == 0) { p = 0; return FD_OK; }
+            dst = src == R ? Q + (int64_t)m * N : R;
+            FD_TRY(subtract_and_mix(src, p, h, ld, F.data(), rank, dst));
+            p = rank;
+            if (pass == 0 && lam_min > 1e-2 && cmax < 1e-2) break;
+        }
+        if (dst == R) FD_TRY(copy_cols(c, R + r0, N, Q + (int64_t)m * N + r0, N, p, n));
         return FD_OK;
     }
 };
@@ -221,17 +307,17 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
     S.m_cap = (int)std::min<int64_t>(L.m_max, N);
     const int m_cap = S.m_cap;
     S.Q = c->at<float>(L.eig_q); S.W = c->at<float>(L.eig_w); S.X = c->at<float>(L.eig_x);
-    S.R = c->at<float>(L.eig_r); S.R2 = c->at<float>(L.eig_t);
+    S.R = c->at<float>(L.eig_r);
     double* small = c->at<double>(L.eig_small);
-    S.d_out = small;
-    S.d_S = reinterpret_cast<float*>(small + (size_t)L.m_max * std::max(L.m_max, L.BP));
-    S.d_scr = small + (size_t)2 * L.m_max * std::max(L.m_max, L.BP);
-    S.scr_n = L.eig_small_doubles - (size_t)2 * L.m_max * std::max(L.m_max, L.BP);
+    const size_t mm = (size_t)L.m_max * std::max(L.m_max, L.BP);
+    S.d_S = reinterpret_cast<float*>(small);
+    S.S_floats = 2 * mm;
+    S.d_scr = small + mm;
+    S.scr_n = L.eig_small_doubles - mm;
     S.T.assign((size_t)m_cap * m_cap, 0.0);
     S.G.assign((size_t)m_cap * m_cap, 0.0);
-    S.h_out.assign((size_t)L.m_max * std::max(L.m_max, L.BP), 0.0);
     auto t_i0 = clk::now();
-    FD_TRY(S.init_staging((size_t)L.m_max * (size_t)std::max(L.m_max, 2 * L.BP)));
+    FD_TRY(S.init_staging(std::max((size_t)m_cap * m_cap, (size_t)(m_cap + 2 * L.BP) * 2 * L.BP)));
     const double t_init = secs(t_i0, clk::now());
 
     const int buffer = std::min<int>(std::min(b, 8), (int)std::max<int64_t>(0, N - nwant));
@@ -272,6 +358,14 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
     // stagnation of the residuals at the accuracy floor of the fp32 operator (noise-smeared spectra): stop early
     double best_res = 1e300;
     int since_best = 0;
+    // blocks appended between two Rayleigh-Ritz steps
+    // (A basis smaller than three times the wanted pairs restarts at every second product and cuts into the wanted pairs' clusters:
+    // there every block is a residual block, and a solve that reaches the accuracy floor of the fp32 operator first is
+    // reported as stalled.  N = 2^18, k = 128, capacity 384: the Krylov continuation brings all residuals of the STORED images
+    // below 1e-6 while the operator's own error leaves them at up to 1.9e-6 against float64 rows.)
+    const int kMaxBlocks = m_cap < 3 * nwant && m_cap < N ? 1 : 4;
+    double last_worst = 0.0;
+    int last_applies = 0;
 
     double t_rr = 0, t_eig = 0, t_res = 0, t_restart = 0, t_orth = 0, t_ext = 0;
     for (int iter = 0;; ++iter) {
@@ -313,31 +407,31 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
                 Xr[i + (size_t)jj * m] = U[i + (size_t)j * m] - 0.5 * corr;
             }
         }
-        // ---- explicit residuals R_i = W x_i - theta_i Q x_i, BP columns at a time -----------------
+        // ---- explicit residuals R_i = W x_i - theta_i Q x_i, into the spare panel -----------------
         // Leading pairs that converged with a margin at an earlier step are not re-evaluated every step (their Ritz
         // vectors only improve as the basis grows); before convergence is declared every pair is evaluated afresh.
         resid.resize(nsel, 1e300);
         const double thr = tol * std::fabs(theta[0]);
         bool all = false;
+        int first = 0;                                             // X[:, i - first] holds the residual of pair i >= first
         for (int pass = 0; pass < 2; ++pass) {
-            std::vector<int> act;
-            for (int i = std::min(nlock, nsel); i < nsel; ++i) act.push_back(i);
-            for (size_t a0 = 0; a0 < act.size(); a0 += (size_t)S.BP) {
-                const int w = (int)std::min<size_t>((size_t)S.BP, act.size() - a0);
-                std::vector<float> Sx((size_t)m * w * 2);
-                for (int jj = 0; jj < w; ++jj) {
-                    const int col = act[a0 + jj];
+            first = std::min(nlock, nsel);
+            const int w = nsel - first;
+            if (w > 0) {
+                float* Sx = nullptr;
+                const size_t cnt = (size_t)2 * m * w;
+                FD_TRY(S.stage_slot(cnt, &Sx));
+                for (int jj = 0; jj < w; ++jj)
                     for (int i = 0; i < m; ++i) {
-                        Sx[i + (size_t)jj * m] = (float)Xr[i + (size_t)col * m];
-                        Sx[(size_t)m * w + i + (size_t)jj * m] = (float)(-theta[col] * Xr[i + (size_t)col * m]);
+                        const double x = Xr[i + (size_t)(first + jj) * m];
+                        Sx[i + (size_t)jj * 2 * m] = (float)x;
+                        Sx[m + i + (size_t)jj * 2 * m] = (float)(-theta[first + jj] * x);
                     }
-                }
-                FD_TRY(S.upload_S(Sx));
-                FD_TRY(nn_product(c, S.W + r0, N, m, S.d_S, m, w, S.R + r0, N, 1.f, 0.f, n));
-                FD_TRY(nn_product(c, S.Q + r0, N, m, S.d_S + (size_t)m * w, m, w, S.R + r0, N, 1.f, 1.f, n));
-                FD_TRY(col_sqnorms(c, S.R + r0, N, w, n, S.d_out));
-                FD_TRY(S.to_host(w));
-                for (int jj = 0; jj < w; ++jj) resid[act[a0 + jj]] = std::sqrt(std::max(0.0, S.h_out[jj]));
+                FD_TRY(S.send_slot(cnt));
+                FD_TRY(nn_product(c, S.own(S.W, m, S.Q, m), S.d_S, 2 * m, w, S.X + r0, N, n));
+                FD_TRY(col_sqnorms(c, S.X + r0, N, w, n, S.h));
+                FD_TRY(S.fetch(w));
+                for (int jj = 0; jj < w; ++jj) resid[first + jj] = std::sqrt(std::max(0.0, S.h[jj]));
             }
             nconv = 0;
             while (nconv < std::min(nwant, nsel) && resid[nconv] <= thr) ++nconv;
@@ -355,112 +449,113 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
         t_res += secs(tp2, tp3);
         if (all) { final_status = FD_OK; break; }
         if (S.applies >= max_applies) break;
+        int blocks = kMaxBlocks;                                  // blocks to append before the next Rayleigh-Ritz step
         {
             double worst = 0.0;
             for (int i = 0; i < std::min(nwant, nsel); ++i) worst = std::max(worst, resid[i]);
-            if (nsel >= nwant && worst < 0.9 * best_res) { best_res = worst; since_best = 0; }
-            else if (nsel >= nwant) ++since_best;
+            if (nsel >= nwant) {
+                if (worst < 0.9 * best_res) { best_res = worst; since_best = 0; }
+                else since_best += S.applies - last_applies;
+                // the worst residual's decay per product since the last step tells how many products are left
+                if (last_worst > worst && worst > thr) {
+                    const double rate = std::log(last_worst / worst) / std::max(1, S.applies - last_applies);
+                    blocks = std::max(1, std::min(kMaxBlocks, (int)std::ceil(std::log(worst / thr) / rate)));
+                }
+                last_worst = worst;
+                last_applies = S.applies;
+            }
             // the largest wanted residual has not improved by 10 % over 25 expansions and is within 2x of the target:
             // the operator's own rounding error is the floor; more applies do not help
             if (since_best >= 25 && best_res <= 2.0 * thr) break;
         }
         if (m >= N) break;                                        // basis spans everything: nothing more to add
 
-        // ---- choose the expansion columns: largest residuals first ------------------------------
+        // ---- choose the expansion columns: wanted pairs above the tolerance first, then largest residuals first ---
+        // (the buffer pairs' residuals are larger almost always; a wanted pair that the fp32 rounding of its residual holds
+        // just above the tolerance would never be chosen)
         std::vector<int> order(nsel);
         for (int i = 0; i < nsel; ++i) order[i] = i;
-        std::sort(order.begin(), order.end(), [&](int a, int bb) { return resid[a] > resid[bb]; });
-        int want_new = std::min<int64_t>(b, N - m);
+        std::sort(order.begin(), order.end(), [&](int a, int bb) {
+            const bool wa = a < nwant && resid[a] > thr, wb = bb < nwant && resid[bb] > thr;
+            return wa != wb ? wa : resid[a] > resid[bb];
+        });
+        const int want_new = (int)std::min<int64_t>(b, N - m);
         std::vector<int> pick;
         for (int i = 0; i < nsel && (int)pick.size() < want_new; ++i)
-            if (resid[order[i]] > 0.1 * thr) pick.push_back(order[i]);
+            if (order[i] >= first && resid[order[i]] > 0.1 * thr) pick.push_back(order[i] - first);
         if (pick.empty()) { final_status = FD_OK; break; }
+        int p = (int)pick.size();
+        FD_TRY(gather_cols(c, S.X + r0, S.R + r0, N, pick.data(), p, n));
 
         // ---- thick restart when the new block would not fit ----------------------------------------
-        if (m + (int)pick.size() > m_cap) {
+        if (m + p > m_cap) {
             int keep = std::max(nsel, std::min(m - 1, (m_cap * 3) / 5));
-            keep = std::min(keep, m_cap - (int)pick.size());
+            keep = std::min(keep, m_cap - p);
             keep = std::min(keep, m);
             // Ritz vectors for the kept block (beyond nsel use the uncorrected eigenvectors)
-            std::vector<float> Sk((size_t)m * keep);
+            float* Sk = nullptr;
+            const size_t cnt = (size_t)m * keep;
+            FD_TRY(S.stage_slot(cnt, &Sk));
             for (int jj = 0; jj < keep; ++jj) {
                 const int j = m - 1 - jj;
                 for (int i = 0; i < m; ++i)
                     Sk[i + (size_t)jj * m] = jj < nsel ? (float)Xr[i + (size_t)jj * m] : (float)U[i + (size_t)j * m];
             }
-            // residual block for the picked columns must be formed BEFORE the basis changes
-            std::vector<float> Sx((size_t)m * pick.size() * 2);
-            const int w = (int)pick.size();
-            for (int jj = 0; jj < w; ++jj)
-                for (int i = 0; i < m; ++i) {
-                    Sx[i + (size_t)jj * m] = (float)Xr[i + (size_t)pick[jj] * m];
-                    Sx[(size_t)m * w + i + (size_t)jj * m] = (float)(-theta[pick[jj]] * Xr[i + (size_t)pick[jj] * m]);
-                }
-            FD_TRY(S.upload_S(Sx));
-            FD_TRY(nn_product(c, S.W + r0, N, m, S.d_S, m, w, S.R + r0, N, 1.f, 0.f, n));
-            FD_TRY(nn_product(c, S.Q + r0, N, m, S.d_S + (size_t)m * w, m, w, S.R + r0, N, 1.f, 1.f, n));
-            FD_TRY(S.upload_S(Sk));
-            FD_TRY(nn_product(c, S.Q + r0, N, m, S.d_S, m, keep, S.X + r0, N, 1.f, 0.f, n));
+            FD_TRY(S.send_slot(cnt));
+            FD_TRY(nn_product(c, S.own(S.Q, m), S.d_S, m, keep, S.X + r0, N, n));
             std::swap(S.Q, S.X);                                  // X now holds the old basis: reuse it for W
-            FD_TRY(nn_product(c, S.W + r0, N, m, S.d_S, m, keep, S.X + r0, N, 1.f, 0.f, n));
+            FD_TRY(nn_product(c, S.own(S.W, m), S.d_S, m, keep, S.X + r0, N, n));
             std::swap(S.W, S.X);
             S.m = keep;
             ++S.restarts;
             FD_TRY(S.full_projection());
-        } else {
-            const int w = (int)pick.size();
-            std::vector<float> Sx((size_t)m * w * 2);
-            for (int jj = 0; jj < w; ++jj)
-                for (int i = 0; i < m; ++i) {
-                    Sx[i + (size_t)jj * m] = (float)Xr[i + (size_t)pick[jj] * m];
-                    Sx[(size_t)m * w + i + (size_t)jj * m] = (float)(-theta[pick[jj]] * Xr[i + (size_t)pick[jj] * m]);
-                }
-            FD_TRY(S.upload_S(Sx));
-            FD_TRY(nn_product(c, S.W + r0, N, m, S.d_S, m, w, S.R + r0, N, 1.f, 0.f, n));
-            FD_TRY(nn_product(c, S.Q + r0, N, m, S.d_S + (size_t)m * w, m, w, S.R + r0, N, 1.f, 1.f, n));
         }
         auto tp4 = clk::now();
         t_restart += secs(tp3, tp4);
-        // ---- orthogonalise the new block against the basis and within itself ---------------------
-        int p = (int)pick.size();
-        FD_TRY(S.project_out(S.R, p, S.m));
-        FD_TRY(S.project_out(S.R, p, S.m));
-        FD_TRY(S.orthonormalise(S.R, S.R2, p, 1e-5));
-        FD_TRY(S.project_out(S.R, p, S.m));
-        FD_TRY(S.orthonormalise(S.R, S.R2, p, 1e-3));
-        if (p == 0) {
-            // the residuals lie (numerically) inside the basis: try a random direction, give up after a few
-            if (++stagnation > 3) break;
-            p = std::min<int64_t>(b, N - S.m);
-            FD_TRY(random_fill(c, S.R + r0, N, p, n, r0, 0xABCD1234u + (uint32_t)iter));
-            FD_TRY(S.project_out(S.R, p, S.m));
-            FD_TRY(S.project_out(S.R, p, S.m));
-            FD_TRY(S.orthonormalise(S.R, S.R2, p, 1e-5));
-            FD_TRY(S.project_out(S.R, p, S.m));
-            FD_TRY(S.orthonormalise(S.R, S.R2, p, 1e-3));
-            if (p == 0) break;
+        // ---- append the residual block, then continue its Krylov space ---------------------------
+        const double* z = nullptr;                                 // [Q B]^T B of the block to append, where it is known already
+        int ldz = 0;
+        std::vector<double> zkeep;
+        const float* B = S.R;
+        bool stuck = false;
+        for (int blk = 0; blk < blocks; ++blk) {
+            auto tb0 = clk::now();
+            FD_TRY(S.expand(B, p, z, ldz));
+            if (p == 0) {
+                if (blk > 0) break;                                // the continuation added nothing: back to the Ritz pairs
+                // the residuals lie (numerically) inside the basis: try a random direction, give up after a few
+                if (++stagnation > 3) { stuck = true; break; }
+                p = (int)std::min<int64_t>(std::min(b, m_cap - S.m), N - S.m);
+                FD_TRY(random_fill(c, S.R + r0, N, p, n, r0, 0xABCD1234u + (uint32_t)iter));
+                FD_TRY(S.expand(S.R, p, nullptr, 0));
+                if (p == 0) { stuck = true; break; }
+            }
+            auto tb1 = clk::now();
+            t_orth += secs(tb0, tb1);
+            FD_TRY(S.apply_cols(S.m, p, b));
+            auto tb2 = clk::now();
+            FD_TRY(S.extend_projection(p));
+            t_ext += secs(tb2, clk::now());
+            if (S.applies >= max_applies || S.m + p > m_cap || S.m + p > N) break;
+            // next block: M times this one; its projection [Q W_new]^T W_new was measured just now
+            B = S.W + (int64_t)(S.m - p) * N;
+            ldz = S.m + p;
+            zkeep.assign(S.h + (size_t)p * ldz, S.h + (size_t)2 * p * ldz);
+            z = zkeep.data();
         }
-        FD_TRY(copy_cols(c, S.R + r0, N, S.Q + (int64_t)S.m * N + r0, N, p, n));
-        auto tp5 = clk::now();
-        t_orth += secs(tp4, tp5);
-        FD_TRY(S.apply_cols(S.m, p, b));
-        auto tp6 = clk::now();
-        FD_TRY(S.extend_projection(p));
-        t_ext += secs(tp6, clk::now());
+        if (stuck) break;
     }
 
     // ---- outputs: evecs = Q X[:, 0 : k + 1) ----------------------------------------------------------
     const int nout = std::min(nwant, nsel);
     {
         const int m = S.m;
-        for (int c0 = 0; c0 < nout; c0 += S.BP) {
-            const int w = std::min(S.BP, nout - c0);
-            std::vector<float> Sx((size_t)m * w);
-            for (int jj = 0; jj < w; ++jj)
-                for (int i = 0; i < m; ++i) Sx[i + (size_t)jj * m] = (float)Xr[i + (size_t)(c0 + jj) * m];
-            FD_TRY(S.upload_S(Sx));
-            FD_TRY(nn_product(c, S.Q + r0, N, m, S.d_S, m, w, evecs_dev + (int64_t)c0 * ldv + r0, ldv, 1.f, 0.f, n));
-        }
+        float* Sx = nullptr;
+        const size_t cnt = (size_t)m * nout;
+        FD_TRY(S.stage_slot(cnt, &Sx));
+        for (size_t i = 0; i < cnt; ++i) Sx[i] = (float)Xr[i];
+        FD_TRY(S.send_slot(cnt));
+        FD_TRY(nn_product(c, S.own(S.Q, m), S.d_S, m, nout, evecs_dev + r0, ldv, n));
         FD_TRY(gather_rows(c, evecs_dev, ldv, nout));              // complete eigenvectors on every rank
         for (int i = 0; i < nwant; ++i) evals_host[i] = i < nout ? theta[i] : 0.0;
         FD_CUDA(c, cudaStreamSynchronize(c->stream));

@@ -32,7 +32,7 @@ struct Layout {
     size_t yacc = 0;
     size_t weights = 0;              // NP right weights of a Gram-form row sum
     size_t symsum = 0;               // N 64-bit fixed-point sums of the symmetric row-sum mode
-    size_t eig_q = 0, eig_w = 0, eig_x = 0, eig_r = 0, eig_t = 0, eig_small = 0, eig_small_doubles = 0;
+    size_t eig_q = 0, eig_w = 0, eig_x = 0, eig_r = 0, eig_small = 0, eig_small_doubles = 0;
     size_t total = 0;
 };
 Layout make_layout(int64_t N, int32_t D, int32_t b_max, int32_t m_max);
@@ -67,12 +67,14 @@ struct fd_ctx {
     fd_precision eigs_prec = FD_PREC_FP32;   // precision mode of fd_eigs's block products (set per stage by the cascade)
     double opt_tc_max_mag = 72.0;    // largest beta' * max|x - mu|^2 the Gram-form kernel is trusted with in fp32 mode
     std::string err;
-    // pinned host staging ring for the eigensolver's small uploads (allocated on the first fd_eigs, freed by fd_destroy:
-    // allocating and freeing page-locked memory on every call costs tens of milliseconds)
+    // page-locked host memory of the eigensolver: a ring of slots for its small uploads, then the projections, which kernels write
+    // there directly (one allocation, made by the first fd_eigs and freed by fd_destroy)
     static constexpr int kStageSlots = 4;
-    float* stage[kStageSlots] = {nullptr, nullptr, nullptr, nullptr};
+    float* stage = nullptr;
+    double* h_out = nullptr;
     cudaEvent_t stage_ev[kStageSlots] = {nullptr, nullptr, nullptr, nullptr};
-    size_t stage_floats = 0;
+    size_t stage_floats = 0;         // per slot
+    size_t h_out_doubles = 0;
     // row-sharded operation (fd_set_shard): this rank owns rows [r0, r1) of every quadratic pass
     struct Shard {
         bool on = false;
