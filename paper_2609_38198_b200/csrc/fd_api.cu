@@ -1,5 +1,6 @@
 // C-ABI entry points: context, degree passes, block product.  Argument checking and
 // dispatch only; every O(N^2) and O(N) step runs in this library's own kernels.
+#include <algorithm>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -53,8 +54,10 @@ Layout make_layout(int64_t N, int32_t D, int32_t b_max, int32_t m_max) {
     L.rowsq = carve(cur, (size_t)N * 8);
     L.sums = carve(cur, (size_t)(2 * 1024 + 8) * 8);
     L.wp = carve(cur, (size_t)N * L.BP * 4);
-    // split-J partials of the SIMT kernel: only small problems split, so this is O(b_max), not O(N b_max)
-    L.part_floats = (size_t)640 * 128 * (size_t)L.BP;
+    // shares of row tiles that a work range's cut falls into: two slots of 256 rows x the widest column tile per CTA (direct-difference
+    // kernels: up to four CTAs on each of 148 SMs, tensor-core product: one; never more CTAs than steps)
+    const int64_t steps = ceil_div(N, 256) * ceil_div(N, 16);
+    L.part_floats = (size_t)std::max<int64_t>(std::min<int64_t>(592, steps), 160) * 2 * 256 * (size_t)L.BP;
     L.part = carve(cur, L.part_floats * 4);
     // tensor-core operands: fp16 hi|lo rows of the augmented points, transposed fp16 hi / lo blocks
     L.xp_col = carve(cur, (size_t)L.NP * L.K16 * 64);
@@ -223,16 +226,14 @@ fd_status fd_degree(fd_ctx* c, double beta, double alpha, fd_precision prec, flo
     a.Y = c->q() + r0; a.ldy = N; a.rowsq = rowsq + r0; a.prec = prec;
     a.sym_ok = !c->sh.on;                                        // K = K^T, unit weights
     if (n > 0) FD_TRY(apply_dispatch(c, a));
-    double sums[2] = {0.0, 0.0};
-    if (n > 0) FD_TRY(reduce_sums(c, c->q() + r0, rowsq + r0, n, &sums[0], &sums[1]));
-    FD_TRY(allreduce_host(c, sums, 2));
+    // the two sums lie beside the tensor-core kernels' status word: one copy brings all three at the end
+    double* sums_dev = reinterpret_cast<double*>(c->at<char>(c->L.status) + 64);
+    if (n > 0) FD_TRY(reduce_sums(c, c->q() + r0, rowsq + r0, n, sums_dev));
     FD_TRY(gather_rows(c, c->q(), N, 1));
-    const double sum_q = sums[0], sum_sq = sums[1];
-    if (!(sum_q == sum_q) || !(sum_q < 1e300)) return fail(c, FD_ERR_NONFINITE, "non-finite degree sum");
+    const float* qa = nullptr;
     if (alpha == 0.0) {
         // d = q, s = q^-1/2
         FD_CUDA(c, cudaMemcpyAsync(c->d(), c->q(), (size_t)N * 4, cudaMemcpyDeviceToDevice, c->stream));
-        FD_TRY(ew_pow(c, c->q(), -0.5, c->s(), N));
     } else {
         // pass 2: d = q^-alpha * K q^-alpha
         FD_TRY(ew_pow(c, c->q(), -alpha, c->w(), N));
@@ -240,12 +241,17 @@ fd_status fd_degree(fd_ctx* c, double beta, double alpha, fd_precision prec, flo
         a2.left = c->w() + r0; a2.right = c->w(); a2.Y = c->d() + r0; a2.rowsq = nullptr; a2.right_pos = true;       // (sym_ok stays: left = right = q^-alpha in (0, 1])
         if (n > 0) FD_TRY(apply_dispatch(c, a2));
         FD_TRY(gather_rows(c, c->d(), N, 1));
-        FD_TRY(ew_scale_vec(c, c->w(), c->d(), c->s(), N));
+        qa = c->w();
     }
-    if (q_dev) FD_CUDA(c, cudaMemcpyAsync(q_dev, c->q(), (size_t)N * 4, cudaMemcpyDeviceToDevice, c->stream));
-    if (d_dev) FD_CUDA(c, cudaMemcpyAsync(d_dev, c->d(), (size_t)N * 4, cudaMemcpyDeviceToDevice, c->stream));
-    if (s_dev) FD_CUDA(c, cudaMemcpyAsync(s_dev, c->s(), (size_t)N * 4, cudaMemcpyDeviceToDevice, c->stream));
-    FD_TRY(tc_check_status(c));
+    FD_TRY(ew_scale_vec(c, qa, c->q(), c->d(), c->s(), N, q_dev, d_dev, s_dev));
+    struct { unsigned int status; unsigned int pad[15]; double sums[2]; } host;
+    FD_CUDA(c, cudaMemcpyAsync(&host, c->at<char>(c->L.status), sizeof host, cudaMemcpyDeviceToHost, c->stream));
+    FD_CUDA(c, cudaStreamSynchronize(c->stream));
+    if (n <= 0) host.sums[0] = host.sums[1] = 0.0;               // a rank that owns no rows
+    FD_TRY(allreduce_host(c, host.sums, 2));                     // (before the status is looked at: every rank takes this step)
+    if (host.status != 0) return tc_check_status(c);             // reports and clears it
+    const double sum_q = host.sums[0], sum_sq = host.sums[1];
+    if (!(sum_q == sum_q) || !(sum_q < 1e300)) return fail(c, FD_ERR_NONFINITE, "non-finite degree sum");
     // the diagonal of K is exactly 1 in both sums
     if (S_off_host) *S_off_host = sum_q - (double)N;
     if (S_off_2beta_host) *S_off_2beta_host = sum_sq - (double)N;

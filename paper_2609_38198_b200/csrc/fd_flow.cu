@@ -13,16 +13,13 @@ namespace {
 constexpr double kKappaP = 10.0;     // Eq. 11
 constexpr int kPExponent = 6;        // Eq. 11
 
-// out[i + j * ldout] /= lambda[j] * den[i]
-__global__ void k_nystrom_finish(float* __restrict__ out, int64_t ldout, int m, const float* __restrict__ den,
-                                 const double* __restrict__ lambda, int64_t n) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// out[i + j * ldout] = num[i + j * n] / (lambda[j] * num[i + m * n]): column m of the product is the denominator.
+struct Lambdas { double v[64]; };
+__global__ void k_nystrom_finish(const float* __restrict__ num, float* __restrict__ out, int64_t ldout, int m, const Lambdas lambda, int64_t n) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const double dn = (double)den[i];
-    for (int j = 0; j < m; ++j) {
-        float* o = out + i + (int64_t)j * ldout;
-        *o = (float)((double)*o / (lambda[j] * dn));
-    }
+    const double dn = (double)num[i + (int64_t)m * n];
+    for (int j = 0; j < m; ++j) out[i + (int64_t)j * ldout] = (float)((double)num[i + (int64_t)j * n] / (lambda.v[j] * dn));
 }
 
 double median_of(std::vector<double> v) {
@@ -208,24 +205,29 @@ extern "C" fd_status fd_nystrom(fd_ctx* c, const float* Xnew_dev, int64_t Nnew, 
     for (int j = 0; j < m; ++j)
         if (!(std::fabs(lambda_host[j]) > 1e-30)) return fail(c, FD_ERR_INVALID, "fd_nystrom: zero eigenvalue");
     const int64_t N = c->L.N;
-    // right scaling q^-alpha (scratch vector w), eigenvalues to the device (scratch: sums buffer)
+    // Numerators and denominator of the formula are columns of one rectangular product: right block [psi | 1] scaled by q^-alpha
+    // (scratch vector w).  N = 65536, D = 30, 40009 new points, 33 vectors: 2.83 -> 1.2 ms against a row-sum pass of its own for the
+    // denominator.  A chunk has one column less than the block buffers hold.
     FD_TRY(ew_pow(c, c->q(), -c->alpha, c->w(), N));
-    double* lam_dev = c->at<double>(c->L.sums);
-    FD_CUDA(c, cudaMemcpyAsync(lam_dev, lambda_host, sizeof(double) * (size_t)m, cudaMemcpyHostToDevice, c->stream));
-    FD_CUDA(c, cudaStreamSynchronize(c->stream));
-    float* den = c->at<float>(c->L.rowsq);                                  // N doubles of scratch = room for N floats
+    const int cap = std::min(c->L.BP, 64) - 1;
+    const int chunks = (m + cap - 1) / cap, step = (m + chunks - 1) / chunks;
     for (int64_t r0 = 0; r0 < Nnew; r0 += N) {
         const int64_t n = std::min(N, Nnew - r0);
-        const float* xr = Xnew_dev + r0 * ldxnew;
-        // the denominator's right vector q^-alpha is positive: it may take the same kernel family as the numerators
-        FD_TRY(apply_general(c, c->beta, nullptr, c->w(), true, xr, n, ldxnew, nullptr, N, 1, den, n, FD_PREC_FP32));
-        for (int c0 = 0; c0 < m; c0 += c->L.b_max) {
-            const int w = std::min<int>(c->L.b_max, m - c0);
-            FD_TRY(fd_apply_general(c, c->beta, nullptr, c->w(), xr, n, ldxnew, psi_dev + (int64_t)c0 * ldpsi, ldpsi, w,
-                                    out_dev + r0 + (int64_t)c0 * ldout, ldout, FD_PREC_FP32));
+        FD_TRY(stage_rows(c, Xnew_dev, ldxnew, r0, n));
+        for (int c0 = 0; c0 < m; c0 += step) {
+            const int w = std::min(step, m - c0);
+            ApplyArgs a{};
+            a.xrow = c->at<float>(c->L.xrow); a.Nrow = n; a.rows_are_ctx = false;
+            a.beta = c->beta; a.right = c->w(); a.right_pos = true; a.prec = FD_PREC_FP32;
+            a.V = psi_dev + (int64_t)c0 * ldpsi; a.ldv = ldpsi; a.b = w + 1; a.ones_last = true;
+            float* num = c->at<float>(c->L.wp);
+            a.Y = num; a.ldy = n;
+            FD_TRY(apply_dispatch(c, a));
+            Lambdas lam;
+            for (int j = 0; j < w; ++j) lam.v[j] = lambda_host[c0 + j];
+            k_nystrom_finish<<<(unsigned)ceil_div(n, 256), 256, 0, c->stream>>>(num, out_dev + r0 + (int64_t)c0 * ldout, ldout, w, lam, n);
+            FD_LAUNCH_CHECK(c, "k_nystrom_finish");
         }
-        k_nystrom_finish<<<(unsigned)ceil_div(n, 256), 256, 0, c->stream>>>(out_dev + r0, ldout, m, den, lam_dev, n);
-        FD_LAUNCH_CHECK(c, "k_nystrom_finish");
     }
     FD_CUDA(c, cudaStreamSynchronize(c->stream));
     return FD_OK;

@@ -27,7 +27,8 @@ struct Layout {
     int64_t NP = 0;                  // N rounded up to the tensor-core column tile
     int32_t K16 = 0;                 // 16-wide K slabs of the augmented Gram operand
     size_t xs = 0, xrow = 0, mu = 0, q = 0, d = 0, s = 0, w = 0, rowsq = 0, sums = 0;
-    size_t wp = 0, part = 0, part_floats = 0;
+    size_t wp = 0;                   // N x BP block of scratch (numerators and denominator of the out-of-sample extension)
+    size_t part = 0, part_floats = 0;
     size_t xp_col = 0, xp_row = 0, wt_hi = 0, wt_lo = 0, colscale = 0, status = 0;
     size_t yacc = 0;
     size_t weights = 0;              // NP right weights of a Gram-form row sum
@@ -133,6 +134,7 @@ struct ApplyArgs {
     const float* V; int64_t ldv; int32_t b;
     float* Y; int64_t ldy;
     double* rowsq;                          // optional: sum_j K_ij^2 per row (rowsum mode, b = 1, V null)
+    bool ones_last;                         // block mode: column b - 1 of the block is the ones vector, V holds the others
     bool right_pos;                         // caller guarantees right > 0 elementwise
     bool sym_ok;                            // square pass with left == right, weights in (0, 1]: the symmetric half-work row sums may serve it
     fd_precision prec;
@@ -162,10 +164,11 @@ fd_status tc_wait_selftest(fd_ctx* c, long long limit_cycles);
 
 // ---- small kernels (fd_elementwise.cu) ------------------------------------------------------
 fd_status ew_pow(fd_ctx* c, const float* in, double p, float* out, int64_t n);            // out = in^p
-fd_status ew_scale_vec(fd_ctx* c, const float* qa, const float* d, float* s, int64_t n);  // s = qa * d^-1/2
+// s = qa * d^-1/2 (qa null: 1); also copies q, d, s to the outputs that are not null.
+fd_status ew_scale_vec(fd_ctx* c, const float* qa, const float* q, const float* d, float* s, int64_t n, float* q_out, float* d_out, float* s_out);
 fd_status ew_fill(fd_ctx* c, float* out, float v, int64_t n);
-// Deterministic fp64 sums of a float vector and a double vector (two-stage tree).  Synchronises.
-fd_status reduce_sums(fd_ctx* c, const float* q, const double* rowsq, int64_t n, double* sum_q, double* sum_sq);
+// Deterministic fp64 sums of a float vector and a double vector (two-stage tree) -> out_dev[0], out_dev[1].
+fd_status reduce_sums(fd_ctx* c, const float* q, const double* rowsq, int64_t n, double* out_dev);
 fd_status scale_cols_by_pow(fd_ctx* c, const float* v, int64_t ldv, int32_t cols, const float* d, double p,
                             float* out, int64_t ldout, int64_t n);
 

@@ -72,9 +72,16 @@ __global__ void k_pow(const float* __restrict__ in, double p, float* __restrict_
     }
 }
 
-__global__ void k_scale_vec(const float* __restrict__ qa, const float* __restrict__ d, float* __restrict__ s, int64_t n) {
+// s = qa * d^-1/2 (qa null: 1), and copies of q, d, s where they are wanted.
+__global__ void k_scale_vec(const float* __restrict__ qa, const float* __restrict__ q, const float* __restrict__ d, float* __restrict__ s, int64_t n,
+                            float* __restrict__ q_out, float* __restrict__ d_out, float* __restrict__ s_out) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) s[i] = (float)((double)qa[i] / sqrt((double)d[i]));
+    if (i >= n) return;
+    const float di = d[i], v = (float)((qa ? (double)qa[i] : 1.0) / sqrt((double)di));
+    s[i] = v;
+    if (q_out) q_out[i] = q[i];
+    if (d_out) d_out[i] = di;
+    if (s_out) s_out[i] = v;
 }
 
 __global__ void k_fill(float* __restrict__ out, float v, int64_t n) {
@@ -101,12 +108,19 @@ __global__ void k_sum_partial(const float* __restrict__ q, const double* __restr
     if (threadIdx.x == 0) { part[2 * blockIdx.x] = s_a[0]; part[2 * blockIdx.x + 1] = s_b[0]; }
 }
 
-__global__ void k_sum_final(const double* __restrict__ part, int blocks, double* __restrict__ out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double a = 0.0, b = 0.0;
-        for (int i = 0; i < blocks; ++i) { a += part[2 * i]; b += part[2 * i + 1]; }
-        out[0] = a; out[1] = b;
+// Fixed order: 256 strided sums, then a tree.
+__global__ void __launch_bounds__(256)
+k_sum_final(const double* __restrict__ part, int blocks, double* __restrict__ out) {
+    __shared__ double s_a[256], s_b[256];
+    double a = 0.0, b = 0.0;
+    for (int i = threadIdx.x; i < blocks; i += 256) { a += part[2 * i]; b += part[2 * i + 1]; }
+    s_a[threadIdx.x] = a; s_b[threadIdx.x] = b;
+    __syncthreads();
+    for (int off = 128; off > 0; off >>= 1) {
+        if ((int)threadIdx.x < off) { s_a[threadIdx.x] += s_a[threadIdx.x + off]; s_b[threadIdx.x] += s_b[threadIdx.x + off]; }
+        __syncthreads();
     }
+    if (threadIdx.x == 0) { out[0] = s_a[0]; out[1] = s_b[0]; }
 }
 
 __global__ void k_scale_cols_pow(const float* __restrict__ v, int64_t ldv, int cols, const float* __restrict__ d, double p,
@@ -187,8 +201,8 @@ fd_status ew_pow(fd_ctx* c, const float* in, double p, float* out, int64_t n) {
     return FD_OK;
 }
 
-fd_status ew_scale_vec(fd_ctx* c, const float* qa, const float* d, float* s, int64_t n) {
-    k_scale_vec<<<grid_for(n, 256), 256, 0, c->stream>>>(qa, d, s, n);
+fd_status ew_scale_vec(fd_ctx* c, const float* qa, const float* q, const float* d, float* s, int64_t n, float* q_out, float* d_out, float* s_out) {
+    k_scale_vec<<<grid_for(n, 256), 256, 0, c->stream>>>(qa, q, d, s, n, q_out, d_out, s_out);
     FD_LAUNCH_CHECK(c, "k_scale_vec");
     return FD_OK;
 }
@@ -199,17 +213,13 @@ fd_status ew_fill(fd_ctx* c, float* out, float v, int64_t n) {
     return FD_OK;
 }
 
-fd_status reduce_sums(fd_ctx* c, const float* q, const double* rowsq, int64_t n, double* sum_q, double* sum_sq) {
+fd_status reduce_sums(fd_ctx* c, const float* q, const double* rowsq, int64_t n, double* out_dev) {
     double* sums = c->at<double>(c->L.sums);
     int nb = grid_for(n, 256, kRedBlocks);
     k_sum_partial<<<nb, 256, 0, c->stream>>>(q, rowsq, n, sums);
     FD_LAUNCH_CHECK(c, "k_sum_partial");
-    k_sum_final<<<1, 32, 0, c->stream>>>(sums, nb, sums + 2 * kRedBlocks);
+    k_sum_final<<<1, 256, 0, c->stream>>>(sums, nb, out_dev);
     FD_LAUNCH_CHECK(c, "k_sum_final");
-    double host[2];
-    FD_CUDA(c, cudaMemcpyAsync(host, sums + 2 * kRedBlocks, sizeof host, cudaMemcpyDeviceToHost, c->stream));
-    FD_CUDA(c, cudaStreamSynchronize(c->stream));
-    *sum_q = host[0]; *sum_sq = host[1];
     return FD_OK;
 }
 

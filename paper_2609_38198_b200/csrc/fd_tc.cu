@@ -345,13 +345,17 @@ __global__ void k_pad_weights(const float* __restrict__ w, int64_t n, int64_t np
     if (j < np) out[j] = j < n ? (w ? w[j] : 1.f) : 0.f;
 }
 
-// Per-block maxima of |right_j V_jc| for each column c.
+// Per-block maxima of |right_j V_jc| for each column c (columns from vcols on are the ones vector).
 __global__ void __launch_bounds__(256)
-k_colmax_partial(const float* __restrict__ V, int64_t ldv, const float* __restrict__ right, int64_t N, int c0, float* __restrict__ part) {
+k_colmax_partial(const float* __restrict__ V, int64_t ldv, int vcols, const float* __restrict__ right, int64_t N, int c0, float* __restrict__ part) {
     __shared__ float sm[8];
-    const float* v = V + (int64_t)(c0 + blockIdx.y) * ldv;
+    const bool ones = c0 + (int)blockIdx.y >= vcols;
+    const float* v = V + (int64_t)(ones ? 0 : c0 + blockIdx.y) * ldv;
     float m = 0.f;
-    for (int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x; j < N; j += (int64_t)gridDim.x * 256) m = fmaxf(m, fabsf(right ? v[j] * right[j] : v[j]));
+    for (int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x; j < N; j += (int64_t)gridDim.x * 256) {
+        const float x = ones ? 1.f : v[j];
+        m = fmaxf(m, fabsf(right ? x * right[j] : x));
+    }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
     if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
@@ -367,7 +371,7 @@ k_colmax_partial(const float* __restrict__ V, int64_t ldv, const float* __restri
 // j >= N and c >= bc.  scale_c = the power of two that puts the column maximum in [2^12, 2^13): every block reduces the
 // partial maxima of its column itself (they are at most 256 values); the first one stores the epilogue factor 2^-bias / scale.
 __global__ void __launch_bounds__(256)
-k_pack_wt(const float* __restrict__ V, int64_t ldv, const float* __restrict__ right, int64_t N, int64_t np, int c0, int bc,
+k_pack_wt(const float* __restrict__ V, int64_t ldv, int vcols, const float* __restrict__ right, int64_t N, int64_t np, int c0, int bc,
           const float* __restrict__ part, int parts, float* __restrict__ inv, __half* __restrict__ wt, int with_lo) {
     __shared__ float sm[8];
     const int c = blockIdx.y;
@@ -386,7 +390,8 @@ k_pack_wt(const float* __restrict__ V, int64_t ldv, const float* __restrict__ ri
         sc = ldexpf(1.0f, 13 - e);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) inv[c] = ldexpf(1.0f, -kBias) / sc;
-    const float* v = V + (int64_t)(c0 + (c < bc ? c : 0)) * ldv;
+    const bool ones = c0 + c >= vcols;
+    const float* v = V + (int64_t)(ones ? 0 : c0 + c) * ldv;
     __half2* hi = reinterpret_cast<__half2*>(wt + (int64_t)c * np);
     __half2* lo = reinterpret_cast<__half2*>(wt + (int64_t)(gridDim.y + c) * np);
     for (int64_t j2 = (int64_t)blockIdx.x * 256 + threadIdx.x; j2 < np / 2; j2 += (int64_t)gridDim.x * 256) {
@@ -395,7 +400,10 @@ k_pack_wt(const float* __restrict__ V, int64_t ldv, const float* __restrict__ ri
         for (int u = 0; u < 2; ++u) {
             const int64_t j = 2 * j2 + u;
             x[u] = 0.f;
-            if (c < bc && j < N) x[u] = (right ? v[j] * right[j] : v[j]) * sc;
+            if (c < bc && j < N) {
+                const float y = ones ? 1.f : v[j];
+                x[u] = (right ? y * right[j] : y) * sc;
+            }
         }
         const __half2 h = __floats2half2_rn(x[0], x[1]);
         hi[j2] = h;
@@ -532,6 +540,7 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
         float* inv = c->at<float>(L.colscale);
         float* part = c->at<float>(L.part);
         const bool fast = a.prec == FD_PREC_FAST;
+        const int vcols = a.ones_last ? a.b - 1 : a.b;
         // column chunks of at most 64, of about equal width (multiples of 16)
         const int cw = fast ? 64 : (int)round_up(ceil_div(a.b, ceil_div(a.b, 64)), 16);
         for (int c0 = 0; c0 < a.b; c0 += cw) {
@@ -539,10 +548,10 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
             const int BT = bc <= 16 ? 16 : bc <= 32 ? 32 : bc <= 48 && !fast ? 48 : 64;
             if (BT > L.BP) return fail(c, FD_ERR_WORKSPACE, "column tile %d wider than the provisioned block buffers (%d)", BT, L.BP);
             const int cm_blocks = (int)std::min<int64_t>(256, ceil_div(N, 1024));
-            k_colmax_partial<<<dim3(cm_blocks, bc), 256, 0, c->stream>>>(a.V, a.ldv, a.right, N, c0, part);
+            k_colmax_partial<<<dim3(cm_blocks, bc), 256, 0, c->stream>>>(a.V, a.ldv, vcols, a.right, N, c0, part);
             FD_LAUNCH_CHECK(c, "k_colmax_partial");
             k_pack_wt<<<dim3((unsigned)std::min<int64_t>(1024, ceil_div(NP, 512)), BT), 256, 0, c->stream>>>(
-                a.V, a.ldv, a.right, N, NP, c0, bc, part, cm_blocks, inv, wt_hi, fast ? 0 : 1);
+                a.V, a.ldv, vcols, a.right, N, NP, c0, bc, part, cm_blocks, inv, wt_hi, fast ? 0 : 1);
             FD_LAUNCH_CHECK(c, "k_pack_wt");
             // one map over W_hi (rows 0 .. BT) and, in the fp32-grade mode, W_lo behind it (rows BT .. 2 BT of the same array)
             if (!make_map_2d(&mh, wt_hi, (uint64_t)NP, (uint64_t)(fast ? BT : 2 * BT), (uint64_t)NP * 2, 64, fast ? BT : 2 * BT, CU_TENSOR_MAP_SWIZZLE_128B))

@@ -65,3 +65,55 @@ def test_symmetric_row_sums_against_every_tile(N, D, beta):
         assert ((a - b).abs() / b).max().item() <= 1e-6
     assert abs(so1 - so0) <= 1e-6 * (so0 + N) and abs(sq1 - sq0) <= 1e-6 * (sq0 + N)
     ctx.close()
+
+
+@pytest.mark.parametrize("N,D,b,splits", [
+    (1, 2, 1, 0), (255, 3, 5, 0), (257, 4, 24, 0), (2049, 2, 8, 0), (4200, 4, 16, 1), (4200, 12, 33, 1), (4200, 16, 64, 1), (2305, 30, 48, 0), (5003, 12, 100, 0),
+])
+def test_direct_difference_edges(N, D, b, splits):
+    """Direct-difference kernels at the edges of their row tiles (256) and column tiles (64), of the work ranges (fewer steps than CTAs,
+    cuts inside row tiles; splits = 1: whole row tiles, so more than 32 column tiles are summed in two levels), of the column
+    widths (4 ... 64, balanced chunks) and of the four-row / two-row layouts.  fp32 products against float64: 1e-6 relative Frobenius
+    (2^-24 per operation, at most 64 x 32 terms per fp32 level, random signs)."""
+    import __graft_entry__ as g
+    g.build()
+    import paper_2609_38198_b200 as fd
+    dev = torch.device("cuda:0")
+    X = workloads.gaussian_cloud(N, D, seed=N, scale=0.7)
+    V = workloads.block(N, b, seed=b)
+    ctx = fd.Context(torch.from_numpy(X).to(dev), b_max=b)
+    ctx.set_option("path", fd.FD_PATH_SIMT)
+    ctx.set_option("splits", splits)
+    beta = 0.8
+    q, d, s, so, so2 = ctx.degree(beta, 1.0)
+    Y = ctx.apply(fd.to_colmajor(V, dev))
+    Y2 = ctx.apply(fd.to_colmajor(V, dev))
+    ctx.synchronize()
+    assert torch.equal(Y, Y2)
+    qo, do, s_o, soo, so2o = dense.degree(X, beta, 1.0)
+    assert np.abs(q.cpu().numpy() / qo - 1).max() <= 1e-6 and np.abs(d.cpu().numpy() / do - 1).max() <= 2e-6
+    assert abs(so2 - so2o) <= 2e-6 * (so2o + N)
+    Yo = dense.apply(X, beta, 1.0, V)
+    assert np.linalg.norm(Y.cpu().numpy().astype(np.float64) - Yo) <= 1e-6 * np.linalg.norm(Yo)
+    ctx.close()
+
+
+@pytest.mark.parametrize("path,m,b_max", [(1, 1, 16), (1, 15, 16), (1, 16, 16), (2, 33, 64), (2, 64, 64), (2, 31, 32), (2, 70, 64)])
+def test_extension_column_chunks(path, m, b_max):
+    """Out-of-sample extension, whose product carries the denominator as one more column: block buffers just wide enough, one column
+    too narrow, several chunks.  Ratio of two products of the same kernel values: 1e-5 entrywise of the largest value."""
+    import __graft_entry__ as g
+    g.build()
+    import paper_2609_38198_b200 as fd
+    from oracle import nystrom
+    dev = torch.device("cuda:0")
+    X, Z = workloads.torus6(1500, seed=5), workloads.torus6(401, seed=6)
+    psi, lam = workloads.block(1500, m, seed=2), np.linspace(1.0, 0.3, m)
+    ctx = fd.Context(torch.from_numpy(X).to(dev), b_max=b_max)
+    ctx.set_option("path", path)
+    q, d, s, so, so2 = ctx.degree(1.0, 1.0)
+    out = ctx.nystrom(torch.from_numpy(Z).to(dev), fd.to_colmajor(psi, dev), lam).cpu().numpy()
+    qo = dense.degree(X, 1.0, 1.0)[0]
+    ref = nystrom.extend(X, qo, 1.0, 1.0, psi.astype(np.float64), lam, Z)
+    assert np.abs(out - ref).max() <= 1e-5 * np.abs(ref).max()
+    ctx.close()
