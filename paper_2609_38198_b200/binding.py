@@ -129,20 +129,39 @@ def fd_version() -> int:
 
 
 def _ptr(t):
-    return None if t is None else c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+class _NoSwitch:
+    def __enter__(self):
+        return None
+
+    def __exit__(self, *exc):
+        return False
+
+
+_NO_SWITCH = _NoSwitch()
+
+
+def _on(device: torch.device):
+    """Makes `device` current for a call; costs nothing when it is current already (a small product takes about as long as the
+    switch back and forth)."""
+    return _NO_SWITCH if torch.cuda.current_device() == device.index else torch.cuda.device(device)
 
 
 def _colmajor(rows: int, cols: int, device) -> torch.Tensor:
     """(rows x cols) float32 tensor whose storage is column-major (ld = rows)."""
-    return torch.empty((cols, rows), dtype=torch.float32, device=device).t()
+    return torch.empty_strided((rows, cols), (1, rows), dtype=torch.float32, device=device)
 
 
 def _ld(t: torch.Tensor) -> int:
     """Leading dimension of a column-major 2-D (or 1-D) float32 tensor."""
     if t.dim() == 1:
         return t.shape[0]
-    assert t.dim() == 2 and t.stride(0) == 1, "blocks must be column-major (use .t() of a contiguous (cols, rows) tensor)"
-    return t.stride(1) if t.shape[1] > 1 else max(t.shape[0], t.stride(1))
+    s0, s1 = t.stride()
+    assert s0 == 1, "blocks must be column-major (use .t() of a contiguous (cols, rows) tensor)"
+    rows, cols = t.shape
+    return s1 if cols > 1 else max(rows, s1)
 
 
 class Context:
@@ -157,7 +176,7 @@ class Context:
         if nbytes == 0:
             raise FdError(FD_ERR_INVALID, "fd_workspace_bytes rejected the shape")
         self.workspace_bytes = nbytes
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             self._ws = torch.empty(nbytes + 256, dtype=torch.uint8, device=self.device)
             off = (-self._ws.data_ptr()) % 256
             self._stream = stream if stream is not None else torch.cuda.current_stream(self.device)
@@ -180,7 +199,7 @@ class Context:
             pass
 
     def _check(self, st: int, ok=(FD_OK,)):
-        if st not in ok:
+        if st != FD_OK and st not in ok:
             shard = getattr(self, "_shard", None)
             if st == FD_ERR_COMM and shard is not None and shard.error is not None:
                 err, shard.error = shard.error, None
@@ -213,12 +232,12 @@ class Context:
         """Returns (q, d, s, S_off(beta), S_off(2 beta))."""
         q, d, s = (torch.empty(self.N, dtype=torch.float32, device=self.device) for _ in range(3))
         so, so2 = c_double(), c_double()
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             self._check(lib.fd_degree(self._h, beta, alpha, prec, _ptr(q), _ptr(d), _ptr(s), byref(so), byref(so2)))
         return q, d, s, so.value, so2.value
 
     def synchronize(self):
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             self._check(lib.fd_synchronize(self._h))
 
     def apply(self, V: torch.Tensor, out: torch.Tensor | None = None, prec: int = FD_PREC_FP32) -> torch.Tensor:
@@ -226,7 +245,7 @@ class Context:
             V = V[:, None]
         b = V.shape[1]
         Y = out if out is not None else _colmajor(self.N, b, self.device)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             self._check(lib.fd_apply(self._h, _ptr(V), _ld(V), b, _ptr(Y), _ld(Y), prec))
         return Y
 
@@ -237,7 +256,7 @@ class Context:
         b = 1 if V is None else V.shape[1]
         nrow = self.N if Xrow is None else int(Xrow.shape[0])
         Y = out if out is not None else _colmajor(nrow, b, self.device)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             self._check(lib.fd_apply_general(self._h, beta, _ptr(left), _ptr(right), _ptr(Xrow), nrow,
                                              0 if Xrow is None else Xrow.stride(0), _ptr(V),
                                              self.N if V is None else _ld(V), b, _ptr(Y), _ld(Y), prec))
@@ -250,7 +269,7 @@ class Context:
         ev = (c_double * (k + 1))()
         U = _colmajor(self.N, k + 1, self.device)
         info = fd_eigs_info()
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             st = lib.fd_eigs(self._h, k, b, tol, max_applies, _ptr(Q0), 0 if Q0 is None else _ld(Q0),
                              0 if Q0 is None else Q0.shape[1], ev, _ptr(U), _ld(U), byref(info))
         self._check(st, ok=(FD_OK, FD_ERR_NOT_CONVERGED) if allow_not_converged else (FD_OK,))
@@ -268,7 +287,7 @@ class Context:
         bx = c_double()
         ev = (c_double * (k + 1))()
         U = _colmajor(self.N, k + 1, self.device)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             st = lib.fd_beta_flow(self._h, byref(opts), _ptr(Q0), 0 if Q0 is None else _ld(Q0),
                                   0 if Q0 is None else Q0.shape[1], log, byref(n), byref(outcome), byref(bx), ev,
                                   _ptr(U), _ld(U))
@@ -293,7 +312,7 @@ class Context:
         bx = c_double()
         ev = (c_double * (k + 1))()
         U = _colmajor(self.N, k + 1, self.device)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             st = lib.fd_beta_flow_cascade(self._h, byref(opts), st_arr, ns, _ptr(Q0), 0 if Q0 is None else _ld(Q0),
                                           0 if Q0 is None else Q0.shape[1], log, byref(n), first, byref(outcome), byref(bx),
                                           ev, _ptr(U), _ld(U))
@@ -306,7 +325,7 @@ class Context:
         m = psi.shape[1]
         lam = (c_double * m)(*[float(v) for v in evals])
         out = _colmajor(int(Xnew.shape[0]), m, self.device)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             self._check(lib.fd_nystrom(self._h, _ptr(Xnew), Xnew.shape[0], Xnew.stride(0), _ptr(psi), _ld(psi), m, lam,
                                        _ptr(out), _ld(out)))
         return out
@@ -316,14 +335,14 @@ class Context:
         m = evecs_old.shape[1]
         lam = (c_double * m)(*[float(v) for v in evals])
         Q0 = _colmajor(self.N, m, self.device)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             self._check(lib.fd_ladder_start(old._h, self._h, _ptr(Xnew), Xnew.stride(0), _ptr(evecs_old), _ld(evecs_old), m,
                                             lam, _ptr(Q0), _ld(Q0)))
         return Q0
 
     def scale_by_degree(self, v: torch.Tensor, power: float) -> torch.Tensor:
         out = _colmajor(self.N, v.shape[1], self.device)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             self._check(lib.fd_scale_by_degree(self._h, _ptr(v), _ld(v), v.shape[1], power, _ptr(out), _ld(out)))
         return out
 
@@ -343,7 +362,7 @@ def fd_apply_general_static(X: torch.Tensor, beta: float, V: torch.Tensor, left=
     N, D, b = int(X.shape[0]), int(X.shape[1]), int(V.shape[1])
     Y = out if out is not None else _colmajor(N, b, X.device)
     err = ctypes.create_string_buffer(256)
-    with torch.cuda.device(X.device):
+    with _on(X.device):
         st = lib.fd_apply_general_static(_ptr(X), N, D, X.stride(0), float(beta), _ptr(left), _ptr(right), _ptr(V), _ld(V), b,
                                          _ptr(Y), _ld(Y), c_void_p(torch.cuda.current_stream(X.device).cuda_stream), err, 256)
     if st != FD_OK:

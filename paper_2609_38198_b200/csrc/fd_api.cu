@@ -319,7 +319,8 @@ fd_status apply_general(fd_ctx* c, double beta, const float* left_dev, const flo
         int64_t n = Nrow - r0 < N ? Nrow - r0 : N;
         FD_TRY(stage_rows(c, Xrow_dev, ldxrow, r0, n));
         a.xrow = c->at<float>(c->L.xrow); a.Nrow = n; a.rows_are_ctx = false;
-        a.left = left_dev ? left_dev + r0 : nullptr; a.Y = Y_dev + r0; a.ldy = ldy;
+        FD_TRY(row_factor(c, left_dev ? left_dev + r0 : nullptr, beta, n, &a.left));
+        a.Y = Y_dev + r0; a.ldy = ldy;
         FD_TRY(apply_dispatch(c, a));
     }
     return FD_OK;

@@ -38,6 +38,13 @@ struct Layout {
 };
 Layout make_layout(int64_t N, int32_t D, int32_t b_max, int32_t m_max);
 
+// Coordinates the kernels work on (keep[0 .. kept)) and those left out because all points share them, with the shared values.
+struct Coords {
+    int kept, dropped;
+    uint8_t keep[64], drop[64];
+    float value[64];
+};
+
 }  // namespace fd
 
 struct fd_ctx {
@@ -49,6 +56,8 @@ struct fd_ctx {
     int centered = 0;
     double mean_sq = 0.0;            // N^-1 sum |x_i - mu|^2 (Eq. 7)
     double max_sq = 0.0;             // max_i |x_i - mu|^2
+    fd::Coords coords{};             // L.DP and L.K16 count the kept coordinates (L.D: the caller's)
+    bool row_extra = false;          // the external rows staged most recently differ from the points in a dropped coordinate
     double row_max_sq = 0.0;         // the same maximum over the external rows staged most recently (rectangular products)
     // current operator state (set by fd_degree)
     bool have_s = false;
@@ -122,6 +131,10 @@ fd_status cuda_fail(fd_ctx* c, cudaError_t e, const char* what);
 fd_status setup_points(fd_ctx* c, const float* X_dev, int64_t ldx);
 // Padded copy of an external row set into the row scratch (rows [r0, r0 + n)).
 fd_status stage_rows(fd_ctx* c, const float* Xrow_dev, int64_t ldxrow, int64_t r0, int64_t n);
+
+// Left scaling of a rectangular product over the rows staged most recently: left_i exp(-beta e_i), e_i = the row's squared distance
+// from the points in the dropped coordinates; *out = left itself when all e_i are 0.
+fd_status row_factor(fd_ctx* c, const float* left, double beta, int64_t n, const float** out);
 
 // ---- quadratic passes -----------------------------------------------------------------------
 // General product on rows [0, Nrow) of `xrow` (padded N x DP layout, device) against the context's

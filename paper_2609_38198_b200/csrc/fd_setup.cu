@@ -1,5 +1,8 @@
 // O(N D) set-up: padded copy of the points, fp64 column means, mean and max of |x - mu|^2
 // (the statistic Eq. 7 needs), and the O(N) elementwise / reduction helpers of the degree pass.
+#include <algorithm>
+#include <cstring>
+
 #include "fd_internal.h"
 
 namespace fd {
@@ -8,32 +11,106 @@ namespace {
 
 constexpr int kRedBlocks = 1024;
 
-// dst[i * DP + k] = src[i * ld + k] for k < D, zero padding for D <= k < DP.
-__global__ void k_pad_copy(const float* __restrict__ src, int64_t ld, int64_t n, int D, int DP, float* __restrict__ dst) {
+// dst[i * DP + k] = src[i * ld + keep[k]] for the kept coordinates, zero padding up to DP.
+__global__ void k_pad_copy(const float* __restrict__ src, int64_t ld, int64_t n, const Coords co, int DP, float* __restrict__ dst) {
     int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int64_t total = n * DP;
     for (; idx < total; idx += (int64_t)gridDim.x * blockDim.x) {
         int64_t i = idx / DP;
         int k = (int)(idx - i * DP);
-        dst[idx] = k < D ? src[i * ld + k] : 0.0f;
+        dst[idx] = k < co.kept ? src[i * ld + co.keep[k]] : 0.0f;
     }
 }
 
-// Stage 1 of the column sums: block b sums rows b, b + gridDim.x, ... into part[b * DP + k] (fp64).
-__global__ void k_colsum_partial(const float* __restrict__ xs, int64_t n, int DP, double* __restrict__ part) {
-    for (int k = threadIdx.x; k < DP; k += blockDim.x) {
-        double acc = 0.0;
-        for (int64_t i = blockIdx.x; i < n; i += gridDim.x) acc += (double)xs[i * DP + k];
+// Column sums, minima and maxima.  Threads run along the rows' contiguous storage (thread t: coordinate t % DP of every
+// (256 / DP)-th row of the block's share), one partial result per block and coordinate.
+__global__ void __launch_bounds__(256)
+k_colsum_partial(const float* __restrict__ xs, int64_t n, int DP, double* __restrict__ part, float2* __restrict__ minmax) {
+    __shared__ double s_sum[256];
+    __shared__ float2 s_mm[256];
+    const int groups = 256 / DP, k = threadIdx.x % DP, g = threadIdx.x / DP;
+    double acc = 0.0;
+    float lo = INFINITY, hi = -INFINITY;
+    if (g < groups)
+        for (int64_t i = (int64_t)blockIdx.x * groups + g; i < n; i += (int64_t)gridDim.x * groups) {
+            const float v = xs[i * DP + k];
+            acc += (double)v;
+            lo = fminf(lo, v); hi = fmaxf(hi, v);
+        }
+    s_sum[threadIdx.x] = acc; s_mm[threadIdx.x] = make_float2(lo, hi);
+    __syncthreads();
+    if (g == 0) {
+        for (int q = 1; q < groups; ++q) {
+            acc += s_sum[q * DP + k];
+            lo = fminf(lo, s_mm[q * DP + k].x); hi = fmaxf(hi, s_mm[q * DP + k].y);
+        }
         part[(size_t)blockIdx.x * DP + k] = acc;
+        minmax[(size_t)blockIdx.x * DP + k] = make_float2(lo, hi);
     }
 }
 
-__global__ void k_colsum_final(const double* __restrict__ part, int blocks, int DP, int64_t n, int center, double* __restrict__ mu) {
-    for (int k = threadIdx.x; k < DP; k += blockDim.x) {
-        double acc = 0.0;
-        for (int b = 0; b < blocks; ++b) acc += part[(size_t)b * DP + k];
-        mu[k] = center ? acc / (double)n : 0.0;
+// mu, and a mask of the coordinates that are not the same for all points (bit k; written as a double's bits to *varying).
+__global__ void __launch_bounds__(1024)
+k_colsum_final(const double* __restrict__ part, const float2* __restrict__ minmax, int blocks, int DP, int64_t n, int center, double* __restrict__ mu,
+               unsigned long long* __restrict__ varying) {
+    __shared__ double s_sum[16][64];
+    __shared__ float2 s_mm[16][64];
+    __shared__ unsigned int mask[2];
+    const int k = threadIdx.x % 64, g = threadIdx.x / 64;
+    double acc = 0.0;
+    float lo = INFINITY, hi = -INFINITY;
+    if (k < DP)
+        for (int b = g; b < blocks; b += 16) {
+            acc += part[(size_t)b * DP + k];
+            const float2 m = minmax[(size_t)b * DP + k];
+            lo = fminf(lo, m.x); hi = fmaxf(hi, m.y);
+        }
+    s_sum[g][k] = acc; s_mm[g][k] = make_float2(lo, hi);
+    __syncthreads();
+    if (g != 0) return;
+    for (int q = 1; q < 16; ++q) {
+        acc += s_sum[q][k];
+        lo = fminf(lo, s_mm[q][k].x); hi = fmaxf(hi, s_mm[q][k].y);
     }
+    if (k < DP) mu[k] = center ? acc / (double)n : 0.0;
+    const unsigned int b = __ballot_sync(0xffffffffu, k < DP && !(lo == hi));
+    if ((k & 31) == 0) mask[k / 32] = b;
+    asm volatile("bar.sync 1, 64;" ::: "memory");
+    if (k == 0) *varying = (unsigned long long)mask[0] | ((unsigned long long)mask[1] << 32);
+}
+
+// mu[k] = mu[keep[k]]
+__global__ void k_compact_mu(double* __restrict__ mu, const Coords co, int DP) {
+    __shared__ double t[64];
+    if ((int)threadIdx.x < DP) t[threadIdx.x] = (int)threadIdx.x < co.kept ? mu[co.keep[threadIdx.x]] : 0.0;
+    __syncthreads();
+    if ((int)threadIdx.x < DP) mu[threadIdx.x] = t[threadIdx.x];
+}
+
+// extra[i] = squared distance of external row i from the points in the dropped coordinates (which all points share); per-block maxima.
+__global__ void __launch_bounds__(256)
+k_row_extra(const float* __restrict__ X, int64_t ld, int64_t n, const Coords co, double* __restrict__ extra, double* __restrict__ part_max) {
+    __shared__ double s_max[256];
+    double mx = 0.0;
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
+        double e = 0.0;
+        for (int k = 0; k < co.dropped; ++k) { const double v = (double)X[i * ld + co.drop[k]] - (double)co.value[k]; e += v * v; }
+        extra[i] = e;
+        mx = e > mx || e != e ? e : mx;
+    }
+    s_max[threadIdx.x] = mx;
+    __syncthreads();
+    for (int off = 128; off > 0; off >>= 1) {
+        if ((int)threadIdx.x < off) { const double o = s_max[threadIdx.x + off]; if (o > s_max[threadIdx.x] || o != o) s_max[threadIdx.x] = o; }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) part_max[blockIdx.x] = s_max[0];
+}
+
+// out[i] = left[i] exp(-beta extra[i])
+__global__ void k_row_factor(const float* __restrict__ left, const double* __restrict__ extra, double beta, int64_t n, float* __restrict__ out) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) out[i] = (float)((left ? (double)left[i] : 1.0) * exp(-beta * extra[i]));
 }
 
 // Per block: sum and max over its rows of |x_i - mu|^2 in fp64.
@@ -139,45 +216,68 @@ inline int grid_for(int64_t n, int block, int cap = 65535 * 8) {
 }  // namespace
 
 fd_status setup_points(fd_ctx* c, const float* X_dev, int64_t ldx) {
-    const Layout& L = c->L;
+    Layout& L = c->L;
     const int64_t N = L.N;
-    k_pad_copy<<<grid_for(N * L.DP, 256, 148 * 16), 256, 0, c->stream>>>(X_dev, ldx, N, L.D, L.DP, c->xs());
+    Coords& co = c->coords;
+    co.kept = L.D; co.dropped = 0;
+    for (int k = 0; k < L.D; ++k) co.keep[k] = (uint8_t)k;
+    k_pad_copy<<<grid_for(N * L.DP, 256, 148 * 16), 256, 0, c->stream>>>(X_dev, ldx, N, co, L.DP, c->xs());
     FD_LAUNCH_CHECK(c, "k_pad_copy");
     double* mu = c->at<double>(L.mu);
-    double* scratch = c->at<double>(L.rowsq);     // reused: (kRedBlocks * DP) doubles needs N >= ... so cap blocks
-    int blocks = (int)(N < kRedBlocks ? N : kRedBlocks);
-    // scratch capacity is N doubles; blocks * DP must fit
-    while ((int64_t)blocks * L.DP > N && blocks > 1) blocks /= 2;
-    double* part = scratch;
-    if ((int64_t)blocks * L.DP > N) {
-        // tiny N with large D: fall back to the sums buffer (2 * 1024 + 8 doubles)
-        part = c->at<double>(L.sums);
-        blocks = 1;
-        if (L.DP > 2 * 1024) return fail(c, FD_ERR_UNSUPPORTED, "D too large");
-    }
-    k_colsum_partial<<<blocks, 128, 0, c->stream>>>(c->xs(), N, L.DP, part);
-    FD_LAUNCH_CHECK(c, "k_colsum_partial");
-    k_colsum_final<<<1, 128, 0, c->stream>>>(part, blocks, L.DP, N, c->centered, mu);
-    FD_LAUNCH_CHECK(c, "k_colsum_final");
     double* sums = c->at<double>(L.sums);
+    // partial results: one per block and coordinate (scratch: the Gram-form operand buffers, at least 16 KB per K slab)
+    double* part = c->at<double>(L.xp_col);
+    float2* minmax = c->at<float2>(L.xp_row);
+    const int64_t room = L.NP * L.K16 * 64 / (8 * L.DP);
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(room, 592), ceil_div(N, 256 / L.DP)));
+    k_colsum_partial<<<blocks, 256, 0, c->stream>>>(c->xs(), N, L.DP, part, minmax);
+    FD_LAUNCH_CHECK(c, "k_colsum_partial");
+    k_colsum_final<<<1, 1024, 0, c->stream>>>(part, minmax, blocks, L.DP, N, c->centered, mu, reinterpret_cast<unsigned long long*>(sums + 2048));
+    FD_LAUNCH_CHECK(c, "k_colsum_final");
     int nb = grid_for(N, 256, 512);
     k_sqnorm_partial<<<nb, 256, 0, c->stream>>>(c->xs(), N, L.DP, mu, sums, sums + 1024);
     FD_LAUNCH_CHECK(c, "k_sqnorm_partial");
-    double host[2048];
-    FD_CUDA(c, cudaMemcpyAsync(host, sums, sizeof(double) * 2048, cudaMemcpyDeviceToHost, c->stream));
+    double host[2049];
+    FD_CUDA(c, cudaMemcpyAsync(host, sums, sizeof host, cudaMemcpyDeviceToHost, c->stream));
     FD_CUDA(c, cudaStreamSynchronize(c->stream));
     double tot = 0.0, mx = 0.0;
     for (int i = 0; i < nb; ++i) { tot += host[i]; if (host[1024 + i] > mx) mx = host[1024 + i]; }
     if (!(tot == tot) || !(tot < 1e300)) return fail(c, FD_ERR_NONFINITE, "non-finite input points");
     c->mean_sq = tot / (double)N;
     c->max_sq = mx;
+    // Coordinates that all points share (zero padding, a frozen degree of freedom) add nothing to any distance between them: where
+    // leaving them out saves padded coordinates, the kernels work on the others alone.  External rows keep their
+    // distance in the dropped coordinates as a factor per row (stage_rows).  D = 32 with 20 zeros, N = 8192, b = 8: 200 -> 105 us a product.
+    unsigned long long varying;
+    std::memcpy(&varying, host + 2048, 8);
+    Coords cut{};
+    for (int k = 0; k < L.D; ++k) {
+        if ((varying >> k) & 1) cut.keep[cut.kept++] = (uint8_t)k;
+        else cut.drop[cut.dropped++] = (uint8_t)k;
+    }
+    if (cut.kept == 0) { cut.keep[0] = cut.drop[--cut.dropped]; cut.kept = 1; }
+    const int DP = (int)round_up(cut.kept, 4);
+    if (DP >= L.DP) return FD_OK;
+    float first[64];
+    FD_CUDA(c, cudaMemcpyAsync(first, X_dev, sizeof(float) * (size_t)L.D, cudaMemcpyDeviceToHost, c->stream));
+    FD_CUDA(c, cudaStreamSynchronize(c->stream));
+    for (int k = 0; k < cut.dropped; ++k) cut.value[k] = first[cut.drop[k]];
+    co = cut;
+    L.DP = DP;
+    L.K16 = (int32_t)ceil_div(cut.kept + 4, 16);
+    k_pad_copy<<<grid_for(N * L.DP, 256, 148 * 16), 256, 0, c->stream>>>(X_dev, ldx, N, co, L.DP, c->xs());
+    FD_LAUNCH_CHECK(c, "k_pad_copy(kept)");
+    k_compact_mu<<<1, 64, 0, c->stream>>>(mu, co, L.DP);
+    FD_LAUNCH_CHECK(c, "k_compact_mu");
+    // (X may be released after the call, as before: the copies above are complete)
+    FD_CUDA(c, cudaStreamSynchronize(c->stream));
     return FD_OK;
 }
 
 fd_status stage_rows(fd_ctx* c, const float* Xrow_dev, int64_t ldxrow, int64_t r0, int64_t n) {
     const Layout& L = c->L;
-    k_pad_copy<<<grid_for(n * L.DP, 256, 148 * 16), 256, 0, c->stream>>>(Xrow_dev + r0 * ldxrow, ldxrow, n, L.D, L.DP,
-                                                                         c->at<float>(L.xrow));
+    const float* X = Xrow_dev + r0 * ldxrow;
+    k_pad_copy<<<grid_for(n * L.DP, 256, 148 * 16), 256, 0, c->stream>>>(X, ldxrow, n, c->coords, L.DP, c->at<float>(L.xrow));
     FD_LAUNCH_CHECK(c, "k_pad_copy(rows)");
     // largest |x - mu|^2 among the staged rows: the Gram-form kernel's exponent budget must hold for them too, and
     // external rows may lie further from the centre than any of the context's own points (scratch: split partials)
@@ -185,13 +285,33 @@ fd_status stage_rows(fd_ctx* c, const float* Xrow_dev, int64_t ldxrow, int64_t r
     const int nb = grid_for(n, 256, 512);
     k_sqnorm_partial<<<nb, 256, 0, c->stream>>>(c->at<float>(L.xrow), n, L.DP, c->at<double>(L.mu), part, part + 1024);
     FD_LAUNCH_CHECK(c, "k_sqnorm_partial(rows)");
-    double host[2048];
-    FD_CUDA(c, cudaMemcpyAsync(host, part, sizeof(double) * 2048, cudaMemcpyDeviceToHost, c->stream));
+    const bool cut = c->coords.dropped > 0;
+    if (cut) {
+        k_row_extra<<<nb, 256, 0, c->stream>>>(X, ldxrow, n, c->coords, c->at<double>(L.rowsq), part + 2048);
+        FD_LAUNCH_CHECK(c, "k_row_extra");
+    }
+    double host[2048 + 512];
+    FD_CUDA(c, cudaMemcpyAsync(host, part, sizeof(double) * (size_t)(cut ? 2048 + 512 : 2048), cudaMemcpyDeviceToHost, c->stream));
     FD_CUDA(c, cudaStreamSynchronize(c->stream));
-    double tot = 0.0, mx = 0.0;
-    for (int i = 0; i < nb; ++i) { tot += host[i]; if (host[1024 + i] > mx) mx = host[1024 + i]; }
-    if (!(tot == tot) || !(tot < 1e300)) return fail(c, FD_ERR_NONFINITE, "non-finite row points");
+    double tot = 0.0, mx = 0.0, ex = 0.0;
+    for (int i = 0; i < nb; ++i) {
+        tot += host[i];
+        if (host[1024 + i] > mx) mx = host[1024 + i];
+        if (cut) ex += host[2048 + i];
+    }
+    if (!(tot == tot) || !(tot < 1e300) || !(ex == ex) || !(ex < 1e300)) return fail(c, FD_ERR_NONFINITE, "non-finite row points");
     c->row_max_sq = mx;
+    c->row_extra = ex > 0.0;
+    return FD_OK;
+}
+
+fd_status row_factor(fd_ctx* c, const float* left, double beta, int64_t n, const float** out) {
+    *out = left;
+    if (!c->row_extra) return FD_OK;
+    float* f = c->at<float>(c->L.symsum);                         // (the symmetric row sums never run between staging and product)
+    k_row_factor<<<grid_for(n, 256), 256, 0, c->stream>>>(left, c->at<double>(c->L.rowsq), beta, n, f);
+    FD_LAUNCH_CHECK(c, "k_row_factor");
+    *out = f;
     return FD_OK;
 }
 

@@ -500,7 +500,7 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
     if (!have_rows || !have_cols) {
         const int first = have_rows ? 1 : 0, roles = (have_rows ? 0 : 1) + (have_cols ? 0 : 1);
         k_pack_points<<<dim3((unsigned)ceil_div(NP, 256), (unsigned)K16, (unsigned)roles), 256, 0, c->stream>>>(
-            rows, cols, first, L.DP, L.D, NP, mu, bprime, std::sqrt(2.0 * bprime), L.D <= 12 * K16);
+            rows, cols, first, L.DP, c->coords.kept, NP, mu, bprime, std::sqrt(2.0 * bprime), c->coords.kept <= 12 * K16);
         FD_LAUNCH_CHECK(c, "k_pack_points");
         if (!have_rows) { c->packed_row_beta = a.rows_are_ctx ? a.beta : -1.0; c->packed_row0 = row0; c->packed_rows = a.Nrow; }
         c->packed_beta = a.beta;

@@ -117,3 +117,38 @@ def test_extension_column_chunks(path, m, b_max):
     ref = nystrom.extend(X, qo, 1.0, 1.0, psi.astype(np.float64), lam, Z)
     assert np.abs(out - ref).max() <= 1e-5 * np.abs(ref).max()
     ctx.close()
+
+
+@pytest.mark.parametrize("N,path,D,const", [(700, 1, 32, 0.0), (700, 2, 32, 2.5), (700, 2, 60, -1.0), (5, 1, 20, 1.0)])
+def test_coordinates_that_all_points_share(N, path, D, const):
+    """Constant coordinates among the points (padding, a frozen degree of freedom) are left out of the kernels' work: same products and
+    degrees, and external rows that differ from the points in such a coordinate keep their distance.  Gates: 1e-5 for the block
+    products as elsewhere; degrees 1e-6 / 2e-5 (direct / Gram form)."""
+    import __graft_entry__ as g
+    g.build()
+    import paper_2609_38198_b200 as fd
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(1)
+    X = np.full((N, D), const, dtype=np.float32)
+    used = np.sort(rng.choice(D, 12, replace=False))
+    X[:, used] = workloads.torus6(N, seed=3)
+    Z = X[: min(N, 300)].copy()
+    Z[:, used] += 0.1 * rng.standard_normal((len(Z), 12)).astype(np.float32)
+    Z[::2, (used[0] + 1) % D if (used[0] + 1) % D not in used else [k for k in range(D) if k not in used][0]] += 0.5
+    b, beta = 8, 1.0
+    V = workloads.block(N, b, seed=2)
+    l = rng.uniform(0.5, 2.0, len(Z)).astype(np.float32)
+    ctx = fd.Context(torch.from_numpy(X).to(dev), b_max=b)
+    ctx.set_option("path", path)
+    q, d, s, so, so2 = ctx.degree(beta, 1.0)
+    qo, do, s_o, soo, so2o = dense.degree(X, beta, 1.0)
+    assert np.abs(q.cpu().numpy() / qo - 1).max() <= (1e-6 if path == 1 else 2e-5)
+    Y = ctx.apply(fd.to_colmajor(V, dev)).cpu().numpy().astype(np.float64)
+    Yo = dense.apply(X, beta, 1.0, V)
+    assert np.linalg.norm(Y - Yo) <= 1e-5 * np.linalg.norm(Yo)
+    for left in (None, l):
+        R = ctx.apply_general(beta, fd.to_colmajor(V, dev), left=None if left is None else torch.from_numpy(left).to(dev), Xrow=torch.from_numpy(Z).to(dev))
+        K = np.exp(-beta * ((Z[:, None, :].astype(np.float64) - X[None].astype(np.float64)) ** 2).sum(-1))
+        Ro = (1.0 if left is None else left[:, None].astype(np.float64)) * (K @ V.astype(np.float64))
+        assert np.linalg.norm(R.cpu().numpy().astype(np.float64) - Ro) <= 1e-5 * np.linalg.norm(Ro)
+    ctx.close()
