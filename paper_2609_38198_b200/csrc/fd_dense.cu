@@ -145,12 +145,18 @@ k_tn_reduce(const double* __restrict__ part, int chunks, int64_t mm, double* __r
 // C[i, c] = sum_k A[i, k] S[k, c] for a strip of PT columns; RPT rows per thread (two where there are enough rows: half the
 // shared-memory reads per FMA).  S is staged 32 rows at a time; the rows of A are read straight from memory, eight columns in flight.
 // N = 2^17, m = 200, p = 32: 48 us against 91 with one row per thread and four loads in flight.
-template <int PT, int RPT>
-__global__ void __launch_bounds__(128)
+// KS groups of 128 threads share the columns of A (partial sums meet in shared memory): few rows leave each thread a long chain of dependent
+// loads otherwise (N = 16384, m = 260, p = 41: 27 -> @NN us with four groups).
+template <int PT, int RPT, int KS>
+__global__ void __launch_bounds__(128 * KS)
 k_nn(const Panel A, const float* __restrict__ S, int lds, int p, float* __restrict__ C, int64_t ldc, int64_t N) {
-    __shared__ __align__(16) float ss[32 * PT];
+    static_assert(KS == 1 || RPT == 1, "split columns with one row per thread only");
+    constexpr int kS = 32 * PT, kRed = KS > 1 ? (KS - 1) * PT * 128 : 0;
+    __shared__ __align__(16) float smem[KS * kS > kRed ? KS * kS : kRed];
     const int m = A.m1 + A.m2;
-    const int64_t i0 = (int64_t)blockIdx.x * (128 * RPT) + threadIdx.x;
+    const int grp = threadIdx.x / 128, tid = threadIdx.x % 128;
+    float* ss = smem + grp * kS;
+    const int64_t i0 = (int64_t)blockIdx.x * (128 * RPT) + tid;
     const int c0 = blockIdx.y * PT;
     int64_t row[RPT];
 #pragma unroll
@@ -160,9 +166,10 @@ k_nn(const Panel A, const float* __restrict__ S, int lds, int p, float* __restri
     for (int r = 0; r < RPT; ++r)
 #pragma unroll
         for (int c = 0; c < PT; ++c) acc[r][c] = 0.f;
-    for (int k0 = 0; k0 < m; k0 += 32) {
+    for (int kb0 = 0; kb0 < m; kb0 += 32 * KS) {
+        const int k0 = kb0 + 32 * grp;                             // this group's 32 columns
         __syncthreads();
-        for (int t = threadIdx.x; t < 32 * PT; t += 128) {
+        for (int t = tid; t < 32 * PT; t += 128) {
             const int kk = t % 32, cc = t / 32;
             ss[kk * PT + cc] = (k0 + kk < m && c0 + cc < p) ? S[(k0 + kk) + (size_t)(c0 + cc) * lds] : 0.f;
         }
@@ -191,6 +198,19 @@ k_nn(const Panel A, const float* __restrict__ S, int lds, int p, float* __restri
                     }
                 }
         }
+    }
+    if (KS > 1) {
+        __syncthreads();
+        if (grp > 0) {
+#pragma unroll
+            for (int c = 0; c < PT; ++c) smem[((grp - 1) * PT + c) * 128 + tid] = acc[0][c];
+        }
+        __syncthreads();
+        if (grp > 0) return;
+#pragma unroll
+        for (int q = 0; q < KS - 1; ++q)
+#pragma unroll
+            for (int c = 0; c < PT; ++c) acc[0][c] += smem[(q * PT + c) * 128 + tid];
     }
 #pragma unroll
     for (int r = 0; r < RPT; ++r)
@@ -303,16 +323,17 @@ fd_status tn_product(fd_ctx* c, const Panel& A, const Panel& B, int64_t N, doubl
 fd_status nn_product(fd_ctx* c, const Panel& A, const float* S_dev, int lds, int p, float* C, int64_t ldc, int64_t N) {
     if (p < 1 || N < 1) return FD_OK;
     if (A.m1 + A.m2 < 1) return fail(c, FD_ERR_INVALID, "nn_product: no columns");
-    // strips of 32 columns and two rows per thread where that still gives every SM a few blocks, else narrower strips
-    const int64_t blocks2 = ceil_div(N, 256) * ceil_div(p, 32), blocks1 = ceil_div(N, 128) * ceil_div(p, 32);
-    if (p > 16 && blocks2 >= 3 * c->sm_count)
-        k_nn<32, 2><<<dim3((unsigned)ceil_div(N, 256), (unsigned)ceil_div(p, 32)), 128, 0, c->stream>>>(A, S_dev, lds, p, C, ldc, N);
-    else if (p > 16 && blocks1 >= 2 * c->sm_count)
-        k_nn<32, 1><<<dim3((unsigned)ceil_div(N, 128), (unsigned)ceil_div(p, 32)), 128, 0, c->stream>>>(A, S_dev, lds, p, C, ldc, N);
-    else if (p > 8 && ceil_div(N, 128) * ceil_div(p, 16) >= 2 * c->sm_count)
-        k_nn<16, 1><<<dim3((unsigned)ceil_div(N, 128), (unsigned)ceil_div(p, 16)), 128, 0, c->stream>>>(A, S_dev, lds, p, C, ldc, N);
+    // strips of 32 columns and two rows per thread where that still gives every SM a few blocks, else strips of 32 / 16 / 8 columns
+    // (the narrowest that holds p, at most 16: more blocks) with the columns of A shared by four groups of threads
+    const unsigned rb = (unsigned)ceil_div(N, 128);
+    if (p > 16 && ceil_div(N, 256) * ceil_div(p, 32) >= 3 * c->sm_count)
+        k_nn<32, 2, 1><<<dim3((unsigned)ceil_div(N, 256), (unsigned)ceil_div(p, 32)), 128, 0, c->stream>>>(A, S_dev, lds, p, C, ldc, N);
+    else if (p > 16 && rb * ceil_div(p, 32) >= 4 * c->sm_count)
+        k_nn<32, 1, 1><<<dim3(rb, (unsigned)ceil_div(p, 32)), 128, 0, c->stream>>>(A, S_dev, lds, p, C, ldc, N);
+    else if (p > 8)
+        k_nn<16, 1, 4><<<dim3(rb, (unsigned)ceil_div(p, 16)), 512, 0, c->stream>>>(A, S_dev, lds, p, C, ldc, N);
     else
-        k_nn<8, 1><<<dim3((unsigned)ceil_div(N, 128), (unsigned)ceil_div(p, 8)), 128, 0, c->stream>>>(A, S_dev, lds, p, C, ldc, N);
+        k_nn<8, 1, 4><<<dim3(rb, 1u), 512, 0, c->stream>>>(A, S_dev, lds, p, C, ldc, N);
     FD_LAUNCH_CHECK(c, "k_nn");
     return FD_OK;
 }

@@ -55,6 +55,7 @@ struct Solver {
     size_t S_floats;                // capacity of d_S and of a staging slot
     std::vector<double> T, G;       // host, column-major, pitch m_cap
     double* h = nullptr;            // page-locked result of the latest projection
+    volatile unsigned int* h_status = nullptr;   // page-locked copy of the tensor-core kernels' status word
     int stage_next = 0;             // next slot of the context's staging ring
     int m = 0;
     int applies = 0, restarts = 0;
@@ -70,7 +71,7 @@ struct Solver {
             FD_CUDA(c, cudaStreamSynchronize(c->stream));
             if (c->stage) { FD_CUDA(c, cudaFreeHost(c->stage)); c->stage = nullptr; c->stage_floats = 0; c->h_out_doubles = 0; }
             const size_t slot = (size_t)round_up((int64_t)S_floats, 64);
-            FD_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->stage), sizeof(float) * slot * fd_ctx::kStageSlots + sizeof(double) * out_doubles));
+            FD_CUDA(c, cudaMallocHost(reinterpret_cast<void**>(&c->stage), sizeof(float) * slot * fd_ctx::kStageSlots + sizeof(double) * (out_doubles + 1)));
             c->stage_floats = slot;
             c->h_out = reinterpret_cast<double*>(c->stage + slot * fd_ctx::kStageSlots);
             c->h_out_doubles = out_doubles;
@@ -78,6 +79,8 @@ struct Solver {
                 if (!c->stage_ev[i]) FD_CUDA(c, cudaEventCreateWithFlags(&c->stage_ev[i], cudaEventDisableTiming));
         }
         h = c->h_out;
+        h_status = reinterpret_cast<unsigned int*>(c->h_out + c->h_out_doubles);
+        *h_status = 0;
         return FD_OK;
     }
     // Slot for a right factor of `floats` entries: the caller fills it and sends it.
@@ -96,7 +99,10 @@ struct Solver {
     // Waits for the projection written to h (cnt doubles) and sums it over the ranks.
     fd_status fetch(int64_t cnt) {
         FD_CUDA(c, cudaStreamSynchronize(c->stream));
-        return allreduce_host(c, h, cnt);
+        FD_TRY(allreduce_host(c, h, cnt));
+        // the status word of the products before this wait (the sum above first: every rank takes that step)
+        if (*h_status != 0) return tc_check_status(c);
+        return FD_OK;
     }
     // h = A^T B (column-major, pitch = columns of A)
     fd_status project(const Panel& A, const Panel& B) {
@@ -116,7 +122,9 @@ struct Solver {
                                  W + (int64_t)(c0 + o) * N, N, c->eigs_prec, /*gather_out=*/false));
             ++applies;
         }
-        FD_TRY(tc_check_status(c));
+        // (looked at after the next projection's wait)
+        if (c->last_path == FD_PATH_TC)
+            FD_CUDA(c, cudaMemcpyAsync(const_cast<unsigned int*>(h_status), c->at<unsigned int>(c->L.status), 4, cudaMemcpyDeviceToHost, c->stream));
         t_apply += secs(t0, clk::now());
         return FD_OK;
     }
@@ -163,9 +171,10 @@ struct Solver {
         return FD_OK;
     }
 
-    // Eigen-decomposition of the p x p Gram matrix g (column-major, overwritten) scaled to a unit diagonal.  On return F
-    // (p x rank, column-major) turns the columns whose Gram matrix g is into orthonormal ones; directions with an
-    // eigenvalue at or below drop_tol are left out.  lam_min: the smallest eigenvalue kept.
+    // F (p x rank, column-major) turns the columns whose p x p Gram matrix is g (column-major, overwritten) into orthonormal ones.  By
+    // Cholesky if every pivot of the matrix scaled to a unit diagonal exceeds kGoodPivot, else by its eigen-decomposition, leaving
+    // out directions with an eigenvalue at or below drop_tol.  lam_min: about the smallest eigenvalue kept.
+    static constexpr double kGoodPivot = 0.1;
     fd_status orthonormal_factor(double* g, int p, double drop_tol, std::vector<double>& F, int& rank, double& lam_min) {
         std::vector<double> dinv(p);
         for (int j = 0; j < p; ++j) {
@@ -177,6 +186,37 @@ struct Solver {
                 const double v = 0.5 * (g[i + (size_t)j * p] + g[j + (size_t)i * p]) * dinv[i] * dinv[j];
                 g[i + (size_t)j * p] = g[j + (size_t)i * p] = v;
             }
+        // well-conditioned (the usual case): Cholesky g = L L^T, F = D^-1/2 L^-T; its pivots bound how close to dependent the columns are
+        {
+            std::vector<double> Lc((size_t)p * p, 0.0);
+            bool good = true;
+            for (int j = 0; j < p && good; ++j) {
+                for (int i = j; i < p; ++i) {
+                    double v = g[i + (size_t)j * p];
+                    for (int l = 0; l < j; ++l) v -= Lc[(size_t)i * p + l] * Lc[(size_t)j * p + l];
+                    if (i == j) {
+                        good = v > kGoodPivot;
+                        if (!good) break;
+                        Lc[(size_t)j * p + j] = std::sqrt(v);
+                    } else Lc[(size_t)i * p + j] = v / Lc[(size_t)j * p + j];
+                }
+            }
+            if (good) {
+                F.assign((size_t)p * p, 0.0);                      // column j of L^-T: back substitution against e_j
+                for (int j = 0; j < p; ++j) {
+                    double* f = &F[(size_t)j * p];
+                    for (int i = j; i >= 0; --i) {
+                        double v = i == j ? 1.0 : 0.0;
+                        for (int l = i + 1; l <= j; ++l) v -= Lc[(size_t)l * p + i] * f[l];
+                        f[i] = v / Lc[(size_t)i * p + i];
+                    }
+                    for (int i = 0; i <= j; ++i) f[i] *= dinv[i];
+                }
+                rank = p;
+                lam_min = kGoodPivot;
+                return FD_OK;
+            }
+        }
         std::vector<double> lam, U;
         if (!sym_eig(g, p, lam, U)) return fail(c, FD_ERR_NOT_CONVERGED, "small eigenproblem (orthonormalise) failed");
         rank = 0;
