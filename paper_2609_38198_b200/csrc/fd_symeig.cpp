@@ -99,20 +99,27 @@ void tridiagonalise(std::vector<double>& z, int n, std::vector<double>& diag, st
             for (int j = 0; j <= l; ++j) {
                 const double* row = &z[(size_t)j * n];
                 double acc = 0.0;
-                for (int k = 0; k <= l; ++k) acc += row[k] * u[k];
+                const double* uu = u.data();
+#pragma omp simd reduction(+ : acc)
+                for (int k = 0; k <= l; ++k) acc += row[k] * uu[k];
                 pv[j] = acc / h;
             }
             // K = u.p / (2 h), q = p - K u
             double up = 0.0;
-            for (int j = 0; j <= l; ++j) up += u[j] * pv[j];
+            const double *uu = u.data(), *pp = pv.data();
+            double* qq = q.data();
+#pragma omp simd reduction(+ : up)
+            for (int j = 0; j <= l; ++j) up += uu[j] * pp[j];
             const double K = up / (h + h);
-            for (int j = 0; j <= l; ++j) q[j] = pv[j] - K * u[j];
+#pragma omp simd
+            for (int j = 0; j <= l; ++j) qq[j] = pp[j] - K * uu[j];
             // A <- A - u q^T - q u^T (both triangles)
 #pragma omp for schedule(static)
             for (int j = 0; j <= l; ++j) {
                 double* row = &z[(size_t)j * n];
-                const double uj = u[j], qj = q[j];
-                for (int k = 0; k <= l; ++k) row[k] -= uj * q[k] + qj * u[k];
+                const double uj = uu[j], qj = qq[j];
+#pragma omp simd
+                for (int k = 0; k <= l; ++k) row[k] -= uj * qq[k] + qj * uu[k];
             }
         }
     }
@@ -131,9 +138,11 @@ void tridiagonalise(std::vector<double>& z, int n, std::vector<double>& diag, st
             const int l = i - 1;
             const double* ui = &U[(size_t)i * n];
             double acc = 0.0;
+#pragma omp simd reduction(+ : acc)
             for (int k = 0; k <= l; ++k) acc += row[k] * ui[k];
             if (acc == 0.0) continue;
             acc /= hval[i];
+#pragma omp simd
             for (int k = 0; k <= l; ++k) row[k] -= acc * ui[k];
         }
     }
@@ -207,6 +216,7 @@ void apply_rotations(double* zt, int n, int pitch, const std::vector<Rotation>& 
             double* a = zt + (size_t)g.row * pitch;
             double* b = a + pitch;
             const double c = g.c, s = g.s;
+#pragma omp simd
             for (int k = k0; k < k1; ++k) {
                 const double ak = a[k], bk = b[k];
                 a[k] = c * ak + s * bk;
@@ -261,6 +271,7 @@ void apply_rotations_reversed(double* w, int cw, const std::vector<Rotation>& ro
         double* a = w + (size_t)g.row * cw;
         double* b = a + cw;
         const double c = g.c, s = g.s;
+#pragma omp simd
         for (int k = 0; k < cw; ++k) {
             const double ak = a[k], bk = b[k];
             a[k] = c * ak - s * bk;
