@@ -146,7 +146,7 @@ k_tn_reduce(const double* __restrict__ part, int chunks, int64_t mm, double* __r
 // shared-memory reads per FMA).  S is staged 32 rows at a time; the rows of A are read straight from memory, eight columns in flight.
 // N = 2^17, m = 200, p = 32: 48 us against 91 with one row per thread and four loads in flight.
 // KS groups of 128 threads share the columns of A (partial sums meet in shared memory): few rows leave each thread a long chain of dependent
-// loads otherwise (N = 16384, m = 260, p = 41: 27 -> @NN us with four groups).
+// loads otherwise (N = 16384, m = 260, p = 41: 27 -> 14 us with four groups).
 template <int PT, int RPT, int KS>
 __global__ void __launch_bounds__(128 * KS)
 k_nn(const Panel A, const float* __restrict__ S, int lds, int p, float* __restrict__ C, int64_t ldc, int64_t N) {

@@ -403,7 +403,9 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
     // there every block is a residual block, and a solve that reaches the accuracy floor of the fp32 operator first is
     // reported as stalled.  N = 2^18, k = 128, capacity 384: the Krylov continuation brings all residuals of the STORED images
     // below 1e-6 while the operator's own error leaves them at up to 1.9e-6 against float64 rows.)
-    const int kMaxBlocks = m_cap < 3 * nwant && m_cap < N ? 1 : 4;
+    const bool small_basis = m_cap < 3 * nwant && m_cap < N;
+    const int kMaxBlocks = small_basis ? 1 : 4;
+    const bool wanted_first = !small_basis;
     double last_worst = 0.0;
     int last_applies = 0;
 
@@ -512,11 +514,11 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
 
         // ---- choose the expansion columns: wanted pairs above the tolerance first, then largest residuals first ---
         // (the buffer pairs' residuals are larger almost always; a wanted pair that the fp32 rounding of its residual holds
-        // just above the tolerance would never be chosen)
+        // just above the tolerance would never be chosen; a small basis takes plain residual blocks throughout)
         std::vector<int> order(nsel);
         for (int i = 0; i < nsel; ++i) order[i] = i;
         std::sort(order.begin(), order.end(), [&](int a, int bb) {
-            const bool wa = a < nwant && resid[a] > thr, wb = bb < nwant && resid[bb] > thr;
+            const bool wa = wanted_first && a < nwant && resid[a] > thr, wb = wanted_first && bb < nwant && resid[bb] > thr;
             return wa != wb ? wa : resid[a] > resid[bb];
         });
         const int want_new = (int)std::min<int64_t>(b, N - m);
