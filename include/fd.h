@@ -86,7 +86,7 @@ fd_status fd_create(fd_ctx** out, const float* X_dev, int64_t N, int32_t D, int6
 fd_status fd_destroy(fd_ctx* ctx);
 
 /* Tuning / test knobs by name: "path" (FD_PATH_*), "splits" (0 = auto), "flush" (column tiles
- * between accumulator flushes of the tensor-core kernels; 0 = default: 2 (up to 32 columns) or 1 in the fp32-grade mode, whose
+ * between accumulator flushes of the tensor-core kernels; 0 = default: 1 in the fp32-grade mode, whose
  * eigenvalue budget the tensor core's round-toward-zero accumulation would otherwise eat, 8 in the reduced-precision mode), "tc_max_mag" (largest beta * log2(e) *
  * max|x - mu|^2 for which the Gram-form tensor-core kernel serves the fp32 mode), "jt_chunk" (column
  * tiles per L2-resident chunk of the tensor-core block product), "sym" (1, default: the degree passes on the Gram-form
@@ -97,7 +97,8 @@ fd_status fd_destroy(fd_ctx* ctx);
  * (value = limit in SM cycles: enqueues
  * a one-thread kernel whose bounded wait on a barrier that nothing completes must expire; the next
  * fd_synchronize then returns FD_ERR_TIMEOUT and the context stays usable).  fd_get_option also reports "last_path" (the
- * family that served the latest pass), "beta", "mean_sq", "max_sq" and "tc_cycles" (SM cycles the first CTA of the most
+ * family that served the latest pass), "beta", "mean_sq", "max_sq", "tile_share" (share of the tiles that the
+ * latest fp32-grade Gram-form block product of the whole point set evaluated; the others hold zeros only) and "tc_cycles" (SM cycles the first CTA of the most
  * recent tensor-core quadratic kernel spent on its work items; synchronises; with the kernel's wall time it
  * gives the SM clock the kernel actually ran at).  Unknown name -> FD_ERR_INVALID. */
 fd_status fd_set_option(fd_ctx* ctx, const char* name, double value);

@@ -55,9 +55,9 @@ Layout make_layout(int64_t N, int32_t D, int32_t b_max, int32_t m_max) {
     L.sums = carve(cur, (size_t)(2 * 1024 + 8) * 8);
     L.wp = carve(cur, (size_t)N * L.BP * 4);
     // shares of row tiles that a work range's cut falls into: two slots of 256 rows x the widest column tile per CTA (direct-difference
-    // kernels: up to four CTAs on each of 148 SMs, tensor-core product: one; never more CTAs than steps)
+    // kernels: up to four CTAs on each of 148 SMs, tensor-core product: one, and a slot for its sums; never more CTAs than steps)
     const int64_t steps = ceil_div(N, 256) * ceil_div(N, 16);
-    L.part_floats = (size_t)std::max<int64_t>(std::min<int64_t>(592, steps), 160) * 2 * 256 * (size_t)L.BP;
+    L.part_floats = (size_t)std::max<int64_t>(std::min<int64_t>(592, steps), 240) * 2 * 256 * (size_t)L.BP;
     L.part = carve(cur, L.part_floats * 4);
     // tensor-core operands: fp16 hi|lo rows of the augmented points, transposed fp16 hi / lo blocks
     L.xp_col = carve(cur, (size_t)L.NP * L.K16 * 64);
@@ -68,6 +68,15 @@ Layout make_layout(int64_t N, int32_t D, int32_t b_max, int32_t m_max) {
     L.status = carve(cur, 256);
     L.symsum = carve(cur, (size_t)N * 8);
     L.weights = carve(cur, (size_t)L.NP * 4);
+    // tile lists: N^2 / 16384 bytes, 17 MB at 2^19 points; larger sets run over all tiles (as do small ones, where nothing is gained)
+    if (N >= 8192 && N <= (int64_t)1 << 19) {
+        const size_t tiles = (size_t)(L.NP / 128), pairs = tiles / 2;
+        L.perm = carve(cur, (size_t)N * 4);
+        L.boxes = carve(cur, tiles * 2 * 8 * 4);
+        if (L.DP > 8) L.zproj = carve(cur, (size_t)N * 8 * 4);
+        L.lists = carve(cur, pairs * tiles * 2);
+        L.list_counts = carve(cur, (4 * pairs + 2) * 4);
+    }
     if (m_max > 0) {
         L.eig_q = carve(cur, (size_t)N * m_max * 4);
         L.eig_w = carve(cur, (size_t)N * m_max * 4);
@@ -194,6 +203,10 @@ fd_status fd_get_option(const fd_ctx* c, const char* name, double* v) {
         if (cudaStreamSynchronize(c->stream) != cudaSuccess ||
             cudaMemcpy(&cyc, c->at<unsigned int>(c->L.status) + 2, 8, cudaMemcpyDeviceToHost) != cudaSuccess) return FD_ERR_CUDA;
         *v = (double)cyc;
+    }
+    else if (!strcmp(name, "tile_share")) {
+        const double tiles = (double)(c->L.NP / 128);
+        *v = c->lists[0].on ? (double)c->lists[0].total / (0.5 * tiles * tiles) : 1.0;
     }
     else if (!strcmp(name, "mean_sq")) *v = c->mean_sq;
     else if (!strcmp(name, "max_sq")) *v = c->max_sq;

@@ -31,6 +31,8 @@ struct Layout {
     size_t part = 0, part_floats = 0;
     size_t xp_col = 0, xp_row = 0, wt_hi = 0, wt_lo = 0, colscale = 0, status = 0;
     size_t yacc = 0;
+    // order of the points and tile lists of the Gram-form kernels (fd_order.cu); 0: not provisioned for this N
+    size_t perm = 0, boxes = 0, zproj = 0, lists = 0, list_counts = 0;
     size_t weights = 0;              // NP right weights of a Gram-form row sum
     size_t symsum = 0;               // N 64-bit fixed-point sums of the symmetric row-sum mode
     size_t eig_q = 0, eig_w = 0, eig_x = 0, eig_r = 0, eig_small = 0, eig_small_doubles = 0;
@@ -66,6 +68,13 @@ struct fd_ctx {
     // (-1: something else)
     double packed_beta = -1.0, packed_row_beta = -1.0;
     int64_t packed_row0 = 0, packed_rows = 0;
+    int order_state = 0;             // 1: the Gram-form operands hold the points in the order of L.perm; -1: no order will be made
+    // tile lists, for block products (0) and degree passes (1), whose exponent limits differ: bandwidth they were decided for, whether
+    // they leave out enough to be used, entries in all; which of the two the workspace holds, and for which bandwidth
+    struct { double beta = -1.0; bool on = false; int64_t total = 0; } lists[2];
+    double refused_beta = 0.0;       // largest bandwidth at which an order was tried and left out too little
+    int listed_kind = -1;
+    double listed_beta = -1.0;
     // options
     int opt_path = FD_PATH_AUTO;
     int opt_splits = 0;
@@ -170,6 +179,9 @@ void shard_range(int64_t N, int world, int rank, int64_t* begin, int64_t* end);
 fd_status gather_rows(fd_ctx* c, float* A, int64_t lda, int cols);
 // In-place sum over the ranks of n host doubles.  No-op for an unsharded context.
 fd_status allreduce_host(fd_ctx* c, double* buf, int64_t n);
+// Tile lists of a bandwidth for block products (kind 0) or degree passes (1) (fd_order.cu): decides c->lists[kind] and, where they are
+// used, brings them into the workspace; orders the points first if that can pay.  Synchronises when the bandwidth is new.
+fd_status tile_lists(fd_ctx* c, double beta, int kind);
 // Reads and clears the tensor-core kernel's status word; FD_ERR_TIMEOUT if a bounded wait expired.  Synchronises.
 fd_status tc_check_status(fd_ctx* c);
 // Launches a one-thread kernel whose bounded wait must expire after limit_cycles (test of the time-out plumbing).

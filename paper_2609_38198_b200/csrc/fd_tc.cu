@@ -202,7 +202,7 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
 
         for (int w = 0; w < my_items && ok; ++w) {
             const int item = (int)blockIdx.x + w * (int)gridDim.x;
-            const int64_t row = (int64_t)item * 256 + t * 128 + row_in_tile;
+            int64_t row = (int64_t)item * 256 + t * 128 + row_in_tile;
             {
                 double dsum = 0.0, dsq = 0.0;
                 for (int j = 0; j < num_jt && ok; ++j) {
@@ -241,6 +241,7 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
                     dsq += (double)(q0 + q1);
                 }
                 if (ok && row < p.Nrow) {
+                    if (p.perm) row = p.perm[row];
                     // undo the 2^bias scaling of P (exact powers of two)
                     constexpr double scale = 1.0 / (double)(1 << kBias);
                     p.q[row] = (float)(p.left ? dsum * (scale * (double)p.left[row]) : dsum * scale);
@@ -282,7 +283,7 @@ __global__ void k_wait_selftest(unsigned int* status, long long limit_cycles) {
 // rounds each MMA at the magnitude of its sum, so this removes most of the exponent's error for far-out points (R^30, exponents
 // up to 60: worst eigenvalue error of 33 pairs 9.7e-7 -> 6.6e-7).  Else coordinates first, the four norm columns after the last one.
 // One thread per (point, slab, role): the 64 bytes it writes are contiguous.
-struct PackRole { const float* xs; __half* out; int64_t n; };   // n: valid points of this role
+struct PackRole { const float* xs; __half* out; int64_t n; const int* perm; };   // n: valid points of this role; perm: point of each position
 __global__ void __launch_bounds__(256)
 k_pack_points(const PackRole rows, const PackRole cols, int first_role, int DP, int D, int64_t np, const double* __restrict__ mu, double bprime,
               double cs, int slab_norms) {
@@ -291,7 +292,7 @@ k_pack_points(const PackRole rows, const PackRole cols, int first_role, int DP, 
     const int s = blockIdx.y, role = first_role + (int)blockIdx.z;
     const PackRole pr = role == 0 ? rows : cols;
     const bool valid = pidx < pr.n;
-    const float* x = pr.xs + pidx * DP;
+    const float* x = pr.xs + (valid && pr.perm ? (int64_t)pr.perm[pidx] : pidx) * DP;
     const int c0 = slab_norms ? 12 * s : 16 * s;                  // first coordinate of this slab
     const int norm0 = slab_norms ? 12 : D - c0;                   // first norm column inside the slab (may lie outside it)
     __half hi[16], lo[16];
@@ -340,9 +341,9 @@ k_pack_points(const PackRole rows, const PackRole cols, int first_role, int DP, 
 }
 
 // out[j] = w[j] (1 without w) for j < n, 0 up to np: the weights of a row sum, padded to whole column tiles.
-__global__ void k_pad_weights(const float* __restrict__ w, int64_t n, int64_t np, float* __restrict__ out) {
+__global__ void k_pad_weights(const float* __restrict__ w, int64_t n, int64_t np, const int* __restrict__ perm, float* __restrict__ out) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < np) out[j] = j < n ? (w ? w[j] : 1.f) : 0.f;
+    if (j < np) out[j] = j < n ? (w ? w[perm ? perm[j] : j] : 1.f) : 0.f;
 }
 
 // Per-block maxima of |right_j V_jc| for each column c (columns from vcols on are the ones vector).
@@ -372,7 +373,7 @@ k_colmax_partial(const float* __restrict__ V, int64_t ldv, int vcols, const floa
 // partial maxima of its column itself (they are at most 256 values); the first one stores the epilogue factor 2^-bias / scale.
 __global__ void __launch_bounds__(256)
 k_pack_wt(const float* __restrict__ V, int64_t ldv, int vcols, const float* __restrict__ right, int64_t N, int64_t np, int c0, int bc,
-          const float* __restrict__ part, int parts, float* __restrict__ inv, __half* __restrict__ wt, int with_lo) {
+          const float* __restrict__ part, int parts, float* __restrict__ inv, __half* __restrict__ wt, int with_lo, const int* __restrict__ perm) {
     __shared__ float sm[8];
     const int c = blockIdx.y;
     float m = c < bc && (int)threadIdx.x < parts ? part[(size_t)c * parts + threadIdx.x] : 0.f;
@@ -401,8 +402,9 @@ k_pack_wt(const float* __restrict__ V, int64_t ldv, int vcols, const float* __re
             const int64_t j = 2 * j2 + u;
             x[u] = 0.f;
             if (c < bc && j < N) {
-                const float y = ones ? 1.f : v[j];
-                x[u] = (right ? y * right[j] : y) * sc;
+                const int64_t i = perm ? (int64_t)perm[j] : j;
+                const float y = ones ? 1.f : v[i];
+                x[u] = (right ? y * right[i] : y) * sc;
             }
         }
         const __half2 h = __floats2half2_rn(x[0], x[1]);
@@ -493,7 +495,14 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
     // pass: the S tiles of the degree passes and of the block product are bit-identical, so any rounding bias of the Gram
     // accumulation is common to q, d and K and cancels in diag(s) K diag(s).  The operands of the context's own points stay
     // packed for the bandwidth: the products of a solve reuse them.
-    const PackRole rows{a.xrow, xp_row, a.Nrow}, cols{c->xs(), xp_col, N};
+    // passes over the context's whole point set may leave out tiles that hold no near pair (fd_order.cu)
+    const bool all_rows = a.rows_are_ctx && a.xrow == c->xs() && a.Nrow == N;
+    const bool prunes = all_rows && !c->sh.on && (rowsum ? sym : a.prec == FD_PREC_FP32);
+    if (prunes) FD_TRY(tile_lists(c, a.beta, rowsum ? 1 : 0));
+    const bool use_lists = prunes && c->L.perm != 0 && c->lists[rowsum ? 1 : 0].on;
+    const int* col_perm = c->order_state == 1 ? c->at<int>(L.perm) : nullptr;
+    const int* row_perm = all_rows ? col_perm : nullptr;
+    const PackRole rows{a.xrow, xp_row, a.Nrow, row_perm}, cols{c->xs(), xp_col, N, col_perm};
     const int64_t row0 = a.rows_are_ctx ? (a.xrow - c->xs()) / L.DP : -1;
     const bool have_rows = a.rows_are_ctx && c->packed_row_beta == a.beta && c->packed_row0 == row0 && c->packed_rows == a.Nrow;
     const bool have_cols = c->packed_beta == a.beta;
@@ -520,17 +529,17 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
     if (p.jt_chunk > p.num_jt) p.jt_chunk = p.num_jt;
     p.num_chunks = (int)ceil_div(p.num_jt, p.jt_chunk);
     p.np_rows = NP; p.np_cols = NP; p.K16 = K16;
-    p.left = a.left; p.status = status;
+    p.left = a.left; p.status = status; p.perm = row_perm; p.use_lists = use_lists ? 1 : 0;
     const int grid = std::min(p.num_work, c->sm_count);
 
     if (rowsum && !a.rowsq) {
         float* w = c->at<float>(L.weights);
-        k_pad_weights<<<(unsigned)ceil_div(NP, 256), 256, 0, c->stream>>>(a.right, N, NP, w);
+        k_pad_weights<<<(unsigned)ceil_div(NP, 256), 256, 0, c->stream>>>(a.right, N, NP, col_perm, w);
         FD_LAUNCH_CHECK(c, "k_pad_weights");
         p.weights = w;
     }
     if (rowsum && sym) {
-        FD_TRY(launch_sym_rowsum(c, mr, mc, p.weights, a.left, a.Y, a.rowsq));
+        FD_TRY(launch_sym_rowsum(c, mr, mc, p.weights, a.left, a.Y, a.rowsq, row_perm, use_lists));
     } else if (rowsum) {
         p.q = a.Y; p.rowsq = a.rowsq; p.b = 1;
         if (p.rowsq) FD_TRY((launch_tc<16>(c, mr, mc, p, grid)));
@@ -551,7 +560,7 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
             k_colmax_partial<<<dim3(cm_blocks, bc), 256, 0, c->stream>>>(a.V, a.ldv, vcols, a.right, N, c0, part);
             FD_LAUNCH_CHECK(c, "k_colmax_partial");
             k_pack_wt<<<dim3((unsigned)std::min<int64_t>(1024, ceil_div(NP, 512)), BT), 256, 0, c->stream>>>(
-                a.V, a.ldv, vcols, a.right, N, NP, c0, bc, part, cm_blocks, inv, wt_hi, fast ? 0 : 1);
+                a.V, a.ldv, vcols, a.right, N, NP, c0, bc, part, cm_blocks, inv, wt_hi, fast ? 0 : 1, col_perm);
             FD_LAUNCH_CHECK(c, "k_pack_wt");
             // one map over W_hi (rows 0 .. BT) and, in the fp32-grade mode, W_lo behind it (rows BT .. 2 BT of the same array)
             if (!make_map_2d(&mh, wt_hi, (uint64_t)NP, (uint64_t)(fast ? BT : 2 * BT), (uint64_t)NP * 2, 64, fast ? BT : 2 * BT, CU_TENSOR_MAP_SWIZZLE_128B))
@@ -567,9 +576,7 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
                 FD_TRY(launch_fast_product(c, BT, mr, mc, mh, pb, std::min(pb.num_work, c->sm_count)));
                 continue;
             }
-            // Accumulator flush: after two column tiles where the small terms have columns of their own (16 additions at the
-            // magnitude of the sum), after every tile where the three terms share them (24); see fd_tc_block.cu.
-            p.flush = c->opt_flush > 0 ? c->opt_flush : (BT <= 32 ? 2 : 1);
+            p.flush = c->opt_flush > 0 ? c->opt_flush : 1;
             FD_TRY(launch_block_product(c, BT, mr, mc, mh, p));
         }
     }

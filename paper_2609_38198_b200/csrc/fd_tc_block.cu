@@ -22,9 +22,9 @@
 // pipes.  Sixteen exponential warps and a product issued per 32-column quarter keep the chain exponentials -> product ->
 // Gram -> exponentials of a buffer shorter than the other row tile's exponentials.  Per tile: 1024 SM clocks of MUFU, 193 K16 clocks of Gram MMAs, 12 BT clocks of product MMAs.  Up to 32 columns
 // the W_lo product shares an instruction with the W_hi one (B operand [W_hi | W_lo], N = 2 BT) and P_lo W_hi is added to
-// the W_lo half of the accumulator: the sum of the large terms then sees 8 round-toward-zero additions per tile instead
-// of 24, so two tiles may be summed before a flush with less rounding than one had with three terms in one accumulator (measured
-// scale error of K V beyond the exponents' own, N = 30000: 2.0e-7 / 2.3e-7 for positive / random-sign V against 2.4e-7 / 5e-7).
+// the W_lo half of the accumulator: 16 MMAs a tile instead of 24, and the sum of the large terms sees 8 round-toward-zero additions
+// per tile instead of 24 (scale error of K V beyond the exponents' own with a flush every tile: 1.5e-7 / 1.2e-7 for positive /
+// random-sign V against 1.5e-7 / 5.4e-7 with three terms in one accumulator; a flush every two tiles is 2 % faster and doubles it).
 // Measured against the layout it replaced (8 exponential warps that also owned the accumulators, three separate terms, whole
 // row pairs per CTA with half-range items for the last round), with the same elected issue: N = 2^20, b = 64: 473 -> 429 ms;
 // N = 2^17, b = 32: 5.91 -> 5.31 ms; N = 2^18, D = 30, b = 32: 28.5 -> 26.5 ms; N = 50021, b = 20: 1.03 -> 0.81 ms.
@@ -42,6 +42,7 @@ namespace {
 
 using namespace tc;
 
+constexpr int kSumFlushes = 32;    // flushes per register sum where the points are ordered
 constexpr int kThreadsB = 896;
 constexpr int kRegsLaunch = 72, kRegsExp = 72, kRegsFlush = 88, kRegsUtil = 40;
 static_assert(kThreadsB * kRegsLaunch == 512 * kRegsExp + 256 * kRegsFlush + 128 * kRegsUtil,
@@ -74,7 +75,7 @@ struct BlockParams {
     int64_t np;                  // padded row count of the operand arrays (row index of K slab c = c * np + p)
     int64_t ldy;
     float* Y;
-    float* part;                 // 2 * gridDim.x slots of [BT][256] floats: shares of row pairs that are cut
+    float* part;                 // slots of [BT][256] floats: two per CTA for shares of row pairs that are cut, then one per CTA for its sums
     const float* left;           // may be null
     const float* colscale_inv;   // per column: 2^-bias / colscale
     unsigned int* status;
@@ -82,31 +83,49 @@ struct BlockParams {
     int jt0, num_jt;             // column tiles [jt0, jt0 + num_jt) of this launch
     int K16, b, flush, stages;
     int accumulate;              // add to Y (later column chunks) instead of storing
+    // tile lists (null: every column tile): column tiles of row pair r at list[r * tiles ..], steps before it offs[r]
+    const unsigned short* list; const unsigned int* offs;
+    int tiles;
+    const int* perm;             // row of Y and left for each row of the operand (null: the same)
 };
 
 // First step of CTA `cta` in the flat sequence of steps, and the work item (part of one row pair) that starts at step g of it.
 __host__ __device__ __forceinline__ long long range_begin(long long total, int cta, int ctas) { return total * cta / ctas; }
-struct Item { int pair, j0, n; };
-struct Steps {                   // walks a CTA's range item by item
-    int pair, j0, left, num_jt;
-    __device__ __forceinline__ Steps(const BlockParams& p) {
-        const long long total = (long long)p.pairs * p.num_jt;
-        const long long g0 = range_begin(total, (int)blockIdx.x, (int)gridDim.x);
-        pair = (int)(g0 / p.num_jt);
-        j0 = (int)(g0 - (long long)pair * p.num_jt);
-        left = (int)(range_begin(total, (int)blockIdx.x + 1, (int)gridDim.x) - g0);
-        num_jt = p.num_jt;
+struct Item { int pair, j0, n; bool whole; };
+// Row pair that holds step g of the lists.
+__device__ __forceinline__ int pair_of(const BlockParams& p, unsigned int g) {
+    int lo = 0, hi = p.pairs - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (p.offs[mid] <= g) lo = mid;
+        else hi = mid - 1;
     }
-    __device__ __forceinline__ bool next(Item& it) {
+    return lo;
+}
+template <bool ORD>
+struct Steps {                   // walks a CTA's range item by item
+    int pair, j0, left;
+    __device__ __forceinline__ Steps(const BlockParams& p) {
+        const bool listed = ORD && p.list;
+        const long long total = listed ? (long long)p.offs[p.pairs] : (long long)p.pairs * p.num_jt;
+        const long long g0 = range_begin(total, (int)blockIdx.x, (int)gridDim.x);
+        pair = listed ? pair_of(p, (unsigned int)g0) : (int)(g0 / p.num_jt);
+        j0 = (int)(g0 - (listed ? (long long)p.offs[pair] : (long long)pair * p.num_jt));
+        left = (int)(range_begin(total, (int)blockIdx.x + 1, (int)gridDim.x) - g0);
+    }
+    __device__ __forceinline__ bool next(const BlockParams& p, Item& it) {
         if (left <= 0) return false;
+        const int full = ORD && p.list ? (int)(p.offs[pair + 1] - p.offs[pair]) : p.num_jt;
         it.pair = pair; it.j0 = j0;
-        it.n = num_jt - j0 < left ? num_jt - j0 : left;
+        it.n = full - j0 < left ? full - j0 : left;
+        it.whole = it.n == full;
         left -= it.n; j0 = 0; ++pair;
         return true;
     }
 };
 
-template <int BT>
+// ORD: the points are ordered (perm, where the rows are the context's own) and tiles may be listed.
+template <int BT, bool ORD>
 __global__ void __launch_bounds__(kThreadsB, 1)
 k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUtensorMap map_xcol,
         const __grid_constant__ CUtensorMap map_w, const BlockParams p) {
@@ -153,8 +172,8 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
             prefetch_tmap(&map_xrow); prefetch_tmap(&map_xcol); prefetch_tmap(&map_w);
             uint32_t issued = 0, s = 0, ph = 1, xph = 1;           // stage ring position and the parity of its "empty" phase
             bool ok = true;
-            Steps steps(p);
-            for (Item it; ok && steps.next(it);) {
+            Steps<ORD> steps(p);
+            for (Item it; ok && steps.next(p, it);) {
                 ok = mbar_wait(&bars->xempty, xph, abort_flag, p.status, 1);
                 if (!ok) break;
                 xph ^= 1u;
@@ -167,7 +186,7 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
                     ok = mbar_wait(&bars->empty[s], ph, abort_flag, p.status, 2);
                     if (!ok) break;
                     uint8_t* st = stage_base + s * SM::stage_bytes(K16);
-                    const int x0 = (p.jt0 + it.j0 + j) * 128;
+                    const int x0 = (ORD && p.list ? (int)p.list[(size_t)it.pair * p.tiles + it.j0 + j] : p.jt0 + it.j0 + j) * 128;
                     mbar_expect_tx(&bars->full[s], SM::stage_bytes(K16));
                     for (int c = 0; c < K16; ++c)
                         tma_load_2d(st + c * SM::kXChunk, &map_xcol, 0, (int)(c * p.np + x0), &bars->full[s]);
@@ -198,8 +217,8 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
             constexpr uint32_t kSlab = SM::kXChunk >> 4;
             uint32_t s = 0, sph = 0, slot = 0, kph = 1, six = 0, xph = 0;
             bool ok = true;
-            Steps steps(p);
-            for (Item it; ok && steps.next(it);) {
+            Steps<ORD> steps(p);
+            for (Item it; ok && steps.next(p, it);) {
                 ok = mbar_wait(&bars->xfull, xph, abort_flag, p.status, 3);
                 if (!ok) break;
                 xph ^= 1u;
@@ -243,8 +262,8 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
             const uint32_t stage_step = (uint32_t)(SM::stage_bytes(K16) >> 4);
             uint32_t s = 0, slot = 0, pph = 0, yph = 1;            // ring positions; yph: parity of the accumulators' "empty" phase
             bool ok = true;
-            Steps steps(p);
-            for (Item it; ok && steps.next(it);) {
+            Steps<ORD> steps(p);
+            for (Item it; ok && steps.next(p, it);) {
                 int in_group = 0;                                  // column tiles accumulated in the current group
                 for (int j = 0; j < it.n && ok; ++j) {
                     const bool group_start = in_group == 0;
@@ -271,13 +290,20 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
                             const uint32_t aq = p_addr + 32u * q;
 #pragma unroll
                             for (int k = 0; k < 2; ++k) {
-                                if (k == 0 && i == 0 && group_start) mma_ts2<0>(y_addr, aq, bq, wdesc_hi, idesc_hi);
-                                else mma_ts2<1>(y_addr, aq + 16 * k, bq + 2 * k, wdesc_hi, idesc_hi);
-                                if (kConcat) mma_ts2<1>(y_addr + BT, aq + 16 * k + 8, bq + 2 * k, wdesc_hi, idesc_lo);
-                                else {
-                                    mma_ts2<1>(y_addr, aq + 16 * k + 8, bq + 2 * k, wdesc_hi, idesc_lo);
+                                if constexpr (kConcat) {
+                                    if (k == 0 && i == 0 && group_start) mma_ts2<0>(y_addr, aq, bq, wdesc_hi, idesc_hi);
+                                    else mma_ts2<1>(y_addr, aq + 16 * k, bq + 2 * k, wdesc_hi, idesc_hi);
+                                    mma_ts2<1>(y_addr + BT, aq + 16 * k + 8, bq + 2 * k, wdesc_hi, idesc_lo);
+                                } else {
+                                    // the two small terms of both K steps first: what they round away is smaller then
+                                    if (k == 0 && i == 0 && group_start) mma_ts2<0>(y_addr, aq + 8, bq, wdesc_hi, idesc_lo);
+                                    else mma_ts2<1>(y_addr, aq + 16 * k + 8, bq + 2 * k, wdesc_hi, idesc_lo);
                                     mma_ts2<1>(y_addr, aq + 16 * k, bq + (uint32_t)(SM::kWPart >> 4) + 2 * k, wdesc_hi, idesc_lo);
                                 }
+                            }
+                            if constexpr (!kConcat) {
+#pragma unroll
+                                for (int k = 0; k < 2; ++k) mma_ts2<1>(y_addr, aq + 16 * k, bq + 2 * k, wdesc_hi, idesc_lo);
                             }
                         }
                         if (!ok) break;
@@ -302,8 +328,8 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
         const int row_in_pair = t * 128 + wq * 32 + lane;
         uint32_t yph = 0;
         bool ok = true;
-        Steps steps(p);
-        for (Item it; ok && steps.next(it);) {
+        Steps<ORD> steps(p);
+        for (Item it; ok && steps.next(p, it);) {
             float acc[BT];
 #pragma unroll
             for (int c = 0; c < BT; ++c) acc[c] = 0.f;
@@ -311,8 +337,24 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
             // keep one sign, n additions lose n / 4 ulp of the result on average (half an ulp each, at a running magnitude that
             // averages half the final one): 2^-25 of the result per addition.  The flush adds that expected loss back.  (With
             // the small terms in columns of their own only the 8 large additions per tile count.)
+            // Two-level sums where the points are ordered: every kSumFlushes groups the registers go to a slot in memory
+            // and restart.  A single fp32 sum over thousands of tiles drops what lies below half a unit in its last place: with ordered
+            // points most of the far tiles' shares (N = 2^17, 6-torus: -8.5e-7 of a row's sum, always of the same sign).  In the
+            // caller's order the tiles' shares are of one size and the single sum loses nothing of one sign.
+            const int period = kSumFlushes * p.flush;
             int left_tiles = it.n;
             while (left_tiles > 0) {
+                if constexpr (ORD) {
+                    const int done = it.n - left_tiles;
+                    if (done > 0 && done % period == 0) {
+                        float* sums = p.part + (size_t)(2 * gridDim.x + blockIdx.x) * BT * 256 + row_in_pair;
+#pragma unroll
+                        for (int c = 0; c < BT; ++c) {
+                            sums[c * 256] = done == period ? acc[c] : sums[c * 256] + acc[c];
+                            acc[c] = 0.f;
+                        }
+                    }
+                }
                 const int tiles_in_group = left_tiles < p.flush ? left_tiles : p.flush;
                 left_tiles -= tiles_in_group;
                 const float corr = 1.0f + (float)(tiles_in_group * (kConcat ? 8 : 24)) * 2.98023224e-8f;
@@ -340,7 +382,13 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
                 }
             }
             if (!ok) break;
-            if (it.n != p.num_jt) {
+            if constexpr (ORD)
+                if (it.n > period) {
+                    const float* sums = p.part + (size_t)(2 * gridDim.x + blockIdx.x) * BT * 256 + row_in_pair;
+#pragma unroll
+                    for (int c = 0; c < BT; ++c) acc[c] += sums[c * 256];
+                }
+            if (!it.whole) {
                 // a share of a row pair that a cut falls into: at most two per CTA (one that starts its row pair, one that does not)
                 float* o = p.part + (size_t)(2 * blockIdx.x + (it.j0 == 0 ? 1 : 0)) * BT * 256 + row_in_pair;
 #pragma unroll
@@ -348,8 +396,9 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
                     if (c < p.b) o[c * 256] = acc[c];
                 continue;
             }
-            const int64_t row = (int64_t)it.pair * 256 + row_in_pair;
+            int64_t row = (int64_t)it.pair * 256 + row_in_pair;
             if (row < p.Nrow) {
+                if (ORD && p.perm) row = p.perm[row];
                 const float l = p.left ? p.left[row] : 1.0f;
 #pragma unroll
                 for (int c = 0; c < BT; ++c)
@@ -371,8 +420,8 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
         const uint32_t lane_addr = ((uint32_t)(wq * 32) << 16) + 64u * h;
         uint32_t slot = (uint32_t)t, six = (uint32_t)t, ph = 0;       // tile index mod 3, mod 6, and the phase of s_full[six]
         bool ok = true;
-        Steps steps(p);
-        for (Item it; ok && steps.next(it);) {
+        Steps<ORD> steps(p);
+        for (Item it; ok && steps.next(p, it);) {
             for (int j = 0; j < it.n; ++j) {
                 ok = mbar_wait(&bars->s_full[six], ph, abort_flag, p.status, 9);
                 if (!ok) break;
@@ -422,15 +471,16 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
 template <int BT>
 __global__ void __launch_bounds__(256)
 k_block_fix(const BlockParams p, int ctas) {
-    const long long total = (long long)p.pairs * p.num_jt;
     const int pair = blockIdx.x;
-    const long long g0 = (long long)pair * p.num_jt, g1 = g0 + p.num_jt;
-    int cta = (int)(g0 * ctas / total);
-    while (cta > 0 && range_begin(total, cta, ctas) > g0) --cta;
-    while (range_begin(total, cta + 1, ctas) <= g0) ++cta;
+    const long long total = p.list ? (long long)p.offs[p.pairs] : (long long)p.pairs * p.num_jt;
+    const long long g0 = p.list ? (long long)p.offs[pair] : (long long)pair * p.num_jt;
+    const long long g1 = p.list ? (long long)p.offs[pair + 1] : g0 + p.num_jt;
+    // the last CTA whose range begins at or before step g0
+    int cta = (int)(((g0 + 1) * ctas - 1) / total);
     if (range_begin(total, cta + 1, ctas) >= g1) return;               // not cut: the CTA stored it
-    const int64_t row = (int64_t)pair * 256 + threadIdx.x;
+    int64_t row = (int64_t)pair * 256 + threadIdx.x;
     if (row >= p.Nrow) return;
+    if (p.perm) row = p.perm[row];
     const int c0 = (int)blockIdx.y * 8;
     float acc[8];
 #pragma unroll
@@ -461,21 +511,24 @@ fd_status launch_one(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, co
     const int smem = SmemB<BT>::total(p.K16, p.stages);
     if (smem > 227 * 1024) return fail(c, FD_ERR_UNSUPPORTED, "block product kernel needs %d B of shared memory", smem);
     // the attribute is per device: set it on every launch (cheap) rather than remembering one device
-    FD_CUDA(c, cudaFuncSetAttribute(k_block<BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    const auto kernel = c->order_state == 1 ? k_block<BT, true> : k_block<BT, false>;
+    FD_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     cudaFuncAttributes fa;
-    FD_CUDA(c, cudaFuncGetAttributes(&fa, k_block<BT>));
+    FD_CUDA(c, cudaFuncGetAttributes(&fa, kernel));
     if (fa.numRegs != kRegsLaunch)
         return fail(c, FD_ERR_UNSUPPORTED, "block product kernel compiled with %d registers per thread, %d expected", fa.numRegs, kRegsLaunch);
+    // (with lists: one launch over everything; consecutive row pairs are neighbours and share most of their column tiles)
+    if (p.list) jt_chunk = jt_total;
     for (int j0 = 0; j0 < jt_total; j0 += jt_chunk) {
         p.jt0 = j0;
         p.num_jt = std::min(jt_chunk, jt_total - j0);
         p.accumulate = j0 > 0;
-        const long long total = (long long)p.pairs * p.num_jt;
+        const long long total = p.list ? c->lists[0].total : (long long)p.pairs * p.num_jt;
         const int grid = (int)std::min<long long>(c->sm_count, total);
-        if ((size_t)2 * grid * BT * 256 > c->L.part_floats) return fail(c, FD_ERR_WORKSPACE, "no room for the shares of cut row pairs");
-        k_block<BT><<<grid, kThreadsB, smem, c->stream>>>(mr, mc, mw, p);
+        if ((size_t)3 * grid * BT * 256 > c->L.part_floats) return fail(c, FD_ERR_WORKSPACE, "no room for the shares of cut row pairs");
+        kernel<<<grid, kThreadsB, smem, c->stream>>>(mr, mc, mw, p);
         FD_LAUNCH_CHECK(c, "k_block");
-        bool cut = false;
+        bool cut = p.list != nullptr;
         for (int i = 1; i < grid && !cut; ++i) cut = range_begin(total, i, grid) % p.num_jt != 0;
         if (cut) {
             k_block_fix<BT><<<dim3((unsigned)p.pairs, (unsigned)ceil_div(p.b, 8)), 256, 0, c->stream>>>(p, grid);
@@ -494,7 +547,12 @@ fd_status launch_block_product(fd_ctx* c, int BT, const CUtensorMap& mr, const C
     BlockParams p{};
     p.Nrow = tp.Nrow; p.np = tp.np_rows; p.ldy = tp.ldy; p.Y = tp.Y; p.left = tp.left; p.colscale_inv = tp.colscale_inv;
     p.status = tp.status; p.part = c->at<float>(c->L.part);
-    p.pairs = tp.num_work; p.K16 = tp.K16; p.b = tp.b; p.flush = tp.flush;
+    p.pairs = tp.num_work; p.K16 = tp.K16; p.b = tp.b; p.flush = tp.flush; p.perm = tp.perm;
+    if (tp.use_lists) {
+        p.list = c->at<unsigned short>(c->L.lists);
+        p.offs = c->at<unsigned int>(c->L.list_counts) + 2 * p.pairs;
+        p.tiles = (int)(c->L.NP / 128);
+    }
     switch (BT) {
         case 16: return launch_one<16>(c, mr, mc, mw, p, tp.num_jt, tp.jt_chunk);
         case 32: return launch_one<32>(c, mr, mc, mw, p, tp.num_jt, tp.jt_chunk);

@@ -30,6 +30,8 @@ struct TcParams {
     float* Y; int64_t ldy;       // block products: output block
     float* q; double* rowsq;     // row-sum modes: outputs
     const float* weights;        // row-sum modes without squares: right weights, padded with zeros to whole tiles
+    const int* perm;             // row of Y, q and left for each row of the operand (null: the same)
+    int use_lists;               // block product: the tile lists of the context hold for this pass
     unsigned int* status;
 };
 
@@ -216,7 +218,7 @@ fd_status launch_fast_product(fd_ctx* c, int BT, const CUtensorMap& mr, const CU
 // Row sums of the context's whole point set from the tiles on or above the diagonal (fd_tc_sym.cu): q = left * sum_j weights_j K_ij (no
 // weights: 1, and the total of rowsq's N entries is sum_ij K_ij^2).
 fd_status launch_sym_rowsum(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, const float* weights, const float* left, float* q,
-                            double* rowsq);
+                            double* rowsq, const int* perm, bool use_lists);
 // fp32-grade block product of BT = 16, 32, 48 or 64 columns (fd_tc_block.cu).
 fd_status launch_block_product(fd_ctx* c, int BT, const CUtensorMap& mr, const CUtensorMap& mc, const CUtensorMap& mw,
                                const TcParams& tp);

@@ -57,14 +57,27 @@ struct SymParams {
     const float* weights;        // padded right weights (weighted instantiation)
     unsigned int* status;
     int pairs, num_jt, K16, shift;
+    // tile lists (null: every tile): the streamed tiles of resident pair r are the last uoffs[r + 1] - uoffs[r] entries of its list
+    const unsigned short* list; const unsigned int* counts; const unsigned int* uoffs;
 };
 
 constexpr int smem_total(int K16) { return 1024 + kStages * K16 * kXChunk + 2 * K16 * kXChunk + kSlots * 4 * 128 * 4 + 1024; }
 
 // Steps before resident pair r: pair r has the streamed tiles 2 r .. num_jt - 1.
 __host__ __device__ __forceinline__ long long steps_before(long long r, long long num_jt) { return r * num_jt - r * (r - 1); }
-struct Item { int pair, j0, n; };
-struct Steps {                   // walks a CTA's range item by item
+// A CTA's range, item by item.  One type without lists and one with them: the exponential warps of the weighted instantiation
+// have no register to spare (one type with a run-time choice spilled 176 B a thread instead of 28: N = 2^18, both passes 21.7 -> 23.0 ms).
+template <bool LISTED> struct Item;
+template <> struct Item<false> {
+    int pair, j0, n;             // streamed tiles j0 ..
+    __device__ __forceinline__ int tile(const SymParams&, int j) const { return j0 + j; }
+};
+template <> struct Item<true> {
+    int pair, first, n;          // entries first .. of the lists
+    __device__ __forceinline__ int tile(const SymParams& p, int j) const { return (int)__ldg(p.list + (first + j)); }
+};
+template <bool LISTED> struct Steps;
+template <> struct Steps<false> {
     int pair, j, left, num_jt;
     __device__ __forceinline__ Steps(const SymParams& p) {
         const long long total = steps_before(p.pairs, p.num_jt);
@@ -80,7 +93,7 @@ struct Steps {                   // walks a CTA's range item by item
         j = 2 * pair + (int)(g0 - steps_before(r, num_jt));
         left = (int)(g1 - g0);
     }
-    __device__ __forceinline__ bool next(Item& it) {
+    __device__ __forceinline__ bool next(const SymParams&, Item<false>& it) {
         if (left <= 0) return false;
         it.pair = pair; it.j0 = j;
         it.n = num_jt - j < left ? num_jt - j : left;
@@ -88,8 +101,33 @@ struct Steps {                   // walks a CTA's range item by item
         return true;
     }
 };
+template <> struct Steps<true> {
+    int pair, done, left;        // `done` steps of the pair lie before the range
+    __device__ __forceinline__ Steps(const SymParams& p) {
+        const long long total = (long long)p.uoffs[p.pairs];
+        const long long g0 = total * blockIdx.x / gridDim.x, g1 = total * (blockIdx.x + 1) / gridDim.x;
+        int lo = 0, hi = p.pairs - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if ((long long)p.uoffs[mid] <= g0) lo = mid;
+            else hi = mid - 1;
+        }
+        pair = lo;
+        done = (int)(g0 - (long long)p.uoffs[pair]);
+        left = (int)(g1 - g0);
+    }
+    __device__ __forceinline__ bool next(const SymParams& p, Item<true>& it) {
+        if (left <= 0) return false;
+        const int full = (int)(p.uoffs[pair + 1] - p.uoffs[pair]);
+        it.pair = pair;
+        it.first = pair * p.num_jt + (int)p.counts[pair] - full + done;
+        it.n = full - done < left ? full - done : left;
+        left -= it.n; ++pair; done = 0;
+        return true;
+    }
+};
 
-template <bool SQ, bool WEIGHTED>
+template <bool SQ, bool WEIGHTED, bool LISTED>
 __global__ void __launch_bounds__(kThreadsS, 1)
 k_sym(const __grid_constant__ CUtensorMap map_res, const __grid_constant__ CUtensorMap map_str, const SymParams p) {
     extern __shared__ uint8_t smem_raw[];
@@ -128,8 +166,8 @@ k_sym(const __grid_constant__ CUtensorMap map_res, const __grid_constant__ CUten
             prefetch_tmap(&map_res); prefetch_tmap(&map_str);
             uint32_t k = 0, xph = 1;                               // step counter; parity of the resident tiles' "empty" phase
             bool ok = true;
-            Steps steps(p);
-            for (Item it; ok && steps.next(it);) {
+            Steps<LISTED> steps(p);
+            for (Item<LISTED> it; ok && steps.next(p, it);) {
                 ok = mbar_wait(&bars->xempty, xph, abort_flag, p.status, 1);
                 if (!ok) break;
                 xph ^= 1u;
@@ -143,7 +181,7 @@ k_sym(const __grid_constant__ CUtensorMap map_res, const __grid_constant__ CUten
                     if (!ok) break;
                     mbar_expect_tx(&bars->full[s], K16 * kXChunk);
                     for (int c = 0; c < K16; ++c)
-                        tma_load_2d(stage_base + (s * K16 + c) * kXChunk, &map_str, 0, (int)(c * p.np + (int64_t)(it.j0 + j) * 128), &bars->full[s]);
+                        tma_load_2d(stage_base + (s * K16 + c) * kXChunk, &map_str, 0, (int)(c * p.np + (int64_t)it.tile(p, j) * 128), &bars->full[s]);
                 }
             }
             if (!ok) {
@@ -164,8 +202,8 @@ k_sym(const __grid_constant__ CUtensorMap map_res, const __grid_constant__ CUten
             constexpr uint32_t kSlab = kXChunk >> 4;
             uint32_t k = 0, xph = 0;
             bool ok = true;
-            Steps steps(p);
-            for (Item it; ok && steps.next(it);) {
+            Steps<LISTED> steps(p);
+            for (Item<LISTED> it; ok && steps.next(p, it);) {
                 ok = mbar_wait(&bars->xfull, xph, abort_flag, p.status, 3);
                 if (!ok) break;
                 xph ^= 1u;
@@ -204,8 +242,8 @@ k_sym(const __grid_constant__ CUtensorMap map_res, const __grid_constant__ CUten
         const int pt0 = (warp - 18) * 64 + lane * 2;
         uint32_t k = 0;
         bool ok = true;
-        Steps steps(p);
-        for (Item it; ok && steps.next(it);) {
+        Steps<LISTED> steps(p);
+        for (Item<LISTED> it; ok && steps.next(p, it);) {
             for (int j = 0; j < it.n; ++j, ++k) {
                 const uint32_t slot = k % kSlots;
                 ok = mbar_wait(&bars->r_ready[slot], (k / kSlots) & 1, abort_flag, p.status, 12);
@@ -215,7 +253,7 @@ k_sym(const __grid_constant__ CUtensorMap map_res, const __grid_constant__ CUten
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&bars->r_free[slot]);
                 const float x = (a.x + b.x) + (c.x + d.x), y = (a.y + b.y) + (c.y + d.y);
-                const int64_t pt = (int64_t)(it.j0 + j) * 128 + pt0;
+                const int64_t pt = (int64_t)it.tile(p, j) * 128 + pt0;
                 if (pt < p.N && x != 0.f) atomicAdd(p.sums + pt, (unsigned long long)__double2ll_rn((double)x * fix));
                 if (pt + 1 < p.N && y != 0.f) atomicAdd(p.sums + pt + 1, (unsigned long long)__double2ll_rn((double)y * fix));
             }
@@ -231,15 +269,15 @@ k_sym(const __grid_constant__ CUtensorMap map_res, const __grid_constant__ CUten
         double dsq = 0.0;
         bool ok = true;
         float acc[64];
-        Steps steps(p);
-        for (Item it; ok && steps.next(it);) {
+        Steps<LISTED> steps(p);
+        for (Item<LISTED> it; ok && steps.next(p, it);) {
             const int It = 2 * it.pair + t;
             const float4* wres = WEIGHTED ? reinterpret_cast<const float4*>(p.weights + (int64_t)It * 128 + 64 * h) : nullptr;
 #pragma unroll
             for (int c = 0; c < 64; ++c) acc[c] = 0.f;
             int pending = 0;                                       // tiles accumulated in acc since the last reduction
             for (int j = 0; j < it.n; ++j, ++k) {
-                const int J = it.j0 + j;
+                const int J = it.tile(p, j);
                 const float wj = WEIGHTED ? __ldg(p.weights + (int64_t)J * 128 + pt_in_tile) : 1.f;
                 const uint32_t buf = (2 * k + (uint32_t)t) & 3;
                 ok = mbar_wait(&bars->s_full[buf], (k >> 1) & 1, abort_flag, p.status, 8);
@@ -332,23 +370,25 @@ k_sym(const __grid_constant__ CUtensorMap map_res, const __grid_constant__ CUten
 
 // Fixed-point sums -> q (times the left weight); clears the squares' slots that no CTA wrote.
 __global__ void k_sym_finish(const unsigned long long* __restrict__ sums, int64_t n, double scale, const float* __restrict__ left,
-                             float* __restrict__ q, double* __restrict__ sq, int ctas) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    q[i] = (float)((double)(long long)sums[i] * (left ? scale * (double)left[i] : scale));
-    if (sq && i >= ctas) sq[i] = 0.0;
+                             float* __restrict__ q, double* __restrict__ sq, int ctas, const int* __restrict__ perm) {
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    const int64_t i = perm ? perm[p] : p;
+    q[i] = (float)((double)(long long)sums[p] * (left ? scale * (double)left[i] : scale));
+    if (sq && p >= ctas) sq[p] = 0.0;
 }
 
 template <bool SQ, bool WEIGHTED>
 fd_status launch_one(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, const SymParams& p, int grid) {
     const int smem = smem_total(p.K16);
     // the attribute is per device: set it on every launch (cheap) rather than remembering one device
-    FD_CUDA(c, cudaFuncSetAttribute(k_sym<SQ, WEIGHTED>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    const auto kernel = p.list ? k_sym<SQ, WEIGHTED, true> : k_sym<SQ, WEIGHTED, false>;
+    FD_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     cudaFuncAttributes fa;
-    FD_CUDA(c, cudaFuncGetAttributes(&fa, k_sym<SQ, WEIGHTED>));
+    FD_CUDA(c, cudaFuncGetAttributes(&fa, kernel));
     if (fa.numRegs != kRegsLaunch)
         return fail(c, FD_ERR_UNSUPPORTED, "symmetric row-sum kernel compiled with %d registers per thread, %d expected", fa.numRegs, kRegsLaunch);
-    k_sym<SQ, WEIGHTED><<<grid, kThreadsS, smem, c->stream>>>(mr, mc, p);
+    kernel<<<grid, kThreadsS, smem, c->stream>>>(mr, mc, p);
     FD_LAUNCH_CHECK(c, "k_sym");
     return FD_OK;
 }
@@ -357,7 +397,8 @@ fd_status launch_one(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, co
 
 namespace tc {
 
-fd_status launch_sym_rowsum(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, const float* weights, const float* left, float* q, double* rowsq) {
+fd_status launch_sym_rowsum(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, const float* weights, const float* left, float* q, double* rowsq,
+                            const int* perm, bool use_lists) {
     const Layout& L = c->L;
     SymParams p{};
     p.N = L.N; p.np = L.NP; p.K16 = L.K16;
@@ -369,10 +410,16 @@ fd_status launch_sym_rowsum(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap&
     while (((int64_t)1 << lg) < L.NP) ++lg;
     p.shift = 61 - kBias - lg;
     FD_CUDA(c, cudaMemsetAsync(p.sums, 0, (size_t)L.N * 8, c->stream));
-    const int grid = (int)std::min<long long>(std::min<long long>(c->sm_count, L.N), steps_before(p.pairs, p.num_jt));
+    if (use_lists) {
+        p.list = c->at<unsigned short>(L.lists);
+        p.counts = c->at<unsigned int>(L.list_counts);
+        p.uoffs = p.counts + 3 * p.pairs + 1;
+    }
+    // (every pair's own two tiles are listed: there are at least two steps per pair)
+    const int grid = (int)std::min<long long>(std::min<long long>(c->sm_count, L.N), use_lists ? 2ll * p.pairs : steps_before(p.pairs, p.num_jt));
     if (rowsq) FD_TRY((launch_one<true, false>(c, mr, mc, p, grid)));
     else FD_TRY((launch_one<false, true>(c, mr, mc, p, grid)));
-    k_sym_finish<<<(unsigned)ceil_div(L.N, 256), 256, 0, c->stream>>>(p.sums, L.N, std::ldexp(1.0, -(p.shift + kBias)), left, q, rowsq, grid);
+    k_sym_finish<<<(unsigned)ceil_div(L.N, 256), 256, 0, c->stream>>>(p.sums, L.N, std::ldexp(1.0, -(p.shift + kBias)), left, q, rowsq, grid, perm);
     FD_LAUNCH_CHECK(c, "k_sym_finish");
     return FD_OK;
 }

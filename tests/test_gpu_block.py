@@ -152,3 +152,55 @@ def test_coordinates_that_all_points_share(N, path, D, const):
         Ro = (1.0 if left is None else left[:, None].astype(np.float64)) * (K @ V.astype(np.float64))
         assert np.linalg.norm(R.cpu().numpy().astype(np.float64) - Ro) <= 1e-5 * np.linalg.norm(Ro)
     ctx.close()
+
+
+@pytest.mark.parametrize("N,kind", [(8192, "manifold"), (8193, "clusters"), (9001, "line"), (8500, "duplicates")])
+def test_far_tiles_are_left_out(N, kind):
+    """Data with many pairs beyond the exponent limit: the points are ordered, tiles without near pairs left out.  Same results as the
+    float64 oracle (gates of the Gram-form path: degrees 2e-5, product 1e-5; what is left out is below 2^-40 of a kernel value's
+    maximum), bit-identical repeats, lists remade when the bandwidth changes, external rows against ordered columns, and the same
+    operator applied through other precision modes and without the symmetric passes."""
+    import __graft_entry__ as g
+    g.build()
+    import paper_2609_38198_b200 as fd
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(N)
+    if kind == "manifold":
+        X, beta = workloads.latent_torus(N, seed=42), 5.0
+    elif kind == "clusters":                       # 5 clusters of unequal size far apart, 12 coordinates
+        X = (rng.standard_normal((5, 12)) * 2.0)[rng.choice(5, N, p=(0.5, 0.2, 0.15, 0.1, 0.05))] + 0.1 * rng.standard_normal((N, 12))
+        X, beta = X.astype(np.float32), 0.8
+    elif kind == "line":                           # one coordinate that matters, unevenly sampled
+        X = np.zeros((N, 3)); X[:, 0] = 8.0 * rng.random(N) ** 1.3; X[:, 1] = 0.01 * rng.standard_normal(N); X[:, 2] = 0.01 * rng.standard_normal(N)
+        X, beta = X.astype(np.float32), 2.0
+    else:                                          # most points coincide
+        X = np.zeros((N, 4)); X[N // 2:] = rng.standard_normal((N - N // 2, 4)) * 0.1 + 2.0
+        X, beta = X.astype(np.float32), 2.0
+    b = 20
+    V = workloads.block(N, b, seed=2)
+    Vd = fd.to_colmajor(V, dev)
+    ctx = fd.Context(torch.from_numpy(X).to(dev), b_max=b)
+    ctx.set_option("path", fd.FD_PATH_TC)
+    ctx.set_option("tc_max_mag", 1e3)
+    shares = []
+    for bt in (beta, 0.1 * beta, beta):
+        q, d, s, so, so2 = ctx.degree(bt, 1.0)
+        Y, Y2, Yf = ctx.apply(Vd), ctx.apply(Vd), ctx.apply(Vd, prec=fd.FD_PREC_FAST)
+        shares.append(ctx.get_option("tile_share"))
+        assert torch.equal(Y, Y2)
+        if bt != beta:
+            continue
+        qo, do, s_o, soo, so2o = dense.degree(X, bt, 1.0)
+        Yo = dense.apply(X, bt, 1.0, V)
+        assert np.abs(q.cpu().numpy() / qo - 1).max() <= 2e-5 and np.abs(d.cpu().numpy() / do - 1).max() <= 4e-5
+        assert abs(so - soo) <= 2e-5 * (soo + N) and abs(so2 - so2o) <= 4e-5 * (so2o + N)
+        assert np.linalg.norm(Y.cpu().numpy().astype(np.float64) - Yo) <= 1e-5 * np.linalg.norm(Yo)
+        assert np.linalg.norm(Yf.cpu().numpy().astype(np.float64) - Yo) <= 3e-3 * np.linalg.norm(Yo)
+        R = ctx.apply_general(bt, Vd, Xrow=torch.from_numpy(X[:77].copy()).to(dev)).cpu().numpy().astype(np.float64)
+        Ro = np.exp(-bt * ((X[:77, None, :].astype(np.float64) - X[None].astype(np.float64)) ** 2).sum(-1)) @ V.astype(np.float64)
+        assert np.linalg.norm(R - Ro) <= 1e-5 * np.linalg.norm(Ro)
+    assert shares[0] < 0.9 and shares[2] == shares[0], shares
+    ctx.set_option("sym", 0)
+    q0, d0, s0, _, _ = ctx.degree(beta, 1.0)
+    assert ((q0 - q).abs() / q0).max().item() <= 2e-6
+    ctx.close()
