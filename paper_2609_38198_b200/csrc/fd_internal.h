@@ -180,8 +180,9 @@ fd_status gather_rows(fd_ctx* c, float* A, int64_t lda, int cols);
 // In-place sum over the ranks of n host doubles.  No-op for an unsharded context.
 fd_status allreduce_host(fd_ctx* c, double* buf, int64_t n);
 // Tile lists of a bandwidth for block products (kind 0) or degree passes (1) (fd_order.cu): decides c->lists[kind] and, where they are
-// used, brings them into the workspace; orders the points first if that can pay.  Synchronises when the bandwidth is new.
-fd_status tile_lists(fd_ctx* c, double beta, int kind);
+// used, brings them into the workspace; orders the points first if that can pay.  A new bandwidth is decided, with a wait, only where
+// `decide` allows it; without, nothing is listed for it.
+fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide);
 // Reads and clears the tensor-core kernel's status word; FD_ERR_TIMEOUT if a bounded wait expired.  Synchronises.
 fd_status tc_check_status(fd_ctx* c);
 // Launches a one-thread kernel whose bounded wait must expire after limit_cycles (test of the time-out plumbing).

@@ -281,7 +281,7 @@ k_lists(const float* __restrict__ box, int DP, int tiles, float limit2, unsigned
 
 }  // namespace
 
-fd_status tile_lists(fd_ctx* c, double beta, int kind) {
+fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide) {
     const Layout& L = c->L;
     auto& st = c->lists[kind];
     if (L.perm == 0 || c->order_state < 0) return FD_OK;
@@ -289,6 +289,7 @@ fd_status tile_lists(fd_ctx* c, double beta, int kind) {
     // Beyond an exponent of 40 both fp16 pieces of a kernel value are zero (2^15 2^-40 = 2^-25 rounds to zero), beyond 60 a degree
     // contribution is below the fixed-point unit; the quarter covers the rounding of the boxes' distance.
     const double limit = kind == 0 ? 40.25 : 60.25;
+    if (!decide && st.beta != beta) return FD_OK;
     const bool known = st.beta == beta;                            // decided before, only overwritten by the other kind's lists
     const int64_t N = L.N;
     const int tiles = (int)(L.NP / 128), pairs = (int)(L.NP / 256);

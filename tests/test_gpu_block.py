@@ -204,3 +204,26 @@ def test_far_tiles_are_left_out(N, kind):
     q0, d0, s0, _, _ = ctx.degree(beta, 1.0)
     assert ((q0 - q).abs() / q0).max().item() <= 2e-6
     ctx.close()
+
+
+def test_product_at_a_bandwidth_without_degrees_takes_every_tile():
+    """Ordered points, and a product at a bandwidth for which no degree pass has decided about the tiles: it returns without waiting and
+    runs over all of them, in the caller's order of rows (float64 oracle, gate of the Gram-form product 1e-5)."""
+    import __graft_entry__ as g
+    g.build()
+    import paper_2609_38198_b200 as fd
+    dev = torch.device("cuda:0")
+    N, b = 8193, 16
+    X = workloads.latent_torus(N, seed=42)
+    V = workloads.block(N, b, seed=3)
+    ctx = fd.Context(torch.from_numpy(X).to(dev), b_max=b)
+    ctx.set_option("path", fd.FD_PATH_TC)
+    ctx.set_option("tc_max_mag", 1e3)
+    ctx.degree(5.0, 1.0)
+    assert ctx.get_option("tile_share") < 0.9
+    rows = np.arange(0, N, 41)
+    for beta in (3.0, 5.0, 3.0):
+        Y = ctx.apply_general(beta, fd.to_colmajor(V, dev)).cpu().numpy().astype(np.float64)[rows]
+        K = np.exp(-beta * ((X[rows, None, :].astype(np.float64) - X[None].astype(np.float64)) ** 2).sum(-1))
+        assert np.linalg.norm(Y - K @ V) <= 1e-5 * np.linalg.norm(K @ V)
+    ctx.close()
