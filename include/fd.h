@@ -98,7 +98,8 @@ fd_status fd_destroy(fd_ctx* ctx);
  * a one-thread kernel whose bounded wait on a barrier that nothing completes must expire; the next
  * fd_synchronize then returns FD_ERR_TIMEOUT and the context stays usable).  fd_get_option also reports "last_path" (the
  * family that served the latest pass), "beta", "mean_sq", "max_sq", "tile_share" (share of the tiles that
- * fp32-grade Gram-form products of the whole point set evaluate at the degree passes' bandwidth; the others hold zeros only) and "tc_cycles" (SM cycles the first CTA of the most
+ * fp32-grade products of the whole point set evaluate at the degree passes' bandwidth, in the kernel family of the latest pass; the others
+ * hold zeros only) and "tc_cycles" (SM cycles the first CTA of the most
  * recent tensor-core quadratic kernel spent on its work items; synchronises; with the kernel's wall time it
  * gives the SM clock the kernel actually ran at).  Unknown name -> FD_ERR_INVALID. */
 fd_status fd_set_option(fd_ctx* ctx, const char* name, double value);

@@ -69,12 +69,15 @@ Layout make_layout(int64_t N, int32_t D, int32_t b_max, int32_t m_max) {
     L.symsum = carve(cur, (size_t)N * 8);
     L.weights = carve(cur, (size_t)L.NP * 4);
     // tile lists: N^2 / 16384 bytes, 17 MB at 2^19 points; larger sets run over all tiles (as do small ones, where nothing is gained)
-    if (N >= 8192 && N <= (int64_t)1 << 19) {
+    if (N >= (L.DP <= 8 ? 16384 : 32768) && N <= (int64_t)1 << 19) {
         const size_t tiles = (size_t)(L.NP / 128), pairs = tiles / 2;
         L.perm = carve(cur, (size_t)N * 4);
-        L.boxes = carve(cur, tiles * 2 * 8 * 4);
+        // (direct-difference kernels: column tiles of 16 points; up to 8 coordinates and 2^17 points, 8.4 MB of lists)
+        const size_t col_tiles = L.DP <= 8 && N <= (int64_t)1 << 17 ? 8 * tiles : tiles;
+        L.direct_lists = col_tiles > tiles;
+        L.boxes = carve(cur, col_tiles * 2 * 8 * 4);
         if (L.DP > 8) L.zproj = carve(cur, (size_t)N * 8 * 4);
-        L.lists = carve(cur, pairs * tiles * 2);
+        L.lists = carve(cur, pairs * col_tiles * 2);
         L.list_counts = carve(cur, (4 * pairs + 2) * 4);
     }
     if (m_max > 0) {
@@ -206,7 +209,9 @@ fd_status fd_get_option(const fd_ctx* c, const char* name, double* v) {
     }
     else if (!strcmp(name, "tile_share")) {
         const double tiles = (double)(c->L.NP / 128);
-        *v = c->lists[0].on ? (double)c->lists[0].total / (0.5 * tiles * tiles) : 1.0;
+        const auto& direct = c->lists[2];
+        if (c->last_path == FD_PATH_SIMT) *v = direct.on ? (double)direct.total / (tiles * tiles) : 1.0;
+        else *v = c->lists[0].on ? (double)c->lists[0].total / (0.5 * tiles * tiles) : 1.0;
     }
     else if (!strcmp(name, "mean_sq")) *v = c->mean_sq;
     else if (!strcmp(name, "max_sq")) *v = c->max_sq;

@@ -18,6 +18,12 @@
 // as it is (column-major) and scaled on the way into shared memory: no packing pass.
 // N = 16384, D = 4, b = 16: 412 -> 309 us a product; N = 12000, D = 12, b = 48: 944 -> 639 us; N = 6000, D = 2, both degree passes:
 // 136 -> 109 us (one row per thread, separate packing pass, one CTA more or less per SM at the end).
+//
+// Up to 8 coordinates, from 16384 points on, column tiles whose kernel values are all exactly zero are left out where the degree passes found
+// enough of them (fd_order.cu): a step is then 64 listed positions of the points' order, gathered through it (which costs a fifth
+// more per step; the next step's indices are looked up during the present one).  2-torus, N = 16384, beta = 100, b = 16: 310 -> 133 us a product
+// with 0.34 of the tiles, both degree passes 335 -> 168 us; N = 80000, beta = 30, b = 32: 12.7 -> 7.6 ms (0.53); circle, N = 20000,
+// beta = 400, b = 4: 230 -> 54 us (0.18).  Above 0.8 of the tiles the gathers cost what the lists save.
 #include <algorithm>
 
 #include "fd_internal.h"
@@ -48,29 +54,81 @@ struct DirectParams {
     double* rowsq;                               // row-sum mode: sum_j K_ij^2 (may be null); Y = the weighted row sums
     void* part;                                  // 2 slots per CTA: shares of row tiles that are cut
     int row_tiles, col_tiles;
+    // tile lists (null: every column tile; fd_order.cu): entries of row tile r at list[r * tiles16 ..], counts[r] of them, tiles of 16
+    // positions each; a step is a column tile of consecutive entries, offs[r] steps lie before row tile r; perm: point of each position
+    const unsigned short* list; const unsigned int* counts; const unsigned int* offs; const int* perm; int tiles16;
     int tj_log2;                                 // log2 of the points per column tile: 6, or 4 where 64 would leave too few steps
 };
 
 __host__ __device__ __forceinline__ long long range_begin(long long total, int cta, int ctas) { return total * cta / ctas; }
 // (A CTA's share of a row tile goes to its slot 1 if its range holds the row tile's first step, else to slot 0.)
 
+// A CTA's range of steps, one row tile after the other.
+template <bool LISTED>
+struct Range {
+    long long g, g_end;
+    int rt = -1, c0, n, full;                        // steps c0 .. c0 + n of the row tile's `full` ones
+    __device__ __forceinline__ Range(const DirectParams& p) {
+        const long long total = LISTED ? (long long)p.offs[p.row_tiles] : (long long)p.row_tiles * p.col_tiles;
+        g = range_begin(total, (int)blockIdx.x, (int)gridDim.x);
+        g_end = range_begin(total, (int)blockIdx.x + 1, (int)gridDim.x);
+    }
+    __device__ __forceinline__ bool next(const DirectParams& p) {
+        if (g >= g_end) return false;                // (the same for the whole CTA)
+        if (!LISTED) {
+            rt = (int)(g / p.col_tiles);
+            c0 = (int)(g - (long long)rt * p.col_tiles);
+            full = p.col_tiles;
+        } else {
+            if (rt < 0) {                            // the last row tile that begins at or before step g: every thread looks at some
+                int before = 0;
+                for (int r0 = 0; r0 < p.row_tiles; r0 += kThr) {
+                    const int r = r0 + (int)threadIdx.x;
+                    before += __syncthreads_count(r < p.row_tiles && (long long)p.offs[r] <= g);
+                }
+                rt = before - 1;
+            } else ++rt;
+            c0 = (int)(g - (long long)p.offs[rt]);
+            full = (int)(p.offs[rt + 1] - p.offs[rt]);
+        }
+        n = (int)(full - c0 < g_end - g ? full - c0 : g_end - g);
+        g += n;
+        return true;
+    }
+};
+
+// Point of slot `jj` of step c of row tile rt; -1: padding.
+__device__ __forceinline__ int listed_point(const DirectParams& p, int rt, int c, int jj) {
+    const int e = (c << (p.tj_log2 - 4)) + (jj >> 4);
+    if (e >= (int)p.counts[rt]) return -1;
+    const int pos = (int)p.list[(size_t)rt * p.tiles16 + e] * 16 + (jj & 15);
+    return pos < (int)p.N ? p.perm[pos] : -1;
+}
+
 // Stages the points of a column tile (padding points lie 1e18 away: kernel value 0).
-template <int DP4>
-__device__ __forceinline__ void stage_points(const DirectParams& p, int64_t j0, float4* sx) {
+template <int DP4, bool LISTED>
+__device__ __forceinline__ void stage_points(const DirectParams& p, int64_t j0, const int* sidx, float4* sx) {
     for (int t = threadIdx.x; t < (DP4 << p.tj_log2); t += kThr) {
-        const int64_t j = j0 + t / DP4;
-        sx[t] = j < p.N ? p.xcol[j0 * DP4 + t] : make_float4(1e18f, 1e18f, 1e18f, 1e18f);
+        if (LISTED) {
+            const int j = sidx[t / DP4];
+            sx[t] = j >= 0 ? p.xcol[(int64_t)j * DP4 + t % DP4] : make_float4(1e18f, 1e18f, 1e18f, 1e18f);
+        } else {
+            const int64_t j = j0 + t / DP4;
+            sx[t] = j < p.N ? p.xcol[j0 * DP4 + t] : make_float4(1e18f, 1e18f, 1e18f, 1e18f);
+        }
     }
 }
 
-// Row r of a thread: lane_row + (256 / R) r.
-template <int DP4, int R>
+// Row r of a thread: position lane_row + (256 / R) r of the row tile.
+template <int DP4, int R, bool LISTED>
 __device__ __forceinline__ void load_rows(const DirectParams& p, int64_t row0, int lane_row, float4 (&xi)[R][DP4]) {
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int64_t i = row0 + lane_row + (kRowsT / R) * r;
+        int64_t i = row0 + lane_row + (kRowsT / R) * r;
+        const bool valid = i < p.Nrow;
+        if (LISTED && valid) i = p.perm[i];
 #pragma unroll
-        for (int k = 0; k < DP4; ++k) xi[r][k] = i < p.Nrow ? p.xrow[i * DP4 + k] : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k = 0; k < DP4; ++k) xi[r][k] = valid ? p.xrow[i * DP4 + k] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
 
@@ -95,7 +153,7 @@ __device__ __forceinline__ void kernel_values(const float4* sx, int jj, const fl
 // Block mode: Y[i, c] = left_i sum_j K_ij right_j V[j, c] for c < b <= BT.
 // (resident CTAs asked for: four, three or two, by the registers that the rows and sums of a thread need)
 constexpr int min_ctas(int regs) { return regs + 40 <= 128 ? 4 : regs + 40 <= 168 ? 3 : 2; }
-template <int DP4, int BT, int R>
+template <int DP4, int BT, int R, bool LISTED>
 __global__ void __launch_bounds__(kThr, min_ctas(R * (4 * DP4 + BT)))
 k_direct(const DirectParams p) {
     constexpr int H = R * kThr / kRowsT;               // column parts of a tile (R = 4: 2)
@@ -107,16 +165,13 @@ k_direct(const DirectParams p) {
     const int part = H == 1 ? 0 : (int)threadIdx.x / (kThr / H);
     const int lane_row = H == 1 ? (int)threadIdx.x : (int)threadIdx.x % (kThr / H);
     const int tj = 1 << p.tj_log2;
-    const long long total = (long long)p.row_tiles * p.col_tiles;
-    long long g = range_begin(total, (int)blockIdx.x, (int)gridDim.x);
-    const long long g_end = range_begin(total, (int)blockIdx.x + 1, (int)gridDim.x);
-    while (g < g_end) {
-        const int rt = (int)(g / p.col_tiles), c0 = (int)(g - (long long)rt * p.col_tiles);
-        const int n = (int)(p.col_tiles - c0 < g_end - g ? p.col_tiles - c0 : g_end - g);
-        g += n;
-        const int64_t row0 = (int64_t)rt * kRowsT;
+    __shared__ int sidx[LISTED ? kTJ : 1];               // points of the column tile
+    for (Range<LISTED> range(p); range.next(p);) {
+        const int c0 = range.c0, n = range.n;
+        const int64_t row0 = (int64_t)range.rt * kRowsT;
+        int point = LISTED && (int)threadIdx.x < tj ? listed_point(p, range.rt, c0, (int)threadIdx.x) : -1;
         float4 xi[R][DP4];
-        load_rows<DP4, R>(p, row0, lane_row, xi);
+        load_rows<DP4, R, LISTED>(p, row0, lane_row, xi);
         float acc[R][BT];
 #pragma unroll
         for (int r = 0; r < R; ++r)
@@ -128,12 +183,20 @@ k_direct(const DirectParams p) {
         for (int t = 0; t < n; ++t) {
             const int64_t j0 = (int64_t)(c0 + t) << p.tj_log2;
             __syncthreads();
-            stage_points<DP4>(p, j0, sx);
+            if (LISTED) {
+                // (the next step's points are looked up while this one is computed)
+                if ((int)threadIdx.x < tj) {
+                    sidx[threadIdx.x] = point;
+                    if (t + 1 < n) point = listed_point(p, range.rt, c0 + t + 1, (int)threadIdx.x);
+                }
+                __syncthreads();
+            }
+            stage_points<DP4, LISTED>(p, j0, sidx, sx);
             for (int e = threadIdx.x; e < (BT << p.tj_log2); e += kThr) {
                 const int jj = e & (tj - 1), c = e >> p.tj_log2;   // rows of V fastest: coalesced
-                const int64_t j = j0 + jj;
+                const int64_t j = LISTED ? (int64_t)sidx[jj] : j0 + jj;
                 float w = 0.f;
-                if (c < p.b && j < p.N) {
+                if (c < p.b && (LISTED ? j >= 0 : j < p.N)) {
                     w = c < p.vcols ? p.V[j + (int64_t)c * p.ldv] : 1.f;
                     if (p.right) w *= p.right[j];
                 }
@@ -192,18 +255,20 @@ k_direct(const DirectParams p) {
             }
         }
         if (part == 0) {
-            const bool whole = n == p.col_tiles;
+            const bool whole = n == range.full;
             float* slot = static_cast<float*>(p.part) +
                           (size_t)(2 * blockIdx.x + (c0 == 0 ? 1 : 0)) * BT * kRowsT + lane_row;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                const int64_t i = row0 + lane_row + (kRowsT / R) * r;
-                const float l = whole && p.left && i < p.Nrow ? p.left[i] : 1.0f;
+                int64_t i = row0 + lane_row + (kRowsT / R) * r;
+                const bool valid = i < p.Nrow;
+                if (LISTED && valid) i = p.perm[i];
+                const float l = whole && p.left && valid ? p.left[i] : 1.0f;
 #pragma unroll
                 for (int c = 0; c < BT; ++c)
                     if (c < p.b) {
                         if (!whole) slot[c * kRowsT + (kRowsT / R) * r] = acc[r][c];
-                        else if (i < p.Nrow) p.Y[i + (int64_t)c * p.ldy] = acc[r][c] * l;
+                        else if (valid) p.Y[i + (int64_t)c * p.ldy] = acc[r][c] * l;
                     }
             }
         }
@@ -212,7 +277,7 @@ k_direct(const DirectParams p) {
 }
 
 // Row-sum mode: sum_j K_ij right_j and sum_j K_ij^2; a column tile (<= 64 terms) in fp32, across tiles in fp64.
-template <int DP4>
+template <int DP4, bool LISTED>
 __global__ void __launch_bounds__(kThr)
 k_direct_rowsum(const DirectParams p) {
     constexpr int R = DP4 <= 4 ? 4 : 2, H = R * kThr / kRowsT;
@@ -222,24 +287,32 @@ k_direct_rowsum(const DirectParams p) {
     const int part = H == 1 ? 0 : (int)threadIdx.x / (kThr / H);
     const int lane_row = H == 1 ? (int)threadIdx.x : (int)threadIdx.x % (kThr / H);
     const int tj = 1 << p.tj_log2;
-    const long long total = (long long)p.row_tiles * p.col_tiles;
-    long long g = range_begin(total, (int)blockIdx.x, (int)gridDim.x);
-    const long long g_end = range_begin(total, (int)blockIdx.x + 1, (int)gridDim.x);
-    while (g < g_end) {
-        const int rt = (int)(g / p.col_tiles), c0 = (int)(g - (long long)rt * p.col_tiles);
-        const int n = (int)(p.col_tiles - c0 < g_end - g ? p.col_tiles - c0 : g_end - g);
-        g += n;
-        const int64_t row0 = (int64_t)rt * kRowsT;
+    __shared__ int sidx[LISTED ? kTJ : 1];               // points of the column tile
+    for (Range<LISTED> range(p); range.next(p);) {
+        const int c0 = range.c0, n = range.n;
+        const int64_t row0 = (int64_t)range.rt * kRowsT;
+        int point = LISTED && (int)threadIdx.x < tj ? listed_point(p, range.rt, c0, (int)threadIdx.x) : -1;
         float4 xi[R][DP4];
-        load_rows<DP4, R>(p, row0, lane_row, xi);
+        load_rows<DP4, R, LISTED>(p, row0, lane_row, xi);
         double dsum[R], dsq[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) { dsum[r] = 0.0; dsq[r] = 0.0; }
         for (int t = 0; t < n; ++t) {
             const int64_t j0 = (int64_t)(c0 + t) << p.tj_log2;
             __syncthreads();
-            stage_points<DP4>(p, j0, sx);
-            if ((int)threadIdx.x < tj) sw[threadIdx.x] = j0 + threadIdx.x < p.N ? (p.right ? p.right[j0 + threadIdx.x] : 1.0f) : 0.f;
+            if (LISTED) {
+                // (the next step's points are looked up while this one is computed)
+                if ((int)threadIdx.x < tj) {
+                    sidx[threadIdx.x] = point;
+                    if (t + 1 < n) point = listed_point(p, range.rt, c0 + t + 1, (int)threadIdx.x);
+                }
+                __syncthreads();
+            }
+            stage_points<DP4, LISTED>(p, j0, sidx, sx);
+            if ((int)threadIdx.x < tj) {
+                const int64_t j = LISTED ? (int64_t)sidx[threadIdx.x] : j0 + threadIdx.x;
+                sw[threadIdx.x] = (LISTED ? j >= 0 : j < p.N) ? (p.right ? p.right[j] : 1.0f) : 0.f;
+            }
             __syncthreads();
             float a[R], q[R];
 #pragma unroll
@@ -272,9 +345,10 @@ k_direct_rowsum(const DirectParams p) {
                             (size_t)(2 * blockIdx.x + (c0 == 0 ? 1 : 0)) * kRowsT + lane_row;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                const int64_t i = row0 + lane_row + (kRowsT / R) * r;
-                if (n != p.col_tiles) slot[(kRowsT / R) * r] = make_double2(dsum[r], dsq[r]);
+                int64_t i = row0 + lane_row + (kRowsT / R) * r;
+                if (n != range.full) slot[(kRowsT / R) * r] = make_double2(dsum[r], dsq[r]);
                 else if (i < p.Nrow) {
+                    if (LISTED) i = p.perm[i];
                     p.Y[i] = (float)(dsum[r] * (p.left ? (double)p.left[i] : 1.0));
                     if (p.rowsq) p.rowsq[i] = dsq[r];
                 }
@@ -290,9 +364,10 @@ constexpr int kFixCols = 8;
 __global__ void __launch_bounds__(256)
 k_direct_fix(const DirectParams p, int BT, int ctas) {
     __shared__ float sm[kFixCols][8][32];
-    const long long total = (long long)p.row_tiles * p.col_tiles;
     const int rt = blockIdx.x / (kRowsT / 32);
-    const long long g0 = (long long)rt * p.col_tiles, g1 = g0 + p.col_tiles;
+    const long long total = p.list ? (long long)p.offs[p.row_tiles] : (long long)p.row_tiles * p.col_tiles;
+    const long long g0 = p.list ? (long long)p.offs[rt] : (long long)rt * p.col_tiles;
+    const long long g1 = p.list ? (long long)p.offs[rt + 1] : g0 + p.col_tiles;
     // the last CTA whose range begins at or before step g0, and the last one whose range begins before g1
     const int first = (int)(((g0 + 1) * ctas - 1) / total), last = (int)((g1 * ctas - 1) / total);
     if (first == last) return;                                         // not cut: its CTA stored it
@@ -315,8 +390,9 @@ k_direct_fix(const DirectParams p, int BT, int ctas) {
     for (int c = 0; c < kFixCols; ++c) sm[c][grp][r] = v[c];
     __syncthreads();
     // group g finishes column col0 + g
-    const int64_t i = (int64_t)rt * kRowsT + row;
+    int64_t i = (int64_t)rt * kRowsT + row;
     if (i >= p.Nrow || col0 + grp >= p.b) return;
+    if (p.perm) i = p.perm[i];
     float x = 0.f;
 #pragma unroll
     for (int q = 0; q < 8; ++q) x += sm[grp][q][r];
@@ -327,9 +403,10 @@ k_direct_fix(const DirectParams p, int BT, int ctas) {
 __global__ void __launch_bounds__(256)
 k_direct_rowsum_fix(const DirectParams p, int ctas) {
     __shared__ double2 sm[8][32];
-    const long long total = (long long)p.row_tiles * p.col_tiles;
     const int rt = blockIdx.x / (kRowsT / 32);
-    const long long g0 = (long long)rt * p.col_tiles, g1 = g0 + p.col_tiles;
+    const long long total = p.list ? (long long)p.offs[p.row_tiles] : (long long)p.row_tiles * p.col_tiles;
+    const long long g0 = p.list ? (long long)p.offs[rt] : (long long)rt * p.col_tiles;
+    const long long g1 = p.list ? (long long)p.offs[rt + 1] : g0 + p.col_tiles;
     const int first = (int)(((g0 + 1) * ctas - 1) / total), last = (int)((g1 * ctas - 1) / total);
     if (first == last) return;
     cudaGridDependencySynchronize();
@@ -341,8 +418,9 @@ k_direct_rowsum_fix(const DirectParams p, int ctas) {
     for (int s = s0; s < s1; ++s) { const double2 o = slots[(size_t)(2 * s + (s == first ? 1 : 0)) * kRowsT]; v.x += o.x; v.y += o.y; }
     sm[grp][r] = v;
     __syncthreads();
-    const int64_t i = (int64_t)rt * kRowsT + row;
+    int64_t i = (int64_t)rt * kRowsT + row;
     if (grp != 0 || i >= p.Nrow) return;
+    if (p.perm) i = p.perm[i];
     v = make_double2(0.0, 0.0);
 #pragma unroll
     for (int q = 0; q < 8; ++q) { v.x += sm[q][r].x; v.y += sm[q][r].y; }
@@ -356,9 +434,11 @@ template <class Kernel>
 fd_status launch(fd_ctx* c, Kernel kernel, int smem, int per_sm, int BT, DirectParams p) {
     // Column tiles of 16 where 64 would give fewer than four steps per CTA: with one or two, the ranges differ by a factor of two and
     // small problems leave SMs idle (N = 1000, b = 64: 29 -> 21 us); more steps make the two barriers per tile dearer.
-    p.tj_log2 = ceil_div(p.N, kTJ) * p.row_tiles < 4ll * c->sm_count * per_sm ? 4 : 6;
+    const auto& lists = c->lists[2];
+    p.tj_log2 = (p.list ? lists.total : ceil_div(p.N, kTJ) * p.row_tiles) < 4ll * c->sm_count * per_sm ? 4 : 6;
     p.col_tiles = (int)ceil_div(p.N, (int64_t)1 << p.tj_log2);
-    const long long total = (long long)p.row_tiles * p.col_tiles;
+    if (p.list && p.tj_log2 == 4) p.offs += p.row_tiles + 1;        // steps of one entry
+    const long long total = !p.list ? (long long)p.row_tiles * p.col_tiles : p.tj_log2 == 4 ? lists.entries : lists.total;
     const size_t slot_floats = (size_t)kRowsT * (BT > 0 ? BT : 4);
     long long ctas = c->opt_splits > 0 ? (long long)p.row_tiles * c->opt_splits : (long long)c->sm_count * per_sm;
     ctas = std::max<long long>(1, std::min<long long>(std::min(ctas, total), (long long)(c->L.part_floats / (2 * slot_floats))));
@@ -366,7 +446,7 @@ fd_status launch(fd_ctx* c, Kernel kernel, int smem, int per_sm, int BT, DirectP
     if (smem > 48 * 1024) FD_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     kernel<<<(unsigned)ctas, kThr, smem, c->stream>>>(p);
     FD_LAUNCH_CHECK(c, "k_direct");
-    bool cut = false;
+    bool cut = p.list != nullptr;
     for (int i = 1; i < ctas && !cut; ++i) cut = range_begin(total, i, (int)ctas) % p.col_tiles != 0;
     if (cut) {
         // launched while the product's last CTAs run (it waits for their stores): the launch costs no gap
@@ -394,16 +474,26 @@ template <int DP4, int BT>
 fd_status launch_block(fd_ctx* c, const DirectParams& p) {
     constexpr int R = 4 * DP4 + BT <= 32 ? 4 : 2, H = R * kThr / kRowsT;
     constexpr int smem = (kTJ * DP4 * 4 + kTJ * (BT + 4) + H * BT * kRowsT) * 4;
-    static const int per_sm = resident(k_direct<DP4, BT, R>, smem);
-    return launch(c, k_direct<DP4, BT, R>, smem, per_sm, BT, p);
+    if constexpr (DP4 <= 2)
+        if (p.list) {
+            static const int per_sm = resident(k_direct<DP4, BT, R, true>, smem);
+            return launch(c, k_direct<DP4, BT, R, true>, smem, per_sm, BT, p);
+        }
+    static const int per_sm = resident(k_direct<DP4, BT, R, false>, smem);
+    return launch(c, k_direct<DP4, BT, R, false>, smem, per_sm, BT, p);
 }
 
 template <int DP4>
 fd_status launch_dp(fd_ctx* c, int BT, const DirectParams& p) {
     switch (BT) {
         case 0: {
-            static const int per_sm = resident(k_direct_rowsum<DP4>, 0);
-            return launch(c, k_direct_rowsum<DP4>, 0, per_sm, 0, p);
+            if constexpr (DP4 <= 2)
+                if (p.list) {
+                    static const int per_sm = resident(k_direct_rowsum<DP4, true>, 0);
+                    return launch(c, k_direct_rowsum<DP4, true>, 0, per_sm, 0, p);
+                }
+            static const int per_sm = resident(k_direct_rowsum<DP4, false>, 0);
+            return launch(c, k_direct_rowsum<DP4, false>, 0, per_sm, 0, p);
         }
         case 4: return launch_block<DP4, 4>(c, p);
         case 8: return launch_block<DP4, 8>(c, p);
@@ -431,6 +521,18 @@ fd_status apply_simt(fd_ctx* c, const ApplyArgs& a) {
     p.part = c->at<float>(L.part);
     p.row_tiles = (int)ceil_div(a.Nrow, kRowsT);
     const bool rowsum = a.V == nullptr;
+    // passes over the context's whole point set may leave out tiles of pairs whose kernel value is exactly zero; the degree passes
+    // decide (they wait for their sums anyway), products follow
+    if (a.rows_are_ctx && a.xrow == c->xs() && a.Nrow == L.N && !c->sh.on && L.direct_lists) {
+        FD_TRY(tile_lists(c, a.beta, 2, rowsum));
+        if (c->lists[2].on && c->lists[2].beta == a.beta) {
+            p.list = c->at<unsigned short>(L.lists);
+            p.counts = c->at<unsigned int>(L.list_counts);
+            p.offs = p.counts + 2 * p.row_tiles;
+            p.perm = c->at<int>(L.perm);
+            p.tiles16 = 16 * p.row_tiles;
+        }
+    }
     const int chunks = rowsum ? 1 : (int)ceil_div(a.b, 64), step = (int)ceil_div(a.b, chunks);
     for (int c0 = 0; c0 < a.b; c0 += step) {
         const int bc = std::min(step, a.b - c0), BT = rowsum ? 0 : pick_bt(bc);

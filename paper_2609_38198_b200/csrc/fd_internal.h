@@ -33,6 +33,7 @@ struct Layout {
     size_t yacc = 0;
     // order of the points and tile lists of the Gram-form kernels (fd_order.cu); 0: not provisioned for this N
     size_t perm = 0, boxes = 0, zproj = 0, lists = 0, list_counts = 0;
+    bool direct_lists = false;       // provisioned for the direct-difference kernels as well
     size_t weights = 0;              // NP right weights of a Gram-form row sum
     size_t symsum = 0;               // N 64-bit fixed-point sums of the symmetric row-sum mode
     size_t eig_q = 0, eig_w = 0, eig_x = 0, eig_r = 0, eig_small = 0, eig_small_doubles = 0;
@@ -69,11 +70,12 @@ struct fd_ctx {
     double packed_beta = -1.0, packed_row_beta = -1.0;
     int64_t packed_row0 = 0, packed_rows = 0;
     int order_state = 0;             // 1: the Gram-form operands hold the points in the order of L.perm; -1: no order will be made
-    // tile lists, for block products (0) and degree passes (1), whose exponent limits differ: bandwidth they were decided for, whether
-    // they leave out enough to be used, entries in all; which of the two the workspace holds, and for which bandwidth
-    struct { double beta = -1.0; bool on = false; int64_t total = 0; } lists[2];
+    // tile lists, for Gram-form block products (0) and degree passes (1) and all passes of the direct-difference kernels (2): bandwidth they were decided for, whether
+    // they leave out enough to be used, entries in all; which of the three the workspace holds, and for which bandwidth
+    // (direct-difference kernels (2): total is in groups of four tiles of 16 points, entries in single ones)
+    struct { double beta = -1.0; bool on = false; int64_t total = 0, entries = 0; } lists[3];
     double refused_beta = 0.0;       // largest bandwidth at which an order was tried and left out too little
-    int listed_kind = -1;
+    int listed_kind = -1, boxes_kind = -1;
     double listed_beta = -1.0;
     // options
     int opt_path = FD_PATH_AUTO;
@@ -179,7 +181,7 @@ void shard_range(int64_t N, int world, int rank, int64_t* begin, int64_t* end);
 fd_status gather_rows(fd_ctx* c, float* A, int64_t lda, int cols);
 // In-place sum over the ranks of n host doubles.  No-op for an unsharded context.
 fd_status allreduce_host(fd_ctx* c, double* buf, int64_t n);
-// Tile lists of a bandwidth for block products (kind 0) or degree passes (1) (fd_order.cu): decides c->lists[kind] and, where they are
+// Tile lists of a bandwidth for c->lists[kind] (fd_order.cu): decides c->lists[kind] and, where they are
 // used, brings them into the workspace; orders the points first if that can pay.  A new bandwidth is decided, with a wait, only where
 // `decide` allows it; without, nothing is listed for it.
 fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide);

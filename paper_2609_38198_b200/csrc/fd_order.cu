@@ -9,16 +9,20 @@
 // distances there are lower bounds too), in which a low-dimensional data set's boxes are tight and cheap (R^30, N = 2^18: 65 %
 // of the tiles remain instead of 73 % with boxes along the coordinates).
 //
-// Order: a k-d tree over 4096 sampled points (each node splits its samples at the median of their widest coordinate) down to leaves
-// of about 128 points; all points are routed through it and sorted by leaf, stably.  It is made once per context, when a
-// bandwidth first leaves at least 15 % of sampled pairs beyond the exponent, and costs about 0.6 ms at N = 2^18.  Vectors stay in
-// the caller's order everywhere: the operand packing gathers through the permutation, the epilogues scatter.
+// Order: a k-d tree over up to 4096 sampled points (each node splits its samples at the median of their widest coordinate) down to
+// leaves of about 128 points (16 where the direct-difference kernels may use it); all points are routed through it and sorted by
+// leaf, stably.  It is made once per context, by the degree passes of a bandwidth with many pairs beyond the exponent limit; the
+// degree passes of a new context then take 0.1 to 0.4 ms longer (N = 16384, D = 4: 335 -> 430 us; N = 2^18, D = 30: 0.6 ms), which one of the
+// two passes or the first products pay back from 16384 points on in the plane and on surfaces (direct differences; N = 8192: 130 us of
+// passes against 300) and from 32768 on in the Gram form.  Vectors stay in the caller's order everywhere: packing and staging
+// gather through the permutation, the epilogues scatter.
 //
-// Lists: for a bandwidth and exponent limit, per row pair (256 points) the column tiles (128 points) whose bounding box comes
-// close enough (distance of the two boxes: a lower bound for every pair).  Data that fill many dimensions (the
-// 6-torus) have no far tiles; then the products run over all tiles as before.
+// Lists: for a bandwidth and exponent limit, per 256 rows the column tiles whose bounding box comes close enough (distance of the
+// two boxes: a lower bound for every pair): tiles of 128 points for the Gram-form kernels, of 16 for the direct-difference
+// ones (there against the 16 boxes of the rows, too: 0.39 -> 0.34 of the tiles remain on the 2-torus, N = 16384, beta = 100).  Data that
+// fill many dimensions (the 6-torus) have no far tiles; then the passes run over all tiles as before.
 // N = 2^18, R^30 on a two-dimensional manifold, beta = 2 (44 % of the pairs are not zero), both at the power limit: b = 32, 25.5 -> 20.1 ms a
-// product; degree passes 23.2 -> 19.9 ms.
+// product; degree passes 23.2 -> 19.9 ms.  Direct differences, exactly zero values only: fd_direct.cu.
 #include <algorithm>
 #include <cmath>
 
@@ -30,14 +34,14 @@ namespace {
 
 constexpr int kSamples = 4096;
 
-// Counts pairs of 1024 sampled points farther apart than limit2 (squared distance).
+// Counts pairs of 512 sampled points farther apart than limit2 (squared distance).
 __global__ void __launch_bounds__(256)
 k_far_pairs(const float* __restrict__ xs, int DP, int64_t n, float limit2, unsigned int* __restrict__ count) {
     const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;      // one sampled row per warp
-    const float* xi = xs + (n * i / 1024) * DP;
+    const float* xi = xs + (n * i / 512) * DP;
     unsigned int far = 0;
-    for (int j = lane; j < 1024; j += 32) {
-        const float* xj = xs + (n * j / 1024) * DP;
+    for (int j = lane; j < 512; j += 32) {
+        const float* xj = xs + (n * j / 512) * DP;
         float d2 = 0.f;
         for (int k = 0; k < DP; ++k) { const float d = xi[k] - xj[k]; d2 = fmaf(d, d, d2); }
         far += d2 > limit2;
@@ -88,51 +92,104 @@ k_project(const float* __restrict__ xs, int DP, int64_t n, const double* __restr
 
 struct Node { int dim; float thr; };
 
-// One level of the tree: block = node, its `len` samples are idx[node * len ..) (level 0: the sample itself).  Sorts them by the
-// widest coordinate; the halves are the children.
-__global__ void __launch_bounds__(512)
-k_kd_level(const float* __restrict__ xs, int DP, int64_t n, int level, int* __restrict__ idx, Node* __restrict__ nodes) {
-    __shared__ float key[kSamples];
-    __shared__ int val[kSamples];
-    __shared__ float s_lo[64], s_hi[64];
-    __shared__ int s_dim;
-    const int len = kSamples >> level, node = blockIdx.x;
-    int* mine = idx + (size_t)node * len;
-    for (int t = threadIdx.x; t < len; t += 512) val[t] = level == 0 ? (int)(n * t / kSamples) : mine[t];
-    __syncthreads();
-    // extent of every coordinate (a warp per coordinate)
-    for (int k = threadIdx.x >> 5; k < DP; k += 16) {
-        float lo = INFINITY, hi = -INFINITY;
-        for (int t = threadIdx.x & 31; t < len; t += 32) { const float v = xs[(int64_t)val[t] * DP + k]; lo = fminf(lo, v); hi = fmaxf(hi, v); }
+// The tree over S = 1024 E evenly spaced points: nodes of level l at nodes[2^l - 1 ..].  One CTA with the samples' coordinates (at most 8) in
+// shared memory; a level is the extent of every node's samples, then one bitonic sort of all nodes' segments at once.  A thread holds
+// entries warp * 32 E + 32 u + lane: exchanges closer than 32 E go through shuffles and registers (S = 2048: 250 of 285; all through
+// shared memory took 146 us, a launch per level 120 us).
+constexpr int kKdThr = 1024;
+constexpr int kd_smem(int samples, int DP) { return samples * (DP * 4 + 8) + (samples / 32) * 16 * 4 + (samples / 2) * 4; }
+template <int E>
+__global__ void __launch_bounds__(kKdThr)
+k_kd_tree(const float* __restrict__ xs, int DP, int64_t n, int depth, Node* __restrict__ nodes) {
+    constexpr int S = kKdThr * E;
+    extern __shared__ __align__(16) float kd[];
+    float* coord = kd;                                             // [DP][S]
+    float* skey = coord + (size_t)S * DP;
+    int* sval = reinterpret_cast<int*>(skey + S);
+    float (*chunk)[2][8] = reinterpret_cast<float(*)[2][8]>(sval + S);             // extents of 32 consecutive entries
+    int* dim = reinterpret_cast<int*>(chunk + S / 32);                             // of each node
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, e0 = warp * 32 * E + lane;
+    for (int t = threadIdx.x; t < S; t += kKdThr) {
+        const float* x = xs + (n * t / S) * DP;
+        for (int k = 0; k < DP; ++k) coord[k * S + t] = x[k];
+    }
+    float key[E];
+    int val[E];
 #pragma unroll
-        for (int m = 16; m >= 1; m >>= 1) { lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, m)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, m)); }
-        if ((threadIdx.x & 31) == 0) { s_lo[k] = lo; s_hi[k] = hi; }
-    }
+    for (int u = 0; u < E; ++u) val[u] = e0 + 32 * u;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int d = 0;
-        for (int k = 1; k < DP; ++k)
-            if (s_hi[k] - s_lo[k] > s_hi[d] - s_lo[d]) d = k;
-        s_dim = d;
-    }
-    __syncthreads();
-    const int dim = s_dim;
-    for (int t = threadIdx.x; t < len; t += 512) key[t] = xs[(int64_t)val[t] * DP + dim];
-    __syncthreads();
-    for (int size = 2; size <= len; size <<= 1)
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int t = threadIdx.x; t < len / 2; t += 512) {
-                const int a = 2 * t - (t & (stride - 1)), b = a + stride;
-                const bool up = (a & size) == 0;
-                const float ka = key[a], kb = key[b];
-                const int va = val[a], vb = val[b];
-                const bool gt = ka > kb || (ka == kb && va > vb);              // ties by index: the order is unique
-                if (gt == up) { key[a] = kb; key[b] = ka; val[a] = vb; val[b] = va; }
+    for (int level = 0; level < depth; ++level) {
+        const int len = S >> level;
+        // widest coordinate of every node
+        const int width = len < 32 ? len : 32;
+#pragma unroll
+        for (int u = 0; u < E; ++u) {
+            float widest = -1.f;
+            int d = 0;
+            for (int k = 0; k < DP; ++k) {
+                float lo = coord[k * S + val[u]], hi = lo;
+                for (int m = width >> 1; m >= 1; m >>= 1) { lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, m)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, m)); }
+                if (hi - lo > widest) { widest = hi - lo; d = k; }
+                if (len >= 32 && lane == 0) { chunk[warp * E + u][0][k] = lo; chunk[warp * E + u][1][k] = hi; }
+            }
+            const int e = e0 + 32 * u;
+            if (len < 32 && e % len == 0) dim[e / len] = d;
+        }
+        __syncthreads();
+        if (len >= 32) {
+            const int per = len / 32;                              // chunks of a node; a warp per node
+            for (int node = warp; node < (1 << level); node += kKdThr / 32) {
+                float widest = -1.f;
+                int d = 0;
+                for (int k = 0; k < DP; ++k) {
+                    float lo = INFINITY, hi = -INFINITY;
+                    for (int q = lane; q < per; q += 32) { lo = fminf(lo, chunk[node * per + q][0][k]); hi = fmaxf(hi, chunk[node * per + q][1][k]); }
+#pragma unroll
+                    for (int m = 16; m >= 1; m >>= 1) { lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, m)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, m)); }
+                    if (hi - lo > widest) { widest = hi - lo; d = k; }
+                }
+                if (lane == 0) dim[node] = d;
             }
             __syncthreads();
         }
-    for (int t = threadIdx.x; t < len; t += 512) mine[t] = val[t];
-    if (threadIdx.x == 0) nodes[(1 << level) - 1 + node] = Node{dim, key[len / 2]};
+#pragma unroll
+        for (int u = 0; u < E; ++u) key[u] = coord[dim[(e0 + 32 * u) / len] * S + val[u]];
+        for (int size = 2; size <= len; size <<= 1)
+            for (int stride = size >> 1; stride > 0; stride >>= 1) {
+                float ok[E];
+                int ov[E];
+                if (stride >= 32 * E) {
+#pragma unroll
+                    for (int u = 0; u < E; ++u) { skey[e0 + 32 * u] = key[u]; sval[e0 + 32 * u] = val[u]; }
+                    __syncthreads();
+#pragma unroll
+                    for (int u = 0; u < E; ++u) { ok[u] = skey[(e0 + 32 * u) ^ stride]; ov[u] = sval[(e0 + 32 * u) ^ stride]; }
+                    __syncthreads();
+                } else if (stride >= 32) {
+#pragma unroll
+                    for (int u = 0; u < E; ++u) {
+                        ok[u] = stride == 32 ? key[(u ^ 1) % E] : key[(u ^ 2) % E];
+                        ov[u] = stride == 32 ? val[(u ^ 1) % E] : val[(u ^ 2) % E];
+                    }
+                } else {
+#pragma unroll
+                    for (int u = 0; u < E; ++u) { ok[u] = __shfl_xor_sync(0xffffffffu, key[u], stride); ov[u] = __shfl_xor_sync(0xffffffffu, val[u], stride); }
+                }
+#pragma unroll
+                for (int u = 0; u < E; ++u) {
+                    const int e = e0 + 32 * u;
+                    const bool up = size == len || (e & size) == 0, lower = (e & stride) == 0;
+                    const bool gt = key[u] > ok[u] || (key[u] == ok[u] && val[u] > ov[u]);     // ties by index: the order is unique
+                    if ((lower == up) == gt) { key[u] = ok[u]; val[u] = ov[u]; }
+                }
+            }
+#pragma unroll
+        for (int u = 0; u < E; ++u) {
+            const int e = e0 + 32 * u;
+            if (e % len == len / 2) nodes[(1 << level) - 1 + e / len] = Node{dim[e / len], key[u]};
+        }
+        __syncthreads();
+    }
 }
 
 // Leaf of every point, and how many points of each block of 1024 fall into each leaf (counts[leaf * blocks + block]).
@@ -174,12 +231,13 @@ k_leaf_scan(unsigned int* __restrict__ counts, int blocks, int leaves, unsigned 
     if (lane == 0) totals[leaf] = base;
 }
 // out[i] = sum of in[0 .. i), out[n] = total (one block; in and out may not overlap).
+// (with a group size g the terms are ceil(in / g).)
 __global__ void __launch_bounds__(1024)
-k_scan(const unsigned int* __restrict__ in, int n, unsigned int* __restrict__ out) {
+k_scan(const unsigned int* __restrict__ in, int n, unsigned int* __restrict__ out, unsigned int g = 1) {
     __shared__ unsigned int s[1024];
     const int per = (n + 1023) / 1024, i0 = threadIdx.x * per;
     unsigned int sum = 0;
-    for (int i = i0; i < min(n, i0 + per); ++i) sum += in[i];
+    for (int i = i0; i < min(n, i0 + per); ++i) sum += (in[i] + g - 1) / g;
     s[threadIdx.x] = sum;
     __syncthreads();
     for (int m = 1; m < 1024; m <<= 1) {
@@ -189,7 +247,7 @@ k_scan(const unsigned int* __restrict__ in, int n, unsigned int* __restrict__ ou
         __syncthreads();
     }
     unsigned int base = s[threadIdx.x] - sum;
-    for (int i = i0; i < min(n, i0 + per); ++i) { out[i] = base; base += in[i]; }
+    for (int i = i0; i < min(n, i0 + per); ++i) { out[i] = base; base += (in[i] + g - 1) / g; }
     if (threadIdx.x == 1023) out[n] = s[1023];
 }
 // perm[position] = index, by leaf and in index order inside a leaf: the warps of a block take their turns.
@@ -215,6 +273,23 @@ k_scatter(const unsigned short* __restrict__ leaf, int64_t n, const unsigned int
     if (i < n) perm[base[l] + counts[(size_t)l * gridDim.x + blockIdx.x] + rank] = (int)i;
 }
 
+// Bounding box of each tile of 16 consecutive positions, for up to 8 coordinates: 16 lanes a tile.
+__global__ void __launch_bounds__(256)
+k_boxes16(const float* __restrict__ xs, int DP, int64_t n, const int* __restrict__ perm, int tiles, float* __restrict__ box) {
+    const int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    const int64_t i = p < n ? perm[p] : -1;
+    for (int k = 0; k < DP; ++k) {
+        float lo = INFINITY, hi = -INFINITY;
+        if (i >= 0) lo = hi = xs[i * DP + k];
+#pragma unroll
+        for (int m = 8; m >= 1; m >>= 1) { lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, m)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, m)); }
+        if ((threadIdx.x & 15) == 0 && p / 16 < tiles) {
+            box[(size_t)(p / 16) * 2 * DP + k] = lo;
+            box[((size_t)(p / 16) * 2 + 1) * DP + k] = hi;
+        }
+    }
+}
+
 // Bounding box of each tile of 128 consecutive positions: box[tile * 2 DP ..] = minima, then maxima.  Empty tiles get an empty box.
 __global__ void __launch_bounds__(128)
 k_boxes(const float* __restrict__ xs, int DP, int64_t n, const int* __restrict__ perm, float* __restrict__ box) {
@@ -235,21 +310,27 @@ k_boxes(const float* __restrict__ xs, int DP, int64_t n, const int* __restrict__
     }
 }
 
-// Column tiles of row pair blockIdx.x whose box comes within limit2 of the pair's box, ascending: list[pair * tiles ..]; counts[pair]
-// of them, of which `upper[pair]` are tiles 2 pair and later (the symmetric row sums start there).
-__global__ void __launch_bounds__(256)
-k_lists(const float* __restrict__ box, int DP, int tiles, float limit2, unsigned short* __restrict__ list, unsigned int* __restrict__ counts,
+// Column tiles (per_pair to a row pair) of row pair blockIdx.x whose box comes within limit2 of the pair's box, ascending: list[pair * tiles ..];
+// counts[pair] of them, of which `upper[pair]` are the pair's own and later ones (the symmetric row sums start there).
+__global__ void __launch_bounds__(1024)
+k_lists(const float* __restrict__ box, int DP, int tiles, int per_pair, float limit2, unsigned short* __restrict__ list, unsigned int* __restrict__ counts,
         unsigned int* __restrict__ upper) {
     __shared__ float lo[64], hi[64];
-    __shared__ unsigned int wsum[8];
+    __shared__ float sub[16][2][8];                                    // boxes of 16 row tiles (per_pair = 16, up to 8 coordinates)
+    __shared__ unsigned int wsum[32];
     const int pair = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int k = threadIdx.x; k < DP; k += 256) {
-        const float *a = box + (size_t)(2 * pair) * 2 * DP, *b = a + 2 * DP;
-        lo[k] = fminf(a[k], b[k]); hi[k] = fmaxf(a[DP + k], b[DP + k]);
+    for (int k = threadIdx.x; k < DP; k += 1024) {
+        float l = INFINITY, h = -INFINITY;
+        for (int t = 0; t < per_pair; ++t) {
+            const float* a = box + ((size_t)pair * per_pair + t) * 2 * DP;
+            l = fminf(l, a[k]); h = fmaxf(h, a[DP + k]);
+            if (per_pair == 16) { sub[t][0][k] = a[k]; sub[t][1][k] = a[DP + k]; }
+        }
+        lo[k] = l; hi[k] = h;
     }
     __syncthreads();
     unsigned int n = 0, below = 0;
-    for (int t0 = 0; t0 < tiles; t0 += 256) {
+    for (int t0 = 0; t0 < tiles; t0 += 1024) {
         const int t = t0 + threadIdx.x;
         bool near = false;
         if (t < tiles) {
@@ -259,16 +340,29 @@ k_lists(const float* __restrict__ box, int DP, int tiles, float limit2, unsigned
                 const float g = fmaxf(fmaxf(b[k] - hi[k], lo[k] - b[DP + k]), 0.f);
                 d2 = fmaf(g, g, d2);
             }
-            near = d2 <= limit2 || (t >> 1) == pair;                   // (an empty box is infinitely far; a pair's own tiles always count)
+            near = d2 <= limit2;
+            if (near && per_pair == 16) {
+                // near the box of all 256 rows: near one of the 16 smaller boxes?
+                near = false;
+                for (int s = 0; s < 16 && !near; ++s) {
+                    float e2 = 0.f;
+                    for (int k = 0; k < DP; ++k) {
+                        const float g = fmaxf(fmaxf(b[k] - sub[s][1][k], sub[s][0][k] - b[DP + k]), 0.f);
+                        e2 = fmaf(g, g, e2);
+                    }
+                    near = e2 <= limit2;
+                }
+            }
+            near = near || t / per_pair == pair;                   // (an empty box is infinitely far; a pair's own tiles always count)
         }
         const unsigned int vote = __ballot_sync(0xffffffffu, near);
         if (lane == 0) wsum[warp] = __popc(vote);
         __syncthreads();
         unsigned int pos = n + __popc(vote & ((1u << lane) - 1u)), all = 0;
-        for (int w = 0; w < 8; ++w) { if (w < warp) pos += wsum[w]; all += wsum[w]; }
+        for (int w = 0; w < 32; ++w) { if (w < warp) pos += wsum[w]; all += wsum[w]; }
         if (near) {
             list[(size_t)pair * tiles + pos] = (unsigned short)t;
-            if (t == 2 * pair) below = pos + 1;                        // (one thread of the block sees it)
+            if (t == per_pair * pair) below = pos + 1;                        // (one thread of the block sees it)
         }
         n += all;
         __syncthreads();
@@ -288,11 +382,15 @@ fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide) {
     if (st.beta == beta && (!st.on || (c->listed_kind == kind && c->listed_beta == beta))) return FD_OK;
     // Beyond an exponent of 40 both fp16 pieces of a kernel value are zero (2^15 2^-40 = 2^-25 rounds to zero), beyond 60 a degree
     // contribution is below the fixed-point unit; the quarter covers the rounding of the boxes' distance.
-    const double limit = kind == 0 ? 40.25 : 60.25;
+    // The direct-difference kernels' exponential gives exactly zero beyond 126.
+    const double limit = kind == 0 ? 40.25 : kind == 1 ? 60.25 : 126.25;
+    const double scaled_beta = beta * (60.25 / limit);             // bandwidths of the kinds on one scale
+    const bool direct = kind == 2;
+    if (direct && !L.direct_lists) return FD_OK;
     if (!decide && st.beta != beta) return FD_OK;
     const bool known = st.beta == beta;                            // decided before, only overwritten by the other kind's lists
     const int64_t N = L.N;
-    const int tiles = (int)(L.NP / 128), pairs = (int)(L.NP / 256);
+    const int per_pair = direct ? 16 : 2, tiles = (int)(L.NP / 256) * per_pair, pairs = (int)(L.NP / 256);
     const float limit2 = (float)(limit / (beta * kLog2e));
     if (!known) { st.on = false; st.beta = beta; }
     unsigned int* small = reinterpret_cast<unsigned int*>(c->at<char>(L.status) + 128);
@@ -305,24 +403,26 @@ fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide) {
     bool fresh = false;
     if (c->order_state == 0) {
         // (an order that left out too little at some bandwidth would leave out less at a smaller one: in units of the degree passes' limit)
-        if (beta * (kind == 0 ? 60.25 / 40.25 : 1.0) <= c->refused_beta * 1.2) return FD_OK;
+        if (scaled_beta <= c->refused_beta * 1.2) return FD_OK;
         fresh = true;
         FD_CUDA(c, cudaMemsetAsync(small, 0, 4, c->stream));
-        k_far_pairs<<<128, 256, 0, c->stream>>>(c->xs(), L.DP, N, limit2, small);
+        k_far_pairs<<<64, 256, 0, c->stream>>>(c->xs(), L.DP, N, limit2, small);
         FD_LAUNCH_CHECK(c, "k_far_pairs");
         unsigned int far = 0;
         FD_CUDA(c, cudaMemcpyAsync(&far, small, 4, cudaMemcpyDeviceToHost, c->stream));
         FD_CUDA(c, cudaStreamSynchronize(c->stream));
-        if ((double)far < 0.15 * 1024.0 * 1024.0) return FD_OK;
+        // (Share of far pairs from which an order is worth making: 0.4, where tiles are small against the data's extent; 0.8 for fewer than
+        // 32768 points.  2-torus, beta = 30, 0.70 of the pairs far: 0.53 of the tiles remain at N = 80000, 0.8 at N = 16384.)
+        if ((double)far < (N < 32768 ? 0.8 : 0.4) * 512.0 * 512.0) return FD_OK;
         // scratch: the operand buffers (re-packed in the new order afterwards); at least 64 bytes per point each
         int depth = 0;
-        while (((int64_t)128 << depth) < N && depth < 12) ++depth;
+        while (((int64_t)(L.direct_lists ? 16 : 128) << depth) < N && depth < 12) ++depth;
+        const int samples = std::min(kSamples, std::max(1024, 2 << depth));        // two to a leaf or more, where there are as many
         const int leaves = 1 << depth, blocks = (int)ceil_div(N, 1024);
         unsigned int* counts = c->at<unsigned int>(L.xp_col);
         char* scratch = c->at<char>(L.xp_row);
         unsigned short* leaf = reinterpret_cast<unsigned short*>(scratch);
-        int* idx = reinterpret_cast<int*>(scratch + round_up(2 * N, 256));
-        Node* nodes = reinterpret_cast<Node*>(idx + kSamples);
+        Node* nodes = reinterpret_cast<Node*>(scratch + round_up(2 * N, 256));
         unsigned int* totals = reinterpret_cast<unsigned int*>(nodes + kSamples);
         unsigned int* base = totals + kSamples;
         if (project) {
@@ -345,10 +445,11 @@ fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide) {
             k_project<<<(unsigned)ceil_div(N, 256), 256, 0, c->stream>>>(c->xs(), L.DP, N, mu, dir, c->at<float>(L.zproj));
             FD_LAUNCH_CHECK(c, "k_project");
         }
-        for (int l = 0; l < depth; ++l) {
-            k_kd_level<<<1 << l, 512, 0, c->stream>>>(z, ZP, N, l, idx, nodes);
-            FD_LAUNCH_CHECK(c, "k_kd_level");
-        }
+        const int smem = kd_smem(samples, ZP);
+        const auto tree = samples == 1024 ? k_kd_tree<1> : samples == 2048 ? k_kd_tree<2> : k_kd_tree<4>;
+        FD_CUDA(c, cudaFuncSetAttribute(tree, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        tree<<<1, kKdThr, smem, c->stream>>>(z, ZP, N, depth, nodes);
+        FD_LAUNCH_CHECK(c, "k_kd_tree");
         k_kd_route<<<blocks, 1024, 0, c->stream>>>(z, ZP, N, depth, nodes, leaf, counts);
         FD_LAUNCH_CHECK(c, "k_kd_route");
         k_leaf_scan<<<(unsigned)ceil_div(leaves, 8), 256, 0, c->stream>>>(counts, blocks, leaves, totals);
@@ -357,30 +458,38 @@ fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide) {
         FD_LAUNCH_CHECK(c, "k_scan");
         k_scatter<<<blocks, 1024, 0, c->stream>>>(leaf, N, counts, base, leaves, perm);
         FD_LAUNCH_CHECK(c, "k_scatter");
-        k_boxes<<<tiles, 128, 0, c->stream>>>(z, ZP, N, perm, box);
-        FD_LAUNCH_CHECK(c, "k_boxes");
         c->order_state = 1;
+        c->boxes_kind = -1;
         c->packed_beta = c->packed_row_beta = -1.0;
     }
+    if (c->boxes_kind != (direct ? 1 : 0)) {
+        if (direct) k_boxes16<<<(unsigned)ceil_div(L.NP, 256), 256, 0, c->stream>>>(z, ZP, N, perm, tiles, box);
+        else k_boxes<<<tiles, 128, 0, c->stream>>>(z, ZP, N, perm, box);
+        FD_LAUNCH_CHECK(c, "k_boxes");
+        c->boxes_kind = direct ? 1 : 0;
+    }
     unsigned int* cnt = c->at<unsigned int>(L.list_counts);
-    k_lists<<<pairs, 256, 0, c->stream>>>(box, ZP, tiles, limit2, c->at<unsigned short>(L.lists), cnt, cnt + pairs);
+    k_lists<<<pairs, 1024, 0, c->stream>>>(box, ZP, tiles, per_pair, limit2, c->at<unsigned short>(L.lists), cnt, cnt + pairs);
     FD_LAUNCH_CHECK(c, "k_lists");
     unsigned int* offs = cnt + 2 * pairs;
-    k_scan<<<1, 1024, 0, c->stream>>>(cnt, pairs, offs);
+    // two offset arrays: all and upper entries; direct-difference kernels: groups of four entries and single ones
+    k_scan<<<1, 1024, 0, c->stream>>>(cnt, pairs, offs, direct ? 4u : 1u);
     FD_LAUNCH_CHECK(c, "k_scan");
-    k_scan<<<1, 1024, 0, c->stream>>>(cnt + pairs, pairs, offs + pairs + 1);
+    k_scan<<<1, 1024, 0, c->stream>>>(direct ? cnt : cnt + pairs, pairs, offs + pairs + 1);
     FD_LAUNCH_CHECK(c, "k_scan");
     c->listed_kind = kind; c->listed_beta = beta;
     if (known) return FD_OK;
-    unsigned int total = 0;
+    unsigned int total = 0, entries = 0;
     FD_CUDA(c, cudaMemcpyAsync(&total, offs + pairs, 4, cudaMemcpyDeviceToHost, c->stream));
+    FD_CUDA(c, cudaMemcpyAsync(&entries, offs + 2 * pairs + 1, 4, cudaMemcpyDeviceToHost, c->stream));
     FD_CUDA(c, cudaStreamSynchronize(c->stream));
-    st.total = total;
-    st.on = (double)total < 0.9 * (double)pairs * (double)tiles;
+    st.total = total; st.entries = entries;
+    // (direct-difference kernels: gathering through the order costs them more)
+    st.on = direct ? 4.0 * (double)total < 0.8 * (double)pairs * (double)tiles : (double)total < 0.9 * (double)pairs * (double)tiles;
     if (fresh && !st.on) {
         // nothing gained: the points keep the caller's order (a larger bandwidth may try again)
         c->order_state = 0;
-        c->refused_beta = std::max(c->refused_beta, beta * (kind == 0 ? 60.25 / 40.25 : 1.0));
+        c->refused_beta = std::max(c->refused_beta, scaled_beta);
     }
     return FD_OK;
 }

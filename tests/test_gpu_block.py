@@ -154,76 +154,130 @@ def test_coordinates_that_all_points_share(N, path, D, const):
     ctx.close()
 
 
-@pytest.mark.parametrize("N,kind", [(8192, "manifold"), (8193, "clusters"), (9001, "line"), (8500, "duplicates")])
+def _gpu_kernel_rows(Xd, rows, beta):
+    """float64 rows of the kernel by direct differences, on the GPU."""
+    return torch.exp(-beta * torch.cdist(Xd[rows], Xd, compute_mode="donot_use_mm_for_euclid_dist") ** 2)
+
+
+def _gpu_degree(Xd, beta):
+    """q, d, sum of q, sum of squares of the kernel, in float64 on the GPU."""
+    N = Xd.shape[0]
+    parts = [torch.arange(i, min(N, i + 2048), device=Xd.device) for i in range(0, N, 2048)]
+    q, so2 = [], 0.0
+    for r in parts:
+        K = _gpu_kernel_rows(Xd, r, beta)
+        q.append(K.sum(1))
+        so2 += (K * K).sum().item()
+    q = torch.cat(q)
+    d = torch.cat([_gpu_kernel_rows(Xd, r, beta) @ (1.0 / q) for r in parts]) / q
+    return q, d, q.sum().item(), so2
+
+
+def _far_points(kind, N, rng):
+    """Points of which many pairs are far apart, and a bandwidth for the Gram-form kernels and one for the direct ones."""
+    t = rng.random((N, 2)) * 2 * np.pi
+    if kind == "manifold":
+        return workloads.latent_torus(N, seed=42), 5.0, None
+    if kind == "torus2":
+        X, bg, bd = np.concatenate([np.cos(t), np.sin(t)], 1), None, 100.0
+    elif kind == "circle":
+        X, bg, bd = np.concatenate([np.cos(t[:, :1]), np.sin(t[:, :1])], 1), None, 400.0
+    elif kind == "clusters":                       # 5 clusters of similar size far apart, 12 coordinates (direct: 7)
+        X = (rng.standard_normal((5, 12)) * 2.0)[rng.choice(5, N, p=(0.25, 0.25, 0.2, 0.15, 0.15))] + 0.1 * rng.standard_normal((N, 12))
+        bg, bd = 0.8, None
+    elif kind == "clusters7":
+        X = (rng.standard_normal((9, 7)) * 2.0)[rng.choice(9, N)] + 0.1 * rng.standard_normal((N, 7))
+        bg, bd = None, 30.0
+    elif kind == "line":                           # one coordinate that matters
+        X = np.concatenate([8.0 * rng.random((N, 1)), 0.01 * rng.standard_normal((N, 2))], 1)
+        bg, bd = 3.4, 100.0
+    else:                                          # a third of the points coincide, between two blobs
+        X, bg, bd = np.zeros((N, 4)), 2.0, 40.0
+        X[N // 3:] = 0.02 * rng.standard_normal((N - N // 3, 4))
+        X[N // 3:, 0] += 3.9 * rng.choice((-1.0, 1.0), N - N // 3)
+    return X.astype(np.float32), bg, bd
+
+
+@pytest.mark.parametrize("N,kind", [(32768, "manifold"), (32769, "clusters"), (33001, "line"), (32900, "duplicates")])
 def test_far_tiles_are_left_out(N, kind):
-    """Data with many pairs beyond the exponent limit: the points are ordered, tiles without near pairs left out.  Same results as the
-    float64 oracle (gates of the Gram-form path: degrees 2e-5, product 1e-5; what is left out is below 2^-40 of a kernel value's
-    maximum), bit-identical repeats, lists remade when the bandwidth changes, external rows against ordered columns, and the same
-    operator applied through other precision modes and without the symmetric passes."""
+    """Data with many pairs beyond the exponent limit: the points are ordered, tiles without near pairs left out.  Same results as float64
+    sums (gates of the Gram-form path: degrees 2e-5, product 1e-5; what is left out is below 2^-40 of a kernel value's
+    maximum), bit-identical repeats, lists remade when the bandwidth changes, external rows against ordered columns, the same
+    operator applied through other precision modes and without the symmetric passes, and a product at a bandwidth that no degree
+    pass has seen, which takes every tile."""
     import __graft_entry__ as g
     g.build()
     import paper_2609_38198_b200 as fd
     dev = torch.device("cuda:0")
-    rng = np.random.default_rng(N)
-    if kind == "manifold":
-        X, beta = workloads.latent_torus(N, seed=42), 5.0
-    elif kind == "clusters":                       # 5 clusters of unequal size far apart, 12 coordinates
-        X = (rng.standard_normal((5, 12)) * 2.0)[rng.choice(5, N, p=(0.5, 0.2, 0.15, 0.1, 0.05))] + 0.1 * rng.standard_normal((N, 12))
-        X, beta = X.astype(np.float32), 0.8
-    elif kind == "line":                           # one coordinate that matters, unevenly sampled
-        X = np.zeros((N, 3)); X[:, 0] = 8.0 * rng.random(N) ** 1.3; X[:, 1] = 0.01 * rng.standard_normal(N); X[:, 2] = 0.01 * rng.standard_normal(N)
-        X, beta = X.astype(np.float32), 2.0
-    else:                                          # most points coincide
-        X = np.zeros((N, 4)); X[N // 2:] = rng.standard_normal((N - N // 2, 4)) * 0.1 + 2.0
-        X, beta = X.astype(np.float32), 2.0
+    X, beta, _ = _far_points(kind, N, np.random.default_rng(N))
+    Xt = torch.from_numpy(X).to(dev)
+    Xd = Xt.double()
     b = 20
-    V = workloads.block(N, b, seed=2)
-    Vd = fd.to_colmajor(V, dev)
-    ctx = fd.Context(torch.from_numpy(X).to(dev), b_max=b)
+    V = fd.to_colmajor(workloads.block(N, b, seed=2), dev)
+    Vd = V.double()
+    rows = torch.arange(0, N, 61, device=dev)
+    ctx = fd.Context(Xt, b_max=b)
     ctx.set_option("path", fd.FD_PATH_TC)
-    ctx.set_option("tc_max_mag", 1e3)
+    ctx.set_option("tc_max_mag", 1e4)
+    qo, do, soo, so2o = _gpu_degree(Xd, beta)
+    sd = 1.0 / (qo * do.sqrt())
+    Yo = sd[rows, None] * (_gpu_kernel_rows(Xd, rows, beta) @ (sd[:, None] * Vd))
     shares = []
     for bt in (beta, 0.1 * beta, beta):
         q, d, s, so, so2 = ctx.degree(bt, 1.0)
-        Y, Y2, Yf = ctx.apply(Vd), ctx.apply(Vd), ctx.apply(Vd, prec=fd.FD_PREC_FAST)
+        Y, Y2, Yf = ctx.apply(V), ctx.apply(V), ctx.apply(V, prec=fd.FD_PREC_FAST)
         shares.append(ctx.get_option("tile_share"))
         assert torch.equal(Y, Y2)
         if bt != beta:
             continue
-        qo, do, s_o, soo, so2o = dense.degree(X, bt, 1.0)
-        Yo = dense.apply(X, bt, 1.0, V)
-        assert np.abs(q.cpu().numpy() / qo - 1).max() <= 2e-5 and np.abs(d.cpu().numpy() / do - 1).max() <= 4e-5
-        assert abs(so - soo) <= 2e-5 * (soo + N) and abs(so2 - so2o) <= 4e-5 * (so2o + N)
-        assert np.linalg.norm(Y.cpu().numpy().astype(np.float64) - Yo) <= 1e-5 * np.linalg.norm(Yo)
-        assert np.linalg.norm(Yf.cpu().numpy().astype(np.float64) - Yo) <= 3e-3 * np.linalg.norm(Yo)
-        R = ctx.apply_general(bt, Vd, Xrow=torch.from_numpy(X[:77].copy()).to(dev)).cpu().numpy().astype(np.float64)
-        Ro = np.exp(-bt * ((X[:77, None, :].astype(np.float64) - X[None].astype(np.float64)) ** 2).sum(-1)) @ V.astype(np.float64)
-        assert np.linalg.norm(R - Ro) <= 1e-5 * np.linalg.norm(Ro)
+        assert (q.double() / qo - 1).abs().max().item() <= 2e-5 and (d.double() / do - 1).abs().max().item() <= 4e-5
+        assert abs(so - (soo - N)) <= 2e-5 * soo and abs(so2 - (so2o - N)) <= 4e-5 * so2o
+        assert ((Y[rows].double() - Yo).norm() / Yo.norm()).item() <= 1e-5
+        assert ((Yf[rows].double() - Yo).norm() / Yo.norm()).item() <= 3e-3
+        R = ctx.apply_general(bt, V, Xrow=Xt[:77].contiguous()).double()
+        Ro = _gpu_kernel_rows(Xd, torch.arange(77, device=dev), bt) @ Vd
+        assert ((R - Ro).norm() / Ro.norm()).item() <= 1e-5
     assert shares[0] < 0.9 and shares[2] == shares[0], shares
+    Z = ctx.apply_general(0.7 * beta, V)[rows].double()
+    Zo = _gpu_kernel_rows(Xd, rows, 0.7 * beta) @ Vd
+    assert ((Z - Zo).norm() / Zo.norm()).item() <= 1e-5
     ctx.set_option("sym", 0)
     q0, d0, s0, _, _ = ctx.degree(beta, 1.0)
     assert ((q0 - q).abs() / q0).max().item() <= 2e-6
     ctx.close()
 
 
-def test_product_at_a_bandwidth_without_degrees_takes_every_tile():
-    """Ordered points, and a product at a bandwidth for which no degree pass has decided about the tiles: it returns without waiting and
-    runs over all of them, in the caller's order of rows (float64 oracle, gate of the Gram-form product 1e-5)."""
+@pytest.mark.parametrize("N,kind,b", [(16384, "torus2", 16), (16385, "circle", 5), (17001, "clusters7", 40), (33001, "duplicates", 24),
+                                      (20011, "torus2", 70), (40000, "line", 3)])
+def test_far_tiles_are_left_out_of_direct_passes(N, kind, b):
+    """Direct-difference passes without the tiles whose kernel values are exactly zero: degrees, sums and products against float64 sums
+    (gate 1e-6 of that family), bit-identical repeats, bandwidths with and without lists, and a product at a bandwidth that no
+    degree pass has seen."""
     import __graft_entry__ as g
     g.build()
     import paper_2609_38198_b200 as fd
     dev = torch.device("cuda:0")
-    N, b = 8193, 16
-    X = workloads.latent_torus(N, seed=42)
-    V = workloads.block(N, b, seed=3)
-    ctx = fd.Context(torch.from_numpy(X).to(dev), b_max=b)
-    ctx.set_option("path", fd.FD_PATH_TC)
-    ctx.set_option("tc_max_mag", 1e3)
-    ctx.degree(5.0, 1.0)
-    assert ctx.get_option("tile_share") < 0.9
-    rows = np.arange(0, N, 41)
-    for beta in (3.0, 5.0, 3.0):
-        Y = ctx.apply_general(beta, fd.to_colmajor(V, dev)).cpu().numpy().astype(np.float64)[rows]
-        K = np.exp(-beta * ((X[rows, None, :].astype(np.float64) - X[None].astype(np.float64)) ** 2).sum(-1))
-        assert np.linalg.norm(Y - K @ V) <= 1e-5 * np.linalg.norm(K @ V)
+    X, _, beta = _far_points(kind, N, np.random.default_rng(N))
+    Xt = torch.from_numpy(X).to(dev)
+    Xd = Xt.double()
+    V = fd.to_colmajor(workloads.block(N, b, seed=2), dev)
+    rows = torch.arange(0, N, 97, device=dev)
+    ctx = fd.Context(Xt, b_max=b)
+    ctx.set_option("path", fd.FD_PATH_SIMT)
+    shares = []
+    for bt in (beta, 0.01 * beta, beta):
+        q, d, s, so, so2 = ctx.degree(bt, 1.0)
+        Y, Y2 = ctx.apply(V), ctx.apply(V)
+        shares.append(ctx.get_option("tile_share"))
+        assert torch.equal(Y, Y2)
+        qo, do, soo, so2o = _gpu_degree(Xd, bt)
+        assert (q.double() / qo - 1).abs().max().item() <= 1e-6 and (d.double() / do - 1).abs().max().item() <= 2e-6
+        assert abs(so - (soo - N)) <= 1e-6 * soo and abs(so2 - (so2o - N)) <= 1e-6 * so2o
+        sd = s.double()
+        Yo = sd[rows, None] * (_gpu_kernel_rows(Xd, rows, bt) @ (sd[:, None] * V.double()))
+        assert ((Y[rows].double() - Yo).norm() / Yo.norm()).item() <= 1e-6
+    assert shares[0] < 0.8 and shares[1] == 1.0 and shares[2] == shares[0], shares
+    Z = ctx.apply_general(0.7 * beta, V)[rows].double()
+    Zo = _gpu_kernel_rows(Xd, rows, 0.7 * beta) @ V.double()
+    assert ((Z - Zo).norm() / Zo.norm()).item() <= 1e-6
     ctx.close()
