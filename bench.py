@@ -39,7 +39,7 @@ UNIT = "pair*cols/s"
 
 # DRAM bytes per launch of the timed block-product kernel (dram__bytes_read.sum + dram__bytes_write.sum of one ncu
 # capture of this kernel at N = 2^20, single-pass metrics), keyed by the kernel that bench times; None = not captured.
-NCU_TRAFFIC_BYTES = {"k_tc<64, block>": 17.139e9 + 2.180e9, "k_simt": None}
+NCU_TRAFFIC_BYTES = {"k_block<64>": None, "k_direct": None}
 
 
 def measured_peaks():
@@ -368,11 +368,11 @@ def run_gpu(args):
             # everything on the FMA pipe: per pair 2 D (difference form) + b (product) + ~3 issue slots
             peak_pairs = fma_peak / (2 * D + b + 3)
             binder = "fma_pipe (direct-difference distance + block product on FFMA)"
-            kernel_name = "k_simt"
+            kernel_name = "k_direct"
         else:
             peak_pairs = mufu_peak
             binder = "mufu (one ex2 per pair; distance and product on the tensor cores)"
-            kernel_name = "k_tc<64, block>"
+            kernel_name = "k_block<64>"
         roofline = {"bound": "alu", "kernel": f"{kernel_name}: block product Y = M V (dominant kernel)", "binder": binder,
                     "achieved": pairs_per_s / 1e9, "peak": peak_pairs / 1e9, "unit": "Gpairs/s",
                     "frac": pairs_per_s / peak_pairs,
