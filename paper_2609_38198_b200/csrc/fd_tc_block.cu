@@ -461,7 +461,11 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
     tc_fence_before();
     __syncthreads();
     // SM cycles CTA 0 spent on its work items (status words 2-3): lets the host relate the kernel time to the SM clock
-    if (blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<long long*>(p.status + 2) = clock64() - t_begin;
+    // (a product in several column chunks adds its launches up)
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        long long* cycles = reinterpret_cast<long long*>(p.status + 2);
+        *cycles = clock64() - t_begin + (p.accumulate ? *cycles : 0);
+    }
     if (warp == 24) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
     }
