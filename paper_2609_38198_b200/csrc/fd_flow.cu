@@ -13,13 +13,16 @@ namespace {
 constexpr double kKappaP = 10.0;     // Eq. 11
 constexpr int kPExponent = 6;        // Eq. 11
 
-// out[i + j * ldout] = num[i + j * n] / (lambda[j] * num[i + m * n]): column m of the product is the denominator.
+// out[i + j * ldout] = num[i + j * n] / (lambda[j] * num[i + m * n]): column m of the product is the denominator.  Where it is zero (a new
+// point whose kernel values all vanish) so are the numerators: the extension is 0 there, not 0 / 0 -- one NaN row would spoil every
+// inner product of a start basis that it becomes part of.
 struct Lambdas { double v[64]; };
 __global__ void k_nystrom_finish(const float* __restrict__ num, float* __restrict__ out, int64_t ldout, int m, const Lambdas lambda, int64_t n) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double dn = (double)num[i + (int64_t)m * n];
-    for (int j = 0; j < m; ++j) out[i + (int64_t)j * ldout] = (float)((double)num[i + (int64_t)j * n] / (lambda.v[j] * dn));
+    for (int j = 0; j < m; ++j)
+        out[i + (int64_t)j * ldout] = dn == 0.0 ? 0.f : (float)((double)num[i + (int64_t)j * n] / (lambda.v[j] * dn));
 }
 
 double median_of(std::vector<double> v) {

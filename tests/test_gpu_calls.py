@@ -1,0 +1,82 @@
+"""Calls and inputs beside the ordinary ones: far new points, arguments that have to be refused, products captured in CUDA
+graphs, non-finite right blocks, results that must not depend on what was asked before."""
+import numpy as np
+import pytest
+import torch
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fd():
+    import __graft_entry__ as g
+    g.build()
+    import paper_2609_38198_b200 as fd
+    assert torch.cuda.is_available()
+    return fd
+
+
+@pytest.fixture(scope="module")
+def dev():
+    return torch.device("cuda:0")
+
+
+# ------------------------------------------------------------------ out-of-sample extension of far points
+@pytest.mark.parametrize("path", [1, 2])
+def test_extension_of_far_points(fd, dev, path):
+    """New points from inside the data to exponents (base 2) of 70 from every point.  Direct differences: the formula.  Gram form: a kernel
+    value carries 2^-40 absolute (one half of the last place of the 16-bit pieces), which is 2^(e - 40) of a value at exponent e and at
+    most twice that of the ratio; beyond 41 every value is zero and so is the extension."""
+    N, m, beta = 3000, 5, 0.8
+    bp = beta * np.log2(np.e)
+    rng = np.random.default_rng(7)
+    X = (0.02 * rng.standard_normal((N, 3))).astype(np.float32)
+    e = np.array([0.0, 4.0, 12.0, 20.0, 30.0, 36.0, 40.5, 44.0, 52.0, 66.0])
+    u = rng.standard_normal((len(e), 3))
+    Z = (u / np.linalg.norm(u, axis=1)[:, None] * np.sqrt(e / bp)[:, None]).astype(np.float32)
+    psi = np.cos(X.astype(np.float64) @ rng.standard_normal((3, m)) * 20.0)
+    lam = np.linspace(1.0, 0.4, m)
+    ctx = fd.Context(torch.from_numpy(X).to(dev), b_max=16)
+    ctx.set_option("path", path)
+    ctx.degree(beta, 1.0)
+    out = ctx.nystrom(torch.from_numpy(Z).to(dev), fd.to_colmajor(psi.astype(np.float32), dev), lam).cpu().numpy().astype(np.float64)
+    X64, Z64 = X.astype(np.float64), Z.astype(np.float64)
+    q = np.exp(-beta * ((X64[:, None] - X64[None]) ** 2).sum(-1)).sum(1)
+    E = bp * ((Z64[:, None] - X64[None]) ** 2).sum(-1)
+    K = 2.0 ** -E / q[None]
+    ref = (K @ psi) / (K.sum(1)[:, None] * lam[None])
+    big = np.abs(psi).max() / lam.min()
+    assert np.isfinite(out).all()
+    for i in range(len(e)):
+        near, far = E[i].min(), E[i].max()
+        if path == 1:
+            assert np.abs(out[i] - ref[i]).max() <= 1e-5 * big
+        elif near > 41.0:
+            assert (out[i] == 0.0).all(), (e[i], out[i])
+        elif far < 39.0:
+            assert np.abs(out[i] - ref[i]).max() <= (1e-5 + 2.0 * 2.0 ** (far - 40.0)) * big, (e[i], out[i], ref[i])
+    ctx.close()
+
+
+def test_ladder_start_with_a_point_far_from_all_others(fd, dev):
+    """One new point beyond the range of the Gram-form product (base-2 exponent 57 from every point) among ordinary ones: a finite
+    start basis with zeros in its row, and a solve that runs."""
+    n_old, N, beta, k, b = 3000, 3400, 1.0, 12, 8
+    X = workloads.torus6(N, seed=13)
+    X[3100] = 0.0
+    X[3100, 0] = 6.9
+    Xt = torch.from_numpy(X).to(dev)
+    old = fd.Context(Xt[:n_old].contiguous(), b_max=b, m_max=64)
+    old.set_option("path", fd.FD_PATH_TC)
+    old.degree(beta, 1.0)
+    lam, U, info = old.eigs(k, b)
+    new = fd.Context(Xt, b_max=b, m_max=64)
+    new.degree(beta, 1.0)
+    Q0 = new.ladder_start(old, Xt, U, lam)
+    assert old.get_option("last_path") == fd.FD_PATH_TC
+    assert torch.isfinite(Q0).all() and (Q0[3100] == 0).all() and (Q0[3099] != 0).all()
+    lam_w, U_w, info_w = new.eigs(k, b, Q0=Q0, max_applies=200)
+    assert info_w.converged == k + 1 and np.isfinite(lam_w).all() and torch.isfinite(U_w).all()
+    old.close(); new.close()
