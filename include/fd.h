@@ -219,7 +219,8 @@ fd_status fd_beta_flow_cascade(fd_ctx* ctx, const fd_flow_opts* opts, const fd_c
  * (Sec. 1, the (n, beta) ladder): psi_j(x) = sum_i K(x, x_i) q_i^-alpha psi_j(x_i) /
  * (lambda_j sum_i K(x, x_i) q_i^-alpha), at the context's current (beta, alpha, q).
  * psi_dev: N x m column-major (Markov vectors d^-1/2 * v); lambda_host: m values;
- * out_dev: Nnew x m column-major.  Numerators and denominator are columns of one rectangular
+ * out_dev: Nnew x m column-major; it must not overlap psi_dev (other rows of one pitched panel do
+ * not).  Numerators and denominator are columns of one rectangular
  * product, at most 63 vectors at a time.  A new point so far from every point of the context that
  * all its kernel values vanish gets 0 (Gram-form kernels: below 2^-40, direct differences: below
  * 2^-126; the value's distance from the formula grows as a row's kernel values approach 2^-40 on

@@ -277,13 +277,6 @@ fd_status fd_degree(fd_ctx* c, double beta, double alpha, fd_precision prec, flo
     return FD_OK;
 }
 
-static fd_status check_block(fd_ctx* c, const float* p, int64_t ld, int64_t rows, const char* what) {
-    if (!p) return fail(c, FD_ERR_INVALID, "%s is null", what);
-    if (ld < rows) return fail(c, FD_ERR_INVALID, "%s: leading dimension %lld < rows %lld", what, (long long)ld, (long long)rows);
-    if ((reinterpret_cast<uintptr_t>(p) & 3) != 0) return fail(c, FD_ERR_INVALID, "%s is not 4-byte aligned", what);
-    return FD_OK;
-}
-
 fd_status fd_apply_general(fd_ctx* c, double beta, const float* left_dev, const float* right_dev,
                            const float* Xrow_dev, int64_t Nrow, int64_t ldxrow, const float* V_dev, int64_t ldv,
                            int32_t b, float* Y_dev, int64_t ldy, fd_precision prec) {
@@ -293,6 +286,29 @@ fd_status fd_apply_general(fd_ctx* c, double beta, const float* left_dev, const 
 }  // extern "C"
 
 namespace fd {
+
+fd_status check_block(fd_ctx* c, const float* p, int64_t ld, int64_t rows, const char* what) {
+    if (!p) return fail(c, FD_ERR_INVALID, "%s is null", what);
+    if (ld < rows) return fail(c, FD_ERR_INVALID, "%s: leading dimension %lld < rows %lld", what, (long long)ld, (long long)rows);
+    if ((reinterpret_cast<uintptr_t>(p) & 3) != 0) return fail(c, FD_ERR_INVALID, "%s is not 4-byte aligned", what);
+    return FD_OK;
+}
+
+fd_status check_in_out(fd_ctx* c, const float* V, int64_t ldv, int64_t vrows, const float* Y, int64_t ldy, int64_t yrows, int32_t b) {
+    FD_TRY(check_block(c, V, ldv, vrows, "V"));
+    FD_TRY(check_block(c, Y, ldy, yrows, "Y"));
+    const char* v0 = (const char*)V; const char* v1 = v0 + ((size_t)ldv * (b - 1) + vrows) * 4;
+    const char* y0 = (const char*)Y; const char* y1 = y0 + ((size_t)ldy * (b - 1) + yrows) * 4;
+    bool overlap = v0 < y1 && y0 < v1;
+    if (overlap && ldv == ldy) {
+        // two row ranges of one pitched panel (e.g. old rows in, new rows out, of the same basis) never touch
+        const int64_t off = Y - V;
+        const int64_t r = ((off % ldv) + ldv) % ldv;              // first row of Y inside V's panel
+        if (r >= vrows && r + yrows <= ldv) overlap = false;
+    }
+    if (overlap) return fail(c, FD_ERR_INVALID, "V and Y overlap");
+    return FD_OK;
+}
 
 fd_status apply_general(fd_ctx* c, double beta, const float* left_dev, const float* right_dev, bool right_pos,
                         const float* Xrow_dev, int64_t Nrow, int64_t ldxrow, const float* V_dev, int64_t ldv, int32_t b,
@@ -306,20 +322,8 @@ fd_status apply_general(fd_ctx* c, double beta, const float* left_dev, const flo
     if (!Xrow_dev) Nrow = N;
     if (Nrow < 1) return fail(c, FD_ERR_INVALID, "Nrow < 1");
     if (Xrow_dev && ldxrow < c->L.D) return fail(c, FD_ERR_INVALID, "ldxrow < D");
-    if (V_dev) FD_TRY(check_block(c, V_dev, ldv, N, "V"));
-    FD_TRY(check_block(c, Y_dev, ldy, Nrow, "Y"));
-    if (V_dev) {
-        const char* v0 = (const char*)V_dev; const char* v1 = v0 + ((size_t)ldv * (b - 1) + N) * 4;
-        const char* y0 = (const char*)Y_dev; const char* y1 = y0 + ((size_t)ldy * (b - 1) + Nrow) * 4;
-        bool overlap = v0 < y1 && y0 < v1;
-        if (overlap && ldv == ldy) {
-            // two row ranges of one pitched panel (e.g. old rows in, new rows out, of the same basis) never touch
-            const int64_t off = ((const float*)Y_dev - (const float*)V_dev);
-            const int64_t r = ((off % ldv) + ldv) % ldv;          // first row of Y inside V's panel
-            if (r >= N && r + Nrow <= ldv) overlap = false;
-        }
-        if (overlap) return fail(c, FD_ERR_INVALID, "V and Y overlap");
-    }
+    if (V_dev) FD_TRY(check_in_out(c, V_dev, ldv, N, Y_dev, ldy, Nrow, b));
+    else FD_TRY(check_block(c, Y_dev, ldy, Nrow, "Y"));
     ApplyArgs a{};
     a.beta = beta; a.right = right_dev; a.V = V_dev; a.ldv = ldv; a.b = b; a.prec = prec; a.rowsq = nullptr;
     a.right_pos = right_pos;

@@ -205,6 +205,7 @@ extern "C" fd_status fd_nystrom(fd_ctx* c, const float* Xnew_dev, int64_t Nnew, 
     if (!Xnew_dev || !psi_dev || !lambda_host || !out_dev || Nnew < 1 || m < 1 || m > 1024)
         return fail(c, FD_ERR_INVALID, "fd_nystrom: bad argument");
     if (ldxnew < c->L.D || ldpsi < c->L.N || ldout < Nnew) return fail(c, FD_ERR_INVALID, "fd_nystrom: bad pitch");
+    FD_TRY(check_in_out(c, psi_dev, ldpsi, c->L.N, out_dev, ldout, Nnew, m));
     for (int j = 0; j < m; ++j)
         if (!(std::fabs(lambda_host[j]) > 1e-30)) return fail(c, FD_ERR_INVALID, "fd_nystrom: zero eigenvalue");
     const int64_t N = c->L.N;

@@ -167,6 +167,9 @@ fd_status apply_simt(fd_ctx* c, const ApplyArgs& a);
 fd_status apply_tc(fd_ctx* c, const ApplyArgs& a);
 bool tc_supported(const fd_ctx* c, const ApplyArgs& a);
 fd_status apply_dispatch(fd_ctx* c, const ApplyArgs& a);
+// Argument checks of a block, and of a product's two blocks of b columns (which must not overlap).
+fd_status check_block(fd_ctx* c, const float* p, int64_t ld, int64_t rows, const char* what);
+fd_status check_in_out(fd_ctx* c, const float* V, int64_t ldv, int64_t vrows, const float* Y, int64_t ldy, int64_t yrows, int32_t b);
 // Body of fd_apply_general with one more promise: right_pos = the caller guarantees right > 0 elementwise, which lets a
 // row-sum (V == nullptr) with a right vector take the same kernel family as the block products of the same operator.
 fd_status apply_general(fd_ctx* c, double beta, const float* left_dev, const float* right_dev, bool right_pos,

@@ -80,3 +80,46 @@ def test_ladder_start_with_a_point_far_from_all_others(fd, dev):
     lam_w, U_w, info_w = new.eigs(k, b, Q0=Q0, max_applies=200)
     assert info_w.converged == k + 1 and np.isfinite(lam_w).all() and torch.isfinite(U_w).all()
     old.close(); new.close()
+
+
+# ------------------------------------------------------------------ arguments of the extension
+def _nystrom(ctx, Xn, n, psi, ldpsi, m, out, ldout):
+    import ctypes
+    from paper_2609_38198_b200 import binding
+    lam = (ctypes.c_double * m)(*([0.5] * m))
+    return binding.lib.fd_nystrom(ctx._h, Xn.data_ptr(), n, Xn.stride(0), psi, ldpsi, m, lam, out, ldout)
+
+
+def _extension_problem(fd, dev, N=300, n=700, m=6):
+    ctx = fd.Context(torch.from_numpy(workloads.torus6(N, seed=1)).to(dev), b_max=8)
+    ctx.degree(0.6, 1.0)
+    Xn = torch.from_numpy(workloads.torus6(n, seed=2)).to(dev)
+    panel = torch.randn((m, N + n), device=dev)               # column-major, pitch N + n
+    return ctx, Xn, panel
+
+
+def test_extension_refuses_overlapping_blocks(fd, dev):
+    """More new points than points: the second chunk of rows would read what the first one wrote.  Other rows of one panel do not overlap."""
+    N, n, m = 300, 700, 6
+    ctx, Xn, panel = _extension_problem(fd, dev, N, n, m)
+    ld = N + n
+    assert _nystrom(ctx, Xn, n, panel.data_ptr(), ld, m, panel.data_ptr(), ld) == fd.FD_ERR_INVALID
+    assert _nystrom(ctx, Xn, n, panel.data_ptr(), ld, m, panel.data_ptr() + 4 * (N - 1), ld) == fd.FD_ERR_INVALID
+    before = panel[:, :N].clone()
+    want = ctx.nystrom(Xn, before.t(), [0.5] * m)
+    assert _nystrom(ctx, Xn, n, panel.data_ptr(), ld, m, panel.data_ptr() + 4 * N, ld) == fd.FD_OK
+    ctx.synchronize()
+    assert torch.equal(panel[:, :N], before) and torch.equal(panel[:, N:].t(), want)
+    ctx.close()
+
+
+def test_extension_refuses_misaligned_blocks(fd, dev):
+    """Found by the host's argument checks, before any launch."""
+    N, n, m = 300, 50, 2
+    ctx, Xn, panel = _extension_problem(fd, dev, N, n, m)
+    out = torch.empty((m, n), device=dev)
+    launches = fd.fd_launch_count()
+    assert _nystrom(ctx, Xn, n, panel.data_ptr() + 2, N + n - 1, m, out.data_ptr(), n) == fd.FD_ERR_INVALID
+    assert _nystrom(ctx, Xn, n, panel.data_ptr(), N + n, m, out.data_ptr() + 1, n - 1) == fd.FD_ERR_INVALID
+    assert fd.fd_launch_count() == launches
+    ctx.close()
