@@ -243,6 +243,7 @@ fd_status fd_degree(fd_ctx* c, double beta, double alpha, fd_precision prec, flo
     a.left = nullptr; a.right = nullptr; a.V = nullptr; a.ldv = N; a.b = 1;
     a.Y = c->q() + r0; a.ldy = N; a.rowsq = rowsq + r0; a.prec = prec;
     a.sym_ok = !c->sh.on;                                        // K = K^T, unit weights
+    a.decide = true;
     if (n > 0) FD_TRY(apply_dispatch(c, a));
     // the two sums lie beside the tensor-core kernels' status word: one copy brings all three at the end
     double* sums_dev = reinterpret_cast<double*>(c->at<char>(c->L.status) + 64);

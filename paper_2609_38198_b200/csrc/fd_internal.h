@@ -161,6 +161,7 @@ struct ApplyArgs {
     bool ones_last;                         // block mode: column b - 1 of the block is the ones vector, V holds the others
     bool right_pos;                         // caller guarantees right > 0 elementwise
     bool sym_ok;                            // square pass with left == right, weights in (0, 1]: the symmetric half-work row sums may serve it
+    bool decide;                            // the pass may wait for the decision which tiles a bandwidth leaves out (degree passes: they wait anyway)
     fd_precision prec;
 };
 fd_status apply_simt(fd_ctx* c, const ApplyArgs& a);

@@ -499,9 +499,10 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
     const bool all_rows = a.rows_are_ctx && a.xrow == c->xs() && a.Nrow == N;
     const bool prunes = all_rows && !c->sh.on && (rowsum ? sym : a.prec == FD_PREC_FP32);
     // The decision reads a count back.  Degree passes return host scalars and wait anyway, so they decide for the products at their
-    // bandwidth too; a product at any other bandwidth returns without waiting and runs over all tiles.
-    if (prunes && rowsum && a.prec == FD_PREC_FP32) FD_TRY(tile_lists(c, a.beta, 0, true));
-    if (prunes) FD_TRY(tile_lists(c, a.beta, rowsum ? 1 : 0, rowsum));
+    // bandwidth too (once: the lists themselves are remade by the first product); any other pass returns without waiting and, at
+    // a bandwidth that is not decided, runs over all tiles.
+    if (prunes && a.decide && a.prec == FD_PREC_FP32 && c->lists[0].beta != a.beta) FD_TRY(tile_lists(c, a.beta, 0, true));
+    if (prunes) FD_TRY(tile_lists(c, a.beta, rowsum ? 1 : 0, a.decide));
     const bool use_lists = prunes && c->lists[rowsum ? 1 : 0].on && c->lists[rowsum ? 1 : 0].beta == a.beta;
     const int* col_perm = c->order_state == 1 ? c->at<int>(L.perm) : nullptr;
     const int* row_perm = all_rows ? col_perm : nullptr;

@@ -123,3 +123,34 @@ def test_extension_refuses_misaligned_blocks(fd, dev):
     assert _nystrom(ctx, Xn, n, panel.data_ptr(), N + n, m, out.data_ptr() + 1, n - 1) == fd.FD_ERR_INVALID
     assert fd.fd_launch_count() == launches
     ctx.close()
+
+
+# ------------------------------------------------------------------ results do not depend on calls in between
+def _listed(fd, dev, kind):
+    """A context whose products at `beta` leave out tiles: (ctx, X, beta)."""
+    if kind == "direct":
+        X, beta = workloads.torus2(16384, seed=1), 100.0
+    else:
+        X, beta = workloads.latent_torus(32768, seed=42), 5.0
+    ctx = fd.Context(torch.from_numpy(X).to(dev), b_max=8)
+    ctx.set_option("path", fd.FD_PATH_SIMT if kind == "direct" else fd.FD_PATH_TC)
+    ctx.set_option("tc_max_mag", 1e4)
+    return ctx, X, beta
+
+
+@pytest.mark.parametrize("kind", ["direct", "gram"])
+def test_only_degree_passes_decide_which_tiles_are_left_out(fd, dev, kind):
+    """A row sum or a product at another bandwidth in between leaves the products at the degree passes' bandwidth as they were, bit for
+    bit, and still without the tiles that hold only zeros."""
+    ctx, X, beta = _listed(fd, dev, kind)
+    V = fd.to_colmajor(workloads.block(X.shape[0], 8, seed=3), dev)
+    ctx.degree(beta, 1.0)
+    Y = ctx.apply(V)
+    share = ctx.get_option("tile_share")
+    assert share < 0.9
+    for other in (0.9 * beta, 0.01 * beta):
+        ctx.apply_general(other, None)
+        ctx.apply_general(other, V)
+        assert torch.equal(ctx.apply(V), Y)
+        assert ctx.get_option("tile_share") == share
+    ctx.close()
