@@ -69,7 +69,8 @@ struct fd_ctx {
     // (-1: something else)
     double packed_beta = -1.0, packed_row_beta = -1.0;
     int64_t packed_row0 = 0, packed_rows = 0;
-    int order_state = 0;             // 1: the Gram-form operands hold the points in the order of L.perm; -1: no order will be made
+    bool packed_ordered = false, packed_row_ordered = false;     // they hold the points in the order of L.perm
+    int order_state = 0;             // 1: L.perm holds an order of the points; -1: none will be made
     // tile lists, for Gram-form block products (0) and degree passes (1) and all passes of the direct-difference kernels (2): bandwidth they were decided for, whether
     // they leave out enough to be used, entries in all; which of the three the workspace holds, and for which bandwidth
     // (direct-difference kernels (2): total is in groups of four tiles of 16 points, entries in single ones)

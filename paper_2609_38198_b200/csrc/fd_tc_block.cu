@@ -83,10 +83,10 @@ struct BlockParams {
     int jt0, num_jt;             // column tiles [jt0, jt0 + num_jt) of this launch
     int K16, b, flush, stages;
     int accumulate;              // add to Y (later column chunks) instead of storing
-    // tile lists (null: every column tile): column tiles of row pair r at list[r * tiles ..], steps before it offs[r]
+    // tile lists (null: every column tile, points in the caller's order): column tiles of row pair r at list[r * tiles ..], steps before it offs[r]
     const unsigned short* list; const unsigned int* offs;
     int tiles;
-    const int* perm;             // row of Y and left for each row of the operand (null: the same)
+    const int* perm;             // with lists: row of Y and left for each row of the operand
 };
 
 // First step of CTA `cta` in the flat sequence of steps, and the work item (part of one row pair) that starts at step g of it.
@@ -106,16 +106,15 @@ template <bool ORD>
 struct Steps {                   // walks a CTA's range item by item
     int pair, j0, left;
     __device__ __forceinline__ Steps(const BlockParams& p) {
-        const bool listed = ORD && p.list;
-        const long long total = listed ? (long long)p.offs[p.pairs] : (long long)p.pairs * p.num_jt;
+        const long long total = ORD ? (long long)p.offs[p.pairs] : (long long)p.pairs * p.num_jt;
         const long long g0 = range_begin(total, (int)blockIdx.x, (int)gridDim.x);
-        pair = listed ? pair_of(p, (unsigned int)g0) : (int)(g0 / p.num_jt);
-        j0 = (int)(g0 - (listed ? (long long)p.offs[pair] : (long long)pair * p.num_jt));
+        pair = ORD ? pair_of(p, (unsigned int)g0) : (int)(g0 / p.num_jt);
+        j0 = (int)(g0 - (ORD ? (long long)p.offs[pair] : (long long)pair * p.num_jt));
         left = (int)(range_begin(total, (int)blockIdx.x + 1, (int)gridDim.x) - g0);
     }
     __device__ __forceinline__ bool next(const BlockParams& p, Item& it) {
         if (left <= 0) return false;
-        const int full = ORD && p.list ? (int)(p.offs[pair + 1] - p.offs[pair]) : p.num_jt;
+        const int full = ORD ? (int)(p.offs[pair + 1] - p.offs[pair]) : p.num_jt;
         it.pair = pair; it.j0 = j0;
         it.n = full - j0 < left ? full - j0 : left;
         it.whole = it.n == full;
@@ -124,7 +123,7 @@ struct Steps {                   // walks a CTA's range item by item
     }
 };
 
-// ORD: the points are ordered (perm, where the rows are the context's own) and tiles may be listed.
+// ORD: a pass over the tile lists; the points are in the order `perm`.
 template <int BT, bool ORD>
 __global__ void __launch_bounds__(kThreadsB, 1)
 k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUtensorMap map_xcol,
@@ -186,7 +185,7 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
                     ok = mbar_wait(&bars->empty[s], ph, abort_flag, p.status, 2);
                     if (!ok) break;
                     uint8_t* st = stage_base + s * SM::stage_bytes(K16);
-                    const int x0 = (ORD && p.list ? (int)p.list[(size_t)it.pair * p.tiles + it.j0 + j] : p.jt0 + it.j0 + j) * 128;
+                    const int x0 = (ORD ? (int)p.list[(size_t)it.pair * p.tiles + it.j0 + j] : p.jt0 + it.j0 + j) * 128;
                     mbar_expect_tx(&bars->full[s], SM::stage_bytes(K16));
                     for (int c = 0; c < K16; ++c)
                         tma_load_2d(st + c * SM::kXChunk, &map_xcol, 0, (int)(c * p.np + x0), &bars->full[s]);
@@ -398,7 +397,7 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
             }
             int64_t row = (int64_t)it.pair * 256 + row_in_pair;
             if (row < p.Nrow) {
-                if (ORD && p.perm) row = p.perm[row];
+                if (ORD) row = p.perm[row];
                 const float l = p.left ? p.left[row] : 1.0f;
 #pragma unroll
                 for (int c = 0; c < BT; ++c)
@@ -515,7 +514,7 @@ fd_status launch_one(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, co
     const int smem = SmemB<BT>::total(p.K16, p.stages);
     if (smem > 227 * 1024) return fail(c, FD_ERR_UNSUPPORTED, "block product kernel needs %d B of shared memory", smem);
     // the attribute is per device: set it on every launch (cheap) rather than remembering one device
-    const auto kernel = c->order_state == 1 ? k_block<BT, true> : k_block<BT, false>;
+    const auto kernel = p.list ? k_block<BT, true> : k_block<BT, false>;
     FD_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     cudaFuncAttributes fa;
     FD_CUDA(c, cudaFuncGetAttributes(&fa, kernel));

@@ -154,3 +154,31 @@ def test_only_degree_passes_decide_which_tiles_are_left_out(fd, dev, kind):
         assert torch.equal(ctx.apply(V), Y)
         assert ctx.get_option("tile_share") == share
     ctx.close()
+
+
+@pytest.mark.parametrize("kind", ["direct", "gram"])
+def test_calls_without_lists_do_not_depend_on_the_order_of_the_points(fd, dev, kind):
+    """A bandwidth so small that no two points are far apart: a context that has ordered its points for another bandwidth gives the bits
+    of one that never did, in every kind of pass."""
+    def passes(ctx, X, small):
+        V = fd.to_colmajor(workloads.block(X.shape[0], 8, seed=3), dev)
+        rows = torch.from_numpy(X[:70].copy()).to(dev)
+        q, d, s, so, so2 = ctx.degree(small, 1.0)
+        out = [q, d, s, ctx.apply(V), ctx.apply_general(1.5 * small, V), ctx.apply_general(small, V, Xrow=rows), ctx.nystrom(rows, V, [0.5] * 8)]
+        if kind == "gram":
+            out.append(ctx.apply(V, prec=fd.FD_PREC_FAST))
+        return out, (so, so2)
+
+    ctx, X, beta = _listed(fd, dev, kind)
+    want, sums = passes(ctx, X, 0.01 * beta)
+    ctx.close()
+    ctx, X, beta = _listed(fd, dev, kind)
+    V = fd.to_colmajor(workloads.block(X.shape[0], 8, seed=4), dev)
+    q, d, s, _, _ = ctx.degree(beta, 1.0)
+    Y = ctx.apply(V)
+    assert ctx.get_option("tile_share") < 0.9
+    got, sums2 = passes(ctx, X, 0.01 * beta)
+    assert sums == sums2 and all(torch.equal(a, b) for a, b in zip(want, got)), [torch.equal(a, b) for a, b in zip(want, got)]
+    q2, d2, s2, _, _ = ctx.degree(beta, 1.0)
+    assert torch.equal(q, q2) and torch.equal(d, d2) and torch.equal(s, s2) and torch.equal(ctx.apply(V), Y)
+    ctx.close()
