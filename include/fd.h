@@ -27,6 +27,11 @@
  *   as void*; NULL = the legacy default stream).  fd_apply and fd_apply_general
  *   return without synchronising; calls that return host scalars synchronise
  *   that stream.
+ *   Both may be recorded into a CUDA graph by a capture of that stream (fd_apply_general: without external
+ *   rows; make one eager call of the kind first).  A graph stands for the call with its pointers, bandwidth
+ *   and kernels as recorded; fd_apply's s is read at replay.  It makes everything it needs from the points
+ *   again, so other calls on the context may come between replays.  After the first recording every
+ *   pass does so (operand packing, tile lists: a few tens of microseconds).  Calls that synchronise cannot be recorded.
  * Errors:  every entry point returns an fd_status; argument errors are found
  *   before any launch; nothing aborts or throws.  There is no CPU fallback.
  * Threads: a context is not thread-safe.

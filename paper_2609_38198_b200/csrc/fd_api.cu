@@ -98,6 +98,13 @@ Layout make_layout(int64_t N, int32_t D, int32_t b_max, int32_t m_max) {
     return L;
 }
 
+fd_status note_capture(fd_ctx* c) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    FD_CUDA(c, cudaStreamIsCapturing(c->stream, &st));
+    if (st != cudaStreamCaptureStatusNone) c->captured = true;
+    return FD_OK;
+}
+
 fd_status apply_dispatch(fd_ctx* c, const ApplyArgs& a) {
     int path = c->opt_path;
     if (path == FD_PATH_TC) {

@@ -524,6 +524,7 @@ fd_status apply_simt(fd_ctx* c, const ApplyArgs& a) {
     // passes over the context's whole point set may leave out tiles of pairs whose kernel value is exactly zero; the degree passes
     // decide (they wait for their sums anyway), products follow
     if (a.rows_are_ctx && a.xrow == c->xs() && a.Nrow == L.N && !c->sh.on && L.direct_lists) {
+        FD_TRY(note_capture(c));
         FD_TRY(tile_lists(c, a.beta, 2, a.decide));
         if (c->lists[2].on && c->lists[2].beta == a.beta) {
             p.list = c->at<unsigned short>(L.lists);

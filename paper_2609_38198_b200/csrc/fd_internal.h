@@ -75,6 +75,9 @@ struct fd_ctx {
     // they leave out enough to be used, entries in all; which of the three the workspace holds, and for which bandwidth
     // (direct-difference kernels (2): total is in groups of four tiles of 16 points, entries in single ones)
     struct { double beta = -1.0; bool on = false; int64_t total = 0, entries = 0; } lists[3];
+    // A pass of this context was recorded into a CUDA graph (set by note_capture, for good).  What the workspace holds is then known to nobody
+    // on the host: recording runs nothing, and a replay packs and lists again.  Every pass packs and lists for itself from then on.
+    bool captured = false;
     double refused_beta = 0.0;       // largest bandwidth at which an order was tried and left out too little
     int listed_kind = -1, boxes_kind = -1;
     double listed_beta = -1.0;
@@ -186,6 +189,8 @@ void shard_range(int64_t N, int world, int rank, int64_t* begin, int64_t* end);
 fd_status gather_rows(fd_ctx* c, float* A, int64_t lda, int cols);
 // In-place sum over the ranks of n host doubles.  No-op for an unsharded context.
 fd_status allreduce_host(fd_ctx* c, double* buf, int64_t n);
+// Sets c->captured if the context's stream is being captured: for passes that would rely on what an earlier one left in the workspace.
+fd_status note_capture(fd_ctx* c);
 // Tile lists of a bandwidth for c->lists[kind] (fd_order.cu): decides c->lists[kind] and, where they are
 // used, brings them into the workspace; orders the points first if that can pay.  A new bandwidth is decided, with a wait, only where
 // `decide` allows it; without, nothing is listed for it.

@@ -379,7 +379,7 @@ fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide) {
     const Layout& L = c->L;
     auto& st = c->lists[kind];
     if (L.perm == 0 || c->order_state < 0) return FD_OK;
-    if (st.beta == beta && (!st.on || (c->listed_kind == kind && c->listed_beta == beta))) return FD_OK;
+    if (st.beta == beta && (!st.on || (!c->captured && c->listed_kind == kind && c->listed_beta == beta))) return FD_OK;
     // Beyond an exponent of 40 both fp16 pieces of a kernel value are zero (2^15 2^-40 = 2^-25 rounds to zero), beyond 60 a degree
     // contribution is below the fixed-point unit; the quarter covers the rounding of the boxes' distance.
     // The direct-difference kernels' exponential gives exactly zero beyond 126.
@@ -462,7 +462,7 @@ fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide) {
         c->boxes_kind = -1;
         c->packed_beta = c->packed_row_beta = -1.0;
     }
-    if (c->boxes_kind != (direct ? 1 : 0)) {
+    if (c->captured || c->boxes_kind != (direct ? 1 : 0)) {
         if (direct) k_boxes16<<<(unsigned)ceil_div(L.NP, 256), 256, 0, c->stream>>>(z, ZP, N, perm, tiles, box);
         else k_boxes<<<tiles, 128, 0, c->stream>>>(z, ZP, N, perm, box);
         FD_LAUNCH_CHECK(c, "k_boxes");

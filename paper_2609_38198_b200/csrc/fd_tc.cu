@@ -479,6 +479,7 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
     const Layout& L = c->L;
     const int64_t N = L.N, NP = L.NP;
     if (!encode_fn()) return fail(c, FD_ERR_CUDA, "cuTensorMapEncodeTiled entry point unavailable");
+    FD_TRY(note_capture(c));
     const double bprime = a.beta * kLog2e;
     const bool rowsum = a.V == nullptr;
     const double* mu = c->at<double>(L.mu);
@@ -507,9 +508,9 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
     const int* perm = use_lists ? c->at<int>(L.perm) : nullptr;
     const PackRole rows{a.xrow, xp_row, a.Nrow, perm}, cols{c->xs(), xp_col, N, perm};
     const int64_t row0 = a.rows_are_ctx ? (a.xrow - c->xs()) / L.DP : -1;
-    const bool have_rows = a.rows_are_ctx && c->packed_row_beta == a.beta && c->packed_row0 == row0 && c->packed_rows == a.Nrow &&
+    const bool have_rows = !c->captured && a.rows_are_ctx && c->packed_row_beta == a.beta && c->packed_row0 == row0 && c->packed_rows == a.Nrow &&
                            c->packed_row_ordered == use_lists;
-    const bool have_cols = c->packed_beta == a.beta && c->packed_ordered == use_lists;
+    const bool have_cols = !c->captured && c->packed_beta == a.beta && c->packed_ordered == use_lists;
     if (!have_rows || !have_cols) {
         const int first = have_rows ? 1 : 0, roles = (have_rows ? 0 : 1) + (have_cols ? 0 : 1);
         k_pack_points<<<dim3((unsigned)ceil_div(NP, 256), (unsigned)K16, (unsigned)roles), 256, 0, c->stream>>>(

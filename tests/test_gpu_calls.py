@@ -182,3 +182,99 @@ def test_calls_without_lists_do_not_depend_on_the_order_of_the_points(fd, dev, k
     q2, d2, s2, _, _ = ctx.degree(beta, 1.0)
     assert torch.equal(q, q2) and torch.equal(d, d2) and torch.equal(s, s2) and torch.equal(ctx.apply(V), Y)
     ctx.close()
+
+
+# ------------------------------------------------------------------ products recorded into CUDA graphs
+@pytest.mark.parametrize("kind,prec", [("direct", 0), ("gram", 0), ("gram", 1)])
+def test_recorded_products_do_not_depend_on_calls_in_between(fd, dev, kind, prec):
+    """Eager calls may come between recording and replay and between replays: external rows (which use the rows' operand buffer), degree
+    passes at another bandwidth (other lists), products at a bandwidth that only a graph has seen.  Every result is that of the same
+    call in a context without graphs, bit for bit."""
+    stream = torch.cuda.Stream()
+    if kind == "direct":
+        X, beta, path = workloads.torus2(16384, seed=1), 100.0, fd.FD_PATH_SIMT
+    else:
+        X, beta, path = workloads.latent_torus(32768, seed=42), 5.0, fd.FD_PATH_TC
+    N, b, other, unseen = X.shape[0], 8, 2.5 * beta, 0.7 * beta
+    Xt = torch.from_numpy(X).to(dev)
+    V = fd.to_colmajor(workloads.block(N, b, seed=3), dev)
+    torch.cuda.synchronize()
+
+    def context(s):
+        ctx = fd.Context(Xt, b_max=b, stream=s)
+        ctx.set_option("path", path)
+        ctx.set_option("tc_max_mag", 1e4)
+        return ctx
+
+    plain = context(stream)
+    s0 = plain.degree(beta, 1.0)[2].clone()
+
+    def general(c, bt, out=None):
+        Y = c.apply_general(bt, V, left=s0, right=s0, out=out, prec=prec)
+        if out is None:
+            torch.cuda.synchronize()                          # (compared on another stream)
+        return Y
+
+    torch.cuda.synchronize()
+    want = general(plain, beta)
+    assert plain.get_option("tile_share") < 0.9
+    want_unseen = general(plain, unseen)
+    torch.cuda.synchronize()
+
+    ctx = context(stream)
+    ctx.degree(beta, 1.0)
+    general(ctx, beta)
+    Y, Z = torch.zeros_like(want), torch.zeros_like(want)
+    torch.cuda.synchronize()
+    g1, g2 = torch.cuda.CUDAGraph(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g1, stream=stream):
+        general(ctx, beta, out=Y)
+    with torch.cuda.graph(g2, stream=stream):
+        general(ctx, unseen, out=Z)
+    torch.cuda.synchronize()
+
+    def replay(g, buf, expect, what):
+        buf.zero_()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(stream):
+            g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(buf, expect), what
+
+    assert torch.equal(general(ctx, unseen), want_unseen), "eager, recorded but never run"
+    replay(g2, Z, want_unseen, "first replay")
+    assert torch.equal(general(ctx, beta), want), "eager after a replay at another bandwidth"
+    replay(g1, Y, want, "after an eager call")
+    ctx.apply_general(beta, V, Xrow=Xt[:500].contiguous())
+    ctx.nystrom(Xt[100:300].contiguous(), V, [0.5] * b)
+    replay(g1, Y, want, "after external rows")
+    ctx.degree(other, 1.0)
+    general(ctx, other)
+    replay(g1, Y, want, "after degree passes at another bandwidth")
+    replay(g2, Z, want_unseen, "after degree passes at another bandwidth")
+    ctx.degree(beta, 1.0)
+    assert torch.equal(general(ctx, beta), want)
+    ctx.synchronize()
+    ctx.close(); plain.close()
+
+
+def test_recorded_row_sums_do_not_wait(fd, dev):
+    """A row sum over the points at a bandwidth that no degree pass has seen returns without waiting, so it can be recorded."""
+    stream = torch.cuda.Stream()
+    X = torch.from_numpy(workloads.torus2(16384, seed=1)).to(dev)
+    torch.cuda.synchronize()
+    ctx = fd.Context(X, b_max=8, stream=stream)
+    ctx.set_option("path", fd.FD_PATH_SIMT)
+    want = ctx.apply_general(150.0, None)
+    torch.cuda.synchronize()
+    ctx.apply_general(100.0, None)
+    Y = torch.zeros_like(want)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream):
+        ctx.apply_general(150.0, None, out=Y)
+    torch.cuda.synchronize()
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(Y, want)
+    ctx.close()
