@@ -359,7 +359,8 @@ k_direct_rowsum(const DirectParams p) {
 }
 
 // Finishes the row tiles that a cut falls into.  Block = (32 rows of a row tile, 8 columns), 8 groups of shares read in parallel (a row
-// tile of a small problem has up to a hundred).
+// tile of a small problem has up to a hundred).  Every block waits for the product, also one that has nothing to add: with lists it may be
+// that no row tile is cut, and what follows this kernel in the stream waits for this kernel only.
 constexpr int kFixCols = 8;
 __global__ void __launch_bounds__(256)
 k_direct_fix(const DirectParams p, int BT, int ctas) {
@@ -370,8 +371,8 @@ k_direct_fix(const DirectParams p, int BT, int ctas) {
     const long long g1 = p.list ? (long long)p.offs[rt + 1] : g0 + p.col_tiles;
     // the last CTA whose range begins at or before step g0, and the last one whose range begins before g1
     const int first = (int)(((g0 + 1) * ctas - 1) / total), last = (int)((g1 * ctas - 1) / total);
-    if (first == last) return;                                         // not cut: its CTA stored it
     cudaGridDependencySynchronize();
+    if (first == last) return;                                         // not cut: its CTA stored it
     const int r = threadIdx.x & 31, grp = threadIdx.x >> 5;
     const int row = (blockIdx.x % (kRowsT / 32)) * 32 + r, col0 = (int)blockIdx.y * kFixCols;
     const int per = (last - first + 8) / 8, s0 = first + grp * per, s1 = min(last + 1, s0 + per);
@@ -408,8 +409,8 @@ k_direct_rowsum_fix(const DirectParams p, int ctas) {
     const long long g0 = p.list ? (long long)p.offs[rt] : (long long)rt * p.col_tiles;
     const long long g1 = p.list ? (long long)p.offs[rt + 1] : g0 + p.col_tiles;
     const int first = (int)(((g0 + 1) * ctas - 1) / total), last = (int)((g1 * ctas - 1) / total);
-    if (first == last) return;
     cudaGridDependencySynchronize();
+    if (first == last) return;
     const int r = threadIdx.x & 31, grp = threadIdx.x >> 5, row = (blockIdx.x % (kRowsT / 32)) * 32 + r;
     const int per = (last - first + 8) / 8, s0 = first + grp * per, s1 = min(last + 1, s0 + per);
     const double2* slots = static_cast<const double2*>(p.part) + row;
