@@ -65,7 +65,7 @@ Layout make_layout(int64_t N, int32_t D, int32_t b_max, int32_t m_max) {
     L.wt_hi = carve(cur, (size_t)L.BP * L.NP * 2);
     L.wt_lo = carve(cur, (size_t)L.BP * L.NP * 2);
     L.colscale = carve(cur, (size_t)(L.BP + 8) * 4 * 2);
-    L.status = carve(cur, 256);
+    L.status = carve(cur, 512);      // status word, cycles, sums (64), counts (128); notes of the direct-difference products (256)
     L.symsum = carve(cur, (size_t)N * 8);
     L.weights = carve(cur, (size_t)L.NP * 4);
     // tile lists: N^2 / 16384 bytes, 17 MB at 2^19 points; larger sets run over all tiles (as do small ones, where nothing is gained)
@@ -148,7 +148,7 @@ fd_status fd_create(fd_ctx** out, const float* X_dev, int64_t N, int32_t D, int6
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device);
     if (e != cudaSuccess) { delete c; return FD_ERR_CUDA; }
-    e = cudaMemsetAsync(c->at<unsigned int>(L.status), 0, 256, c->stream);
+    e = cudaMemsetAsync(c->at<unsigned int>(L.status), 0, 512, c->stream);
     if (e != cudaSuccess) { delete c; return FD_ERR_CUDA; }
     fd_status st = setup_points(c, X_dev, ldx);
     if (st != FD_OK) { delete c; return st; }

@@ -58,6 +58,10 @@ struct DirectParams {
     // positions each; a step is a column tile of consecutive entries, offs[r] steps lie before row tile r; perm: point of each position
     const unsigned short* list; const unsigned int* counts; const unsigned int* offs; const int* perm; int tiles16;
     int tj_log2;                                 // log2 of the points per column tile: 6, or 4 where 64 would leave too few steps
+    int dp4;                                     // float4 per point
+    // with lists: bad[c] = epoch where a sum of column c (row sums: a weighted sum) is not finite.  An entry of the right block that is not finite
+    // shows in its own point's row at least (kernel value 1); looking at the sums costs 1 %, at the staged entries 6 % (N = 16384, D = 4, b = 16).
+    unsigned int* bad; unsigned int epoch;
 };
 
 __host__ __device__ __forceinline__ long long range_begin(long long total, int cta, int ctas) { return total * cta / ctas; }
@@ -255,6 +259,22 @@ k_direct(const DirectParams p) {
             }
         }
         if (part == 0) {
+            if (LISTED) {
+                float zero = 0.f;                                  // NaN if any sum is not finite
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int c = 0; c < BT; ++c) zero = fmaf(acc[r][c], 0.f, zero);
+                if (zero != 0.f) {
+#pragma unroll
+                    for (int c = 0; c < BT; ++c) {
+                        float z = 0.f;
+#pragma unroll
+                        for (int r = 0; r < R; ++r) z = fmaf(acc[r][c], 0.f, z);
+                        if (z != 0.f) p.bad[c] = p.epoch;
+                    }
+                }
+            }
             const bool whole = n == range.full;
             float* slot = static_cast<float*>(p.part) +
                           (size_t)(2 * blockIdx.x + (c0 == 0 ? 1 : 0)) * BT * kRowsT + lane_row;
@@ -346,6 +366,7 @@ k_direct_rowsum(const DirectParams p) {
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 int64_t i = row0 + lane_row + (kRowsT / R) * r;
+                if (LISTED && !isfinite(dsum[r])) p.bad[0] = p.epoch;
                 if (n != range.full) slot[(kRowsT / R) * r] = make_double2(dsum[r], dsq[r]);
                 else if (i < p.Nrow) {
                     if (LISTED) i = p.perm[i];
@@ -358,75 +379,116 @@ k_direct_rowsum(const DirectParams p) {
     cudaTriggerProgrammaticLaunchCompletion();
 }
 
+// Row i's sum over every point for column c of the right block (row sums, V null: for the weights).  For columns that `bad` names: the product
+// of an entry that is not finite with a kernel value of zero is NaN, so tiles of zeros count as well and the lists do not hold.
+__device__ __forceinline__ float sum_over_all_points(const DirectParams& p, int64_t i, int c) {
+    float acc = 0.f;
+#pragma unroll 1
+    for (int64_t j = 0; j < p.N; ++j) {
+        float h = 0.f;
+#pragma unroll 1
+        for (int k = 0; k < p.dp4; ++k) {
+            const float4 a = p.xrow[i * p.dp4 + k], b = p.xcol[j * p.dp4 + k];
+            const float d0 = a.x - b.x, d1 = a.y - b.y, d2 = a.z - b.z, d3 = a.w - b.w;
+            h = fmaf(d0, d0, h); h = fmaf(d1, d1, h); h = fmaf(d2, d2, h); h = fmaf(d3, d3, h);
+        }
+        float w = p.V && c < p.vcols ? p.V[j + (int64_t)c * p.ldv] : 1.f;
+        if (p.right) w *= p.right[j];
+        acc = fmaf(ex2_approx(h * p.nbeta2), w, acc);
+    }
+    return acc;
+}
+
 // Finishes the row tiles that a cut falls into.  Block = (32 rows of a row tile, 8 columns), 8 groups of shares read in parallel (a row
 // tile of a small problem has up to a hundred).  Every block waits for the product, also one that has nothing to add: with lists it may be
 // that no row tile is cut, and what follows this kernel in the stream waits for this kernel only.
 constexpr int kFixCols = 8;
+template <bool LISTED>
 __global__ void __launch_bounds__(256)
 k_direct_fix(const DirectParams p, int BT, int ctas) {
     __shared__ float sm[kFixCols][8][32];
     const int rt = blockIdx.x / (kRowsT / 32);
-    const long long total = p.list ? (long long)p.offs[p.row_tiles] : (long long)p.row_tiles * p.col_tiles;
-    const long long g0 = p.list ? (long long)p.offs[rt] : (long long)rt * p.col_tiles;
-    const long long g1 = p.list ? (long long)p.offs[rt + 1] : g0 + p.col_tiles;
+    const long long total = LISTED ? (long long)p.offs[p.row_tiles] : (long long)p.row_tiles * p.col_tiles;
+    const long long g0 = LISTED ? (long long)p.offs[rt] : (long long)rt * p.col_tiles;
+    const long long g1 = LISTED ? (long long)p.offs[rt + 1] : g0 + p.col_tiles;
     // the last CTA whose range begins at or before step g0, and the last one whose range begins before g1
     const int first = (int)(((g0 + 1) * ctas - 1) / total), last = (int)((g1 * ctas - 1) / total);
     cudaGridDependencySynchronize();
-    if (first == last) return;                                         // not cut: its CTA stored it
+    const bool cut = first != last;                                    // else its CTA stored it
+    if (!LISTED && !cut) return;
     const int r = threadIdx.x & 31, grp = threadIdx.x >> 5;
     const int row = (blockIdx.x % (kRowsT / 32)) * 32 + r, col0 = (int)blockIdx.y * kFixCols;
-    const int per = (last - first + 8) / 8, s0 = first + grp * per, s1 = min(last + 1, s0 + per);
-    const float* slots = static_cast<const float*>(p.part) + (size_t)col0 * kRowsT + row;
-    float v[kFixCols];
+    // (read beside the shares, looked at after them: one latency)
+    const unsigned int note = LISTED && col0 + grp < p.b ? p.bad[col0 + grp] : p.epoch + 1;
+    if (cut) {
+        const int per = (last - first + 8) / 8, s0 = first + grp * per, s1 = min(last + 1, s0 + per);
+        const float* slots = static_cast<const float*>(p.part) + (size_t)col0 * kRowsT + row;
+        float v[kFixCols];
 #pragma unroll
-    for (int c = 0; c < kFixCols; ++c) v[c] = 0.f;
+        for (int c = 0; c < kFixCols; ++c) v[c] = 0.f;
 #pragma unroll 4
-    for (int s = s0; s < s1; ++s) {
-        const float* o = slots + (size_t)(2 * s + (s == first ? 1 : 0)) * BT * kRowsT;
+        for (int s = s0; s < s1; ++s) {
+            const float* o = slots + (size_t)(2 * s + (s == first ? 1 : 0)) * BT * kRowsT;
 #pragma unroll
-        for (int c = 0; c < kFixCols; ++c)
-            if (col0 + c < p.b) v[c] += o[c * kRowsT];
+            for (int c = 0; c < kFixCols; ++c)
+                if (col0 + c < p.b) v[c] += o[c * kRowsT];
+        }
+#pragma unroll
+        for (int c = 0; c < kFixCols; ++c) sm[c][grp][r] = v[c];
+        __syncthreads();
     }
-#pragma unroll
-    for (int c = 0; c < kFixCols; ++c) sm[c][grp][r] = v[c];
-    __syncthreads();
     // group g finishes column col0 + g
     int64_t i = (int64_t)rt * kRowsT + row;
     if (i >= p.Nrow || col0 + grp >= p.b) return;
-    if (p.perm) i = p.perm[i];
+    const bool bad = LISTED && note == p.epoch;
+    if (!cut && !bad) return;
+    if (LISTED) i = p.perm[i];
     float x = 0.f;
+    if (bad) x = sum_over_all_points(p, i, col0 + grp);
+    else {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) x += sm[grp][q][r];
+        for (int q = 0; q < 8; ++q) x += sm[grp][q][r];
+    }
     p.Y[i + (int64_t)(col0 + grp) * p.ldy] = x * (p.left ? p.left[i] : 1.0f);
 }
 
 // The same for row sums: block = 32 rows.
+template <bool LISTED>
 __global__ void __launch_bounds__(256)
 k_direct_rowsum_fix(const DirectParams p, int ctas) {
     __shared__ double2 sm[8][32];
     const int rt = blockIdx.x / (kRowsT / 32);
-    const long long total = p.list ? (long long)p.offs[p.row_tiles] : (long long)p.row_tiles * p.col_tiles;
-    const long long g0 = p.list ? (long long)p.offs[rt] : (long long)rt * p.col_tiles;
-    const long long g1 = p.list ? (long long)p.offs[rt + 1] : g0 + p.col_tiles;
+    const long long total = LISTED ? (long long)p.offs[p.row_tiles] : (long long)p.row_tiles * p.col_tiles;
+    const long long g0 = LISTED ? (long long)p.offs[rt] : (long long)rt * p.col_tiles;
+    const long long g1 = LISTED ? (long long)p.offs[rt + 1] : g0 + p.col_tiles;
     const int first = (int)(((g0 + 1) * ctas - 1) / total), last = (int)((g1 * ctas - 1) / total);
     cudaGridDependencySynchronize();
-    if (first == last) return;
+    const bool cut = first != last;
+    if (!LISTED && !cut) return;
     const int r = threadIdx.x & 31, grp = threadIdx.x >> 5, row = (blockIdx.x % (kRowsT / 32)) * 32 + r;
-    const int per = (last - first + 8) / 8, s0 = first + grp * per, s1 = min(last + 1, s0 + per);
-    const double2* slots = static_cast<const double2*>(p.part) + row;
-    double2 v = make_double2(0.0, 0.0);
+    const unsigned int note = LISTED ? p.bad[0] : p.epoch + 1;
+    if (cut) {
+        const int per = (last - first + 8) / 8, s0 = first + grp * per, s1 = min(last + 1, s0 + per);
+        const double2* slots = static_cast<const double2*>(p.part) + row;
+        double2 v = make_double2(0.0, 0.0);
 #pragma unroll 8
-    for (int s = s0; s < s1; ++s) { const double2 o = slots[(size_t)(2 * s + (s == first ? 1 : 0)) * kRowsT]; v.x += o.x; v.y += o.y; }
-    sm[grp][r] = v;
-    __syncthreads();
+        for (int s = s0; s < s1; ++s) { const double2 o = slots[(size_t)(2 * s + (s == first ? 1 : 0)) * kRowsT]; v.x += o.x; v.y += o.y; }
+        sm[grp][r] = v;
+        __syncthreads();
+    }
     int64_t i = (int64_t)rt * kRowsT + row;
     if (grp != 0 || i >= p.Nrow) return;
-    if (p.perm) i = p.perm[i];
-    v = make_double2(0.0, 0.0);
+    const bool bad = LISTED && note == p.epoch;
+    if (!cut && !bad) return;
+    if (LISTED) i = p.perm[i];
+    double2 v = make_double2(0.0, 0.0);
+    if (cut) {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) { v.x += sm[q][r].x; v.y += sm[q][r].y; }
+        for (int q = 0; q < 8; ++q) { v.x += sm[q][r].x; v.y += sm[q][r].y; }
+        if (p.rowsq) p.rowsq[i] = v.y;
+    }
+    if (bad) v.x = (double)sum_over_all_points(p, i, 0);
     p.Y[i] = (float)(v.x * (p.left ? (double)p.left[i] : 1.0));
-    if (p.rowsq) p.rowsq[i] = v.y;
 }
 
 // Launches one CTA per equal range of steps: as many as are resident at once (more would leave a last round partly filled), or as
@@ -457,8 +519,8 @@ fd_status launch(fd_ctx* c, Kernel kernel, int smem, int per_sm, int BT, DirectP
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3((unsigned)p.row_tiles * (kRowsT / 32), BT > 0 ? (unsigned)ceil_div(p.b, kFixCols) : 1u);
         cfg.blockDim = dim3(256); cfg.stream = c->stream; cfg.attrs = &attr; cfg.numAttrs = 1;
-        if (BT > 0) FD_CUDA(c, cudaLaunchKernelEx(&cfg, k_direct_fix, p, BT, (int)ctas));
-        else FD_CUDA(c, cudaLaunchKernelEx(&cfg, k_direct_rowsum_fix, p, (int)ctas));
+        if (BT > 0) FD_CUDA(c, cudaLaunchKernelEx(&cfg, p.list ? k_direct_fix<true> : k_direct_fix<false>, p, BT, (int)ctas));
+        else FD_CUDA(c, cudaLaunchKernelEx(&cfg, p.list ? k_direct_rowsum_fix<true> : k_direct_rowsum_fix<false>, p, (int)ctas));
         FD_LAUNCH_CHECK(c, "k_direct_fix");
     }
     return FD_OK;
@@ -519,7 +581,7 @@ fd_status apply_simt(fd_ctx* c, const ApplyArgs& a) {
     p.xcol = reinterpret_cast<const float4*>(c->xs()); p.N = L.N;
     p.nbeta2 = (float)(-a.beta * kLog2e);
     p.right = a.right; p.left = a.left; p.ldv = a.ldv; p.ldy = a.ldy;
-    p.part = c->at<float>(L.part);
+    p.part = c->at<float>(L.part); p.dp4 = DP4;
     p.row_tiles = (int)ceil_div(a.Nrow, kRowsT);
     const bool rowsum = a.V == nullptr;
     // passes over the context's whole point set may leave out tiles of pairs whose kernel value is exactly zero; the degree passes
@@ -533,6 +595,7 @@ fd_status apply_simt(fd_ctx* c, const ApplyArgs& a) {
             p.offs = p.counts + 2 * p.row_tiles;
             p.perm = c->at<int>(L.perm);
             p.tiles16 = 16 * p.row_tiles;
+            p.bad = reinterpret_cast<unsigned int*>(c->at<char>(L.status) + 256);
         }
     }
     const int chunks = rowsum ? 1 : (int)ceil_div(a.b, 64), step = (int)ceil_div(a.b, chunks);
@@ -543,6 +606,11 @@ fd_status apply_simt(fd_ctx* c, const ApplyArgs& a) {
         p.b = bc;
         p.Y = a.Y + (int64_t)c0 * a.ldy;
         p.rowsq = a.rowsq;
+        if (p.list) {
+            // (a replayed graph brings the same epoch again; what an earlier replay noted would cost time, not the result)
+            p.epoch = ++c->direct_epoch;
+            if (c->captured) FD_CUDA(c, cudaMemsetAsync(p.bad, 0, 64 * 4, c->stream));
+        }
         switch (DP4) {
             case 1: FD_TRY(launch_dp<1>(c, BT, p)); break;
             case 2: FD_TRY(launch_dp<2>(c, BT, p)); break;

@@ -78,6 +78,7 @@ struct fd_ctx {
     // A pass of this context was recorded into a CUDA graph (set by note_capture, for good).  What the workspace holds is then known to nobody
     // on the host: recording runs nothing, and a replay packs and lists again.  Every pass packs and lists for itself from then on.
     bool captured = false;
+    unsigned int direct_epoch = 0;   // number of the latest listed pass of the direct-difference kernels
     double refused_beta = 0.0;       // largest bandwidth at which an order was tried and left out too little
     int listed_kind = -1, boxes_kind = -1;
     double listed_beta = -1.0;

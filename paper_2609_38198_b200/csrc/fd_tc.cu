@@ -345,7 +345,7 @@ __global__ void k_pad_weights(const float* __restrict__ w, int64_t n, int64_t np
     if (j < np) out[j] = j < n ? (w ? w[perm ? perm[j] : j] : 1.f) : 0.f;
 }
 
-// Per-block maxima of |right_j V_jc| for each column c (columns from vcols on are the ones vector).
+// Per-block maxima of |right_j V_jc| for each column c (columns from vcols on are the ones vector); infinite where an entry is not finite.
 __global__ void __launch_bounds__(256)
 k_colmax_partial(const float* __restrict__ V, int64_t ldv, int vcols, const float* __restrict__ right, int64_t N, int c0, float* __restrict__ part) {
     __shared__ float sm[8];
@@ -353,8 +353,9 @@ k_colmax_partial(const float* __restrict__ V, int64_t ldv, int vcols, const floa
     const float* v = V + (int64_t)(ones ? 0 : c0 + blockIdx.y) * ldv;
     float m = 0.f;
     for (int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x; j < N; j += (int64_t)gridDim.x * 256) {
-        const float x = ones ? 1.f : v[j];
-        m = fmaxf(m, fabsf(right ? x * right[j] : x));
+        float x = ones ? 1.f : v[j];
+        if (right) x *= right[j];
+        m = fmaxf(m, isfinite(x) ? fabsf(x) : INFINITY);
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
@@ -370,6 +371,8 @@ k_colmax_partial(const float* __restrict__ V, int64_t ldv, int vcols, const floa
 // wt [c * np + j] = fp16 hi piece of scale_c * right_j * V[j, c0 + c], and the lo piece BT rows below when `with_lo`; zero padding for
 // j >= N and c >= bc.  scale_c = the power of two that puts the column maximum in [2^12, 2^13): every block reduces the
 // partial maxima of its column itself (they are at most 256 values); the first one stores the epilogue factor 2^-bias / scale.
+// An entry that is not finite makes its whole column NaN in the fp32-grade mode (the lo piece of Inf is NaN, and 0 NaN = NaN in every
+// row): the factor is NaN then, so that rows whose tiles leave the entry out get it too.
 __global__ void __launch_bounds__(256)
 k_pack_wt(const float* __restrict__ V, int64_t ldv, int vcols, const float* __restrict__ right, int64_t N, int64_t np, int c0, int bc,
           const float* __restrict__ part, int parts, float* __restrict__ inv, __half* __restrict__ wt, int with_lo, const int* __restrict__ perm) {
@@ -389,7 +392,7 @@ k_pack_wt(const float* __restrict__ V, int64_t ldv, int vcols, const float* __re
         frexpf(m, &e);                               // m = f * 2^e, f in [0.5, 1)
         sc = ldexpf(1.0f, 13 - e);
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) inv[c] = ldexpf(1.0f, -kBias) / sc;
+    if (blockIdx.x == 0 && threadIdx.x == 0) inv[c] = with_lo && isinf(m) ? NAN : ldexpf(1.0f, -kBias) / sc;
     const bool ones = c0 + c >= vcols;
     const float* v = V + (int64_t)(ones ? 0 : c0 + c) * ldv;
     __half2* hi = reinterpret_cast<__half2*>(wt + (int64_t)c * np);

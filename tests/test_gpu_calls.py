@@ -278,3 +278,65 @@ def test_recorded_row_sums_do_not_wait(fd, dev):
     torch.cuda.synchronize()
     assert torch.equal(Y, want)
     ctx.close()
+
+
+# ------------------------------------------------------------------ non-finite right blocks
+@pytest.mark.parametrize("kind", ["direct", "gram"])
+def test_entries_that_are_not_finite_reach_every_row(fd, dev, kind):
+    """0 * Inf and 0 * NaN are NaN: with far tiles left out the product has NaN and Inf where the product over all tiles (a context whose
+    degree passes have not seen the bandwidth) has them; the other columns are untouched.  Also in a recorded product, whose later
+    replays with finite entries are as before, and in row sums with such weights."""
+    ctx, X, beta = _listed(fd, dev, kind)
+    N, b = X.shape[0], 24
+    path = ctx.get_option("path")
+    ctx.close()
+    stream = torch.cuda.Stream()
+    Xt = torch.from_numpy(X).to(dev)
+    good = fd.to_colmajor(workloads.block(N, b, seed=3), dev)
+    V = good.clone(memory_format=torch.preserve_format)
+    V[100, 1] = float("nan"); V[200, 2] = float("inf"); V[300, 3] = float("-inf"); V[300, 17] = float("inf"); V[9000, 17] = float("-inf")
+    V[17, 23] = float("inf"); V[18, 23] = float("nan"); V[:, 7] = 3e38                  # (finite, though its sums are not)
+    w = torch.rand(N, device=dev) + 0.5
+    w[12] = float("inf")
+    torch.cuda.synchronize()
+    ctx = fd.Context(Xt, b_max=b, stream=stream)
+    ctx.set_option("path", path)
+    ctx.set_option("tc_max_mag", 1e4)
+    ctx.degree(beta, 1.0)
+    want_good = ctx.apply(good)
+    assert ctx.get_option("tile_share") < 0.9
+    Y = ctx.apply(V)
+    torch.cuda.synchronize()
+    # every tile
+    ref = fd.Context(Xt, b_max=b, stream=stream)
+    ref.set_option("path", path)
+    ref.set_option("tc_max_mag", 1e4)
+    s = torch.empty(N, device=dev)
+    s.copy_(ctx.degree(beta, 1.0)[2])
+    torch.cuda.synchronize()
+    Yr = ref.apply_general(beta, V, left=s, right=s)
+    torch.cuda.synchronize()
+    cls = lambda t: torch.where(torch.isnan(t), 3, torch.where(torch.isposinf(t), 1, torch.where(torch.isneginf(t), 2, 0)))
+    assert torch.equal(cls(Y), cls(Yr))
+    finite = torch.isfinite(Yr).all(0)
+    assert 0 < (~finite).sum() <= 6 and ((Y[:, finite] - Yr[:, finite]).norm() / Yr[:, finite].norm()).item() <= 2e-6
+    if kind == "direct":
+        R, Rr = ctx.apply_general(beta, None, right=w), ref.apply_general(beta, None, right=w)
+        torch.cuda.synchronize()
+        assert torch.equal(cls(R), cls(Rr)) and not torch.isfinite(R).any()
+    # recorded: bad entries, then finite ones in the same buffer
+    buf, out = V.clone(memory_format=torch.preserve_format), torch.zeros_like(Y)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream):
+        ctx.apply(buf, out=out)
+    for v, want in ((V, Y), (good, want_good), (V, Y)):
+        buf.copy_(v)
+        torch.cuda.synchronize()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(cls(out), cls(want)) and torch.equal(torch.nan_to_num(out), torch.nan_to_num(want))
+    last = ctx.apply(good)
+    torch.cuda.synchronize()
+    assert torch.equal(last, want_good)
+    ctx.close(); ref.close()
