@@ -35,10 +35,10 @@
  * Errors:  every entry point returns an fd_status; argument errors are found
  *   before any launch; nothing aborts or throws.  There is no CPU fallback.
  * Threads: a context is not thread-safe.
- * Repeats: the same call in the same state gives the same bits.  Passes at a bandwidth that a degree
- *   pass has seen may leave out tiles of the kernel that hold only zeros ("tile_share"); they add in
- *   another order than passes over all tiles, and bandwidths asked earlier can tip the decision.  Every
- *   other pass gives the bits of a new context.
+ * Repeats: the same call in the same state gives the same bits.  At the bandwidth of the latest degree
+ *   passes, passes over the points may leave out tiles of the kernel that hold only zeros ("tile_share"); all
+ *   tensor-core passes at that bandwidth then add in another order than at others, and bandwidths asked
+ *   earlier can tip the decision.  Passes at any other bandwidth give the bits of a new context.
  * k:       counts NONTRIVIAL eigenpairs; the Perron pair (eigenvalue 1) is
  *   returned in slot 0, so k + 1 pairs come back (Sec. 2.3, Sec. 3).
  */

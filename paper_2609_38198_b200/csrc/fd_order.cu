@@ -15,7 +15,8 @@
 // degree passes of a new context then take 0.1 (N = 16384, D = 4) to 0.6 ms (N = 2^18, D = 30) longer, which one of the
 // two passes or the first products pay back from 16384 points on in the plane and on surfaces (direct differences; N = 8192: 130 us of
 // passes against 300) and from 32768 on in the Gram form.  Vectors stay in the caller's order everywhere: packing and staging
-// gather through the permutation, the epilogues scatter.  Only passes over lists work in the order; all others in the caller's.
+// gather through the permutation, the epilogues scatter.  Gram-form passes at a bandwidth with lists work in the order, all others (and
+// direct-difference passes without lists) in the caller's.
 //
 // Lists: for a bandwidth and exponent limit, per 256 rows the column tiles whose bounding box comes close enough (distance of the
 // two boxes: a lower bound for every pair): tiles of 128 points for the Gram-form kernels, of 16 for the direct-difference

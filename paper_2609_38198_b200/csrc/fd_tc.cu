@@ -202,7 +202,7 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
 
         for (int w = 0; w < my_items && ok; ++w) {
             const int item = (int)blockIdx.x + w * (int)gridDim.x;
-            const int64_t row = (int64_t)item * 256 + t * 128 + row_in_tile;
+            int64_t row = (int64_t)item * 256 + t * 128 + row_in_tile;
             {
                 double dsum = 0.0, dsq = 0.0;
                 for (int j = 0; j < num_jt && ok; ++j) {
@@ -241,6 +241,7 @@ k_tc(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
                     dsq += (double)(q0 + q1);
                 }
                 if (ok && row < p.Nrow) {
+                    if (p.perm) row = p.perm[row];
                     // undo the 2^bias scaling of P (exact powers of two)
                     constexpr double scale = 1.0 / (double)(1 << kBias);
                     p.q[row] = (float)(p.left ? dsum * (scale * (double)p.left[row]) : dsum * scale);
@@ -507,13 +508,17 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
     if (prunes && a.decide && a.prec == FD_PREC_FP32 && c->lists[0].beta != a.beta) FD_TRY(tile_lists(c, a.beta, 0, true));
     if (prunes) FD_TRY(tile_lists(c, a.beta, rowsum ? 1 : 0, a.decide));
     const bool use_lists = prunes && c->lists[rowsum ? 1 : 0].on && c->lists[rowsum ? 1 : 0].beta == a.beta;
-    // The points' order is used where lists are: any other pass gives the same bits as in a context that never made an order.
-    const int* perm = use_lists ? c->at<int>(L.perm) : nullptr;
-    const PackRole rows{a.xrow, xp_row, a.Nrow, perm}, cols{c->xs(), xp_col, N, perm};
+    // The points' order is used, by every Gram-form pass, at the bandwidths that have lists (external rows against ordered columns: neighbouring
+    // kernel values alike draw less power; N = 65536, 40009 rows of R^30, 33 vectors: 1.19 ms against 1.23).  At any other bandwidth a pass
+    // gives the bits of a context that never made an order.
+    const bool ordered = !c->sh.on && ((c->lists[0].on && c->lists[0].beta == a.beta) || (c->lists[1].on && c->lists[1].beta == a.beta));
+    const int* col_perm = ordered ? c->at<int>(L.perm) : nullptr;
+    const int* row_perm = all_rows ? col_perm : nullptr;
+    const PackRole rows{a.xrow, xp_row, a.Nrow, row_perm}, cols{c->xs(), xp_col, N, col_perm};
     const int64_t row0 = a.rows_are_ctx ? (a.xrow - c->xs()) / L.DP : -1;
     const bool have_rows = !c->captured && a.rows_are_ctx && c->packed_row_beta == a.beta && c->packed_row0 == row0 && c->packed_rows == a.Nrow &&
-                           c->packed_row_ordered == use_lists;
-    const bool have_cols = !c->captured && c->packed_beta == a.beta && c->packed_ordered == use_lists;
+                           c->packed_row_ordered == ordered;
+    const bool have_cols = !c->captured && c->packed_beta == a.beta && c->packed_ordered == ordered;
     if (!have_rows || !have_cols) {
         const int first = have_rows ? 1 : 0, roles = (have_rows ? 0 : 1) + (have_cols ? 0 : 1);
         k_pack_points<<<dim3((unsigned)ceil_div(NP, 256), (unsigned)K16, (unsigned)roles), 256, 0, c->stream>>>(
@@ -521,9 +526,9 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
         FD_LAUNCH_CHECK(c, "k_pack_points");
         if (!have_rows) {
             c->packed_row_beta = a.rows_are_ctx ? a.beta : -1.0;
-            c->packed_row0 = row0; c->packed_rows = a.Nrow; c->packed_row_ordered = use_lists;
+            c->packed_row0 = row0; c->packed_rows = a.Nrow; c->packed_row_ordered = ordered;
         }
-        c->packed_beta = a.beta; c->packed_ordered = use_lists;
+        c->packed_beta = a.beta; c->packed_ordered = ordered;
     }
 
     CUtensorMap mr, mc, mh;
@@ -540,17 +545,17 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
     if (p.jt_chunk > p.num_jt) p.jt_chunk = p.num_jt;
     p.num_chunks = (int)ceil_div(p.num_jt, p.jt_chunk);
     p.np_rows = NP; p.np_cols = NP; p.K16 = K16;
-    p.left = a.left; p.status = status; p.perm = perm; p.use_lists = use_lists ? 1 : 0;
+    p.left = a.left; p.status = status; p.perm = row_perm; p.ordered = ordered ? 1 : 0; p.use_lists = use_lists ? 1 : 0;
     const int grid = std::min(p.num_work, c->sm_count);
 
     if (rowsum && !a.rowsq) {
         float* w = c->at<float>(L.weights);
-        k_pad_weights<<<(unsigned)ceil_div(NP, 256), 256, 0, c->stream>>>(a.right, N, NP, perm, w);
+        k_pad_weights<<<(unsigned)ceil_div(NP, 256), 256, 0, c->stream>>>(a.right, N, NP, col_perm, w);
         FD_LAUNCH_CHECK(c, "k_pad_weights");
         p.weights = w;
     }
     if (rowsum && sym) {
-        FD_TRY(launch_sym_rowsum(c, mr, mc, p.weights, a.left, a.Y, a.rowsq, perm, use_lists));
+        FD_TRY(launch_sym_rowsum(c, mr, mc, p.weights, a.left, a.Y, a.rowsq, row_perm, use_lists));
     } else if (rowsum) {
         p.q = a.Y; p.rowsq = a.rowsq; p.b = 1;
         if (p.rowsq) FD_TRY((launch_tc<16>(c, mr, mc, p, grid)));
@@ -571,7 +576,7 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
             k_colmax_partial<<<dim3(cm_blocks, bc), 256, 0, c->stream>>>(a.V, a.ldv, vcols, a.right, N, c0, part);
             FD_LAUNCH_CHECK(c, "k_colmax_partial");
             k_pack_wt<<<dim3((unsigned)std::min<int64_t>(1024, ceil_div(NP, 512)), BT), 256, 0, c->stream>>>(
-                a.V, a.ldv, vcols, a.right, N, NP, c0, bc, part, cm_blocks, inv, wt_hi, fast ? 0 : 1, perm);
+                a.V, a.ldv, vcols, a.right, N, NP, c0, bc, part, cm_blocks, inv, wt_hi, fast ? 0 : 1, col_perm);
             FD_LAUNCH_CHECK(c, "k_pack_wt");
             // one map over W_hi (rows 0 .. BT) and, in the fp32-grade mode, W_lo behind it (rows BT .. 2 BT of the same array)
             if (!make_map_2d(&mh, wt_hi, (uint64_t)NP, (uint64_t)(fast ? BT : 2 * BT), (uint64_t)NP * 2, 64, fast ? BT : 2 * BT, CU_TENSOR_MAP_SWIZZLE_128B))

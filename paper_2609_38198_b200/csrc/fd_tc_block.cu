@@ -83,10 +83,10 @@ struct BlockParams {
     int jt0, num_jt;             // column tiles [jt0, jt0 + num_jt) of this launch
     int K16, b, flush, stages;
     int accumulate;              // add to Y (later column chunks) instead of storing
-    // tile lists (null: every column tile, points in the caller's order): column tiles of row pair r at list[r * tiles ..], steps before it offs[r]
+    // tile lists (null: every column tile): column tiles of row pair r at list[r * tiles ..], steps before it offs[r]
     const unsigned short* list; const unsigned int* offs;
     int tiles;
-    const int* perm;             // with lists: row of Y and left for each row of the operand
+    const int* perm;             // row of Y and left for each row of the operand (null: the same)
 };
 
 // First step of CTA `cta` in the flat sequence of steps, and the work item (part of one row pair) that starts at step g of it.
@@ -106,15 +106,16 @@ template <bool ORD>
 struct Steps {                   // walks a CTA's range item by item
     int pair, j0, left;
     __device__ __forceinline__ Steps(const BlockParams& p) {
-        const long long total = ORD ? (long long)p.offs[p.pairs] : (long long)p.pairs * p.num_jt;
+        const bool listed = ORD && p.list;
+        const long long total = listed ? (long long)p.offs[p.pairs] : (long long)p.pairs * p.num_jt;
         const long long g0 = range_begin(total, (int)blockIdx.x, (int)gridDim.x);
-        pair = ORD ? pair_of(p, (unsigned int)g0) : (int)(g0 / p.num_jt);
-        j0 = (int)(g0 - (ORD ? (long long)p.offs[pair] : (long long)pair * p.num_jt));
+        pair = listed ? pair_of(p, (unsigned int)g0) : (int)(g0 / p.num_jt);
+        j0 = (int)(g0 - (listed ? (long long)p.offs[pair] : (long long)pair * p.num_jt));
         left = (int)(range_begin(total, (int)blockIdx.x + 1, (int)gridDim.x) - g0);
     }
     __device__ __forceinline__ bool next(const BlockParams& p, Item& it) {
         if (left <= 0) return false;
-        const int full = ORD ? (int)(p.offs[pair + 1] - p.offs[pair]) : p.num_jt;
+        const int full = ORD && p.list ? (int)(p.offs[pair + 1] - p.offs[pair]) : p.num_jt;
         it.pair = pair; it.j0 = j0;
         it.n = full - j0 < left ? full - j0 : left;
         it.whole = it.n == full;
@@ -123,7 +124,7 @@ struct Steps {                   // walks a CTA's range item by item
     }
 };
 
-// ORD: a pass over the tile lists; the points are in the order `perm`.
+// ORD: the points are ordered (perm, where the rows are the context's own) and tiles may be listed.
 template <int BT, bool ORD>
 __global__ void __launch_bounds__(kThreadsB, 1)
 k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUtensorMap map_xcol,
@@ -185,7 +186,7 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
                     ok = mbar_wait(&bars->empty[s], ph, abort_flag, p.status, 2);
                     if (!ok) break;
                     uint8_t* st = stage_base + s * SM::stage_bytes(K16);
-                    const int x0 = (ORD ? (int)p.list[(size_t)it.pair * p.tiles + it.j0 + j] : p.jt0 + it.j0 + j) * 128;
+                    const int x0 = (ORD && p.list ? (int)p.list[(size_t)it.pair * p.tiles + it.j0 + j] : p.jt0 + it.j0 + j) * 128;
                     mbar_expect_tx(&bars->full[s], SM::stage_bytes(K16));
                     for (int c = 0; c < K16; ++c)
                         tma_load_2d(st + c * SM::kXChunk, &map_xcol, 0, (int)(c * p.np + x0), &bars->full[s]);
@@ -397,7 +398,7 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
             }
             int64_t row = (int64_t)it.pair * 256 + row_in_pair;
             if (row < p.Nrow) {
-                if (ORD) row = p.perm[row];
+                if (ORD && p.perm) row = p.perm[row];
                 const float l = p.left ? p.left[row] : 1.0f;
 #pragma unroll
                 for (int c = 0; c < BT; ++c)
@@ -508,13 +509,13 @@ k_block_fix(const BlockParams p, int ctas) {
 }
 
 template <int BT>
-fd_status launch_one(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, const CUtensorMap& mw, BlockParams p, int jt_total, int jt_chunk) {
+fd_status launch_one(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, const CUtensorMap& mw, BlockParams p, bool ordered, int jt_total, int jt_chunk) {
     p.stages = kStages;
     while (p.stages > 2 && SmemB<BT>::total(p.K16, p.stages) > 227 * 1024) --p.stages;
     const int smem = SmemB<BT>::total(p.K16, p.stages);
     if (smem > 227 * 1024) return fail(c, FD_ERR_UNSUPPORTED, "block product kernel needs %d B of shared memory", smem);
     // the attribute is per device: set it on every launch (cheap) rather than remembering one device
-    const auto kernel = p.list ? k_block<BT, true> : k_block<BT, false>;
+    const auto kernel = ordered ? k_block<BT, true> : k_block<BT, false>;
     FD_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     cudaFuncAttributes fa;
     FD_CUDA(c, cudaFuncGetAttributes(&fa, kernel));
@@ -557,10 +558,10 @@ fd_status launch_block_product(fd_ctx* c, int BT, const CUtensorMap& mr, const C
         p.tiles = (int)(c->L.NP / 128);
     }
     switch (BT) {
-        case 16: return launch_one<16>(c, mr, mc, mw, p, tp.num_jt, tp.jt_chunk);
-        case 32: return launch_one<32>(c, mr, mc, mw, p, tp.num_jt, tp.jt_chunk);
-        case 48: return launch_one<48>(c, mr, mc, mw, p, tp.num_jt, tp.jt_chunk);
-        case 64: return launch_one<64>(c, mr, mc, mw, p, tp.num_jt, tp.jt_chunk);
+        case 16: return launch_one<16>(c, mr, mc, mw, p, tp.ordered != 0, tp.num_jt, tp.jt_chunk);
+        case 32: return launch_one<32>(c, mr, mc, mw, p, tp.ordered != 0, tp.num_jt, tp.jt_chunk);
+        case 48: return launch_one<48>(c, mr, mc, mw, p, tp.ordered != 0, tp.num_jt, tp.jt_chunk);
+        case 64: return launch_one<64>(c, mr, mc, mw, p, tp.ordered != 0, tp.num_jt, tp.jt_chunk);
     }
     return fail(c, FD_ERR_UNSUPPORTED, "no block product instantiation for column tile %d", BT);
 }

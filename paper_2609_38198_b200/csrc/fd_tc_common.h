@@ -30,8 +30,9 @@ struct TcParams {
     float* Y; int64_t ldy;       // block products: output block
     float* q; double* rowsq;     // row-sum modes: outputs
     const float* weights;        // row-sum modes without squares: right weights, padded with zeros to whole tiles
-    const int* perm;             // fp32-grade block product over the tile lists: row of Y and left for each row of the operand (null: the same)
-    int use_lists;               // fp32-grade block product: the tile lists of the context hold for this pass
+    const int* perm;             // row of Y, q and left for each row of the operand (null: the same)
+    int ordered;                 // the columns are in the points' order
+    int use_lists;               // block product: the tile lists of the context hold for this pass
     unsigned int* status;
 };
 

@@ -264,7 +264,7 @@ k_bp(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
         bool ok = true;
         for (int w = 0; w < my_items && ok; ++w) {
             FD_ITEM_P(w);
-            const int64_t row = (int64_t)item * 128 + row_in_tile;
+            int64_t row = (int64_t)item * 128 + row_in_tile;
             float acc[BT];
 #pragma unroll
             for (int c = 0; c < BT; ++c) acc[c] = 0.f;
@@ -292,6 +292,7 @@ k_bp(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
                 for (int c = 0; c < BT; ++c) acc[c] = fmaf(__uint_as_float(v[c / 16][c % 16]), corr, acc[c]);
             }
             if (ok && row < p.Nrow) {
+                if (p.perm) row = p.perm[row];
                 const float l = p.left ? p.left[row] : 1.0f;
 #pragma unroll
                 for (int c = 0; c < BT; ++c)
