@@ -550,6 +550,9 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
             std::swap(S.W, S.X);
             S.m = keep;
             ++S.restarts;
+            // the kept columns are the Ritz vectors themselves (the loop may end below without another Rayleigh-Ritz step)
+            Xr.assign((size_t)keep * nsel, 0.0);
+            for (int jj = 0; jj < std::min(nsel, keep); ++jj) Xr[jj + (size_t)jj * keep] = 1.0;
             FD_TRY(S.full_projection());
         }
         auto tp4 = clk::now();

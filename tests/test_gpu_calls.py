@@ -340,3 +340,42 @@ def test_entries_that_are_not_finite_reach_every_row(fd, dev, kind):
     torch.cuda.synchronize()
     assert torch.equal(last, want_good)
     ctx.close(); ref.close()
+
+
+# ------------------------------------------------------------------ eigensolver
+class _NothingNewAfterRestart:
+    """A one-rank transport that turns every projection after the first thick restart into zeros, as if the basis held everything: the
+    solver then finds no direction to add and leaves.  (kept = columns that a restart keeps: their projections are kept x kept.)"""
+    rank, world = 0, 1
+
+    def __init__(self, kept):
+        self.kept, self.seen = kept, 0
+
+    def allreduce_sum_host(self, arr, device, stream):
+        if self.seen >= 2:
+            arr[:] = 0.0
+        elif arr.size == self.kept * self.kept:
+            self.seen += 1
+
+    def allgather(self, send, recv, stream):
+        with torch.cuda.stream(stream):
+            recv.copy_(send)
+
+
+def test_vectors_of_a_solve_that_ends_right_after_a_restart(fd, dev):
+    """FD_ERR_NOT_CONVERGED returns the best Ritz pairs, also where the basis has just been compressed onto them."""
+    from oracle import dense
+    X = workloads.torus6(600, seed=2)
+    k, b, beta, cap = 4, 4, 0.5, 14
+    kept = k + 1 + b                                          # every Ritz vector of a step: more than 3/5 of the capacity
+    ctx = fd.Context(torch.from_numpy(X).to(dev), b_max=b, m_max=cap)
+    transport = _NothingNewAfterRestart(kept)
+    ctx.set_shard(fd.Shard(transport, X.shape[0], b, dev))
+    ctx.degree(beta, 1.0)
+    lam, U, info = ctx.eigs(k, b, tol=1e-9, max_applies=50, allow_not_converged=True)
+    assert transport.seen == 2 and info.restarts == 1 and info.basis_cols == kept and info.converged < k + 1
+    U = U.cpu().numpy().astype(np.float64)
+    assert np.abs(U.T @ U - np.eye(k + 1)).max() <= 1e-5
+    R = dense.apply(X, beta, 1.0, U) - U * lam[None, :]
+    assert np.linalg.norm(R, axis=0).max() <= info.max_residual + 5e-6 and info.max_residual < 0.3
+    ctx.close()
