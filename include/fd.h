@@ -155,7 +155,7 @@ typedef struct {
     int32_t converged;         /* leading pairs (of k + 1) with residual <= tol * theta_0     */
     int32_t basis_cols;        /* columns in the basis at exit                                */
     double  max_residual;      /* largest residual norm among the k + 1 returned pairs       */
-    double  seconds_apply;     /* host wall time spent inside the quadratic applies          */
+    double  seconds_apply;     /* time on the GPU of the quadratic applies (with row gathers) */
     double  seconds_total;
 } fd_eigs_info;
 

@@ -160,6 +160,8 @@ fd_status fd_destroy(fd_ctx* ctx) {
     if (ctx) {
         for (int i = 0; i < fd_ctx::kStageSlots; ++i)
             if (ctx->stage_ev[i]) cudaEventDestroy(ctx->stage_ev[i]);
+        for (int i = 0; i < 2; ++i)
+            if (ctx->apply_ev[i]) cudaEventDestroy(ctx->apply_ev[i]);
         if (ctx->stage) cudaFreeHost(ctx->stage);
     }
     delete ctx;

@@ -99,6 +99,7 @@ struct fd_ctx {
     float* stage = nullptr;
     double* h_out = nullptr;
     cudaEvent_t stage_ev[kStageSlots] = {nullptr, nullptr, nullptr, nullptr};
+    cudaEvent_t apply_ev[2] = {nullptr, nullptr};        // around the latest products of a solve
     size_t stage_floats = 0;         // per slot
     size_t h_out_doubles = 0;
     // row-sharded operation (fd_set_shard): this rank owns rows [r0, r1) of every quadratic pass

@@ -379,3 +379,23 @@ def test_vectors_of_a_solve_that_ends_right_after_a_restart(fd, dev):
     R = dense.apply(X, beta, 1.0, U) - U * lam[None, :]
     assert np.linalg.norm(R, axis=0).max() <= info.max_residual + 5e-6 and info.max_residual < 0.3
     ctx.close()
+
+
+def test_reported_time_in_applies_is_the_products_time(fd, dev):
+    """info.seconds_apply against the same number of products timed on their own (events; half to twice: clocks and neighbours differ)."""
+    N, k, b, beta = 50021, 12, 32, 2.0
+    ctx = fd.Context(torch.from_numpy(workloads.torus6(N, seed=3)).to(dev), b_max=b, m_max=3 * (k + 1) + 2 * b)
+    ctx.degree(beta, 1.0)
+    lam, U, info = ctx.eigs(k, b)
+    V = fd.to_colmajor(workloads.block(N, b, seed=1), dev)
+    ctx.apply(V)
+    t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    t0.record()
+    for _ in range(info.applies):
+        ctx.apply(V)
+    t1.record()
+    torch.cuda.synchronize()
+    seconds = 1e-3 * t0.elapsed_time(t1)
+    assert 0.5 * seconds <= info.seconds_apply <= 2.0 * seconds, (info.seconds_apply, seconds)
+    assert info.seconds_apply <= info.seconds_total
+    ctx.close()
