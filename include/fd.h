@@ -167,7 +167,12 @@ typedef struct {
  * column-major, orthonormal.  Needs m_max >= 2 (k + 1) + b at fd_create; the thick restart keeps 3/5 of m_max, so a
  * capacity near 3 (k + 1) + 2 b keeps room for the rest of an eigenvalue cluster that the request cuts (on the
  * 6-torus, k = 128 cuts a 160-fold cluster: 129 of 129 pairs converge in 43 block products with m_max = 576, 73 of
- * 129 in 125 with 384).  info->converged counts the LEADING pairs below tol.  On FD_ERR_NOT_CONVERGED the outputs hold
+ * 129 in 125 with 384).  Below 3 (k + 1) every block is a residual block, with a projected eigenproblem after each product, and a
+ * solve that stalls just above tol is reported as it is; from there on M is applied to the basis again first.
+ * info->converged counts the LEADING pairs below tol.  Residuals (tol, max_residual) are formed from the basis's stored images
+ * M Q, which carry the rounding of fp32 products and restarts: with M applied afresh to the returned vectors they are up to
+ * 1e-6 theta_0 larger, against a float64 operator up to 3e-6 (6-torus, 2-torus and latent torus, N = 2^14 .. 2^18), so a tol
+ * below that is a tolerance on the iteration, not on the error.  On FD_ERR_NOT_CONVERGED the outputs hold
  * the best current Ritz pairs.  Synchronous. */
 fd_status fd_eigs(fd_ctx* ctx, int32_t k, int32_t b, double tol, int32_t max_applies,
                   const float* Q0_dev, int64_t ldq0, int32_t q0_cols,

@@ -399,3 +399,33 @@ def test_reported_time_in_applies_is_the_products_time(fd, dev):
     assert 0.5 * seconds <= info.seconds_apply <= 2.0 * seconds, (info.seconds_apply, seconds)
     assert info.seconds_apply <= info.seconds_total
     ctx.close()
+
+
+@pytest.mark.parametrize("data,N,seed,beta,k,b,cap", [
+    ("torus6", 40000, 42, 2.0, 64, 32, 192), ("torus6", 40000, 42, 2.0, 64, 32, 195), ("torus6", 30000, 7, 2.0, 64, 32, 259),
+    ("torus2", 16384, 42, 100.0, 32, 16, 98), ("torus2", 16384, 42, 100.0, 32, 16, 99), ("torus2", 16384, 42, 300.0, 32, 16, 131),
+    ("latent", 65536, 42, 2.0, 32, 32, 98), ("latent", 65536, 42, 2.0, 32, 32, 163)])
+def test_solves_at_the_accuracy_floor_on_both_sides_of_the_capacity_rule(fd, dev, data, N, seed, beta, k, b, cap):
+    """Spectra whose residuals end near tol = 1e-6.  From a capacity of 3 (k + 1) on a solve that stalls above tol applies M to its basis again
+    and converges.  On both sides the returned pairs' float64 residuals exceed the reported ones, which are measured with stored fp32
+    images, by at most 3e-6: 1e-6 for the images' rounding, 2e-6 for the operator's own error.  (All rows: the far-out points of the
+    latent torus carry most of that error, so a sample of rows would not do.)"""
+    X = {"torus6": workloads.torus6, "torus2": workloads.torus2, "latent": workloads.latent_torus}[data](N, seed=seed)
+    Xt = torch.from_numpy(X).to(dev)
+    Xd = Xt.double()
+    ctx = fd.Context(Xt, b_max=b, m_max=cap)
+    s = ctx.degree(beta, 1.0)[2].double()
+    lam, U, info = ctx.eigs(k, b, max_applies=600, allow_not_converged=True)
+    lt, Ud = torch.tensor(lam, device=dev), U.double()
+    sq = torch.zeros(k + 1, dtype=torch.float64, device=dev)
+    for r in torch.arange(N, device=dev).split(1024):
+        K = torch.exp(-beta * torch.cdist(Xd[r], Xd, compute_mode="donot_use_mm_for_euclid_dist") ** 2)
+        sq += ((s[r, None] * (K @ (s[:, None] * Ud)) - Ud[r] * lt) ** 2).sum(0)
+    est = sq.sqrt().max().item()
+    print(f"{data} cap {cap}: {info.converged}/{k + 1} after {info.applies} products, reported {info.max_residual:.2e}, float64 {est:.2e}")
+    assert est <= info.max_residual + 3e-6
+    if cap >= 3 * (k + 1):
+        assert info.converged == k + 1
+    else:
+        assert info.converged == k + 1 or 1e-6 < info.max_residual <= 2.5e-6
+    ctx.close()
