@@ -57,7 +57,8 @@ Layout make_layout(int64_t N, int32_t D, int32_t b_max, int32_t m_max) {
     // shares of row tiles that a work range's cut falls into: two slots of 256 rows x the widest column tile per CTA (direct-difference
     // kernels: up to four CTAs on each of 148 SMs, tensor-core product: one, and a slot for its sums; never more CTAs than steps)
     const int64_t steps = ceil_div(N, 256) * ceil_div(N, 16);
-    L.part_floats = (size_t)std::max<int64_t>(std::min<int64_t>(592, steps), 240) * 2 * 256 * (size_t)L.BP;
+    // (no launch has more than 64 columns, however wide the blocks are)
+    L.part_floats = (size_t)std::max<int64_t>(std::min<int64_t>(592, steps), 240) * 2 * 256 * (size_t)std::min(L.BP, 64);
     L.part = carve(cur, L.part_floats * 4);
     // tensor-core operands: fp16 hi|lo rows of the augmented points, transposed fp16 hi / lo blocks
     L.xp_col = carve(cur, (size_t)L.NP * L.K16 * 64);

@@ -56,3 +56,11 @@ def test_argument_errors_before_any_launch(fd):
     assert b"workspace" in fd.lib.fd_status_string(2)
     assert fd.fd_version() >= 100
     assert fd.fd_launch_count() == 0           # nothing ran on this CPU-only path
+
+
+def test_workspace_shares_do_not_grow_with_wide_blocks(fd):
+    """A launch has at most 64 columns, so the slots for the shares of cut row tiles stop growing there: beyond b_max = 64 the workspace grows by
+    the three N x b block buffers (fp32 scratch, two fp16 operands) and a few words per column."""
+    for N, D in ((2048, 2), (100000, 12)):
+        per_column = 4 * N + 2 * 2 * ((N + 255) // 256 * 256) + 16
+        assert fd.fd_workspace_bytes(N, D, 256, 0) - fd.fd_workspace_bytes(N, D, 64, 0) <= 192 * per_column + 4096
