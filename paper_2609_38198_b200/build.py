@@ -13,7 +13,7 @@ LIB = os.path.join(HERE, "libfd.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-    "-Xcompiler", "-fPIC,-O3,-mavx2,-mfma,-Wall,-Wno-unused-function,-fopenmp", "--expt-relaxed-constexpr",
+    "-Xcompiler", "-fPIC,-O3,-Wall,-Wno-unused-function,-fopenmp", "--expt-relaxed-constexpr",
 ]
 
 

@@ -26,6 +26,10 @@ fd_status random_fill(fd_ctx* c, float* A, int64_t lda, int p, int64_t N, int64_
 fd_status sqrt_vec(fd_ctx* c, const float* d, float* out, int64_t N);
 fd_status copy_cols(fd_ctx* c, const float* src, int64_t lds, float* dst, int64_t ldd, int p, int64_t N);
 
+// y += a x, and x . y, on the host (fd_symeig.cpp: with the widest vectors the machine has).
+void host_axpy(double* y, const double* x, double a, int n);
+double host_dot(const double* x, const double* y, int n);
+
 // Eigen-decomposition of a dense symmetric n x n matrix (column-major, only read).  On return evals ascending (all n) and
 // evecs n x n column-major with orthonormal columns; with 0 <= nvec < n only the columns of the nvec LARGEST eigenvalues
 // (columns n - nvec .. n - 1) are computed, the others are zero.  Householder tridiagonalisation followed by implicit

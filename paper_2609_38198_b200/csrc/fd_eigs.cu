@@ -273,8 +273,7 @@ struct Solver {
             for (int l = 0; l < p; ++l) {
                 const double fl = f[l];
                 if (fl == 0.0) continue;
-                const double* zl = z + (size_t)l * ldz;
-                for (int i = 0; i < m; ++i) col[i] -= zl[i] * fl;
+                host_axpy(col.data(), z + (size_t)l * ldz, -fl, m);
             }
             for (int i = 0; i < m; ++i) S[i + (size_t)j * (m + p)] = (float)col[i];
             for (int l = 0; l < p; ++l) S[m + l + (size_t)j * (m + p)] = (float)f[l];
@@ -439,7 +438,7 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
                 const double t = S.T[l + (size_t)j * m_cap];
                 const double* Ecol = &S.G[(size_t)l * m_cap];
                 double* o = &ET[(size_t)j * m];
-                for (int i = 0; i < m; ++i) o[i] += Ecol[i] * t;          // G column l ...
+                host_axpy(o, Ecol, t, m);                                 // G column l ...
                 o[l] -= t;                                                 // ... minus the identity
             }
         for (int j = 0; j < m; ++j)

@@ -64,3 +64,13 @@ def test_workspace_shares_do_not_grow_with_wide_blocks(fd):
     for N, D in ((2048, 2), (100000, 12)):
         per_column = 4 * N + 2 * 2 * ((N + 255) // 256 * 256) + 16
         assert fd.fd_workspace_bytes(N, D, 256, 0) - fd.fd_workspace_bytes(N, D, 64, 0) <= 192 * per_column + 4096
+
+
+def test_host_code_is_built_for_every_host():
+    """No instruction-set option of one processor family in the build: the long host loops choose at load time (fd_symeig.cpp)."""
+    import importlib.util
+    spec = importlib.util.spec_from_file_location("_build", os.path.join(ROOT, "paper_2609_38198_b200", "build.py"))
+    build = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(build)
+    options = ",".join(build.NVCC_FLAGS).split(",")
+    assert not [o for o in options if o.startswith("-m")], options
