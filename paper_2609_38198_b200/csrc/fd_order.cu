@@ -26,6 +26,7 @@
 // product; degree passes 23.2 -> 19.9 ms.  Direct differences, exactly zero values only: fd_direct.cu.
 #include <algorithm>
 #include <cmath>
+#include <new>
 
 #include "fd_dense.h"
 
@@ -436,13 +437,18 @@ fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide) {
             double* cov = part + (size_t)(kSamples / 128) * n2;
             k_cov_sum<<<(unsigned)ceil_div(n2, 256), 256, 0, c->stream>>>(part, kSamples / 128, n2, cov);
             FD_LAUNCH_CHECK(c, "k_cov_sum");
-            std::vector<double> C((size_t)n2), lam, U;
-            FD_CUDA(c, cudaMemcpyAsync(C.data(), cov, sizeof(double) * (size_t)n2, cudaMemcpyDeviceToHost, c->stream));
+            double C[64 * 64];
+            FD_CUDA(c, cudaMemcpyAsync(C, cov, sizeof(double) * (size_t)n2, cudaMemcpyDeviceToHost, c->stream));
             FD_CUDA(c, cudaStreamSynchronize(c->stream));
-            if (!sym_eig(C.data(), L.DP, lam, U)) { c->order_state = -1; return FD_OK; }
             Directions dir{};
-            for (int d = 0; d < 8; ++d)
-                for (int k = 0; k < L.DP; ++k) dir.v[d][k] = (float)U[k + (size_t)(L.DP - 1 - d) * L.DP];
+            bool solved = false;
+            try {
+                std::vector<double> lam, U;
+                solved = sym_eig(C, L.DP, lam, U);
+                for (int d = 0; d < 8 && solved; ++d)
+                    for (int k = 0; k < L.DP; ++k) dir.v[d][k] = (float)U[k + (size_t)(L.DP - 1 - d) * L.DP];
+            } catch (const std::bad_alloc&) {}                     // (nothing may be thrown through the C interface)
+            if (!solved) { c->order_state = -1; return FD_OK; }
             k_project<<<(unsigned)ceil_div(N, 256), 256, 0, c->stream>>>(c->xs(), L.DP, N, mu, dir, c->at<float>(L.zproj));
             FD_LAUNCH_CHECK(c, "k_project");
         }
