@@ -30,7 +30,6 @@ struct Layout {
     size_t wp = 0;                   // N x BP block of scratch (numerators and denominator of the out-of-sample extension)
     size_t part = 0, part_floats = 0;
     size_t xp_col = 0, xp_row = 0, wt_hi = 0, wt_lo = 0, colscale = 0, status = 0;
-    size_t yacc = 0;
     // order of the points and tile lists of the Gram-form kernels (fd_order.cu); 0: not provisioned for this N
     size_t perm = 0, boxes = 0, zproj = 0, lists = 0, list_counts = 0;
     bool direct_lists = false;       // provisioned for the direct-difference kernels as well
@@ -206,7 +205,6 @@ fd_status tc_wait_selftest(fd_ctx* c, long long limit_cycles);
 fd_status ew_pow(fd_ctx* c, const float* in, double p, float* out, int64_t n);            // out = in^p
 // s = qa * d^-1/2 (qa null: 1); also copies q, d, s to the outputs that are not null.
 fd_status ew_scale_vec(fd_ctx* c, const float* qa, const float* q, const float* d, float* s, int64_t n, float* q_out, float* d_out, float* s_out);
-fd_status ew_fill(fd_ctx* c, float* out, float v, int64_t n);
 // Deterministic fp64 sums of a float vector and a double vector (two-stage tree) -> out_dev[0], out_dev[1].
 fd_status reduce_sums(fd_ctx* c, const float* q, const double* rowsq, int64_t n, double* out_dev);
 fd_status scale_cols_by_pow(fd_ctx* c, const float* v, int64_t ldv, int32_t cols, const float* d, double p,

@@ -161,11 +161,6 @@ __global__ void k_scale_vec(const float* __restrict__ qa, const float* __restric
     if (s_out) s_out[i] = v;
 }
 
-__global__ void k_fill(float* __restrict__ out, float v, int64_t n) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = v;
-}
-
 // Stage 1: block partial sums (fixed assignment of elements to threads -> deterministic).
 __global__ void k_sum_partial(const float* __restrict__ q, const double* __restrict__ rowsq, int64_t n,
                               double* __restrict__ part) {
@@ -324,12 +319,6 @@ fd_status ew_pow(fd_ctx* c, const float* in, double p, float* out, int64_t n) {
 fd_status ew_scale_vec(fd_ctx* c, const float* qa, const float* q, const float* d, float* s, int64_t n, float* q_out, float* d_out, float* s_out) {
     k_scale_vec<<<grid_for(n, 256), 256, 0, c->stream>>>(qa, q, d, s, n, q_out, d_out, s_out);
     FD_LAUNCH_CHECK(c, "k_scale_vec");
-    return FD_OK;
-}
-
-fd_status ew_fill(fd_ctx* c, float* out, float v, int64_t n) {
-    k_fill<<<grid_for(n, 256), 256, 0, c->stream>>>(out, v, n);
-    FD_LAUNCH_CHECK(c, "k_fill");
     return FD_OK;
 }
 
