@@ -88,7 +88,7 @@ size_t fd_workspace_bytes(int64_t N, int32_t D, int32_t b_max, int32_t m_max);
 /* Creates a context over N points.  Copies X into the library's padded layouts inside the
  * workspace (so X_dev may be released after the call), computes the column means and, if
  * center != 0, the centred copy used by the Gram-form kernels (Eq. 4) and by fd_beta0.
- * ws_dev must be 256-byte aligned and stay valid until fd_destroy.  Synchronises once. */
+ * ws_dev must be 256-byte aligned and stay valid until fd_destroy.  Synchronises. */
 fd_status fd_create(fd_ctx** out, const float* X_dev, int64_t N, int32_t D, int64_t ldx,
                     int32_t center, int32_t b_max, int32_t m_max,
                     void* ws_dev, size_t ws_bytes, void* cuda_stream);

@@ -11,7 +11,8 @@
 // results are bit-reproducible run to run.  (Letting the CTA that comes last add them needs no second launch but puts one
 // CTA's chain of dependent reads at the end: 183 us instead of 8 at N = 2048.)
 //
-// What bounds it: instruction issue, 2 D + b + 2 FMA-pipe operations per pair.  A thread owns two or four rows (four: the two halves of the
+// What bounds it: instruction issue and the latency between dependent instructions, 2 D + b + 2 FMA-pipe operations per pair (N = 16384, listed:
+// two of three issue slots taken, FMA pipe 54 %, 1.6 eligible warps a scheduler).  A thread owns two or four rows (four: the two halves of the
 // CTA take half the columns of a tile each), which share the broadcast reads of x_j and w_j from shared memory; with one row per
 // thread these cost as many slots as a fifth of the FMAs.  (Two rows per packed instruction, add / fma.rn.f32x2, halve
 // the instruction count but ran at half the FMA rate: 5 to 15 % slower in every shape.)  Right-hand columns are read from V

@@ -19,7 +19,8 @@
 //                shared memory, so that a pair of tiles costs one atomic per streamed point.
 // Work is a flat sequence of (resident pair, streamed tile) steps, cut into equal ranges, one per CTA.
 //
-// What bounds it: the MUFU (1024 SM clocks per tile) with the additions beside it.  Both degree passes at N = 2^18 (one with squares, one
+// What bounds it: the MUFU (1024 SM clocks per tile; 76 % busy at N = 65536) and the queue that feeds it, with the additions beside it (issue
+// slots 60 to 63 %).  Both degree passes at N = 2^18 (one with squares, one
 // with weights): 26.2 -> 21.6 ms against two warpgroups with 128 accumulators a thread, whole row pairs per CTA and an atomic per
 // point and tile.
 #include <algorithm>
