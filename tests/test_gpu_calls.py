@@ -429,3 +429,10 @@ def test_solves_at_the_accuracy_floor_on_both_sides_of_the_capacity_rule(fd, dev
     else:
         assert info.converged == k + 1 or 1e-6 < info.max_residual <= 2.5e-6
     ctx.close()
+
+
+def test_c3_full_size_certificate_at_the_benchmark_capacity(fd, dev):
+    """The 6-torus at N = 2^17 with the capacity the benchmark gives its solve (3 (k + 1) + 2 b, rounded up): Krylov blocks between
+    Rayleigh-Ritz steps, which the smaller capacity of the other full-size certificate does not take."""
+    from test_gpu_tc import full_size_certificate
+    full_size_certificate(fd, dev, workloads.torus6(131072, seed=42), 2.0, 64, 32, 288, min_converged=65, sample=128)
