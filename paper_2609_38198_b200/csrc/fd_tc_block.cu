@@ -5,8 +5,10 @@
 //   1. Gram MMA of augmented fp16 hi|lo points: the tile leaves the tensor core as the base-2 exponent
 //        S_ij = 2 b' x_i.x_j - b' r_i - b' r_j + bias      (Eq. 4; the norms ride as extra K columns)
 //      into one of three 128-column TMEM buffers.
-//   2. Exponential warps (thread = row, 64 columns each) read S, take P = 2^S on the MUFU, split it into fp16 hi + lo and write
-//      both halves back IN PLACE as the TMEM A operand of the product.
+//   2. Exponential warps (thread = row, 64 columns each) read S, take P = 2^S on the MUFU, split it into fp16 hi (rounded to nearest) and
+//      the rest and write both back IN PLACE as the TMEM A operand of the product.  Two values take six instructions: two exponentials, one
+//      conversion to a pair of fp16, two mixed-precision subtractions hi - P, one conversion of these; the product MMAs of the
+//      second piece negate their A operand.
 //   3. Product MMAs per 16-column K step: Y += P_hi W_hi + P_lo W_hi + P_hi W_lo with W = diag(right) V split the same way.
 //   4. Every `flush` column tiles a separate warpgroup per row tile adds Y into fp32 registers and the accumulator restarts,
 //      so tensor-core accumulation error does not grow with N.
@@ -18,8 +20,11 @@
 //   warp 24      TMA producer; warp 25 / 26 product-MMA issuer / Gram-MMA issuer (one elected thread each).
 // TMEM (512 columns): three S/P buffers at [0, 384), one accumulator of 64 columns per row tile at 384 + 64 t.
 //
-// What bounds it: at N >= 2^17 the board's power limit (1000 W; 1390 SM clocks per tile, at about 1480 MHz), below that the overlap of the
-// pipes: at N = 65536, b = 64 the MUFU is busy 74 % of the time and the tensor pipe 70 to 78 %, issue slots 65 %.  Sixteen exponential warps and a product issued per 32-column quarter keep the chain exponentials -> product ->
+// What bounds it: at N >= 2^17 the board's power limit (1000 W), below that the chain of steps that a buffer goes through: 1260 SM clocks a tile at
+// N = 50021, b = 20, where the MUFU needs 1024.  Without the exponentials (a probe) the chain still takes 1105, without the product MMAs
+// 1210, without two of the three Gram MMAs 1245; exponentials moved to the FMA pipe (a polynomial for one or two columns in sixteen) cost 4 to 10 %.
+// Instructions count twice, as issue slots in the chain and as power: hi cut from the bits and subtracted (eight instructions for two values) and
+// scalar flushes took 798 instead of 749 us there, 5.45 instead of 5.19 ms at N = 2^17, b = 32, 26.7 instead of 25.6 ms at N = 2^18, b = 64.  Sixteen exponential warps and a product issued per 32-column quarter keep the chain exponentials -> product ->
 // Gram -> exponentials of a buffer shorter than the other row tile's exponentials.  Per tile: 1024 SM clocks of MUFU, 193 K16 clocks of Gram MMAs, 12 BT clocks of product MMAs.  Up to 32 columns
 // the W_lo product shares an instruction with the W_hi one (B operand [W_hi | W_lo], N = 2 BT) and P_lo W_hi is added to
 // the W_lo half of the accumulator: 16 MMAs a tile instead of 24, and the sum of the large terms sees 8 round-toward-zero additions
@@ -255,7 +260,7 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
       } else if (warp == 25) {
         // =============================================================== product MMA issuer (one thread)
         if (elect_one()) {
-            constexpr uint32_t idesc_hi = idesc_f16(kConcat ? 2 * BT : BT), idesc_lo = idesc_f16(BT);
+            constexpr uint32_t idesc_hi = idesc_f16(kConcat ? 2 * BT : BT), idesc_lo = idesc_f16(BT), idesc_res = idesc_lo | kNegateA;
             // W stage descriptor as (low, high) words: 128 B rows (SWIZZLE_128B), 1024 B between 8-row groups
             const uint64_t wd = smem_desc(smem_u32(stage_base + K16 * SM::kXChunk), 1024, 2);
             const uint32_t wbase_lo = (uint32_t)wd, wdesc_hi = (uint32_t)(wd >> 32);
@@ -293,11 +298,11 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
                                 if constexpr (kConcat) {
                                     if (k == 0 && i == 0 && group_start) mma_ts2<0>(y_addr, aq, bq, wdesc_hi, idesc_hi);
                                     else mma_ts2<1>(y_addr, aq + 16 * k, bq + 2 * k, wdesc_hi, idesc_hi);
-                                    mma_ts2<1>(y_addr + BT, aq + 16 * k + 8, bq + 2 * k, wdesc_hi, idesc_lo);
+                                    mma_ts2<1>(y_addr + BT, aq + 16 * k + 8, bq + 2 * k, wdesc_hi, idesc_res);
                                 } else {
                                     // the two small terms of both K steps first: what they round away is smaller then
-                                    if (k == 0 && i == 0 && group_start) mma_ts2<0>(y_addr, aq + 8, bq, wdesc_hi, idesc_lo);
-                                    else mma_ts2<1>(y_addr, aq + 16 * k + 8, bq + 2 * k, wdesc_hi, idesc_lo);
+                                    if (k == 0 && i == 0 && group_start) mma_ts2<0>(y_addr, aq + 8, bq, wdesc_hi, idesc_res);
+                                    else mma_ts2<1>(y_addr, aq + 16 * k + 8, bq + 2 * k, wdesc_hi, idesc_res);
                                     mma_ts2<1>(y_addr, aq + 16 * k, bq + (uint32_t)(SM::kWPart >> 4) + 2 * k, wdesc_hi, idesc_lo);
                                 }
                             }
@@ -330,9 +335,9 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
         bool ok = true;
         Steps<ORD> steps(p);
         for (Item it; ok && steps.next(p, it);) {
-            float acc[BT];
+            uint64_t acc2[BT / 2];
 #pragma unroll
-            for (int c = 0; c < BT; ++c) acc[c] = 0.f;
+            for (int c = 0; c < BT / 2; ++c) acc2[c] = 0;
             // The tensor core adds each K step into the TMEM accumulator with round-toward-zero.  For a sum whose partial sums
             // keep one sign, n additions lose n / 4 ulp of the result on average (half an ulp each, at a running magnitude that
             // averages half the final one): 2^-25 of the result per addition.  The flush adds that expected loss back.  (With
@@ -350,14 +355,17 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
                         float* sums = p.part + (size_t)(2 * gridDim.x + blockIdx.x) * BT * 256 + row_in_pair;
 #pragma unroll
                         for (int c = 0; c < BT; ++c) {
-                            sums[c * 256] = done == period ? acc[c] : sums[c * 256] + acc[c];
-                            acc[c] = 0.f;
+                            const float2 a = split2(acc2[c / 2]);
+                            const float v = c & 1 ? a.y : a.x;
+                            sums[c * 256] = done == period ? v : sums[c * 256] + v;
+                            if (c & 1) acc2[c / 2] = 0;
                         }
                     }
                 }
                 const int tiles_in_group = left_tiles < p.flush ? left_tiles : p.flush;
                 left_tiles -= tiles_in_group;
-                const float corr = 1.0f + (float)(tiles_in_group * (kConcat ? 8 : 24)) * 2.98023224e-8f;
+                const float corr1 = 1.0f + (float)(tiles_in_group * (kConcat ? 8 : 24)) * 2.98023224e-8f;
+                const uint64_t corr = pair2(corr1, corr1);
                 ok = mbar_wait(&bars->y_full[t], yph, abort_flag, p.status, 10);
                 if (!ok) break;
                 yph ^= 1u;
@@ -375,13 +383,18 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
                         if (lane == 0) mbar_arrive(&bars->y_empty[t]);
                     }
 #pragma unroll
-                    for (int c = 0; c < kStep; ++c) {
-                        if constexpr (kConcat) acc[c0 + c] += fmaf(__uint_as_float(hi[c]), corr, __uint_as_float(lo[c]));
-                        else acc[c0 + c] = fmaf(__uint_as_float(hi[c]), corr, acc[c0 + c]);
+                    for (int c = 0; c < kStep; c += 2) {
+                        const uint64_t h2 = pair2(__uint_as_float(hi[c]), __uint_as_float(hi[c + 1]));
+                        uint64_t& a2 = acc2[(c0 + c) / 2];
+                        if constexpr (kConcat) a2 = add2(a2, fma2(h2, corr, pair2(__uint_as_float(lo[c]), __uint_as_float(lo[c + 1]))));
+                        else a2 = fma2(h2, corr, a2);
                     }
                 }
             }
             if (!ok) break;
+            float acc[BT];
+#pragma unroll
+            for (int c = 0; c < BT; c += 2) { const float2 a = split2(acc2[c / 2]); acc[c] = a.x; acc[c + 1] = a.y; }
             if constexpr (ORD)
                 if (it.n > period) {
                     const float* sums = p.part + (size_t)(2 * gridDim.x + blockIdx.x) * BT * 256 + row_in_pair;
@@ -439,10 +452,8 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
                         for (int i = 0; i < 8; ++i) {
                             const float p0 = ex2f(__uint_as_float(sv[16 * ch + 2 * i]));
                             const float p1 = ex2f(__uint_as_float(sv[16 * ch + 2 * i + 1]));
-                            const float h0 = __uint_as_float(__float_as_uint(p0) & 0xFFFFE000u);
-                            const float h1 = __uint_as_float(__float_as_uint(p1) & 0xFFFFE000u);
-                            hi[i] = pack_f16x2(h0, h1);
-                            lo[i] = pack_f16x2(p0 - h0, p1 - h1);
+                            hi[i] = pack_f16x2(p0, p1);
+                            lo[i] = pack_f16x2(sub_lo_f16(hi[i], p0), sub_hi_f16(hi[i], p1));
                         }
                         tmem_st8(addr + 32 * q32 + 16 * ch, hi);
                         tmem_st8(addr + 32 * q32 + 16 * ch + 8, lo);

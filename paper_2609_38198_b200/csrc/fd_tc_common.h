@@ -182,6 +182,17 @@ __device__ __forceinline__ uint32_t pack_f16x2(float lo, float hi) {
     return r;
 }
 
+// h - x for the low / high half h of a packed pair of fp16 values and an fp32 x: one instruction (the conversion of h alone takes two and a half).
+__device__ __forceinline__ float sub_lo_f16(uint32_t h, float x) {
+    float d;
+    asm("{\n\t.reg .b16 l, u;\n\tmov.b32 {l, u}, %1;\n\tsub.f32.f16 %0, l, %2;\n\t}" : "=f"(d) : "r"(h), "f"(x));
+    return d;
+}
+__device__ __forceinline__ float sub_hi_f16(uint32_t h, float x) {
+    float d;
+    asm("{\n\t.reg .b16 l, u;\n\tmov.b32 {l, u}, %1;\n\tsub.f32.f16 %0, u, %2;\n\t}" : "=f"(d) : "r"(h), "f"(x));
+    return d;
+}
 // K-major shared-memory operand descriptor (sm_100 format): start address, stride between 8-row groups,
 // swizzle mode (2 = 128 B rows, 4 = 64 B rows).
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t sbo_bytes, uint32_t layout) {
@@ -196,6 +207,7 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t sbo_bytes,
 __host__ __device__ constexpr uint32_t idesc_f16(int n) {
     return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
+constexpr uint32_t kNegateA = 1u << 13;      // instruction descriptor: D (+)= -A B
 
 // Reduced-precision block product (fd_tc_fast.cu): one row tile per CTA, work items of 128 rows.
 fd_status launch_fast_product(fd_ctx* c, int BT, const CUtensorMap& mr, const CUtensorMap& mc, const CUtensorMap& mh,
