@@ -20,8 +20,10 @@
 // Work is a flat sequence of (resident pair, streamed tile) steps, cut into equal ranges, one per CTA.
 //
 // What bounds it: the MUFU (1024 SM clocks per tile; 76 % busy at N = 65536) and the queue that feeds it, with the additions beside it (issue
-// slots 60 to 63 %).  Both degree passes at N = 2^18 (one with squares, one
-// with weights): 26.2 -> 21.6 ms against two warpgroups with 128 accumulators a thread, whole row pairs per CTA and an atomic per
+// slots 60 to 63 % with scalar additions).  The additions work on two columns an instruction (add / fma.rn.f32x2): half their issue slots, the same
+// bits.  N = 65536: 1440 -> 1376 us both passes, N = 2^18: 21.55 -> 20.4 ms.  (Loads of 8 columns one step ahead: 1.5 % slower; a polynomial
+// on the FMA pipe for two of sixteen columns: 4 % slower.)  Both degree passes at N = 2^18 (one with squares, one
+// with weights), scalar: 26.2 -> 21.6 ms against two warpgroups with 128 accumulators a thread, whole row pairs per CTA and an atomic per
 // point and tile.
 #include <algorithm>
 #include <cmath>
@@ -269,23 +271,24 @@ k_sym(const __grid_constant__ CUtensorMap map_res, const __grid_constant__ CUten
         uint32_t k = 0;
         double dsq = 0.0;
         bool ok = true;
-        float acc[64];
+        uint64_t acc2[32];                                         // two columns each
         Steps<LISTED> steps(p);
         for (Item<LISTED> it; ok && steps.next(p, it);) {
             const int It = 2 * it.pair + t;
-            const float4* wres = WEIGHTED ? reinterpret_cast<const float4*>(p.weights + (int64_t)It * 128 + 64 * h) : nullptr;
+            const ulonglong2* wres = WEIGHTED ? reinterpret_cast<const ulonglong2*>(p.weights + (int64_t)It * 128 + 64 * h) : nullptr;
 #pragma unroll
-            for (int c = 0; c < 64; ++c) acc[c] = 0.f;
+            for (int c = 0; c < 32; ++c) acc2[c] = 0;
             int pending = 0;                                       // tiles accumulated in acc since the last reduction
             for (int j = 0; j < it.n; ++j, ++k) {
                 const int J = it.tile(p, j);
                 const float wj = WEIGHTED ? __ldg(p.weights + (int64_t)J * 128 + pt_in_tile) : 1.f;
+                const uint64_t wj2 = pair2(wj, wj);
                 const uint32_t buf = (2 * k + (uint32_t)t) & 3;
                 ok = mbar_wait(&bars->s_full[buf], (k >> 1) & 1, abort_flag, p.status, 8);
                 if (!ok) break;
                 tc_fence_after();
                 const bool use = J >= It;
-                float r0 = 0.f, r1 = 0.f, q0 = 0.f, q1 = 0.f;
+                uint64_t r2 = 0, q2 = 0;
                 if (use) {
 #pragma unroll
                     for (int ch = 0; ch < 4; ++ch) {
@@ -294,20 +297,15 @@ k_sym(const __grid_constant__ CUtensorMap map_res, const __grid_constant__ CUten
                         tmem_wait_ld();
 #pragma unroll
                         for (int i = 0; i < 16; i += 4) {
-                            float4 w4;
+                            ulonglong2 w4;
                             if (WEIGHTED) w4 = __ldg(wres + 4 * ch + i / 4);
 #pragma unroll
                             for (int u = 0; u < 4; u += 2) {
-                                const int c = 16 * ch + i + u;
-                                const float p0 = ex2f(__uint_as_float(sv[i + u])), p1 = ex2f(__uint_as_float(sv[i + u + 1]));
-                                if (WEIGHTED) {
-                                    acc[c] = fmaf(p0, wj, acc[c]); acc[c + 1] = fmaf(p1, wj, acc[c + 1]);
-                                    r0 = fmaf(p0, u ? w4.z : w4.x, r0); r1 = fmaf(p1, u ? w4.w : w4.y, r1);
-                                } else {
-                                    acc[c] += p0; acc[c + 1] += p1;
-                                    r0 += p0; r1 += p1;
-                                }
-                                if (SQ) { q0 = fmaf(p0, p0, q0); q1 = fmaf(p1, p1, q1); }
+                                uint64_t& a = acc2[(16 * ch + i + u) / 2];
+                                const uint64_t p2 = pair2(ex2f(__uint_as_float(sv[i + u])), ex2f(__uint_as_float(sv[i + u + 1])));
+                                if (WEIGHTED) { a = fma2(p2, wj2, a); r2 = fma2(p2, u ? w4.y : w4.x, r2); }
+                                else { a = add2(a, p2); r2 = add2(r2, p2); }
+                                if (SQ) q2 = fma2(p2, p2, q2);
                             }
                         }
                     }
@@ -320,14 +318,23 @@ k_sym(const __grid_constant__ CUtensorMap map_res, const __grid_constant__ CUten
                 const uint32_t slot = k % kSlots;
                 ok = mbar_wait(&bars->r_free[slot], ((k / kSlots) & 1) ^ 1, abort_flag, p.status, 13);
                 if (!ok) break;
-                rbuf[slot * 512 + wg * 128 + pt_in_tile] = both ? r0 + r1 : 0.f;
+                const float2 rp = split2(r2);
+                const float r = rp.x + rp.y;
+                rbuf[slot * 512 + wg * 128 + pt_in_tile] = both ? r : 0.f;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&bars->r_ready[slot]);
-                if (SQ && use) dsq += (double)(q0 + q1) * (both ? 2.0 : 1.0);
+                if (SQ && use) {
+                    const float2 qp = split2(q2);
+                    const float q = qp.x + qp.y;
+                    dsq += (double)q * (both ? 2.0 : 1.0);
+                }
                 if (use) ++pending;
                 if (pending == kSymFlush || (j + 1 == it.n && pending > 0)) {
                     // sums of acc over the 32 lanes: lane l ends up with columns l and 32 + l
                     const double fix = (double)(1ull << p.shift);
+                    float acc[64];
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) { const float2 a = split2(acc2[c]); acc[2 * c] = a.x; acc[2 * c + 1] = a.y; }
 #pragma unroll
                     for (int ch = 0; ch < 2; ++ch) {
 #pragma unroll
@@ -344,7 +351,7 @@ k_sym(const __grid_constant__ CUtensorMap map_res, const __grid_constant__ CUten
                         if (pt < p.N) atomicAdd(p.sums + pt, (unsigned long long)__double2ll_rn((double)acc[32 * ch] * fix));
                     }
 #pragma unroll
-                    for (int c = 0; c < 64; ++c) acc[c] = 0.f;
+                    for (int c = 0; c < 32; ++c) acc2[c] = 0;
                     pending = 0;
                 }
             }
