@@ -73,13 +73,17 @@ Layout make_layout(int64_t N, int32_t D, int32_t b_max, int32_t m_max) {
     if (N >= (L.DP <= 8 ? 16384 : 32768) && N <= (int64_t)1 << 19) {
         const size_t tiles = (size_t)(L.NP / 128), pairs = tiles / 2;
         L.perm = carve(cur, (size_t)N * 4);
-        // (direct-difference kernels: column tiles of 16 points; up to 8 coordinates and 2^17 points, 8.4 MB of lists)
-        const size_t col_tiles = L.DP <= 8 && N <= (int64_t)1 << 17 ? 8 * tiles : tiles;
-        L.direct_lists = col_tiles > tiles;
+        // (direct-difference kernels: 64 rows x 16 points; up to 8 coordinates and 2^17 points, 33 MB of lists)
+        L.direct_lists = L.DP <= 8 && N <= (int64_t)1 << 17;
+        const size_t groups = L.direct_lists ? 2 * tiles : pairs, col_tiles = L.direct_lists ? 8 * tiles : tiles;
         L.boxes = carve(cur, col_tiles * 2 * 8 * 4);
         if (L.DP > 8) L.zproj = carve(cur, (size_t)N * 8 * 4);
-        L.lists = carve(cur, pairs * col_tiles * 2);
-        L.list_counts = carve(cur, (4 * pairs + 2) * 4);
+        for (int i = 0; i < 2; ++i) {
+            L.lists[i] = carve(cur, groups * col_tiles * 2);
+            L.list_counts[i] = carve(cur, (4 * groups + 2) * 4);
+        }
+        L.near = carve(cur, std::max(2 * tiles * tiles, L.direct_lists ? groups * col_tiles : 0));
+        if (L.direct_lists) L.xord = carve(cur, (size_t)L.NP * L.DP * 4);
     }
     if (m_max > 0) {
         L.eig_q = carve(cur, (size_t)N * m_max * 4);
@@ -220,7 +224,7 @@ fd_status fd_get_option(const fd_ctx* c, const char* name, double* v) {
     else if (!strcmp(name, "tile_share")) {
         const double tiles = (double)(c->L.NP / 128);
         const auto& direct = c->lists[2];
-        if (c->last_path == FD_PATH_SIMT) *v = direct.on ? (double)direct.total / (tiles * tiles) : 1.0;
+        if (c->last_path == FD_PATH_SIMT) *v = direct.on ? (double)direct.total / (16.0 * tiles * tiles) : 1.0;
         else *v = c->lists[0].on ? (double)c->lists[0].total / (0.5 * tiles * tiles) : 1.0;
     }
     else if (!strcmp(name, "mean_sq")) *v = c->mean_sq;
@@ -273,12 +277,21 @@ fd_status fd_degree(fd_ctx* c, double beta, double alpha, fd_precision prec, flo
         qa = c->w();
     }
     FD_TRY(ew_scale_vec(c, qa, c->q(), c->d(), c->s(), N, q_dev, d_dev, s_dev));
-    struct { unsigned int status; unsigned int pad[15]; double sums[2]; } host;
+    struct { unsigned int status; unsigned int pad[15]; double sums[2]; unsigned int listed, pad2; } host;
+    // the products' lists by what pass 1 noted, and how many tiles they hold
+    const int kind = c->near_direct ? 2 : 0;
+    const bool listed = n > 0 && c->near_beta == beta && c->lists[kind].on && c->lists[kind].beta == beta;
+    if (listed) {
+        FD_TRY(tile_lists(c, beta, c->near_direct ? 4 : 0, false));
+        const int64_t lists = c->L.NP / (c->near_direct ? 64 : 256);
+        FD_CUDA(c, cudaMemcpyAsync(c->at<char>(c->L.status) + 80, c->at<unsigned int>(c->L.list_counts[0]) + 3 * lists, 4, cudaMemcpyDeviceToDevice, c->stream));
+    }
     FD_CUDA(c, cudaMemcpyAsync(&host, c->at<char>(c->L.status), sizeof host, cudaMemcpyDeviceToHost, c->stream));
     FD_CUDA(c, cudaStreamSynchronize(c->stream));
     if (n <= 0) host.sums[0] = host.sums[1] = 0.0;               // a rank that owns no rows
     FD_TRY(allreduce_host(c, host.sums, 2));                     // (before the status is looked at: every rank takes this step)
     if (host.status != 0) return tc_check_status(c);             // reports and clears it
+    if (listed) c->lists[kind].total = host.listed;
     const double sum_q = host.sums[0], sum_sq = host.sums[1];
     if (!(sum_q == sum_q) || !(sum_q < 1e300)) return fail(c, FD_ERR_NONFINITE, "non-finite degree sum");
     // the diagonal of K is exactly 1 in both sums

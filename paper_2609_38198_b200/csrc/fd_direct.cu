@@ -20,30 +20,22 @@
 // N = 16384, D = 4, b = 16: 412 -> 309 us a product; N = 12000, D = 12, b = 48: 944 -> 639 us; N = 6000, D = 2, both degree passes:
 // 136 -> 109 us (one row per thread, separate packing pass, one CTA more or less per SM at the end).
 //
-// Up to 8 coordinates, from 16384 points on, column tiles whose kernel values are all exactly zero are left out where the degree passes found
-// enough of them (fd_order.cu): a step is then 64 listed positions of the points' order, gathered through it (which costs a fifth
-// more per step; the next step's indices are looked up during the present one).  2-torus, N = 16384, beta = 100, b = 16: 310 -> 133 us a product
-// with 0.34 of the tiles, both degree passes 335 -> 168 us; N = 80000, beta = 30, b = 32: 12.7 -> 7.6 ms (0.53); circle, N = 20000,
-// beta = 400, b = 4: 230 -> 54 us (0.18).  Above 0.8 of the tiles the gathers cost what the lists save.
+// Up to 8 coordinates, from 16384 points on, passes over the whole point set may run over tile lists instead: fd_direct_listed.cu.
 #include <algorithm>
 
-#include "fd_internal.h"
+#include "fd_direct.h"
 
 namespace fd {
 
 namespace {
+
+using namespace direct;
 
 constexpr int kThr = 128;        // threads per CTA
 constexpr int kRowsT = 256;      // rows per row tile
 constexpr int kTJ = 64;          // points per column tile, at most (DirectParams::tj_log2)
 constexpr int kFlushCols = 2048; // columns between flushes of the fp32 tile accumulators
 constexpr int kMaxCtasPerSm = 4; // (the shares of cut row tiles are provisioned for four)
-
-__device__ __forceinline__ float ex2_approx(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 
 struct DirectParams {
     const float4* xrow; const float4* xcol;      // padded points, DP4 float4 each
@@ -55,110 +47,56 @@ struct DirectParams {
     double* rowsq;                               // row-sum mode: sum_j K_ij^2 (may be null); Y = the weighted row sums
     void* part;                                  // 2 slots per CTA: shares of row tiles that are cut
     int row_tiles, col_tiles;
-    // tile lists (null: every column tile; fd_order.cu): entries of row tile r at list[r * tiles16 ..], counts[r] of them, tiles of 16
-    // positions each; a step is a column tile of consecutive entries, offs[r] steps lie before row tile r; perm: point of each position
-    const unsigned short* list; const unsigned int* counts; const unsigned int* offs; const int* perm; int tiles16;
     int tj_log2;                                 // log2 of the points per column tile: 6, or 4 where 64 would leave too few steps
-    int dp4;                                     // float4 per point
-    // with lists: bad[c] = epoch where a sum of column c (row sums: a weighted sum) is not finite.  An entry of the right block that is not finite
-    // shows in its own point's row at least (kernel value 1); looking at the sums costs 1 %, at the staged entries 6 % (N = 16384, D = 4, b = 16).
-    unsigned int* bad; unsigned int epoch;
 };
 
 __host__ __device__ __forceinline__ long long range_begin(long long total, int cta, int ctas) { return total * cta / ctas; }
 // (A CTA's share of a row tile goes to its slot 1 if its range holds the row tile's first step, else to slot 0.)
 
 // A CTA's range of steps, one row tile after the other.
-template <bool LISTED>
 struct Range {
     long long g, g_end;
-    int rt = -1, c0, n, full;                        // steps c0 .. c0 + n of the row tile's `full` ones
+    int rt = -1, c0, n;                              // steps c0 .. c0 + n of the row tile
     __device__ __forceinline__ Range(const DirectParams& p) {
-        const long long total = LISTED ? (long long)p.offs[p.row_tiles] : (long long)p.row_tiles * p.col_tiles;
+        const long long total = (long long)p.row_tiles * p.col_tiles;
         g = range_begin(total, (int)blockIdx.x, (int)gridDim.x);
         g_end = range_begin(total, (int)blockIdx.x + 1, (int)gridDim.x);
     }
     __device__ __forceinline__ bool next(const DirectParams& p) {
         if (g >= g_end) return false;                // (the same for the whole CTA)
-        if (!LISTED) {
-            rt = (int)(g / p.col_tiles);
-            c0 = (int)(g - (long long)rt * p.col_tiles);
-            full = p.col_tiles;
-        } else {
-            if (rt < 0) {                            // the last row tile that begins at or before step g: every thread looks at some
-                int before = 0;
-                for (int r0 = 0; r0 < p.row_tiles; r0 += kThr) {
-                    const int r = r0 + (int)threadIdx.x;
-                    before += __syncthreads_count(r < p.row_tiles && (long long)p.offs[r] <= g);
-                }
-                rt = before - 1;
-            } else ++rt;
-            c0 = (int)(g - (long long)p.offs[rt]);
-            full = (int)(p.offs[rt + 1] - p.offs[rt]);
-        }
-        n = (int)(full - c0 < g_end - g ? full - c0 : g_end - g);
+        rt = (int)(g / p.col_tiles);
+        c0 = (int)(g - (long long)rt * p.col_tiles);
+        n = (int)(p.col_tiles - c0 < g_end - g ? p.col_tiles - c0 : g_end - g);
         g += n;
         return true;
     }
 };
 
-// Point of slot `jj` of step c of row tile rt; -1: padding.
-__device__ __forceinline__ int listed_point(const DirectParams& p, int rt, int c, int jj) {
-    const int e = (c << (p.tj_log2 - 4)) + (jj >> 4);
-    if (e >= (int)p.counts[rt]) return -1;
-    const int pos = (int)p.list[(size_t)rt * p.tiles16 + e] * 16 + (jj & 15);
-    return pos < (int)p.N ? p.perm[pos] : -1;
-}
-
 // Stages the points of a column tile (padding points lie 1e18 away: kernel value 0).
-template <int DP4, bool LISTED>
-__device__ __forceinline__ void stage_points(const DirectParams& p, int64_t j0, const int* sidx, float4* sx) {
+template <int DP4>
+__device__ __forceinline__ void stage_points(const DirectParams& p, int64_t j0, float4* sx) {
     for (int t = threadIdx.x; t < (DP4 << p.tj_log2); t += kThr) {
-        if (LISTED) {
-            const int j = sidx[t / DP4];
-            sx[t] = j >= 0 ? p.xcol[(int64_t)j * DP4 + t % DP4] : make_float4(1e18f, 1e18f, 1e18f, 1e18f);
-        } else {
-            const int64_t j = j0 + t / DP4;
-            sx[t] = j < p.N ? p.xcol[j0 * DP4 + t] : make_float4(1e18f, 1e18f, 1e18f, 1e18f);
-        }
+        const int64_t j = j0 + t / DP4;
+        sx[t] = j < p.N ? p.xcol[j0 * DP4 + t] : make_float4(1e18f, 1e18f, 1e18f, 1e18f);
     }
 }
 
 // Row r of a thread: position lane_row + (256 / R) r of the row tile.
-template <int DP4, int R, bool LISTED>
+template <int DP4, int R>
 __device__ __forceinline__ void load_rows(const DirectParams& p, int64_t row0, int lane_row, float4 (&xi)[R][DP4]) {
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        int64_t i = row0 + lane_row + (kRowsT / R) * r;
+        const int64_t i = row0 + lane_row + (kRowsT / R) * r;
         const bool valid = i < p.Nrow;
-        if (LISTED && valid) i = p.perm[i];
 #pragma unroll
         for (int k = 0; k < DP4; ++k) xi[r][k] = valid ? p.xrow[i * DP4 + k] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
 
-template <int DP4, int R>
-__device__ __forceinline__ void kernel_values(const float4* sx, int jj, const float4 (&xi)[R][DP4], float nbeta2, float (&kij)[R]) {
-    float h[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) h[r] = 0.f;
-#pragma unroll
-    for (int k = 0; k < DP4; ++k) {
-        const float4 xj = sx[jj * DP4 + k];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const float d0 = xi[r][k].x - xj.x, d1 = xi[r][k].y - xj.y, d2 = xi[r][k].z - xj.z, d3 = xi[r][k].w - xj.w;
-            h[r] = fmaf(d0, d0, h[r]); h[r] = fmaf(d1, d1, h[r]); h[r] = fmaf(d2, d2, h[r]); h[r] = fmaf(d3, d3, h[r]);
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) kij[r] = ex2_approx(h[r] * nbeta2);
-}
-
 // Block mode: Y[i, c] = left_i sum_j K_ij right_j V[j, c] for c < b <= BT.
 // (resident CTAs asked for: four, three or two, by the registers that the rows and sums of a thread need)
 constexpr int min_ctas(int regs) { return regs + 40 <= 128 ? 4 : regs + 40 <= 168 ? 3 : 2; }
-template <int DP4, int BT, int R, bool LISTED>
+template <int DP4, int BT, int R>
 __global__ void __launch_bounds__(kThr, min_ctas(R * (4 * DP4 + BT)))
 k_direct(const DirectParams p) {
     constexpr int H = R * kThr / kRowsT;               // column parts of a tile (R = 4: 2)
@@ -170,38 +108,25 @@ k_direct(const DirectParams p) {
     const int part = H == 1 ? 0 : (int)threadIdx.x / (kThr / H);
     const int lane_row = H == 1 ? (int)threadIdx.x : (int)threadIdx.x % (kThr / H);
     const int tj = 1 << p.tj_log2;
-    __shared__ int sidx[LISTED ? kTJ : 1];               // points of the column tile
-    for (Range<LISTED> range(p); range.next(p);) {
+    for (Range range(p); range.next(p);) {
         const int c0 = range.c0, n = range.n;
         const int64_t row0 = (int64_t)range.rt * kRowsT;
-        int point = LISTED && (int)threadIdx.x < tj ? listed_point(p, range.rt, c0, (int)threadIdx.x) : -1;
         float4 xi[R][DP4];
-        load_rows<DP4, R, LISTED>(p, row0, lane_row, xi);
-        float acc[R][BT];
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-#pragma unroll
-            for (int c = 0; c < BT; ++c) acc[r][c] = 0.f;
+        load_rows<DP4, R>(p, row0, lane_row, xi);
+        Sums<R, BT> acc;
+        acc.clear();
         // a thread's own slots of sacc: row r, column c at mine[c * 256 + (256 / R) * r]
         float* mine = sacc + part * BT * kRowsT + lane_row;
         bool flushed = false;
         for (int t = 0; t < n; ++t) {
             const int64_t j0 = (int64_t)(c0 + t) << p.tj_log2;
             __syncthreads();
-            if (LISTED) {
-                // (the next step's points are looked up while this one is computed)
-                if ((int)threadIdx.x < tj) {
-                    sidx[threadIdx.x] = point;
-                    if (t + 1 < n) point = listed_point(p, range.rt, c0 + t + 1, (int)threadIdx.x);
-                }
-                __syncthreads();
-            }
-            stage_points<DP4, LISTED>(p, j0, sidx, sx);
+            stage_points<DP4>(p, j0, sx);
             for (int e = threadIdx.x; e < (BT << p.tj_log2); e += kThr) {
                 const int jj = e & (tj - 1), c = e >> p.tj_log2;   // rows of V fastest: coalesced
-                const int64_t j = LISTED ? (int64_t)sidx[jj] : j0 + jj;
+                const int64_t j = j0 + jj;
                 float w = 0.f;
-                if (c < p.b && (LISTED ? j >= 0 : j < p.N)) {
+                if (c < p.b && j < p.N) {
                     w = c < p.vcols ? p.V[j + (int64_t)c * p.ldv] : 1.f;
                     if (p.right) w *= p.right[j];
                 }
@@ -212,17 +137,7 @@ k_direct(const DirectParams p) {
             for (int jj = part * (tj / H); jj < (part + 1) * (tj / H); ++jj) {
                 float kij[R];
                 kernel_values<DP4, R>(sx, jj, xi, p.nbeta2, kij);
-#pragma unroll
-                for (int c4 = 0; c4 < BT / 4; ++c4) {
-                    const float4 w = *reinterpret_cast<const float4*>(&sw[jj * BP + 4 * c4]);
-#pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        acc[r][4 * c4 + 0] = fmaf(kij[r], w.x, acc[r][4 * c4 + 0]);
-                        acc[r][4 * c4 + 1] = fmaf(kij[r], w.y, acc[r][4 * c4 + 1]);
-                        acc[r][4 * c4 + 2] = fmaf(kij[r], w.z, acc[r][4 * c4 + 2]);
-                        acc[r][4 * c4 + 3] = fmaf(kij[r], w.w, acc[r][4 * c4 + 3]);
-                    }
-                }
+                acc.add(kij, reinterpret_cast<const float4*>(&sw[jj * BP]));
             }
             if (((t + 1) & (kFlushCols / tj - 1)) == 0 && t + 1 < n) {
                 // two-level summation keeps the rounding error of long column ranges at the 1e-7 level
@@ -231,74 +146,58 @@ k_direct(const DirectParams p) {
 #pragma unroll
                     for (int c = 0; c < BT; ++c) {
                         float* s = mine + c * kRowsT + (kRowsT / R) * r;
-                        *s = flushed ? *s + acc[r][c] : acc[r][c];
-                        acc[r][c] = 0.f;
+                        *s = flushed ? *s + acc.get(r, c) : acc.get(r, c);
                     }
+                acc.clear();
                 flushed = true;
             }
         }
-        if (flushed) {
+        float sum[R][BT];
 #pragma unroll
-            for (int r = 0; r < R; ++r)
+        for (int r = 0; r < R; ++r)
 #pragma unroll
-                for (int c = 0; c < BT; ++c) acc[r][c] += mine[c * kRowsT + (kRowsT / R) * r];
-        }
+            for (int c = 0; c < BT; ++c) {
+                sum[r][c] = acc.get(r, c);
+                if (flushed) sum[r][c] += mine[c * kRowsT + (kRowsT / R) * r];
+            }
         if (H == 2) {
             // the second half hands its sums to the first
             if (part == 1) {
 #pragma unroll
                 for (int r = 0; r < R; ++r)
 #pragma unroll
-                    for (int c = 0; c < BT; ++c) mine[c * kRowsT + (kRowsT / R) * r] = acc[r][c];
+                    for (int c = 0; c < BT; ++c) mine[c * kRowsT + (kRowsT / R) * r] = sum[r][c];
             }
             __syncthreads();
             if (part == 0) {
 #pragma unroll
                 for (int r = 0; r < R; ++r)
 #pragma unroll
-                    for (int c = 0; c < BT; ++c) acc[r][c] += mine[(BT + c) * kRowsT + (kRowsT / R) * r];
+                    for (int c = 0; c < BT; ++c) sum[r][c] += mine[(BT + c) * kRowsT + (kRowsT / R) * r];
             }
         }
         if (part == 0) {
-            if (LISTED) {
-                float zero = 0.f;                                  // NaN if any sum is not finite
-#pragma unroll
-                for (int r = 0; r < R; ++r)
-#pragma unroll
-                    for (int c = 0; c < BT; ++c) zero = fmaf(acc[r][c], 0.f, zero);
-                if (zero != 0.f) {
-#pragma unroll
-                    for (int c = 0; c < BT; ++c) {
-                        float z = 0.f;
-#pragma unroll
-                        for (int r = 0; r < R; ++r) z = fmaf(acc[r][c], 0.f, z);
-                        if (z != 0.f) p.bad[c] = p.epoch;
-                    }
-                }
-            }
-            const bool whole = n == range.full;
+            const bool whole = n == p.col_tiles;
             float* slot = static_cast<float*>(p.part) +
                           (size_t)(2 * blockIdx.x + (c0 == 0 ? 1 : 0)) * BT * kRowsT + lane_row;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                int64_t i = row0 + lane_row + (kRowsT / R) * r;
+                const int64_t i = row0 + lane_row + (kRowsT / R) * r;
                 const bool valid = i < p.Nrow;
-                if (LISTED && valid) i = p.perm[i];
                 const float l = whole && p.left && valid ? p.left[i] : 1.0f;
 #pragma unroll
                 for (int c = 0; c < BT; ++c)
                     if (c < p.b) {
-                        if (!whole) slot[c * kRowsT + (kRowsT / R) * r] = acc[r][c];
-                        else if (valid) p.Y[i + (int64_t)c * p.ldy] = acc[r][c] * l;
+                        if (!whole) slot[c * kRowsT + (kRowsT / R) * r] = sum[r][c];
+                        else if (valid) p.Y[i + (int64_t)c * p.ldy] = sum[r][c] * l;
                     }
             }
         }
     }
-    cudaTriggerProgrammaticLaunchCompletion();
 }
 
 // Row-sum mode: sum_j K_ij right_j and sum_j K_ij^2; a column tile (<= 64 terms) in fp32, across tiles in fp64.
-template <int DP4, bool LISTED>
+template <int DP4>
 __global__ void __launch_bounds__(kThr)
 k_direct_rowsum(const DirectParams p) {
     constexpr int R = DP4 <= 4 ? 4 : 2, H = R * kThr / kRowsT;
@@ -308,31 +207,21 @@ k_direct_rowsum(const DirectParams p) {
     const int part = H == 1 ? 0 : (int)threadIdx.x / (kThr / H);
     const int lane_row = H == 1 ? (int)threadIdx.x : (int)threadIdx.x % (kThr / H);
     const int tj = 1 << p.tj_log2;
-    __shared__ int sidx[LISTED ? kTJ : 1];               // points of the column tile
-    for (Range<LISTED> range(p); range.next(p);) {
+    for (Range range(p); range.next(p);) {
         const int c0 = range.c0, n = range.n;
         const int64_t row0 = (int64_t)range.rt * kRowsT;
-        int point = LISTED && (int)threadIdx.x < tj ? listed_point(p, range.rt, c0, (int)threadIdx.x) : -1;
         float4 xi[R][DP4];
-        load_rows<DP4, R, LISTED>(p, row0, lane_row, xi);
+        load_rows<DP4, R>(p, row0, lane_row, xi);
         double dsum[R], dsq[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) { dsum[r] = 0.0; dsq[r] = 0.0; }
         for (int t = 0; t < n; ++t) {
             const int64_t j0 = (int64_t)(c0 + t) << p.tj_log2;
             __syncthreads();
-            if (LISTED) {
-                // (the next step's points are looked up while this one is computed)
-                if ((int)threadIdx.x < tj) {
-                    sidx[threadIdx.x] = point;
-                    if (t + 1 < n) point = listed_point(p, range.rt, c0 + t + 1, (int)threadIdx.x);
-                }
-                __syncthreads();
-            }
-            stage_points<DP4, LISTED>(p, j0, sidx, sx);
+            stage_points<DP4>(p, j0, sx);
             if ((int)threadIdx.x < tj) {
-                const int64_t j = LISTED ? (int64_t)sidx[threadIdx.x] : j0 + threadIdx.x;
-                sw[threadIdx.x] = (LISTED ? j >= 0 : j < p.N) ? (p.right ? p.right[j] : 1.0f) : 0.f;
+                const int64_t j = j0 + threadIdx.x;
+                sw[threadIdx.x] = j < p.N ? (p.right ? p.right[j] : 1.0f) : 0.f;
             }
             __syncthreads();
             float a[R], q[R];
@@ -366,129 +255,85 @@ k_direct_rowsum(const DirectParams p) {
                             (size_t)(2 * blockIdx.x + (c0 == 0 ? 1 : 0)) * kRowsT + lane_row;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                int64_t i = row0 + lane_row + (kRowsT / R) * r;
-                if (LISTED && !isfinite(dsum[r])) p.bad[0] = p.epoch;
-                if (n != range.full) slot[(kRowsT / R) * r] = make_double2(dsum[r], dsq[r]);
+                const int64_t i = row0 + lane_row + (kRowsT / R) * r;
+                if (n != p.col_tiles) slot[(kRowsT / R) * r] = make_double2(dsum[r], dsq[r]);
                 else if (i < p.Nrow) {
-                    if (LISTED) i = p.perm[i];
                     p.Y[i] = (float)(dsum[r] * (p.left ? (double)p.left[i] : 1.0));
                     if (p.rowsq) p.rowsq[i] = dsq[r];
                 }
             }
         }
     }
-    cudaTriggerProgrammaticLaunchCompletion();
-}
-
-// Row i's sum over every point for column c of the right block (row sums, V null: for the weights).  For columns that `bad` names: the product
-// of an entry that is not finite with a kernel value of zero is NaN, so tiles of zeros count as well and the lists do not hold.
-__device__ __forceinline__ float sum_over_all_points(const DirectParams& p, int64_t i, int c) {
-    float acc = 0.f;
-#pragma unroll 1
-    for (int64_t j = 0; j < p.N; ++j) {
-        float h = 0.f;
-#pragma unroll 1
-        for (int k = 0; k < p.dp4; ++k) {
-            const float4 a = p.xrow[i * p.dp4 + k], b = p.xcol[j * p.dp4 + k];
-            const float d0 = a.x - b.x, d1 = a.y - b.y, d2 = a.z - b.z, d3 = a.w - b.w;
-            h = fmaf(d0, d0, h); h = fmaf(d1, d1, h); h = fmaf(d2, d2, h); h = fmaf(d3, d3, h);
-        }
-        float w = p.V && c < p.vcols ? p.V[j + (int64_t)c * p.ldv] : 1.f;
-        if (p.right) w *= p.right[j];
-        acc = fmaf(ex2_approx(h * p.nbeta2), w, acc);
-    }
-    return acc;
 }
 
 // Finishes the row tiles that a cut falls into.  Block = (32 rows of a row tile, 8 columns), 8 groups of shares read in parallel (a row
-// tile of a small problem has up to a hundred).  Every block waits for the product, also one that has nothing to add: with lists it may be
-// that no row tile is cut, and what follows this kernel in the stream waits for this kernel only.
+// tile of a small problem has up to a hundred).  Every block waits for the product, also one that has nothing to add: what follows
+// this kernel in the stream waits for this kernel only.
 constexpr int kFixCols = 8;
-template <bool LISTED>
 __global__ void __launch_bounds__(256)
 k_direct_fix(const DirectParams p, int BT, int ctas) {
     __shared__ float sm[kFixCols][8][32];
     const int rt = blockIdx.x / (kRowsT / 32);
-    const long long total = LISTED ? (long long)p.offs[p.row_tiles] : (long long)p.row_tiles * p.col_tiles;
-    const long long g0 = LISTED ? (long long)p.offs[rt] : (long long)rt * p.col_tiles;
-    const long long g1 = LISTED ? (long long)p.offs[rt + 1] : g0 + p.col_tiles;
+    const long long total = (long long)p.row_tiles * p.col_tiles;
+    const long long g0 = (long long)rt * p.col_tiles;
+    const long long g1 = g0 + p.col_tiles;
     // the last CTA whose range begins at or before step g0, and the last one whose range begins before g1
     const int first = (int)(((g0 + 1) * ctas - 1) / total), last = (int)((g1 * ctas - 1) / total);
-    cudaGridDependencySynchronize();
-    const bool cut = first != last;                                    // else its CTA stored it
-    if (!LISTED && !cut) return;
+    grid_wait();
+    grid_go();
+    if (first == last) return;                                         // not cut: its CTA stored it
     const int r = threadIdx.x & 31, grp = threadIdx.x >> 5;
     const int row = (blockIdx.x % (kRowsT / 32)) * 32 + r, col0 = (int)blockIdx.y * kFixCols;
-    // (read beside the shares, looked at after them: one latency)
-    const unsigned int note = LISTED && col0 + grp < p.b ? p.bad[col0 + grp] : p.epoch + 1;
-    if (cut) {
-        const int per = (last - first + 8) / 8, s0 = first + grp * per, s1 = min(last + 1, s0 + per);
-        const float* slots = static_cast<const float*>(p.part) + (size_t)col0 * kRowsT + row;
-        float v[kFixCols];
+    const int per = (last - first + 8) / 8, s0 = first + grp * per, s1 = min(last + 1, s0 + per);
+    const float* slots = static_cast<const float*>(p.part) + (size_t)col0 * kRowsT + row;
+    float v[kFixCols];
 #pragma unroll
-        for (int c = 0; c < kFixCols; ++c) v[c] = 0.f;
+    for (int c = 0; c < kFixCols; ++c) v[c] = 0.f;
 #pragma unroll 4
-        for (int s = s0; s < s1; ++s) {
-            const float* o = slots + (size_t)(2 * s + (s == first ? 1 : 0)) * BT * kRowsT;
+    for (int s = s0; s < s1; ++s) {
+        const float* o = slots + (size_t)(2 * s + (s == first ? 1 : 0)) * BT * kRowsT;
 #pragma unroll
-            for (int c = 0; c < kFixCols; ++c)
-                if (col0 + c < p.b) v[c] += o[c * kRowsT];
-        }
-#pragma unroll
-        for (int c = 0; c < kFixCols; ++c) sm[c][grp][r] = v[c];
-        __syncthreads();
+        for (int c = 0; c < kFixCols; ++c)
+            if (col0 + c < p.b) v[c] += o[c * kRowsT];
     }
+#pragma unroll
+    for (int c = 0; c < kFixCols; ++c) sm[c][grp][r] = v[c];
+    __syncthreads();
     // group g finishes column col0 + g
-    int64_t i = (int64_t)rt * kRowsT + row;
+    const int64_t i = (int64_t)rt * kRowsT + row;
     if (i >= p.Nrow || col0 + grp >= p.b) return;
-    const bool bad = LISTED && note == p.epoch;
-    if (!cut && !bad) return;
-    if (LISTED) i = p.perm[i];
     float x = 0.f;
-    if (bad) x = sum_over_all_points(p, i, col0 + grp);
-    else {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) x += sm[grp][q][r];
-    }
+    for (int q = 0; q < 8; ++q) x += sm[grp][q][r];
     p.Y[i + (int64_t)(col0 + grp) * p.ldy] = x * (p.left ? p.left[i] : 1.0f);
 }
 
 // The same for row sums: block = 32 rows.
-template <bool LISTED>
 __global__ void __launch_bounds__(256)
 k_direct_rowsum_fix(const DirectParams p, int ctas) {
     __shared__ double2 sm[8][32];
     const int rt = blockIdx.x / (kRowsT / 32);
-    const long long total = LISTED ? (long long)p.offs[p.row_tiles] : (long long)p.row_tiles * p.col_tiles;
-    const long long g0 = LISTED ? (long long)p.offs[rt] : (long long)rt * p.col_tiles;
-    const long long g1 = LISTED ? (long long)p.offs[rt + 1] : g0 + p.col_tiles;
+    const long long total = (long long)p.row_tiles * p.col_tiles;
+    const long long g0 = (long long)rt * p.col_tiles;
+    const long long g1 = g0 + p.col_tiles;
     const int first = (int)(((g0 + 1) * ctas - 1) / total), last = (int)((g1 * ctas - 1) / total);
-    cudaGridDependencySynchronize();
-    const bool cut = first != last;
-    if (!LISTED && !cut) return;
+    grid_wait();
+    grid_go();
+    if (first == last) return;
     const int r = threadIdx.x & 31, grp = threadIdx.x >> 5, row = (blockIdx.x % (kRowsT / 32)) * 32 + r;
-    const unsigned int note = LISTED ? p.bad[0] : p.epoch + 1;
-    if (cut) {
-        const int per = (last - first + 8) / 8, s0 = first + grp * per, s1 = min(last + 1, s0 + per);
-        const double2* slots = static_cast<const double2*>(p.part) + row;
-        double2 v = make_double2(0.0, 0.0);
-#pragma unroll 8
-        for (int s = s0; s < s1; ++s) { const double2 o = slots[(size_t)(2 * s + (s == first ? 1 : 0)) * kRowsT]; v.x += o.x; v.y += o.y; }
-        sm[grp][r] = v;
-        __syncthreads();
-    }
-    int64_t i = (int64_t)rt * kRowsT + row;
-    if (grp != 0 || i >= p.Nrow) return;
-    const bool bad = LISTED && note == p.epoch;
-    if (!cut && !bad) return;
-    if (LISTED) i = p.perm[i];
+    const int per = (last - first + 8) / 8, s0 = first + grp * per, s1 = min(last + 1, s0 + per);
+    const double2* slots = static_cast<const double2*>(p.part) + row;
     double2 v = make_double2(0.0, 0.0);
-    if (cut) {
+#pragma unroll 8
+    for (int s = s0; s < s1; ++s) { const double2 o = slots[(size_t)(2 * s + (s == first ? 1 : 0)) * kRowsT]; v.x += o.x; v.y += o.y; }
+    sm[grp][r] = v;
+    __syncthreads();
+    const int64_t i = (int64_t)rt * kRowsT + row;
+    if (grp != 0 || i >= p.Nrow) return;
+    v = make_double2(0.0, 0.0);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) { v.x += sm[q][r].x; v.y += sm[q][r].y; }
-        if (p.rowsq) p.rowsq[i] = v.y;
-    }
-    if (bad) v.x = (double)sum_over_all_points(p, i, 0);
+    for (int q = 0; q < 8; ++q) { v.x += sm[q][r].x; v.y += sm[q][r].y; }
+    if (p.rowsq) p.rowsq[i] = v.y;
     p.Y[i] = (float)(v.x * (p.left ? (double)p.left[i] : 1.0));
 }
 
@@ -498,30 +343,23 @@ template <class Kernel>
 fd_status launch(fd_ctx* c, Kernel kernel, int smem, int per_sm, int BT, DirectParams p) {
     // Column tiles of 16 where 64 would give fewer than four steps per CTA: with one or two, the ranges differ by a factor of two and
     // small problems leave SMs idle (N = 1000, b = 64: 29 -> 21 us); more steps make the two barriers per tile dearer.
-    const auto& lists = c->lists[2];
-    p.tj_log2 = (p.list ? lists.total : ceil_div(p.N, kTJ) * p.row_tiles) < 4ll * c->sm_count * per_sm ? 4 : 6;
+    p.tj_log2 = ceil_div(p.N, kTJ) * p.row_tiles < 4ll * c->sm_count * per_sm ? 4 : 6;
     p.col_tiles = (int)ceil_div(p.N, (int64_t)1 << p.tj_log2);
-    if (p.list && p.tj_log2 == 4) p.offs += p.row_tiles + 1;        // steps of one entry
-    const long long total = !p.list ? (long long)p.row_tiles * p.col_tiles : p.tj_log2 == 4 ? lists.entries : lists.total;
+    const long long total = (long long)p.row_tiles * p.col_tiles;
     const size_t slot_floats = (size_t)kRowsT * (BT > 0 ? BT : 4);
     long long ctas = c->opt_splits > 0 ? (long long)p.row_tiles * c->opt_splits : (long long)c->sm_count * per_sm;
     ctas = std::max<long long>(1, std::min<long long>(std::min(ctas, total), (long long)(c->L.part_floats / (2 * slot_floats))));
     if (c->opt_splits <= 0) ctas = ceil_div(total, ceil_div(total, ctas));      // same longest range, fewer shares
     if (smem > 48 * 1024) FD_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    kernel<<<(unsigned)ctas, kThr, smem, c->stream>>>(p);
+    kernel<<<dim3((unsigned)ctas), dim3(kThr), smem, c->stream>>>(p);
     FD_LAUNCH_CHECK(c, "k_direct");
-    bool cut = p.list != nullptr;
+    bool cut = false;
     for (int i = 1; i < ctas && !cut; ++i) cut = range_begin(total, i, (int)ctas) % p.col_tiles != 0;
     if (cut) {
         // launched while the product's last CTAs run (it waits for their stores): the launch costs no gap
-        cudaLaunchAttribute attr{};
-        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr.val.programmaticStreamSerializationAllowed = 1;
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3((unsigned)p.row_tiles * (kRowsT / 32), BT > 0 ? (unsigned)ceil_div(p.b, kFixCols) : 1u);
-        cfg.blockDim = dim3(256); cfg.stream = c->stream; cfg.attrs = &attr; cfg.numAttrs = 1;
-        if (BT > 0) FD_CUDA(c, cudaLaunchKernelEx(&cfg, p.list ? k_direct_fix<true> : k_direct_fix<false>, p, BT, (int)ctas));
-        else FD_CUDA(c, cudaLaunchKernelEx(&cfg, p.list ? k_direct_rowsum_fix<true> : k_direct_rowsum_fix<false>, p, (int)ctas));
+        const dim3 grid((unsigned)p.row_tiles * (kRowsT / 32), BT > 0 ? (unsigned)ceil_div(p.b, kFixCols) : 1u);
+        if (BT > 0) FD_CUDA(c, launch_behind(c->stream, grid, dim3(256), 0, k_direct_fix, p, BT, (int)ctas));
+        else FD_CUDA(c, launch_behind(c->stream, grid, dim3(256), 0, k_direct_rowsum_fix, p, (int)ctas));
         FD_LAUNCH_CHECK(c, "k_direct_fix");
     }
     return FD_OK;
@@ -538,26 +376,16 @@ template <int DP4, int BT>
 fd_status launch_block(fd_ctx* c, const DirectParams& p) {
     constexpr int R = 4 * DP4 + BT <= 32 ? 4 : 2, H = R * kThr / kRowsT;
     constexpr int smem = (kTJ * DP4 * 4 + kTJ * (BT + 4) + H * BT * kRowsT) * 4;
-    if constexpr (DP4 <= 2)
-        if (p.list) {
-            static const int per_sm = resident(k_direct<DP4, BT, R, true>, smem);
-            return launch(c, k_direct<DP4, BT, R, true>, smem, per_sm, BT, p);
-        }
-    static const int per_sm = resident(k_direct<DP4, BT, R, false>, smem);
-    return launch(c, k_direct<DP4, BT, R, false>, smem, per_sm, BT, p);
+    static const int per_sm = resident(k_direct<DP4, BT, R>, smem);
+    return launch(c, k_direct<DP4, BT, R>, smem, per_sm, BT, p);
 }
 
 template <int DP4>
 fd_status launch_dp(fd_ctx* c, int BT, const DirectParams& p) {
     switch (BT) {
         case 0: {
-            if constexpr (DP4 <= 2)
-                if (p.list) {
-                    static const int per_sm = resident(k_direct_rowsum<DP4, true>, 0);
-                    return launch(c, k_direct_rowsum<DP4, true>, 0, per_sm, 0, p);
-                }
-            static const int per_sm = resident(k_direct_rowsum<DP4, false>, 0);
-            return launch(c, k_direct_rowsum<DP4, false>, 0, per_sm, 0, p);
+            static const int per_sm = resident(k_direct_rowsum<DP4>, 0);
+            return launch(c, k_direct_rowsum<DP4>, 0, per_sm, 0, p);
         }
         case 4: return launch_block<DP4, 4>(c, p);
         case 8: return launch_block<DP4, 8>(c, p);
@@ -568,8 +396,6 @@ fd_status launch_dp(fd_ctx* c, int BT, const DirectParams& p) {
         default: return launch_block<DP4, 64>(c, p);
     }
 }
-
-int pick_bt(int bc) { return bc <= 4 ? 4 : bc <= 8 ? 8 : bc <= 16 ? 16 : bc <= 24 ? 24 : bc <= 32 ? 32 : bc <= 48 ? 48 : 64; }
 
 }  // namespace
 
@@ -582,22 +408,16 @@ fd_status apply_simt(fd_ctx* c, const ApplyArgs& a) {
     p.xcol = reinterpret_cast<const float4*>(c->xs()); p.N = L.N;
     p.nbeta2 = (float)(-a.beta * kLog2e);
     p.right = a.right; p.left = a.left; p.ldv = a.ldv; p.ldy = a.ldy;
-    p.part = c->at<float>(L.part); p.dp4 = DP4;
+    p.part = c->at<float>(L.part);
     p.row_tiles = (int)ceil_div(a.Nrow, kRowsT);
     const bool rowsum = a.V == nullptr;
     // passes over the context's whole point set may leave out tiles of pairs whose kernel value is exactly zero; the degree passes
     // decide (they wait for their sums anyway), products follow
     if (a.rows_are_ctx && a.xrow == c->xs() && a.Nrow == L.N && !c->sh.on && L.direct_lists) {
+        const int kind = rowsum && a.rowsq ? 2 : 4;
         FD_TRY(note_capture(c));
-        FD_TRY(tile_lists(c, a.beta, 2, a.decide));
-        if (c->lists[2].on && c->lists[2].beta == a.beta) {
-            p.list = c->at<unsigned short>(L.lists);
-            p.counts = c->at<unsigned int>(L.list_counts);
-            p.offs = p.counts + 2 * p.row_tiles;
-            p.perm = c->at<int>(L.perm);
-            p.tiles16 = 16 * p.row_tiles;
-            p.bad = reinterpret_cast<unsigned int*>(c->at<char>(L.status) + 256);
-        }
+        FD_TRY(tile_lists(c, a.beta, kind, a.decide));
+        if (c->lists[2].on && c->lists[2].beta == a.beta) return apply_direct_listed(c, a, kind);
     }
     const int chunks = rowsum ? 1 : (int)ceil_div(a.b, 64), step = (int)ceil_div(a.b, chunks);
     for (int c0 = 0; c0 < a.b; c0 += step) {
@@ -607,11 +427,6 @@ fd_status apply_simt(fd_ctx* c, const ApplyArgs& a) {
         p.b = bc;
         p.Y = a.Y + (int64_t)c0 * a.ldy;
         p.rowsq = a.rowsq;
-        if (p.list) {
-            // (a replayed graph brings the same epoch again; what an earlier replay noted would cost time, not the result)
-            p.epoch = ++c->direct_epoch;
-            if (c->captured) FD_CUDA(c, cudaMemsetAsync(p.bad, 0, 64 * 4, c->stream));
-        }
         switch (DP4) {
             case 1: FD_TRY(launch_dp<1>(c, BT, p)); break;
             case 2: FD_TRY(launch_dp<2>(c, BT, p)); break;

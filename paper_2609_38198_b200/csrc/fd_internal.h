@@ -31,7 +31,7 @@ struct Layout {
     size_t part = 0, part_floats = 0;
     size_t xp_col = 0, xp_row = 0, wt_hi = 0, wt_lo = 0, colscale = 0, status = 0;
     // order of the points and tile lists of the Gram-form kernels (fd_order.cu); 0: not provisioned for this N
-    size_t perm = 0, boxes = 0, zproj = 0, lists = 0, list_counts = 0;
+    size_t perm = 0, boxes = 0, zproj = 0, lists[2] = {0, 0}, list_counts[2] = {0, 0}, near = 0, xord = 0;
     bool direct_lists = false;       // provisioned for the direct-difference kernels as well
     size_t weights = 0;              // NP right weights of a Gram-form row sum
     size_t symsum = 0;               // N 64-bit fixed-point sums of the symmetric row-sum mode
@@ -72,15 +72,18 @@ struct fd_ctx {
     int order_state = 0;             // 1: L.perm holds an order of the points; -1: none will be made
     // tile lists, for Gram-form block products (0) and degree passes (1) and all passes of the direct-difference kernels (2): bandwidth they were decided for, whether
     // they leave out enough to be used, entries in all; which of the three the workspace holds, and for which bandwidth
-    // (direct-difference kernels (2): total is in groups of four tiles of 16 points, entries in single ones)
-    struct { double beta = -1.0; bool on = false; int64_t total = 0, entries = 0; } lists[3];
+    struct { double beta = -1.0; bool on = false; int64_t total = 0; } lists[3];
     // A pass of this context was recorded into a CUDA graph (set by note_capture, for good).  What the workspace holds is then known to nobody
     // on the host: recording runs nothing, and a replay packs and lists again.  Every pass packs and lists for itself from then on.
     bool captured = false;
     unsigned int direct_epoch = 0;   // number of the latest listed pass of the direct-difference kernels
     double refused_beta = 0.0;       // largest bandwidth at which an order was tried and left out too little
-    int listed_kind = -1, boxes_kind = -1;
-    double listed_beta = -1.0;
+    struct { int kind = -1; double beta = -1.0; } listed[2];     // what the two list buffers hold: of the products (0), of the degree passes (1)
+    int boxes_kind = -1;
+    // bandwidth whose near tiles a degree pass noted in L.near (fd_order.cu).  No pass writes notes once products have been recorded: a
+    // replay lists by what they say.
+    double near_beta = -1.0;
+    bool near_direct = false;        // (by a direct-difference pass)
     // options
     int opt_path = FD_PATH_AUTO;
     int opt_splits = 0;
@@ -213,7 +216,23 @@ fd_status scale_cols_by_pow(fd_ctx* c, const float* v, int64_t ldv, int32_t cols
 }  // namespace fd
 
 #ifdef __CUDACC__
+#include <utility>
+
 namespace fd {
+
+// Launches a kernel that may start while the kernel before it in the stream ends: it calls grid_wait() in every thread before it touches memory
+// (also in blocks that have nothing to do: what follows waits for this kernel only).  grid_go() lets the one after it do the same.
+template <class... Params, class... Args>
+cudaError_t launch_behind(cudaStream_t stream, dim3 grid, dim3 block, size_t smem, void (*kernel)(Params...), Args&&... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream; cfg.attrs = &attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+__device__ __forceinline__ void grid_wait() { cudaGridDependencySynchronize(); }
+__device__ __forceinline__ void grid_go() { cudaTriggerProgrammaticLaunchCompletion(); }
 
 // Two fp32 values in a register pair: an instruction on both takes one issue slot and the time of two on the FMA pipe.
 __device__ __forceinline__ uint64_t pair2(float a, float b) {

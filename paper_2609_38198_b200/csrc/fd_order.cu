@@ -18,12 +18,19 @@
 // gather through the permutation, the epilogues scatter.  Gram-form passes at a bandwidth with lists work in the order, all others (and
 // direct-difference passes without lists) in the caller's.
 //
-// Lists: for a bandwidth and exponent limit, per 256 rows the column tiles whose bounding box comes close enough (distance of the
-// two boxes: a lower bound for every pair): tiles of 128 points for the Gram-form kernels, of 16 for the direct-difference
-// ones (there against the 16 boxes of the rows, too: 0.39 -> 0.34 of the tiles remain on the 2-torus, N = 16384, beta = 100).  Data that
-// fill many dimensions (the 6-torus) have no far tiles; then the passes run over all tiles as before.
-// N = 2^18, R^30 on a two-dimensional manifold, beta = 2 (44 % of the pairs are not zero), both at the power limit: b = 32, 25.5 -> 20.1 ms a
-// product; degree passes 23.2 -> 19.9 ms.  Direct differences, exactly zero values only: fd_direct.cu.
+// Lists by the boxes: for a bandwidth and exponent limit, per 256 rows the column tiles of 128 points whose bounding box comes close enough
+// (distance of the two boxes: a lower bound for every pair); for the direct-difference kernels per 64 rows the tiles of 16 points, there
+// against the 4 boxes of the rows, too.  Data that fill many dimensions (the 6-torus) have no far tiles; then the passes run over all
+// tiles as before.
+//
+// Lists by notes: boxes of curved patches leave a third more tiles than hold a near pair.  The first degree pass computes every kernel value
+// anyway, so it notes which tiles had one within the limits (from the sums of squares that it forms anyway; direct differences: from the
+// sums), and the second pass and the products at that bandwidth go by these notes.  R^30 on a two-dimensional manifold, beta = 2: 0.80 -> 0.64 of the
+// tiles at N = 65536 (b = 32: 1225 -> 975 us a product), 0.67 -> 0.58 at N = 2^18 (20.0 -> 17.3 ms); 2-torus, direct differences: 0.26 -> 0.17 at
+// N = 16384, beta = 100, 0.56 -> 0.39 at N = 65536, beta = 30.  The first pass goes by the boxes always, so that its results do not depend on earlier calls.
+//
+// (The extension's new points in an order of their own, listed by the boxes: 40009 points against 65536 leave 0.88 of the tiles, and what
+// that saves goes into the order: 985 -> 965 us; 16500 against 33000: 290 -> 319.  They are taken as they come.)
 #include <algorithm>
 #include <cmath>
 #include <new>
@@ -233,13 +240,12 @@ k_leaf_scan(unsigned int* __restrict__ counts, int blocks, int leaves, unsigned 
     if (lane == 0) totals[leaf] = base;
 }
 // out[i] = sum of in[0 .. i), out[n] = total (one block; in and out may not overlap).
-// (with a group size g the terms are ceil(in / g).)
 __global__ void __launch_bounds__(1024)
-k_scan(const unsigned int* __restrict__ in, int n, unsigned int* __restrict__ out, unsigned int g = 1) {
+k_scan(const unsigned int* __restrict__ in, int n, unsigned int* __restrict__ out) {
     __shared__ unsigned int s[1024];
     const int per = (n + 1023) / 1024, i0 = threadIdx.x * per;
     unsigned int sum = 0;
-    for (int i = i0; i < min(n, i0 + per); ++i) sum += (in[i] + g - 1) / g;
+    for (int i = i0; i < min(n, i0 + per); ++i) sum += in[i];
     s[threadIdx.x] = sum;
     __syncthreads();
     for (int m = 1; m < 1024; m <<= 1) {
@@ -249,7 +255,7 @@ k_scan(const unsigned int* __restrict__ in, int n, unsigned int* __restrict__ ou
         __syncthreads();
     }
     unsigned int base = s[threadIdx.x] - sum;
-    for (int i = i0; i < min(n, i0 + per); ++i) { out[i] = base; base += (in[i] + g - 1) / g; }
+    for (int i = i0; i < min(n, i0 + per); ++i) { out[i] = base; base += in[i]; }
     if (threadIdx.x == 1023) out[n] = s[1023];
 }
 // perm[position] = index, by leaf and in index order inside a leaf: the warps of a block take their turns.
@@ -273,6 +279,15 @@ k_scatter(const unsigned short* __restrict__ leaf, int64_t n, const unsigned int
         __syncthreads();
     }
     if (i < n) perm[base[l] + counts[(size_t)l * gridDim.x + blockIdx.x] + rank] = (int)i;
+}
+
+// The points in their order, padded with points 1e18 away (kernel value 0).
+__global__ void __launch_bounds__(256)
+k_order_points(const float4* __restrict__ xs, int DP4, int64_t n, int64_t np, const int* __restrict__ perm, float4* __restrict__ out) {
+    const int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (p >= np) return;
+    const int64_t i = p < n ? perm[p] : -1;
+    for (int k = 0; k < DP4; ++k) out[p * DP4 + k] = i >= 0 ? xs[i * DP4 + k] : make_float4(1e18f, 1e18f, 1e18f, 1e18f);
 }
 
 // Bounding box of each tile of 16 consecutive positions, for up to 8 coordinates: 16 lanes a tile.
@@ -314,19 +329,20 @@ k_boxes(const float* __restrict__ xs, int DP, int64_t n, const int* __restrict__
 
 // Column tiles (per_pair to a row pair) of row pair blockIdx.x whose box comes within limit2 of the pair's box, ascending: list[pair * tiles ..];
 // counts[pair] of them, of which `upper[pair]` are the pair's own and later ones (the symmetric row sums start there).
+// noted (null: by the boxes): what a row-sum pass saw, note_rows rows of `tiles` entries for a pair, not 0 for near ones.
 __global__ void __launch_bounds__(1024)
-k_lists(const float* __restrict__ box, int DP, int tiles, int per_pair, float limit2, unsigned short* __restrict__ list, unsigned int* __restrict__ counts,
-        unsigned int* __restrict__ upper) {
+k_lists(const float* __restrict__ box, int DP, int tiles, int per_pair, float limit2, const unsigned char* __restrict__ noted, int note_rows,
+        unsigned short* __restrict__ list, unsigned int* __restrict__ counts, unsigned int* __restrict__ upper) {
     __shared__ float lo[64], hi[64];
-    __shared__ float sub[16][2][8];                                    // boxes of 16 row tiles (per_pair = 16, up to 8 coordinates)
+    __shared__ float sub[4][2][8];                                     // boxes of the row tiles (per_pair = 4, up to 8 coordinates)
     __shared__ unsigned int wsum[32];
     const int pair = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int k = threadIdx.x; k < DP; k += 1024) {
+    for (int k = threadIdx.x; k < DP && !noted; k += 1024) {
         float l = INFINITY, h = -INFINITY;
         for (int t = 0; t < per_pair; ++t) {
             const float* a = box + ((size_t)pair * per_pair + t) * 2 * DP;
             l = fminf(l, a[k]); h = fmaxf(h, a[DP + k]);
-            if (per_pair == 16) { sub[t][0][k] = a[k]; sub[t][1][k] = a[DP + k]; }
+            if (per_pair == 4) { sub[t][0][k] = a[k]; sub[t][1][k] = a[DP + k]; }
         }
         lo[k] = l; hi[k] = h;
     }
@@ -335,7 +351,10 @@ k_lists(const float* __restrict__ box, int DP, int tiles, int per_pair, float li
     for (int t0 = 0; t0 < tiles; t0 += 1024) {
         const int t = t0 + threadIdx.x;
         bool near = false;
-        if (t < tiles) {
+        if (t < tiles && noted) {
+            for (int s = 0; s < note_rows; ++s) near = near || noted[((size_t)pair * note_rows + s) * tiles + t] != 0;
+            near = near || t / per_pair == pair;
+        } else if (t < tiles) {
             const float* b = box + (size_t)t * 2 * DP;
             float d2 = 0.f;
             for (int k = 0; k < DP; ++k) {
@@ -343,10 +362,10 @@ k_lists(const float* __restrict__ box, int DP, int tiles, int per_pair, float li
                 d2 = fmaf(g, g, d2);
             }
             near = d2 <= limit2;
-            if (near && per_pair == 16) {
-                // near the box of all 256 rows: near one of the 16 smaller boxes?
+            if (near && per_pair == 4) {
+                // near the box of all 64 rows: near one of the 4 smaller boxes?
                 near = false;
-                for (int s = 0; s < 16 && !near; ++s) {
+                for (int s = 0; s < 4 && !near; ++s) {
                     float e2 = 0.f;
                     for (int k = 0; k < DP; ++k) {
                         const float g = fmaxf(fmaxf(b[k] - sub[s][1][k], sub[s][0][k] - b[DP + k]), 0.f);
@@ -379,20 +398,25 @@ k_lists(const float* __restrict__ box, int DP, int tiles, int per_pair, float li
 
 fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide) {
     const Layout& L = c->L;
-    auto& st = c->lists[kind];
+    auto& st = c->lists[kind == 3 ? 1 : kind == 4 ? 2 : kind];
     if (L.perm == 0 || c->order_state < 0) return FD_OK;
-    if (st.beta == beta && (!st.on || (!c->captured && c->listed_kind == kind && c->listed_beta == beta))) return FD_OK;
+    const bool direct = kind == 2 || kind == 4;
+    const bool noted = c->near_beta == beta && c->near_direct == direct && kind != 1 && kind != 2;
+    const int buf = kind == 0 || kind == 4 ? 0 : 1;
+    auto& listed = c->listed[buf];
+    const int held = noted ? 8 + kind : kind;                      // what the buffer would hold
+    if (st.beta == beta && (!st.on || (!c->captured && listed.kind == held && listed.beta == beta))) return FD_OK;
     // Beyond an exponent of 40 both fp16 pieces of a kernel value are zero (2^15 2^-40 = 2^-25 rounds to zero), beyond 60 a degree
     // contribution is below the fixed-point unit; the quarter covers the rounding of the boxes' distance.
     // The direct-difference kernels' exponential gives exactly zero beyond 126.
-    const double limit = kind == 0 ? 40.25 : kind == 1 ? 60.25 : 126.25;
+    const double limit = kind == 0 ? 40.25 : direct ? 126.25 : 60.25;
     const double scaled_beta = beta * (60.25 / limit);             // bandwidths of the kinds on one scale
-    const bool direct = kind == 2;
     if (direct && !L.direct_lists) return FD_OK;
     if (!decide && st.beta != beta) return FD_OK;
     const bool known = st.beta == beta;                            // decided before, only overwritten by the other kind's lists
     const int64_t N = L.N;
-    const int per_pair = direct ? 16 : 2, tiles = (int)(L.NP / 256) * per_pair, pairs = (int)(L.NP / 256);
+    // rows of a list, tiles of a row of tiles
+    const int per_pair = direct ? 4 : 2, pairs = (int)(L.NP / (direct ? 64 : 256)), tiles = pairs * per_pair;
     const float limit2 = (float)(limit / (beta * kLog2e));
     if (!known) { st.on = false; st.beta = beta; }
     unsigned int* small = reinterpret_cast<unsigned int*>(c->at<char>(L.status) + 128);
@@ -415,7 +439,7 @@ fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide) {
         FD_CUDA(c, cudaStreamSynchronize(c->stream));
         // (Share of far pairs from which an order is worth making: 0.4, where tiles are small against the data's extent; 0.8 for fewer than
         // 32768 points.  2-torus, beta = 30, 0.70 of the pairs far: 0.53 of the tiles remain at N = 80000, 0.8 at N = 16384.)
-        if ((double)far < (N < 32768 ? 0.8 : 0.4) * 512.0 * 512.0) return FD_OK;
+        if ((double)far < 0.4 * 512.0 * 512.0) return FD_OK;
         // scratch: the operand buffers (re-packed in the new order afterwards); at least 64 bytes per point each
         int depth = 0;
         while (((int64_t)(L.direct_lists ? 16 : 128) << depth) < N && depth < 12) ++depth;
@@ -465,6 +489,10 @@ fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide) {
         FD_LAUNCH_CHECK(c, "k_scan");
         k_scatter<<<blocks, 1024, 0, c->stream>>>(leaf, N, counts, base, leaves, perm);
         FD_LAUNCH_CHECK(c, "k_scatter");
+        if (L.direct_lists) {
+            k_order_points<<<(unsigned)ceil_div(L.NP, 256), 256, 0, c->stream>>>(reinterpret_cast<const float4*>(c->xs()), L.DP / 4, N, L.NP, perm, c->at<float4>(L.xord));
+            FD_LAUNCH_CHECK(c, "k_order_points");
+        }
         c->order_state = 1;
         c->boxes_kind = -1;
         c->packed_beta = c->packed_row_beta = -1.0;
@@ -475,24 +503,25 @@ fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide) {
         FD_LAUNCH_CHECK(c, "k_boxes");
         c->boxes_kind = direct ? 1 : 0;
     }
-    unsigned int* cnt = c->at<unsigned int>(L.list_counts);
-    k_lists<<<pairs, 1024, 0, c->stream>>>(box, ZP, tiles, per_pair, limit2, c->at<unsigned short>(L.lists), cnt, cnt + pairs);
+    unsigned int* cnt = c->at<unsigned int>(L.list_counts[buf]);
+    const unsigned char* notes = noted ? c->at<unsigned char>(L.near) + (kind == 3 ? (size_t)tiles * tiles : 0) : nullptr;
+    k_lists<<<pairs, 1024, 0, c->stream>>>(box, ZP, tiles, per_pair, limit2, notes, direct ? 1 : 2, c->at<unsigned short>(L.lists[buf]), cnt, cnt + pairs);
     FD_LAUNCH_CHECK(c, "k_lists");
     unsigned int* offs = cnt + 2 * pairs;
-    // two offset arrays: all and upper entries; direct-difference kernels: groups of four entries and single ones
-    k_scan<<<1, 1024, 0, c->stream>>>(cnt, pairs, offs, direct ? 4u : 1u);
+    // offsets of all entries, and of the upper ones
+    k_scan<<<1, 1024, 0, c->stream>>>(cnt, pairs, offs);
     FD_LAUNCH_CHECK(c, "k_scan");
-    k_scan<<<1, 1024, 0, c->stream>>>(direct ? cnt : cnt + pairs, pairs, offs + pairs + 1);
-    FD_LAUNCH_CHECK(c, "k_scan");
-    c->listed_kind = kind; c->listed_beta = beta;
+    if (!direct) {
+        k_scan<<<1, 1024, 0, c->stream>>>(cnt + pairs, pairs, offs + pairs + 1);
+        FD_LAUNCH_CHECK(c, "k_scan");
+    }
+    listed.kind = held; listed.beta = beta;
     if (known) return FD_OK;
-    unsigned int total = 0, entries = 0;
+    unsigned int total = 0;
     FD_CUDA(c, cudaMemcpyAsync(&total, offs + pairs, 4, cudaMemcpyDeviceToHost, c->stream));
-    FD_CUDA(c, cudaMemcpyAsync(&entries, offs + 2 * pairs + 1, 4, cudaMemcpyDeviceToHost, c->stream));
     FD_CUDA(c, cudaStreamSynchronize(c->stream));
-    st.total = total; st.entries = entries;
-    // (direct-difference kernels: gathering through the order costs them more)
-    st.on = direct ? 4.0 * (double)total < 0.8 * (double)pairs * (double)tiles : (double)total < 0.9 * (double)pairs * (double)tiles;
+    st.total = total;
+    st.on = (double)total < (direct ? 0.8 : 0.9) * (double)pairs * (double)tiles;
     if (fresh && !st.on) {
         // nothing gained: the points keep the caller's order (a larger bandwidth may try again)
         c->order_state = 0;

@@ -506,7 +506,7 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
     // bandwidth too (once: the lists themselves are remade by the first product); any other pass returns without waiting and, at
     // a bandwidth that is not decided, runs over all tiles.
     if (prunes && a.decide && a.prec == FD_PREC_FP32 && c->lists[0].beta != a.beta) FD_TRY(tile_lists(c, a.beta, 0, true));
-    if (prunes) FD_TRY(tile_lists(c, a.beta, rowsum ? 1 : 0, a.decide));
+    if (prunes) FD_TRY(tile_lists(c, a.beta, !rowsum ? 0 : a.rowsq ? 1 : 3, a.decide));
     const bool use_lists = prunes && c->lists[rowsum ? 1 : 0].on && c->lists[rowsum ? 1 : 0].beta == a.beta;
     // The points' order is used, by every Gram-form pass, at the bandwidths that have lists (external rows against ordered columns: neighbouring
     // kernel values alike draw less power; N = 65536, 40009 rows of R^30, 33 vectors: 1.19 ms against 1.23).  At any other bandwidth a pass
@@ -555,7 +555,11 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
         p.weights = w;
     }
     if (rowsum && sym) {
-        FD_TRY(launch_sym_rowsum(c, mr, mc, p.weights, a.left, a.Y, a.rowsq, row_perm, use_lists));
+        // the pass with squares notes which tiles hold values that count, for the lists of the pass and the products after it
+        const bool note_near = ordered && a.rowsq && a.decide && !c->captured && (c->near_beta != a.beta || c->near_direct);
+        if (note_near) c->near_beta = -1.0;
+        FD_TRY(launch_sym_rowsum(c, mr, mc, p.weights, a.left, a.Y, a.rowsq, row_perm, use_lists, note_near));
+        if (note_near) { c->near_beta = a.beta; c->near_direct = false; }
     } else if (rowsum) {
         p.q = a.Y; p.rowsq = a.rowsq; p.b = 1;
         if (p.rowsq) FD_TRY((launch_tc<16>(c, mr, mc, p, grid)));
@@ -573,10 +577,9 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
             const int BT = bc <= 16 ? 16 : bc <= 32 ? 32 : bc <= 48 && !fast ? 48 : 64;
             if (BT > L.BP) return fail(c, FD_ERR_WORKSPACE, "column tile %d wider than the provisioned block buffers (%d)", BT, L.BP);
             const int cm_blocks = (int)std::min<int64_t>(256, ceil_div(N, 1024));
-            k_colmax_partial<<<dim3(cm_blocks, bc), 256, 0, c->stream>>>(a.V, a.ldv, vcols, a.right, N, c0, part);
+            k_colmax_partial<<<dim3(cm_blocks, bc), dim3(256), 0, c->stream>>>(a.V, a.ldv, vcols, a.right, N, c0, part);
             FD_LAUNCH_CHECK(c, "k_colmax_partial");
-            k_pack_wt<<<dim3((unsigned)std::min<int64_t>(1024, ceil_div(NP, 512)), BT), 256, 0, c->stream>>>(
-                a.V, a.ldv, vcols, a.right, N, NP, c0, bc, part, cm_blocks, inv, wt_hi, fast ? 0 : 1, col_perm);
+            k_pack_wt<<<dim3((unsigned)std::min<int64_t>(1024, ceil_div(NP, 512)), BT), dim3(256), 0, c->stream>>>(a.V, a.ldv, vcols, a.right, N, NP, c0, bc, (const float*)part, cm_blocks, inv, wt_hi, fast ? 0 : 1, col_perm);
             FD_LAUNCH_CHECK(c, "k_pack_wt");
             // one map over W_hi (rows 0 .. BT) and, in the fp32-grade mode, W_lo behind it (rows BT .. 2 BT of the same array)
             if (!make_map_2d(&mh, wt_hi, (uint64_t)NP, (uint64_t)(fast ? BT : 2 * BT), (uint64_t)NP * 2, 64, fast ? BT : 2 * BT, CU_TENSOR_MAP_SWIZZLE_128B))

@@ -96,6 +96,8 @@ struct BlockParams {
 
 // First step of CTA `cta` in the flat sequence of steps, and the work item (part of one row pair) that starts at step g of it.
 __host__ __device__ __forceinline__ long long range_begin(long long total, int cta, int ctas) { return total * cta / ctas; }
+// (a range without steps would leave its slots as they were: no more ranges than steps)
+__host__ __device__ __forceinline__ int range_count(long long total, int ctas) { return total < ctas ? (int)total : ctas; }
 struct Item { int pair, j0, n; bool whole; };
 // Row pair that holds step g of the lists.
 __device__ __forceinline__ int pair_of(const BlockParams& p, unsigned int g) {
@@ -113,10 +115,12 @@ struct Steps {                   // walks a CTA's range item by item
     __device__ __forceinline__ Steps(const BlockParams& p) {
         const bool listed = ORD && p.list;
         const long long total = listed ? (long long)p.offs[p.pairs] : (long long)p.pairs * p.num_jt;
-        const long long g0 = range_begin(total, (int)blockIdx.x, (int)gridDim.x);
+        const int ctas = range_count(total, (int)gridDim.x), cta = (int)blockIdx.x;
+        if (cta >= ctas) { pair = j0 = left = 0; return; }
+        const long long g0 = range_begin(total, cta, ctas);
         pair = listed ? pair_of(p, (unsigned int)g0) : (int)(g0 / p.num_jt);
         j0 = (int)(g0 - (listed ? (long long)p.offs[pair] : (long long)pair * p.num_jt));
-        left = (int)(range_begin(total, (int)blockIdx.x + 1, (int)gridDim.x) - g0);
+        left = (int)(range_begin(total, cta + 1, ctas) - g0);
     }
     __device__ __forceinline__ bool next(const BlockParams& p, Item& it) {
         if (left <= 0) return false;
@@ -490,6 +494,7 @@ k_block_fix(const BlockParams p, int ctas) {
     const long long total = p.list ? (long long)p.offs[p.pairs] : (long long)p.pairs * p.num_jt;
     const long long g0 = p.list ? (long long)p.offs[pair] : (long long)pair * p.num_jt;
     const long long g1 = p.list ? (long long)p.offs[pair + 1] : g0 + p.num_jt;
+    ctas = range_count(total, ctas);
     // the last CTA whose range begins at or before step g0
     int cta = (int)(((g0 + 1) * ctas - 1) / total);
     if (range_begin(total, cta + 1, ctas) >= g1) return;               // not cut: the CTA stored it
@@ -538,15 +543,16 @@ fd_status launch_one(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, co
         p.jt0 = j0;
         p.num_jt = std::min(jt_chunk, jt_total - j0);
         p.accumulate = j0 > 0;
-        const long long total = p.list ? c->lists[0].total : (long long)p.pairs * p.num_jt;
+        // (with lists the number of steps is known to the device only)
+        const long long total = (long long)p.pairs * p.num_jt;
         const int grid = (int)std::min<long long>(c->sm_count, total);
         if ((size_t)3 * grid * BT * 256 > c->L.part_floats) return fail(c, FD_ERR_WORKSPACE, "no room for the shares of cut row pairs");
-        kernel<<<grid, kThreadsB, smem, c->stream>>>(mr, mc, mw, p);
+        kernel<<<dim3((unsigned)grid), dim3(kThreadsB), (size_t)smem, c->stream>>>(mr, mc, mw, p);
         FD_LAUNCH_CHECK(c, "k_block");
         bool cut = p.list != nullptr;
         for (int i = 1; i < grid && !cut; ++i) cut = range_begin(total, i, grid) % p.num_jt != 0;
         if (cut) {
-            k_block_fix<BT><<<dim3((unsigned)p.pairs, (unsigned)ceil_div(p.b, 8)), 256, 0, c->stream>>>(p, grid);
+            k_block_fix<BT><<<dim3((unsigned)p.pairs, (unsigned)ceil_div(p.b, 8)), dim3(256), 0, c->stream>>>(p, grid);
             FD_LAUNCH_CHECK(c, "k_block_fix");
         }
     }
@@ -564,8 +570,8 @@ fd_status launch_block_product(fd_ctx* c, int BT, const CUtensorMap& mr, const C
     p.status = tp.status; p.part = c->at<float>(c->L.part);
     p.pairs = tp.num_work; p.K16 = tp.K16; p.b = tp.b; p.flush = tp.flush; p.perm = tp.perm;
     if (tp.use_lists) {
-        p.list = c->at<unsigned short>(c->L.lists);
-        p.offs = c->at<unsigned int>(c->L.list_counts) + 2 * p.pairs;
+        p.list = c->at<unsigned short>(c->L.lists[0]);
+        p.offs = c->at<unsigned int>(c->L.list_counts[0]) + 2 * p.pairs;
         p.tiles = (int)(c->L.NP / 128);
     }
     switch (BT) {

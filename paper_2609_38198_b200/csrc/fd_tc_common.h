@@ -215,7 +215,7 @@ fd_status launch_fast_product(fd_ctx* c, int BT, const CUtensorMap& mr, const CU
 // Row sums of the context's whole point set from the tiles on or above the diagonal (fd_tc_sym.cu): q = left * sum_j weights_j K_ij (no
 // weights: 1, and the total of rowsq's N entries is sum_ij K_ij^2).
 fd_status launch_sym_rowsum(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, const float* weights, const float* left, float* q,
-                            double* rowsq, const int* perm, bool use_lists);
+                            double* rowsq, const int* perm, bool use_lists, bool note_near);
 // fp32-grade block product of BT = 16, 32, 48 or 64 columns (fd_tc_block.cu).
 fd_status launch_block_product(fd_ctx* c, int BT, const CUtensorMap& mr, const CUtensorMap& mc, const CUtensorMap& mw,
                                const TcParams& tp);

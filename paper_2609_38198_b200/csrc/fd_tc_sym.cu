@@ -42,6 +42,8 @@ static_assert(kThreadsS * kRegsLaunch == 512 * kRegsExp + 128 * kRegsUtil, "setm
 constexpr int kSymFlush = 64;          // tiles between reductions of the resident sums
 constexpr int kXChunk = 128 * 64;      // one K slab (hi|lo) of 128 points: 8 KB
 constexpr int kSlots = 4;              // ring of streamed partial sums
+// 2^(bias - 40) and 2^(bias - 60), squared (a tenth below: the same value comes out of another kernel's accumulator as well)
+constexpr float kNearProduct2 = 0.9f * 0x1p-50f, kNearSums2 = 0.9f * 0x1p-90f;
 
 struct BarriersS {
     uint64_t full[kStages], empty[kStages];   // streamed tile: TMA -> Gram issuer -> TMA
@@ -62,6 +64,8 @@ struct SymParams {
     int pairs, num_jt, K16, shift;
     // tile lists (null: every tile): the streamed tiles of resident pair r are the last uoffs[r + 1] - uoffs[r] entries of its list
     const unsigned short* list; const unsigned int* counts; const unsigned int* uoffs;
+    // notes of the tiles that hold a value of the product's / the row sums' range, num_jt x num_jt bytes each (null: not wanted)
+    unsigned char* near_product; unsigned char* near_sums;
 };
 
 constexpr int smem_total(int K16) { return 1024 + kStages * K16 * kXChunk + 2 * K16 * kXChunk + kSlots * 4 * 128 * 4 + 1024; }
@@ -130,7 +134,7 @@ template <> struct Steps<true> {
     }
 };
 
-template <bool SQ, bool WEIGHTED, bool LISTED>
+template <bool SQ, bool WEIGHTED, bool LISTED, bool NOTED>
 __global__ void __launch_bounds__(kThreadsS, 1)
 k_sym(const __grid_constant__ CUtensorMap map_res, const __grid_constant__ CUtensorMap map_str, const SymParams p) {
     extern __shared__ uint8_t smem_raw[];
@@ -327,6 +331,15 @@ k_sym(const __grid_constant__ CUtensorMap map_res, const __grid_constant__ CUten
                     const float2 qp = split2(q2);
                     const float q = qp.x + qp.y;
                     dsq += (double)q * (both ? 2.0 : 1.0);
+                    if (NOTED) {
+                        // a value at or above a limit shows in its thread's sum of squares
+                        const bool sums = __any_sync(0xffffffffu, q >= kNearSums2), product = __any_sync(0xffffffffu, q >= kNearProduct2);
+                        if (lane == 0 && sums) {
+                            const size_t a = (size_t)It * p.num_jt + J, b = (size_t)J * p.num_jt + It;
+                            p.near_sums[a] = 1; p.near_sums[b] = 1;
+                            if (product) { p.near_product[a] = 1; p.near_product[b] = 1; }
+                        }
+                    }
                 }
                 if (use) ++pending;
                 if (pending == kSymFlush || (j + 1 == it.n && pending > 0)) {
@@ -390,7 +403,9 @@ template <bool SQ, bool WEIGHTED>
 fd_status launch_one(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, const SymParams& p, int grid) {
     const int smem = smem_total(p.K16);
     // the attribute is per device: set it on every launch (cheap) rather than remembering one device
-    const auto kernel = p.list ? k_sym<SQ, WEIGHTED, true> : k_sym<SQ, WEIGHTED, false>;
+    // (notes are taken by the pass with squares only)
+    const auto kernel = p.near_sums ? (p.list ? k_sym<SQ, WEIGHTED, true, SQ> : k_sym<SQ, WEIGHTED, false, SQ>)
+                                    : (p.list ? k_sym<SQ, WEIGHTED, true, false> : k_sym<SQ, WEIGHTED, false, false>);
     FD_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     cudaFuncAttributes fa;
     FD_CUDA(c, cudaFuncGetAttributes(&fa, kernel));
@@ -406,7 +421,7 @@ fd_status launch_one(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, co
 namespace tc {
 
 fd_status launch_sym_rowsum(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, const float* weights, const float* left, float* q, double* rowsq,
-                            const int* perm, bool use_lists) {
+                            const int* perm, bool use_lists, bool note_near) {
     const Layout& L = c->L;
     SymParams p{};
     p.N = L.N; p.np = L.NP; p.K16 = L.K16;
@@ -419,9 +434,15 @@ fd_status launch_sym_rowsum(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap&
     p.shift = 61 - kBias - lg;
     FD_CUDA(c, cudaMemsetAsync(p.sums, 0, (size_t)L.N * 8, c->stream));
     if (use_lists) {
-        p.list = c->at<unsigned short>(L.lists);
-        p.counts = c->at<unsigned int>(L.list_counts);
+        p.list = c->at<unsigned short>(L.lists[1]);
+        p.counts = c->at<unsigned int>(L.list_counts[1]);
         p.uoffs = p.counts + 3 * p.pairs + 1;
+    }
+    if (note_near) {
+        const size_t plane = (size_t)p.num_jt * p.num_jt;
+        p.near_product = c->at<unsigned char>(L.near);
+        p.near_sums = p.near_product + plane;
+        FD_CUDA(c, cudaMemsetAsync(p.near_product, 0, 2 * plane, c->stream));
     }
     // (every pair's own two tiles are listed: there are at least two steps per pair)
     const int grid = (int)std::min<long long>(std::min<long long>(c->sm_count, L.N), use_lists ? 2ll * p.pairs : steps_before(p.pairs, p.num_jt));
