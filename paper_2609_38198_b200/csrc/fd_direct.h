@@ -41,9 +41,12 @@ __device__ __forceinline__ void kernel_values(const float4* sx, int jj, const fl
     for (int r = 0; r < R; ++r) kij[r] = ex2_approx(h[r] * nbeta2);
 }
 
-// Sums of BT columns for R rows.  add(): sum[r][c] += kij[r] w[c].
+// Sums of BT columns for R rows.  add(): sum[r][c] += kij[r] w[c].  64 columns use packed arithmetic (two columns an instruction: half the issue
+// slots, the same time on the FMA pipe): N = 12000, D = 4: 744 -> 627 us a product.  Narrower blocks are 2 to 8 % slower with it.
+template <int R, int BT, bool PACKED = (BT > 48)>
+struct Sums;
 template <int R, int BT>
-struct Sums {
+struct Sums<R, BT, false> {
     float v[R][BT];
     __device__ __forceinline__ void clear() {
 #pragma unroll
@@ -66,6 +69,34 @@ struct Sums {
     }
     __device__ __forceinline__ float get(int r, int c) const { return v[r][c]; }
 };
+template <int R, int BT>
+struct Sums<R, BT, true> {
+    uint64_t v[R][BT / 2];
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < BT / 2; ++c) v[r][c] = 0;
+    }
+    __device__ __forceinline__ void add(const float (&kij)[R], const float4* w) {
+        uint64_t kk[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) kk[r] = pair2(kij[r], kij[r]);
+#pragma unroll
+        for (int c4 = 0; c4 < BT / 4; ++c4) {
+            const ulonglong2 w4 = reinterpret_cast<const ulonglong2*>(w)[c4];
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r][2 * c4] = fma2(kk[r], w4.x, v[r][2 * c4]);
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r][2 * c4 + 1] = fma2(kk[r], w4.y, v[r][2 * c4 + 1]);
+        }
+    }
+    __device__ __forceinline__ float get(int r, int c) const {
+        const float2 a = split2(v[r][c / 2]);
+        return c & 1 ? a.y : a.x;
+    }
+};
+
 }  // namespace direct
 
 }  // namespace fd
