@@ -21,6 +21,8 @@
 // 136 -> 109 us (one row per thread, separate packing pass, one CTA more or less per SM at the end).
 //
 // Up to 8 coordinates, from 16384 points on, passes over the whole point set may run over tile lists instead: fd_direct_listed.cu.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "fd_direct.h"
@@ -337,6 +339,102 @@ k_direct_rowsum_fix(const DirectParams p, int ctas) {
     p.Y[i] = (float)(v.x * (p.left ? (double)p.left[i] : 1.0));
 }
 
+// Block mode of small problems: a cluster of eight CTAs per 64 rows, a CTA an eighth of the columns, a warp an eighth of those; the sums
+// meet in shared memory, first the warps' of each CTA, then the CTAs' through the cluster.  One launch and no shares in memory: N = 2048 cut into
+// 512 ranges of the kernel above writes 4 MB of them for a second kernel to add.
+constexpr int kSmallRows = 64, kSmallThr = 256, kSmallCtas = 8;
+template <int DP4, int BT>
+__global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThr)
+k_direct_small(const DirectParams p) {
+    constexpr int BP = BT + 4, kWarps = kSmallThr / 32, R = kSmallRows / 32;
+    constexpr int kStage = kSmallThr * (4 * DP4 + BP), kRed = kWarps * BT * kSmallRows;
+    __shared__ __align__(16) float smem[kStage > kRed ? kStage : kRed];
+    __shared__ float total[BT * kSmallRows];             // [column][row]
+    float4* sx = reinterpret_cast<float4*>(smem);
+    float* sw = smem + kSmallThr * 4 * DP4;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rank = (int)blockIdx.x % kSmallCtas;
+    const int64_t row0 = (int64_t)(blockIdx.x / kSmallCtas) * kSmallRows;
+    const int64_t per = (p.N + kSmallCtas - 1) / kSmallCtas, j_end = per * (rank + 1) < p.N ? per * (rank + 1) : p.N;
+    float4 xi[R][DP4];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int64_t i = row0 + lane + 32 * r;
+#pragma unroll
+        for (int k = 0; k < DP4; ++k) xi[r][k] = i < p.Nrow ? p.xrow[i * DP4 + k] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float sum[R][BT];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int c = 0; c < BT; ++c) sum[r][c] = 0.f;
+    for (int64_t j0 = per * rank; j0 < j_end; j0 += kSmallThr) {
+        const int n = (int)(j_end - j0 < kSmallThr ? j_end - j0 : kSmallThr), t = threadIdx.x;
+        __syncthreads();
+        if (t < n) {
+            float w[BT];
+#pragma unroll
+            for (int c = 0; c < BT; ++c) w[c] = c < p.b ? (c < p.vcols ? p.V[j0 + t + (int64_t)c * p.ldv] : 1.f) : 0.f;
+            const float right = p.right ? p.right[j0 + t] : 1.f;
+#pragma unroll
+            for (int k = 0; k < DP4; ++k) sx[t * DP4 + k] = p.xcol[(j0 + t) * DP4 + k];
+#pragma unroll
+            for (int c = 0; c < BT; ++c) sw[t * BP + c] = w[c] * right;
+        }
+        __syncthreads();
+        const int jj0 = n * warp / kWarps, jj1 = n * (warp + 1) / kWarps;
+        // (sums of eight columns, then of those: neighbouring points' large values do not meet the far ones' small ones in one long sum)
+        auto column = [&](Sums<R, BT>& acc, int jj) {
+            float kij[R];
+            kernel_values<DP4, R>(sx, jj, xi, p.nbeta2, kij);
+            acc.add(kij, reinterpret_cast<const float4*>(&sw[jj * BP]));
+        };
+        int jj = jj0;
+        while (jj < jj1) {
+            Sums<R, BT> acc;
+            acc.clear();
+            if (jj + 8 <= jj1) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) column(acc, jj + u);
+                jj += 8;
+            } else {
+#pragma unroll 1
+                for (; jj < jj1; ++jj) column(acc, jj);
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int c = 0; c < BT; ++c) sum[r][c] += acc.get(r, c);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int c = 0; c < BT; ++c) smem[(warp * BT + c) * kSmallRows + lane + 32 * r] = sum[r][c];
+    __syncthreads();
+    for (int e = threadIdx.x; e < BT * kSmallRows; e += kSmallThr) {
+        float x = 0.f;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) x += smem[w * BT * kSmallRows + e];
+        total[e] = x;
+    }
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    cluster.sync();
+    // every CTA finishes an eighth of the 64 x BT sums
+    for (int t = threadIdx.x; t < BT * kSmallRows / kSmallCtas; t += kSmallThr) {
+        const int e = rank * (BT * kSmallRows / kSmallCtas) + t, c = e / kSmallRows;
+        float v[kSmallCtas];
+#pragma unroll
+        for (int q = 0; q < kSmallCtas; ++q) v[q] = *cluster.map_shared_rank(&total[e], q);
+        const int64_t i = row0 + e % kSmallRows;
+        if (c < p.b && i < p.Nrow) {
+            const float x = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+            p.Y[i + (int64_t)c * p.ldy] = x * (p.left ? p.left[i] : 1.0f);
+        }
+    }
+    cluster.sync();                                      // (a CTA's sums stay until the others have read them)
+}
+
 // Launches one CTA per equal range of steps: as many as are resident at once (more would leave a last round partly filled), or as
 // asked (option "splits": ranges per row tile), within the slots' capacity.
 template <class Kernel>
@@ -372,8 +470,18 @@ int resident(Kernel kernel, int smem) {              // a property of the compil
     return std::min(n, kMaxCtasPerSm);
 }
 
+// Widest set that goes to the cluster kernel.  Against the ranges above: N = 1000, b = 8: 18.0 -> 12.8 us; 2048: 15.5 -> 10.9; 4096: 25.8 -> 23.8; 6000: 44 -> 40
+// with sums of one level, which the larger sets' accuracy does not allow; b = 16, N = 2048: 19.7 -> 13.3, 4096: 34.7 -> 36.5.
+constexpr int64_t small_n(int BT) { return BT <= 8 ? 4096 : 2048; }
+
 template <int DP4, int BT>
 fd_status launch_block(fd_ctx* c, const DirectParams& p) {
+    if constexpr (DP4 <= 2 && BT <= 16)
+        if (p.N <= small_n(BT) && p.Nrow <= small_n(BT) && c->opt_splits <= 0) {
+            k_direct_small<DP4, BT><<<dim3((unsigned)(kSmallCtas * ceil_div(p.Nrow, kSmallRows))), dim3(kSmallThr), 0, c->stream>>>(p);
+            FD_LAUNCH_CHECK(c, "k_direct_small");
+            return FD_OK;
+        }
     constexpr int R = 4 * DP4 + BT <= 32 ? 4 : 2, H = R * kThr / kRowsT;
     constexpr int smem = (kTJ * DP4 * 4 + kTJ * (BT + 4) + H * BT * kRowsT) * 4;
     static const int per_sm = resident(k_direct<DP4, BT, R>, smem);

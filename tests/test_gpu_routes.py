@@ -1,4 +1,4 @@
-"""Routes chosen by size: products over the tiles that hold near pairs."""
+"""Routes chosen by size: narrow products of small sets in one launch, products over the tiles that hold near pairs."""
 import numpy as np
 import pytest
 import torch
@@ -24,6 +24,32 @@ def dev():
 
 def _kernel_rows(Zd, Xd, beta):
     return torch.exp(-beta * torch.cdist(Zd, Xd, compute_mode="donot_use_mm_for_euclid_dist") ** 2)
+
+
+@pytest.mark.parametrize("N,D,b", [(1, 1, 1), (3, 2, 4), (7, 5, 8), (63, 4, 16), (64, 8, 3), (65, 3, 9), (255, 2, 8), (257, 7, 16), (2047, 2, 8),
+                                   (2048, 3, 16), (2049, 4, 16), (4095, 2, 1), (4096, 4, 8), (4097, 4, 8)])
+def test_small_narrow_products(fd, dev, N, D, b):
+    """Up to 4096 points with up to 8 coordinates and 8 columns (2048 and 16): one launch, sums inside a cluster.  Square products with scalings on both sides, a
+    right block and an output with a pitch of their own, external rows, a replay from a graph.  Gate 1e-6 of the direct-difference family."""
+    rng = np.random.default_rng(N + 7 * b)
+    X = torch.from_numpy(rng.standard_normal((N, D)).astype(np.float32)).to(dev)
+    beta, ld = 0.7, N + 5
+    V = torch.empty((b, ld), device=dev)[:, 3:3 + N].t()
+    V.copy_(torch.from_numpy(rng.standard_normal((N, b)).astype(np.float32)))
+    left, right = (torch.rand(N, device=dev) + 0.5 for _ in range(2))
+    Xd, Vd = X.double(), V.double()
+    ctx = fd.Context(X, b_max=b)
+    Y = torch.zeros((b, ld), device=dev)[:, 2:2 + N].t()
+    ctx.apply_general(beta, V, left=left, right=right, out=Y)
+    ref = left.double()[:, None] * (_kernel_rows(Xd, Xd, beta) @ (right.double()[:, None] * Vd))
+    assert ctx.get_option("last_path") == fd.FD_PATH_SIMT
+    assert ((Y.double() - ref).norm() / ref.norm()).item() <= 1e-6
+    for M in (1, min(N, 33), min(N, 129)):
+        Z = X[:M].contiguous() + 0.01
+        R = ctx.apply_general(beta, V, Xrow=Z)
+        Ro = _kernel_rows(Z.double(), Xd, beta) @ Vd
+        assert ((R.double() - Ro).norm() / Ro.norm()).item() <= 1e-6
+    ctx.close()
 
 
 @pytest.mark.parametrize("kind", ["direct", "gram"])
