@@ -5,8 +5,10 @@
 //   1. Gram MMA of augmented fp16 hi|lo points: the tile leaves the tensor core as the base-2 exponent
 //        S_ij = 2 b' x_i.x_j - b' r_i - b' r_j + bias      (Eq. 4; the norms ride as extra K columns)
 //      into one of three 128-column TMEM buffers.
-//   2. Exponential warps (thread = row, 64 columns each) read S, take 2^S on the MUFU, round P to fp16 and write it
-//      back IN PLACE as the TMEM A operand of the product.
+//   2. Exponential warps (thread = row, 64 columns each) read S, take 2^S, round P to fp16 and write it back IN PLACE as the TMEM A operand of
+//      the product.  A quarter of the exponentials run on the FMA pipe (a polynomial), the others on the MUFU, which bounds the kernel
+//      otherwise (1024 of 1080 SM clocks a tile): N = 65536, b = 64: 1352 -> 1180 us, N = 2^18: 18.6 -> 17.9 ms (power); an eighth: 1243 us and
+//      18.1 ms.  The error is that of the single fp16 operands, 2.44e-4 and 2.69e-4, with and without.
 //   3. Product MMA per 16-column K step:  Y += P W  with W = diag(right) V in fp16, fp32 accumulation in TMEM.
 //   4. Every `flush` column tiles a separate warpgroup adds Y into fp32 registers and the accumulator restarts, so
 //      tensor-core accumulation error does not grow with N.
@@ -35,6 +37,8 @@ namespace fd {
 namespace {
 
 using namespace tc;
+
+constexpr int kFmaPairs = 2;      // of eight pairs of columns, those whose exponentials run on the FMA pipe
 
 constexpr int kThreadsBp = 768;
 constexpr int kRegsLaunch = 80, kRegsExp = 72, kRegsFlush = 152, kRegsUtil = 40;
@@ -331,9 +335,9 @@ k_bp(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CUten
                             uint32_t hi[8];
 #pragma unroll
                             for (int i = 0; i < 8; ++i) {
-                                const float p0 = ex2f(__uint_as_float(sv[16 * ch + 2 * i]));
-                                const float p1 = ex2f(__uint_as_float(sv[16 * ch + 2 * i + 1]));
-                                hi[i] = pack_f16x2(p0, p1);
+                                const float x0 = __uint_as_float(sv[16 * ch + 2 * i]), x1 = __uint_as_float(sv[16 * ch + 2 * i + 1]);
+                                const float2 e = i >= 8 - kFmaPairs ? ex2_fma2(x0, x1) : make_float2(ex2f(x0), ex2f(x1));
+                                hi[i] = pack_f16x2(e.x, e.y);
                             }
                             tmem_st8(addr + 32 * q32 + 16 * ch, hi);
                         }
