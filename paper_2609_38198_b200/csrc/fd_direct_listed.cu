@@ -10,7 +10,7 @@
 // What bounds it: instruction issue, 2 D + b + 2 FMA-pipe operations per pair (N = 16384, D = 4, b = 16: about 60 % of the issue slots).  Against
 // steps of 256 rows x 64 points gathered through the order, by a whole block and from boxes alone: 2-torus, N = 16384, beta = 100, b = 16: 134 -> 69 us
 // a product (0.34 -> 0.17 of the tiles), both degree passes 164 -> 125; beta = 30: 310 (all tiles; not worth lists then) -> 157; N = 65536,
-// b = 32, beta = 100: 1805 -> 1046.  The error against float64 fell from 1.8e-7 to 1.4e-7 and from 4.3e-7 to 2.1e-7: short first sums.
+// b = 32, beta = 100: 1805 -> 1046.  Error against float64: 1.75e-7 -> 1.32e-7, 1.43e-7 -> 1.48e-7 and 4.3e-7 -> 2.1e-7 (short first sums).
 #include <algorithm>
 
 #include "fd_direct.h"
@@ -153,7 +153,7 @@ k_near(const NearParams p) {
         // Two-level sums: the points are in their order, so one long fp32 sum would add the far points' small values to the near ones' large sum and
         // drop them, always with the same sign.  Up to 16 columns the second level is in registers, for wider blocks in the warp's slot.
         constexpr bool kInRegs = BT <= 16;
-        constexpr int kFlush = kInRegs ? 2 : 4;                    // entries between flushes
+        constexpr int kFlush = kInRegs ? 2 : 8;                    // entries between flushes (4 to memory: 1046 -> 1127 us at N = 65536, b = 32)
         float sum[kRows][kInRegs ? BT : 1];
         if (kInRegs) {
 #pragma unroll
