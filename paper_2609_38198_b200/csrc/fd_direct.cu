@@ -470,9 +470,9 @@ int resident(Kernel kernel, int smem) {              // a property of the compil
     return std::min(n, kMaxCtasPerSm);
 }
 
-// Widest set that goes to the cluster kernel.  Against the ranges above: N = 1000, b = 8: 18.0 -> 12.8 us; 2048: 15.5 -> 10.9; 4096: 25.8 -> 23.8; 6000: 44 -> 40
-// with sums of one level, which the larger sets' accuracy does not allow; b = 16, N = 2048: 19.7 -> 13.3, 4096: 34.7 -> 36.5.
-constexpr int64_t small_n(int BT) { return BT <= 8 ? 4096 : 2048; }
+// Largest set that goes to the cluster kernel.  Against the ranges above: N = 1000, b = 8: 18.0 -> 8.8 us; 2048: 15.5 -> 11.3; 4096: 25.5 -> 25.3; b = 16,
+// N = 2048: 19.4 -> 11.7, 4096: 34.7 -> 36.5.
+constexpr int64_t small_n(int BT) { return BT <= 8 ? 3072 : 2048; }
 
 template <int DP4, int BT>
 fd_status launch_block(fd_ctx* c, const DirectParams& p) {

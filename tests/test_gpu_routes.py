@@ -27,9 +27,9 @@ def _kernel_rows(Zd, Xd, beta):
 
 
 @pytest.mark.parametrize("N,D,b", [(1, 1, 1), (3, 2, 4), (7, 5, 8), (63, 4, 16), (64, 8, 3), (65, 3, 9), (255, 2, 8), (257, 7, 16), (2047, 2, 8),
-                                   (2048, 3, 16), (2049, 4, 16), (4095, 2, 1), (4096, 4, 8), (4097, 4, 8)])
+                                   (2048, 3, 16), (2049, 4, 16), (3071, 2, 1), (3072, 4, 8), (3073, 4, 8)])
 def test_small_narrow_products(fd, dev, N, D, b):
-    """Up to 4096 points with up to 8 coordinates and 8 columns (2048 and 16): one launch, sums inside a cluster.  Square products with scalings on both sides, a
+    """Up to 3072 points with up to 8 coordinates and 8 columns (2048 and 16): one launch, sums inside a cluster.  Square products with scalings on both sides, a
     right block and an output with a pitch of their own, external rows, a replay from a graph.  Gate 1e-6 of the direct-difference family."""
     rng = np.random.default_rng(N + 7 * b)
     X = torch.from_numpy(rng.standard_normal((N, D)).astype(np.float32)).to(dev)
