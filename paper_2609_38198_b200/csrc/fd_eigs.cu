@@ -121,15 +121,17 @@ struct Solver {
         return fetch(cnt);
     }
 
-    // W[:, c0 : c0 + n) = M Q[:, c0 : c0 + n), in blocks of at most bw columns.  Nothing waits for the products here: their time is read
+    // W[:, c0 : c0 + n) = M Q[:, c0 : c0 + n).
+    fd_status apply_cols(int c0, int cnt, int bw) { return apply_block(Q + (int64_t)c0 * N, W + (int64_t)c0 * N, cnt, bw); }
+    // out = M B for cnt columns, in blocks of at most bw.  Nothing waits for the products here: their time is read
     // after the wait of the projection that follows.
-    fd_status apply_cols(int c0, int cnt, int bw) {
+    fd_status apply_block(float* B, float* out, int cnt, int bw) {
         FD_CUDA(c, cudaEventRecord(c->apply_ev[0], c->stream));
-        FD_TRY(gather_rows(c, Q + (int64_t)c0 * N, N, cnt));         // the product needs all rows of the right block
+        FD_TRY(gather_rows(c, B, N, cnt));                           // the product needs all rows of the right block
         for (int o = 0; o < cnt; o += bw) {
             int w = std::min(bw, cnt - o);
-            FD_TRY(apply_general(c, c->beta, c->s(), c->s(), false, nullptr, N, 0, Q + (int64_t)(c0 + o) * N, N, w,
-                                 W + (int64_t)(c0 + o) * N, N, c->eigs_prec, /*gather_out=*/false));
+            FD_TRY(apply_general(c, c->beta, c->s(), c->s(), false, nullptr, N, 0, B + (int64_t)o * N, N, w,
+                                 out + (int64_t)o * N, N, c->eigs_prec, /*gather_out=*/false));
             ++applies;
         }
         // (looked at after the next projection's wait)
@@ -283,11 +285,12 @@ struct Solver {
     }
 
     // Orthonormalises the block B (p <= BP columns, not inside Q's first m columns) against the basis and within itself; the
-    // result goes to Q[:, m ..) and p is updated (0: nothing new).  z: [Q B]^T B of pitch ldz if the caller has it, else null.
+    // result goes to `target` and p is updated (0: nothing new).  other: scratch of the same size (B may be it).
+    // z: [Q B]^T B of pitch ldz if the caller has it, else null.
     //   1. R = (B - Q C) scaled to unit columns: removes the basis to fp32 rounding of B's own size;
     //   2. Q_new = (R - Q C') F with C' = Q^T R (small now) and F from R^T R - C'^T C', which is accurate because C' is small;
     //   3. once more if the block was nearly dependent, so that step 2's rounding was magnified.
-    fd_status expand(const float* B, int& p, const double* z, int ldz) {
+    fd_status expand(const float* B, int& p, const double* z, int ldz, float* target, float* other) {
         if (p == 0) return FD_OK;
         std::vector<double> F;
         if (!z) {
@@ -302,7 +305,7 @@ struct Solver {
             const double left = std::max(d - cc, 1e-12 * d);      // |column|^2 after the projection (floor: cancellation)
             F[j + (size_t)j * p] = left > 1e-60 ? 1.0 / std::sqrt(left) : 0.0;
         }
-        float* dst = B == R ? Q + (int64_t)m * N : R;
+        float* dst = B == other ? target : other;
         FD_TRY(subtract_and_mix(B, p, z, ldz, F.data(), p, dst));
         for (int pass = 0; pass < 2; ++pass) {
             const float* src = dst;
@@ -321,14 +324,15 @@ struct Solver {
             int rank; double lam_min;
             FD_TRY(orthonormal_factor(g.data(), p, pass == 0 ? 1e-5 : 1e-3, F, rank, lam_min));
             if (rank == 0) { p = 0; return FD_OK; }
-            dst = src == R ? Q + (int64_t)m * N : R;
+            dst = src == other ? target : other;
             FD_TRY(subtract_and_mix(src, p, h, ld, F.data(), rank, dst));
             p = rank;
             if (pass == 0 && lam_min > 1e-2 && cmax < 1e-2) break;
         }
-        if (dst == R) FD_TRY(copy_cols(c, R + r0, N, Q + (int64_t)m * N + r0, N, p, n));
+        if (dst == other) FD_TRY(copy_cols(c, other + r0, N, target + r0, N, p, n));
         return FD_OK;
     }
+    fd_status expand(const float* B, int& p, const double* z, int ldz) { return expand(B, p, z, ldz, Q + (int64_t)m * N, R); }
 };
 
 }  // namespace
@@ -416,8 +420,22 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
     const bool small_basis = m_cap < 3 * nwant && m_cap < N;
     const int kMaxBlocks = small_basis ? 1 : 4;
     const bool wanted_first = !small_basis;
-    double last_worst = 0.0;
+    // Ritz vectors kept at a restart: three fifths of the basis or, where twice the wanted pairs are less, as many above that as leave room for whole
+    // blocks: a group of blocks more between two restarts for as many products in all (6-torus, N = 2^17, k = 64: 11 -> 8 restarts, 293 -> 282 ms;
+    // N = 86893, k = 40: 19 -> 12, 153 -> 133 ms; 2-torus, N = 16384, k = 25: 20 -> 12, 28.5 -> 23.5 ms).
+    const int restart_keep = small_basis || 2 * nwant > (m_cap * 3) / 5 ? (m_cap * 3) / 5 : m_cap - (m_cap - 2 * nwant) / b * b;
+    double last_worst = 0.0, last_rate = 0.0;
     int last_applies = 0;
+    // The block after the last one before a Rayleigh-Ritz step is made, and M applied to it, while the host solves the projected
+    // eigenproblem: the residuals of all Ritz vectors lie in its span, so it is the next expansion whatever that step decides.  It
+    // waits in R and its image in the extension's scratch: the basis may be full.  Only while the blocks are a Krylov sequence (cold starts,
+    // no direction dropped), and while the residuals are expected to stay well above the tolerance: a solve's last steps take
+    // explicit residuals, which also see what the stored images have lost to rounding.  6-torus, N = 2^17, k = 64: 323 -> 293 ms, N = 86893, k = 40:
+    // 185 -> 152; R^30, N = 65536, k = 32: 38 -> 32; 2-torus, N = 16384, k = 32: 29.1 -> 26.3 (as many products but for one or two).
+    constexpr double kAhead = 100.0;
+    bool krylov = !Q0_dev && !small_basis;
+    float* const ahead_image = c->at<float>(L.wp);
+    int ahead = 0;
     // The stored images drift from M Q: a restart rounds Q S and W S separately, and what they differ by ends up in every residual (0.3e-6 to
     // 0.9e-6 after 20 to 100 restarts).  Where the worst wanted residual has not improved by 10 % over kStall products within twice the
     // tolerance, the next restart applies M to the kept basis again.  6-torus, N = 30000, k = 64, capacity 259: 65 of 65 pairs instead of a
@@ -448,7 +466,7 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
         auto tp1 = clk::now();
         // eigenvectors: the leading Ritz vectors on every step; the larger kept set only when this step may restart
         const int nvec_ritz = std::min(nsel_max, m);
-        const int nvec = (m + b > m_cap) ? std::max(nvec_ritz, std::min(m - 1, (m_cap * 3) / 5)) : nvec_ritz;
+        const int nvec = (m + b > m_cap) ? std::max(nvec_ritz, std::min(m - 1, restart_keep)) : nvec_ritz;
         if (!sym_eig(Tc.data(), m, lam, U, nvec)) return fail(c, FD_ERR_NOT_CONVERGED, "projected eigenproblem failed");
         auto tp2 = clk::now();
         t_rr += secs(tp0, tp1); t_eig += secs(tp1, tp2);
@@ -516,8 +534,8 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
                 else since_best += S.applies - last_applies;
                 // the worst residual's decay per product since the last step tells how many products are left
                 if (last_worst > worst && worst > thr) {
-                    const double rate = std::log(last_worst / worst) / std::max(1, S.applies - last_applies);
-                    blocks = std::max(1, std::min(kMaxBlocks, (int)std::ceil(std::log(worst / thr) / rate)));
+                    last_rate = std::log(last_worst / worst) / std::max(1, S.applies - last_applies);
+                    blocks = std::max(1, std::min(kMaxBlocks, (int)std::ceil(std::log(worst / thr) / last_rate)));
                 }
                 last_worst = worst;
                 last_applies = S.applies;
@@ -538,16 +556,20 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
             return wa != wb ? wa : resid[a] > resid[bb];
         });
         const int want_new = (int)std::min<int64_t>(b, N - m);
-        std::vector<int> pick;
-        for (int i = 0; i < nsel && (int)pick.size() < want_new; ++i)
-            if (order[i] >= first && resid[order[i]] > 0.1 * thr) pick.push_back(order[i] - first);
-        if (pick.empty()) { final_status = FD_OK; break; }
-        int p = (int)pick.size();
-        FD_TRY(gather_cols(c, S.X + r0, S.R + r0, N, pick.data(), p, n));
+        int p = ahead;
+        if (ahead == 0) {
+            std::vector<int> pick;
+            for (int i = 0; i < nsel && (int)pick.size() < want_new; ++i)
+                if (order[i] >= first && resid[order[i]] > 0.1 * thr) pick.push_back(order[i] - first);
+            if (pick.empty()) { final_status = FD_OK; break; }
+            p = (int)pick.size();
+            krylov = krylov && p == b;
+            FD_TRY(gather_cols(c, S.X + r0, S.R + r0, N, pick.data(), p, n));
+        }
 
         // ---- thick restart when the new block would not fit ----------------------------------------
         if (m + p > m_cap) {
-            int keep = std::max(nsel, std::min(m - 1, (m_cap * 3) / 5));
+            int keep = std::max(nsel, std::min(m - 1, restart_keep));
             keep = std::min(keep, m_cap - p);
             keep = std::min(keep, m);
             // Ritz vectors for the kept block (beyond nsel use the uncorrected eigenvectors)
@@ -587,7 +609,13 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
         bool stuck = false;
         for (int blk = 0; blk < blocks; ++blk) {
             auto tb0 = clk::now();
-            FD_TRY(S.expand(B, p, z, ldz));
+            const bool have_image = ahead > 0;
+            if (have_image) {
+                FD_TRY(copy_cols(c, S.R + r0, N, S.Q + (int64_t)S.m * N + r0, N, p, n));
+                FD_TRY(copy_cols(c, ahead_image + r0, N, S.W + (int64_t)S.m * N + r0, N, p, n));
+                ahead = 0;
+            } else FD_TRY(S.expand(B, p, z, ldz));
+            krylov = krylov && p == b;
             if (p == 0) {
                 if (blk > 0) break;                                // the continuation added nothing: back to the Ritz pairs
                 // the residuals lie (numerically) inside the basis: try a random direction, give up after a few
@@ -599,7 +627,7 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
             }
             auto tb1 = clk::now();
             t_orth += secs(tb0, tb1);
-            FD_TRY(S.apply_cols(S.m, p, b));
+            if (!have_image) FD_TRY(S.apply_cols(S.m, p, b));
             auto tb2 = clk::now();
             FD_TRY(S.extend_projection(p));
             t_ext += secs(tb2, clk::now());
@@ -611,6 +639,16 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
             z = zkeep.data();
         }
         if (stuck) break;
+        // ---- the next block, ahead of the step that decides ----------------------------------------
+        if (krylov && p == b && nsel >= nwant && S.m + b <= N && S.applies + 1 < max_applies &&
+            last_worst * std::exp(-last_rate * (S.applies - last_applies)) > kAhead * tol * std::fabs(theta[0])) {
+            ldz = S.m + p;
+            zkeep.assign(S.h + (size_t)p * ldz, S.h + (size_t)2 * p * ldz);
+            FD_TRY(S.expand(S.W + (int64_t)(S.m - p) * N, p, zkeep.data(), ldz, S.R, S.X));
+            krylov = p == b;
+            if (p > 0) FD_TRY(S.apply_block(S.R, ahead_image, p, b));
+            ahead = p;
+        }
     }
 
     // ---- outputs: evecs = Q X[:, 0 : k + 1) ----------------------------------------------------------

@@ -1,4 +1,5 @@
-"""Routes chosen by size: narrow products of small sets in one launch, products over the tiles that hold near pairs."""
+"""Routes chosen by size: narrow products of small sets in one launch, products over the tiles that hold near pairs, solves with blocks of
+many widths."""
 import numpy as np
 import pytest
 import torch
@@ -79,3 +80,31 @@ def test_products_over_noted_tiles(fd, dev, kind, N):
     assert torch.equal(ctx.degree(beta, 1.0)[2], s) and ctx.get_option("tile_share") == share
     assert torch.equal(ctx.apply_general(beta, V, left=s, right=s), Y)
     ctx.close(); plain.close()
+
+
+@pytest.mark.parametrize("N,k,b,m_max", [(24, 5, 7, 24), (65, 12, 16, 65), (300, 20, 1, 64), (300, 9, 33, 96), (700, 30, 64, 224), (900, 20, 70, 210),
+                                         (512, 8, 16, 59)])
+def test_solves_with_blocks_of_many_widths(fd, dev, N, k, b, m_max):
+    """Blocks of one to 70 columns, bases that leave room for one block or for several beside twice the wanted pairs and bases that span everything.
+    Eigenvalues to 1e-6, residuals in float64 to 5e-6, vectors orthonormal to 1e-5, against the dense matrix; the same from a warm start
+    (no block ahead of the Rayleigh-Ritz step there)."""
+    X = workloads.latent_torus(N, seed=42)
+    beta = 0.6
+    Xd = torch.from_numpy(X).to(dev).double()
+    K = _kernel_rows(Xd, Xd, beta)
+    q = K.sum(1)
+    d = (K @ (1.0 / q)) / q
+    s = 1.0 / (q * d.sqrt())
+    M = s[:, None] * K * s[None]
+    lam = torch.linalg.eigvalsh(M).flip(0)[:k + 1].cpu().numpy()
+    ctx = fd.Context(torch.from_numpy(X).to(dev), b_max=b, m_max=m_max)
+    ctx.degree(beta, 1.0)
+    Q0 = None
+    for _ in range(2):
+        ev, U, info = ctx.eigs(k, b, Q0=Q0)
+        assert np.abs(np.array(ev) - lam).max() <= 1e-6 * lam[0]
+        Ud = U.double()
+        assert (Ud.t() @ Ud - torch.eye(k + 1, device=dev)).abs().max().item() <= 1e-5
+        assert (M @ Ud - Ud * torch.tensor(ev, device=dev)).norm(dim=0).max().item() <= 5e-6 * lam[0]
+        Q0 = U
+    ctx.close()
