@@ -42,6 +42,8 @@ __device__ __forceinline__ void copy4(uint32_t dst, const float* src, int valid)
 template <int UI, int UJ, bool ALIGNED>
 __global__ void __launch_bounds__(128)
 k_tn_partial(const Panel A, const Panel B, int64_t N, int64_t rows_per_chunk, double* __restrict__ part) {
+    grid_wait();
+    grid_go();
     extern __shared__ __align__(16) float sm[];
     constexpr int TI = 16 * UI, TJ = 8 * UJ, kStage = (TI + TJ) * kTnPitch;
     const int m = A.m1 + A.m2, n = B.m1 + B.m2;
@@ -124,6 +126,8 @@ k_tn_partial(const Panel A, const Panel B, int64_t N, int64_t rows_per_chunk, do
 // parallel.  `out` may be page-locked host memory: the values are stored there directly, no copy follows.
 __global__ void __launch_bounds__(256)
 k_tn_reduce(const double* __restrict__ part, int chunks, int64_t mm, double* __restrict__ out) {
+    grid_wait();
+    grid_go();
     __shared__ double sm[8][33];
     const int64_t e = (int64_t)blockIdx.x * 32 + threadIdx.x;
     double a0 = 0.0, a1 = 0.0;
@@ -150,6 +154,8 @@ k_tn_reduce(const double* __restrict__ part, int chunks, int64_t mm, double* __r
 template <int PT, int RPT, int KS>
 __global__ void __launch_bounds__(128 * KS)
 k_nn(const Panel A, const float* __restrict__ S, int lds, int p, float* __restrict__ C, int64_t ldc, int64_t N) {
+    grid_wait();
+    grid_go();
     static_assert(KS == 1 || RPT == 1, "split columns with one row per thread only");
     constexpr int kS = 32 * PT, kRed = KS > 1 ? (KS - 1) * PT * 128 : 0;
     __shared__ __align__(16) float smem[KS * kS > kRed ? KS * kS : kRed];
@@ -224,6 +230,8 @@ k_nn(const Panel A, const float* __restrict__ S, int lds, int p, float* __restri
 // dst[:, c] = src[:, idx[c]]
 struct ColumnList { int n; uint16_t idx[256]; };
 __global__ void k_gather_cols(const float* __restrict__ src, float* __restrict__ dst, int64_t ld, const ColumnList list, int64_t N) {
+    grid_wait();
+    grid_go();
     const int c = blockIdx.y;
     const float* s = src + (int64_t)list.idx[c] * ld;
     float* d = dst + (int64_t)c * ld;
@@ -233,6 +241,8 @@ __global__ void k_gather_cols(const float* __restrict__ src, float* __restrict__
 // out[c] = sum_i A[i, c]^2 in fp64; one block per column, fixed summation order (bit-reproducible).
 __global__ void __launch_bounds__(1024)
 k_col_sqnorms(const float* __restrict__ A, int64_t lda, int64_t N, double* __restrict__ out) {
+    grid_wait();
+    grid_go();
     __shared__ double sm[1024];
     const float* col = A + (int64_t)blockIdx.x * lda;
     double acc = 0.0;
@@ -290,7 +300,7 @@ fd_status launch_tn(fd_ctx* c, const Panel& A, const Panel& B, int64_t N, int64_
     chunks = ceil_div(N, rpc);
     FD_CUDA(c, cudaFuncSetAttribute(k_tn_partial<UI, UJ, ALIGNED>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     const dim3 grid((unsigned)ceil_div(m, TI), (unsigned)ceil_div(n, TJ), (unsigned)chunks);
-    k_tn_partial<UI, UJ, ALIGNED><<<grid, 128, smem, c->stream>>>(A, B, N, rpc, scratch);
+    FD_CUDA(c, launch_behind(c->stream, grid, dim3(128), smem, k_tn_partial<UI, UJ, ALIGNED>, A, B, N, rpc, scratch));
     FD_LAUNCH_CHECK(c, "k_tn_partial");
     *chunks_out = (int)chunks;
     return FD_OK;
@@ -315,7 +325,7 @@ fd_status tn_product(fd_ctx* c, const Panel& A, const Panel& B, int64_t N, doubl
         else { if (n > 16) FD_TN(4, 4); else FD_TN(4, 2); }
 #undef FD_TN
     }
-    k_tn_reduce<<<(unsigned)ceil_div((int64_t)mm, 32), dim3(32, 8), 0, c->stream>>>(scratch, chunks, (int64_t)mm, out);
+    FD_CUDA(c, launch_behind(c->stream, dim3((unsigned)ceil_div((int64_t)mm, 32)), dim3(32, 8), 0, k_tn_reduce, (const double*)scratch, chunks, (int64_t)mm, out));
     FD_LAUNCH_CHECK(c, "k_tn_reduce");
     return FD_OK;
 }
@@ -327,13 +337,13 @@ fd_status nn_product(fd_ctx* c, const Panel& A, const float* S_dev, int lds, int
     // (the narrowest that holds p, at most 16: more blocks) with the columns of A shared by four groups of threads
     const unsigned rb = (unsigned)ceil_div(N, 128);
     if (p > 16 && ceil_div(N, 256) * ceil_div(p, 32) >= 3 * c->sm_count)
-        k_nn<32, 2, 1><<<dim3((unsigned)ceil_div(N, 256), (unsigned)ceil_div(p, 32)), 128, 0, c->stream>>>(A, S_dev, lds, p, C, ldc, N);
+        FD_CUDA(c, launch_behind(c->stream, dim3((unsigned)ceil_div(N, 256), (unsigned)ceil_div(p, 32)), dim3(128), 0, k_nn<32, 2, 1>, A, S_dev, lds, p, C, ldc, N));
     else if (p > 16 && rb * ceil_div(p, 32) >= 4 * c->sm_count)
-        k_nn<32, 1, 1><<<dim3(rb, (unsigned)ceil_div(p, 32)), 128, 0, c->stream>>>(A, S_dev, lds, p, C, ldc, N);
+        FD_CUDA(c, launch_behind(c->stream, dim3(rb, (unsigned)ceil_div(p, 32)), dim3(128), 0, k_nn<32, 1, 1>, A, S_dev, lds, p, C, ldc, N));
     else if (p > 8)
-        k_nn<16, 1, 4><<<dim3(rb, (unsigned)ceil_div(p, 16)), 512, 0, c->stream>>>(A, S_dev, lds, p, C, ldc, N);
+        FD_CUDA(c, launch_behind(c->stream, dim3(rb, (unsigned)ceil_div(p, 16)), dim3(512), 0, k_nn<16, 1, 4>, A, S_dev, lds, p, C, ldc, N));
     else
-        k_nn<8, 1, 4><<<dim3(rb, 1u), 512, 0, c->stream>>>(A, S_dev, lds, p, C, ldc, N);
+        FD_CUDA(c, launch_behind(c->stream, dim3(rb, 1u), dim3(512), 0, k_nn<8, 1, 4>, A, S_dev, lds, p, C, ldc, N));
     FD_LAUNCH_CHECK(c, "k_nn");
     return FD_OK;
 }
@@ -344,14 +354,14 @@ fd_status gather_cols(fd_ctx* c, const float* src, float* dst, int64_t ld, const
     ColumnList list;
     list.n = p;
     for (int i = 0; i < p; ++i) list.idx[i] = (uint16_t)idx[i];
-    k_gather_cols<<<dim3((unsigned)std::min<int64_t>(64, ceil_div(N, 256)), (unsigned)p), 256, 0, c->stream>>>(src, dst, ld, list, N);
+    FD_CUDA(c, launch_behind(c->stream, dim3((unsigned)std::min<int64_t>(64, ceil_div(N, 256)), (unsigned)p), dim3(256), 0, k_gather_cols, src, dst, ld, list, N));
     FD_LAUNCH_CHECK(c, "k_gather_cols");
     return FD_OK;
 }
 
 fd_status col_sqnorms(fd_ctx* c, const float* A, int64_t lda, int p, int64_t N, double* out) {
     if (p < 1) return FD_OK;
-    k_col_sqnorms<<<(unsigned)p, 1024, 0, c->stream>>>(A, lda, N, out);
+    FD_CUDA(c, launch_behind(c->stream, dim3((unsigned)p), dim3(1024), 0, k_col_sqnorms, A, lda, N, out));
     FD_LAUNCH_CHECK(c, "k_col_sqnorms");
     return FD_OK;
 }

@@ -101,6 +101,8 @@ constexpr int min_ctas(int regs) { return regs + 40 <= 128 ? 4 : regs + 40 <= 16
 template <int DP4, int BT, int R>
 __global__ void __launch_bounds__(kThr, min_ctas(R * (4 * DP4 + BT)))
 k_direct(const DirectParams p) {
+    grid_wait();
+    grid_go();
     constexpr int H = R * kThr / kRowsT;               // column parts of a tile (R = 4: 2)
     constexpr int BP = BT + 4;                         // pitch of the staged block (16-byte rows; spreads the transposing stores)
     extern __shared__ __align__(16) float smem[];
@@ -202,6 +204,8 @@ k_direct(const DirectParams p) {
 template <int DP4>
 __global__ void __launch_bounds__(kThr)
 k_direct_rowsum(const DirectParams p) {
+    grid_wait();
+    grid_go();
     constexpr int R = DP4 <= 4 ? 4 : 2, H = R * kThr / kRowsT;
     __shared__ float4 sx[kTJ * DP4];
     __shared__ float sw[kTJ];
@@ -346,6 +350,8 @@ constexpr int kSmallRows = 64, kSmallThr = 256, kSmallCtas = 8;
 template <int DP4, int BT>
 __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThr)
 k_direct_small(const DirectParams p) {
+    grid_wait();
+    grid_go();
     constexpr int BP = BT + 4, kWarps = kSmallThr / 32, R = kSmallRows / 32;
     constexpr int kStage = kSmallThr * (4 * DP4 + BP), kRed = kWarps * BT * kSmallRows;
     __shared__ __align__(16) float smem[kStage > kRed ? kStage : kRed];
@@ -449,7 +455,7 @@ fd_status launch(fd_ctx* c, Kernel kernel, int smem, int per_sm, int BT, DirectP
     ctas = std::max<long long>(1, std::min<long long>(std::min(ctas, total), (long long)(c->L.part_floats / (2 * slot_floats))));
     if (c->opt_splits <= 0) ctas = ceil_div(total, ceil_div(total, ctas));      // same longest range, fewer shares
     if (smem > 48 * 1024) FD_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    kernel<<<dim3((unsigned)ctas), dim3(kThr), smem, c->stream>>>(p);
+    FD_CUDA(c, launch_behind(c->stream, dim3((unsigned)ctas), dim3(kThr), smem, kernel, p));
     FD_LAUNCH_CHECK(c, "k_direct");
     bool cut = false;
     for (int i = 1; i < ctas && !cut; ++i) cut = range_begin(total, i, (int)ctas) % p.col_tiles != 0;
@@ -478,7 +484,7 @@ template <int DP4, int BT>
 fd_status launch_block(fd_ctx* c, const DirectParams& p) {
     if constexpr (DP4 <= 2 && BT <= 16)
         if (p.N <= small_n(BT) && p.Nrow <= small_n(BT) && c->opt_splits <= 0) {
-            k_direct_small<DP4, BT><<<dim3((unsigned)(kSmallCtas * ceil_div(p.Nrow, kSmallRows))), dim3(kSmallThr), 0, c->stream>>>(p);
+            FD_CUDA(c, launch_behind(c->stream, dim3((unsigned)(kSmallCtas * ceil_div(p.Nrow, kSmallRows))), dim3(kSmallThr), 0, k_direct_small<DP4, BT>, p));
             FD_LAUNCH_CHECK(c, "k_direct_small");
             return FD_OK;
         }

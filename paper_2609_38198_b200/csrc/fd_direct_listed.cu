@@ -140,6 +140,8 @@ constexpr int near_ctas(int DP4, int BT) { return BT <= 8 ? (4 * DP4 + BT <= 8 ?
 template <int DP4, int BT>
 __global__ void __launch_bounds__(kThr, near_ctas(DP4, BT))
 k_near(const NearParams p) {
+    grid_wait();
+    grid_go();
     constexpr int WF4 = BT / 4, kSlot = kEntry * (DP4 + WF4);
     extern __shared__ __align__(16) float4 smem_near[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, warp = (int)blockIdx.x * kWarps + wib, warps = (int)gridDim.x * kWarps;
@@ -211,6 +213,8 @@ k_near(const NearParams p) {
 template <int DP4, bool WEIGHTED>
 __global__ void __launch_bounds__(kThr, 8)
 k_near_rowsum(const NearParams p) {
+    grid_wait();
+    grid_go();
     constexpr int kSlot = kEntry * DP4;
     __shared__ float4 ring_store[kWarps * kRing * kSlot];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, warp = (int)blockIdx.x * kWarps + wib, warps = (int)gridDim.x * kWarps;
@@ -364,6 +368,8 @@ k_near_fix(const NearParams p, int BT, int warps) {
 __global__ void __launch_bounds__(256)
 k_near_pack(const float* __restrict__ V, int64_t ldv, int vcols, const float* __restrict__ right, const int* __restrict__ perm, int64_t N, int64_t NP, int b, int BT,
             float4* __restrict__ w, unsigned int* __restrict__ bad, unsigned int epoch) {
+    grid_wait();
+    grid_go();
     const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
     const bool vec = BT == 1;
     const int per = vec ? 1 : BT / 4;
@@ -394,7 +400,7 @@ fd_status launch(fd_ctx* c, Kernel kernel, int smem, int per_sm, int BT, NearPar
     ctas = std::max<long long>(1, std::min<long long>(ctas, (long long)(c->L.part_floats / (2 * kWarps * slot_floats))));
     const int warps = (int)ctas * kWarps;
     if (smem > 48 * 1024) FD_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    kernel<<<dim3((unsigned)ctas), dim3(kThr), smem, c->stream>>>(p);
+    FD_CUDA(c, launch_behind(c->stream, dim3((unsigned)ctas), dim3(kThr), smem, kernel, p));
     FD_LAUNCH_CHECK(c, "k_near");
     FD_CUDA(c, launch_behind(c->stream, dim3((unsigned)p.groups * (kRowsG / 32), BT > 0 ? (unsigned)ceil_div(p.b, kFixCols) : 1u), dim3(256), 0,
                              BT > 0 ? k_near_fix<false> : k_near_fix<true>, p, BT, warps));
@@ -469,7 +475,8 @@ fd_status apply_direct_listed(fd_ctx* c, const ApplyArgs& a, int kind) {
             p.bad = bad;
             if (c->captured) FD_CUDA(c, cudaMemsetAsync(bad, 0, 64 * 4, c->stream));
             const int64_t threads = rowsum ? L.NP / 4 : L.NP * (BT / 4);
-            k_near_pack<<<dim3((unsigned)ceil_div(threads, 256)), dim3(256), 0, c->stream>>>(p.V, p.ldv, p.vcols, p.right, p.perm, L.N, L.NP, bc, rowsum ? 1 : BT, reinterpret_cast<float4*>(w), bad, p.epoch);
+            FD_CUDA(c, launch_behind(c->stream, dim3((unsigned)ceil_div(threads, 256)), dim3(256), 0, k_near_pack, p.V, p.ldv, p.vcols, p.right, p.perm,
+                                     L.N, L.NP, bc, rowsum ? 1 : BT, reinterpret_cast<float4*>(w), bad, p.epoch));
             FD_LAUNCH_CHECK(c, "k_near_pack");
             p.w = w;
         }

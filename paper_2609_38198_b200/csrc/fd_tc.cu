@@ -349,6 +349,8 @@ __global__ void k_pad_weights(const float* __restrict__ w, int64_t n, int64_t np
 // Per-block maxima of |right_j V_jc| for each column c (columns from vcols on are the ones vector); infinite where an entry is not finite.
 __global__ void __launch_bounds__(256)
 k_colmax_partial(const float* __restrict__ V, int64_t ldv, int vcols, const float* __restrict__ right, int64_t N, int c0, float* __restrict__ part) {
+    grid_wait();
+    grid_go();
     __shared__ float sm[8];
     const bool ones = c0 + (int)blockIdx.y >= vcols;
     const float* v = V + (int64_t)(ones ? 0 : c0 + blockIdx.y) * ldv;
@@ -377,6 +379,8 @@ k_colmax_partial(const float* __restrict__ V, int64_t ldv, int vcols, const floa
 __global__ void __launch_bounds__(256)
 k_pack_wt(const float* __restrict__ V, int64_t ldv, int vcols, const float* __restrict__ right, int64_t N, int64_t np, int c0, int bc,
           const float* __restrict__ part, int parts, float* __restrict__ inv, __half* __restrict__ wt, int with_lo, const int* __restrict__ perm) {
+    grid_wait();
+    grid_go();
     __shared__ float sm[8];
     const int c = blockIdx.y;
     float m = c < bc && (int)threadIdx.x < parts ? part[(size_t)c * parts + threadIdx.x] : 0.f;
@@ -577,9 +581,10 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
             const int BT = bc <= 16 ? 16 : bc <= 32 ? 32 : bc <= 48 && !fast ? 48 : 64;
             if (BT > L.BP) return fail(c, FD_ERR_WORKSPACE, "column tile %d wider than the provisioned block buffers (%d)", BT, L.BP);
             const int cm_blocks = (int)std::min<int64_t>(256, ceil_div(N, 1024));
-            k_colmax_partial<<<dim3(cm_blocks, bc), dim3(256), 0, c->stream>>>(a.V, a.ldv, vcols, a.right, N, c0, part);
+            FD_CUDA(c, launch_behind(c->stream, dim3(cm_blocks, bc), dim3(256), 0, k_colmax_partial, a.V, a.ldv, vcols, a.right, N, c0, part));
             FD_LAUNCH_CHECK(c, "k_colmax_partial");
-            k_pack_wt<<<dim3((unsigned)std::min<int64_t>(1024, ceil_div(NP, 512)), BT), dim3(256), 0, c->stream>>>(a.V, a.ldv, vcols, a.right, N, NP, c0, bc, (const float*)part, cm_blocks, inv, wt_hi, fast ? 0 : 1, col_perm);
+            FD_CUDA(c, launch_behind(c->stream, dim3((unsigned)std::min<int64_t>(1024, ceil_div(NP, 512)), BT), dim3(256), 0, k_pack_wt,
+                                     a.V, a.ldv, vcols, a.right, N, NP, c0, bc, (const float*)part, cm_blocks, inv, wt_hi, fast ? 0 : 1, col_perm));
             FD_LAUNCH_CHECK(c, "k_pack_wt");
             // one map over W_hi (rows 0 .. BT) and, in the fp32-grade mode, W_lo behind it (rows BT .. 2 BT of the same array)
             if (!make_map_2d(&mh, wt_hi, (uint64_t)NP, (uint64_t)(fast ? BT : 2 * BT), (uint64_t)NP * 2, 64, fast ? BT : 2 * BT, CU_TENSOR_MAP_SWIZZLE_128B))

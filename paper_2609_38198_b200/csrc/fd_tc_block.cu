@@ -171,6 +171,8 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
+    grid_wait();
+    grid_go();
     const long long t_begin = clock64();
 
     if (warp >= 24) {
@@ -490,6 +492,8 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
 template <int BT>
 __global__ void __launch_bounds__(256)
 k_block_fix(const BlockParams p, int ctas) {
+    grid_wait();
+    grid_go();
     const int pair = blockIdx.x;
     const long long total = p.list ? (long long)p.offs[p.pairs] : (long long)p.pairs * p.num_jt;
     const long long g0 = p.list ? (long long)p.offs[pair] : (long long)pair * p.num_jt;
@@ -547,12 +551,12 @@ fd_status launch_one(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap& mc, co
         const long long total = (long long)p.pairs * p.num_jt;
         const int grid = (int)std::min<long long>(c->sm_count, total);
         if ((size_t)3 * grid * BT * 256 > c->L.part_floats) return fail(c, FD_ERR_WORKSPACE, "no room for the shares of cut row pairs");
-        kernel<<<dim3((unsigned)grid), dim3(kThreadsB), (size_t)smem, c->stream>>>(mr, mc, mw, p);
+        FD_CUDA(c, launch_behind(c->stream, dim3((unsigned)grid), dim3(kThreadsB), (size_t)smem, kernel, mr, mc, mw, p));
         FD_LAUNCH_CHECK(c, "k_block");
         bool cut = p.list != nullptr;
         for (int i = 1; i < grid && !cut; ++i) cut = range_begin(total, i, grid) % p.num_jt != 0;
         if (cut) {
-            k_block_fix<BT><<<dim3((unsigned)p.pairs, (unsigned)ceil_div(p.b, 8)), dim3(256), 0, c->stream>>>(p, grid);
+            FD_CUDA(c, launch_behind(c->stream, dim3((unsigned)p.pairs, (unsigned)ceil_div(p.b, 8)), dim3(256), 0, k_block_fix<BT>, p, grid));
             FD_LAUNCH_CHECK(c, "k_block_fix");
         }
     }
