@@ -38,7 +38,8 @@
  * Repeats: the same call in the same state gives the same bits.  At the bandwidth of the latest degree
  *   passes, passes over the points may leave out tiles of the kernel that hold only zeros ("tile_share"); all
  *   tensor-core passes at that bandwidth then add in another order than at others, and bandwidths asked
- *   earlier can tip the decision.  Passes at any other bandwidth give the bits of a new context.
+ *   earlier can tip the decision.  Passes at any other bandwidth give the bits of a new context.  Once a product has been
+ *   recorded into a graph, later degree passes at other bandwidths leave out a few tiles less.
  * k:       counts NONTRIVIAL eigenpairs; the Perron pair (eigenvalue 1) is
  *   returned in slot 0, so k + 1 pairs come back (Sec. 2.3, Sec. 3).
  */
@@ -80,7 +81,8 @@ enum { FD_PATH_AUTO = 0, FD_PATH_SIMT = 1, FD_PATH_TC = 2 };
  * max|x - mu|^2 >= "tc_max_mag", then returns FD_ERR_UNSUPPORTED).  fd_create refuses D > FD_MAX_D. */
 #define FD_MAX_D 60
 
-/* Bytes of device workspace fd_create needs.  O(N (D + b_max + m_max)); no N^2 term.
+/* Bytes of device workspace fd_create needs.  O(N (D + b_max + m_max)); beside that, up to 2^19 points, tile lists and notes of N^2 / 4096 bytes
+ * (N^2 / 200 with up to 8 coordinates and 2^17 points).
  * b_max: widest block passed to fd_apply / fd_apply_general (1..256).
  * m_max: basis capacity for fd_eigs (columns); 0 if fd_eigs will not be called. */
 size_t fd_workspace_bytes(int64_t N, int32_t D, int32_t b_max, int32_t m_max);
@@ -164,7 +166,7 @@ typedef struct {
  * implicitly restarted Lanczos and gives no further detail; Sec. 2.3).  b = block size,
  * tol = residual tolerance relative to theta_0, Q0_dev = optional warm-start basis (N x q0_cols,
  * need not be orthonormal).  evals_host: k + 1 doubles, descending.  evecs_dev: N x (k + 1)
- * column-major, orthonormal.  Needs m_max >= 2 (k + 1) + b at fd_create; the thick restart keeps 3/5 of m_max, so a
+ * column-major, orthonormal.  Needs m_max >= 2 (k + 1) + b at fd_create; the thick restart keeps up to 3/5 of m_max, so a
  * capacity near 3 (k + 1) + 2 b keeps room for the rest of an eigenvalue cluster that the request cuts (on the
  * 6-torus, k = 128 cuts a 160-fold cluster: 129 of 129 pairs converge in 44 block products with m_max = 576, 384
  * stalls above tol).  Below 3 (k + 1) every block is a residual block, with a projected eigenproblem after each product, and a
