@@ -7,7 +7,7 @@
 // barrier of the block: neighbouring warps need not agree on which tiles are near.  The flat sequence of (64 rows, entry) steps is cut
 // into equal ranges, one per warp; shares of row groups that a cut falls into are added by k_near_fix in the order of the warps.
 //
-// What bounds it: instruction issue, 2 D + b + 2 FMA-pipe operations per pair (N = 16384, D = 4, b = 16: about 60 % of the issue slots).  Against
+// What bounds it: instruction issue, 2 D + b + 2 FMA-pipe operations per pair (N = 16384, D = 4, b = 16: 76 % of the issue slots taken, FMA pipe 60 %).  Against
 // steps of 256 rows x 64 points gathered through the order, by a whole block and from boxes alone: 2-torus, N = 16384, beta = 100, b = 16: 134 -> 69 us
 // a product (0.34 -> 0.17 of the tiles), both degree passes 164 -> 125; beta = 30: 310 (all tiles; not worth lists then) -> 157; N = 65536,
 // b = 32, beta = 100: 1805 -> 1046.  Error against float64: 1.75e-7 -> 1.32e-7, 1.43e-7 -> 1.48e-7 and 4.3e-7 -> 2.1e-7 (short first sums).
