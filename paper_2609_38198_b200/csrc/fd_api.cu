@@ -82,6 +82,8 @@ Layout make_layout(int64_t N, int32_t D, int32_t b_max, int32_t m_max) {
             L.lists[i] = carve(cur, groups * col_tiles * 2);
             L.list_counts[i] = carve(cur, (4 * groups + 2) * 4);
         }
+        L.lists[2] = carve(cur, pairs * tiles * 2);
+        L.list_counts[2] = carve(cur, (4 * pairs + 2) * 4);
         L.near = carve(cur, std::max(2 * tiles * tiles, L.direct_lists ? groups * col_tiles : 0));
         if (L.direct_lists) L.xord = carve(cur, (size_t)L.NP * L.DP * 4);
     }

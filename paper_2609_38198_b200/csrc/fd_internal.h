@@ -31,7 +31,7 @@ struct Layout {
     size_t part = 0, part_floats = 0;
     size_t xp_col = 0, xp_row = 0, wt_hi = 0, wt_lo = 0, colscale = 0, status = 0;
     // order of the points and tile lists of the Gram-form kernels (fd_order.cu); 0: not provisioned for this N
-    size_t perm = 0, boxes = 0, zproj = 0, lists[2] = {0, 0}, list_counts[2] = {0, 0}, near = 0, xord = 0;
+    size_t perm = 0, boxes = 0, zproj = 0, lists[3] = {0, 0, 0}, list_counts[3] = {0, 0, 0}, near = 0, xord = 0;
     bool direct_lists = false;       // provisioned for the direct-difference kernels as well
     size_t weights = 0;              // NP right weights of a Gram-form row sum
     size_t symsum = 0;               // N 64-bit fixed-point sums of the symmetric row-sum mode
@@ -78,7 +78,7 @@ struct fd_ctx {
     bool captured = false;
     unsigned int direct_epoch = 0;   // number of the latest listed pass of the direct-difference kernels
     double refused_beta = 0.0;       // largest bandwidth at which an order was tried and left out too little
-    struct { int kind = -1; double beta = -1.0; } listed[2];     // what the two list buffers hold: of the products (0), of the degree passes (1)
+    struct { int kind = -1; double beta = -1.0; } listed[3];     // what the list buffers hold: of the products (0), of the first (1) and the second degree pass (2; Gram form)
     int boxes_kind = -1;
     // bandwidth whose near tiles a degree pass noted in L.near (fd_order.cu).  No pass writes notes once products have been recorded: a
     // replay lists by what they say.

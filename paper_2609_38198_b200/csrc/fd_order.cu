@@ -402,7 +402,7 @@ fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide) {
     if (L.perm == 0 || c->order_state < 0) return FD_OK;
     const bool direct = kind == 2 || kind == 4;
     const bool noted = c->near_beta == beta && c->near_direct == direct && kind != 1 && kind != 2;
-    const int buf = kind == 0 || kind == 4 ? 0 : 1;
+    const int buf = kind == 0 || kind == 4 ? 0 : kind == 3 ? 2 : 1;
     auto& listed = c->listed[buf];
     const int held = noted ? 8 + kind : kind;                      // what the buffer would hold
     if (st.beta == beta && (!st.on || (!c->captured && listed.kind == held && listed.beta == beta))) return FD_OK;
@@ -508,10 +508,12 @@ fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide) {
     k_lists<<<pairs, 1024, 0, c->stream>>>(box, ZP, tiles, per_pair, limit2, notes, direct ? 1 : 2, c->at<unsigned short>(L.lists[buf]), cnt, cnt + pairs);
     FD_LAUNCH_CHECK(c, "k_lists");
     unsigned int* offs = cnt + 2 * pairs;
-    // offsets of all entries, and of the upper ones
-    k_scan<<<1, 1024, 0, c->stream>>>(cnt, pairs, offs);
-    FD_LAUNCH_CHECK(c, "k_scan");
-    if (!direct) {
+    // offsets of all entries, and of the upper ones (degree passes in the Gram form)
+    if (kind != 3) {
+        k_scan<<<1, 1024, 0, c->stream>>>(cnt, pairs, offs);
+        FD_LAUNCH_CHECK(c, "k_scan");
+    }
+    if (kind == 1 || kind == 3) {
         k_scan<<<1, 1024, 0, c->stream>>>(cnt + pairs, pairs, offs + pairs + 1);
         FD_LAUNCH_CHECK(c, "k_scan");
     }

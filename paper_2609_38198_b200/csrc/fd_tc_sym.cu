@@ -19,8 +19,8 @@
 //                shared memory, so that a pair of tiles costs one atomic per streamed point.
 // Work is a flat sequence of (resident pair, streamed tile) steps, cut into equal ranges, one per CTA.
 //
-// What bounds it: the MUFU (1024 SM clocks per tile; 76 % busy at N = 65536) and the queue that feeds it, with the additions beside it (issue
-// slots 60 to 63 % with scalar additions).  The additions work on two columns an instruction (add / fma.rn.f32x2): half their issue slots, the same
+// What bounds it: the MUFU (1024 SM clocks per tile; 78 to 81 % busy at N = 65536) and the queue that feeds it, with the additions beside it (issue
+// slots 53 to 55 %, 60 to 63 % with scalar additions).  The additions work on two columns an instruction (add / fma.rn.f32x2): half their issue slots, the same
 // bits.  N = 65536: 1440 -> 1376 us both passes, N = 2^18: 21.55 -> 20.4 ms.  (Loads of 8 columns one step ahead: 1.5 % slower; a polynomial
 // on the FMA pipe for two of sixteen columns: 4 % slower.)  Both degree passes at N = 2^18 (one with squares, one
 // with weights), scalar: 26.2 -> 21.6 ms against two warpgroups with 128 accumulators a thread, whole row pairs per CTA and an atomic per
@@ -434,8 +434,8 @@ fd_status launch_sym_rowsum(fd_ctx* c, const CUtensorMap& mr, const CUtensorMap&
     p.shift = 61 - kBias - lg;
     FD_CUDA(c, cudaMemsetAsync(p.sums, 0, (size_t)L.N * 8, c->stream));
     if (use_lists) {
-        p.list = c->at<unsigned short>(L.lists[1]);
-        p.counts = c->at<unsigned int>(L.list_counts[1]);
+        p.list = c->at<unsigned short>(L.lists[rowsq ? 1 : 2]);
+        p.counts = c->at<unsigned int>(L.list_counts[rowsq ? 1 : 2]);
         p.uoffs = p.counts + 3 * p.pairs + 1;
     }
     if (note_near) {
