@@ -117,7 +117,7 @@ k_direct(const DirectParams p) {
         const int64_t row0 = (int64_t)range.rt * kRowsT;
         float4 xi[R][DP4];
         load_rows<DP4, R>(p, row0, lane_row, xi);
-        Sums<R, BT> acc;
+        Sums<R, BT, (BT > 48 && DP4 != 5 && DP4 != 6)> acc;              // (packed, 17 to 24 coordinates spill 72 and 236 bytes a thread)
         acc.clear();
         // a thread's own slots of sacc: row r, column c at mine[c * 256 + (256 / R) * r]
         float* mine = sacc + part * BT * kRowsT + lane_row;
