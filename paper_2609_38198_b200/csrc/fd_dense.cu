@@ -300,7 +300,8 @@ fd_status launch_tn(fd_ctx* c, const Panel& A, const Panel& B, int64_t N, int64_
     chunks = ceil_div(N, rpc);
     FD_CUDA(c, cudaFuncSetAttribute(k_tn_partial<UI, UJ, ALIGNED>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     const dim3 grid((unsigned)ceil_div(m, TI), (unsigned)ceil_div(n, TJ), (unsigned)chunks);
-    FD_CUDA(c, launch_behind(c->stream, grid, dim3(128), smem, k_tn_partial<UI, UJ, ALIGNED>, A, B, N, rpc, scratch));
+    // (not behind the kernel before: two blocks per SM, evenly)
+    k_tn_partial<UI, UJ, ALIGNED><<<grid, 128, smem, c->stream>>>(A, B, N, rpc, scratch);
     FD_LAUNCH_CHECK(c, "k_tn_partial");
     *chunks_out = (int)chunks;
     return FD_OK;
