@@ -101,8 +101,6 @@ constexpr int min_ctas(int regs) { return regs + 40 <= 128 ? 4 : regs + 40 <= 16
 template <int DP4, int BT, int R>
 __global__ void __launch_bounds__(kThr, min_ctas(R * (4 * DP4 + BT)))
 k_direct(const DirectParams p) {
-    grid_wait();
-    grid_go();
     constexpr int H = R * kThr / kRowsT;               // column parts of a tile (R = 4: 2)
     constexpr int BP = BT + 4;                         // pitch of the staged block (16-byte rows; spreads the transposing stores)
     extern __shared__ __align__(16) float smem[];
@@ -198,14 +196,13 @@ k_direct(const DirectParams p) {
             }
         }
     }
+    grid_go();
 }
 
 // Row-sum mode: sum_j K_ij right_j and sum_j K_ij^2; a column tile (<= 64 terms) in fp32, across tiles in fp64.
 template <int DP4>
 __global__ void __launch_bounds__(kThr)
 k_direct_rowsum(const DirectParams p) {
-    grid_wait();
-    grid_go();
     constexpr int R = DP4 <= 4 ? 4 : 2, H = R * kThr / kRowsT;
     __shared__ float4 sx[kTJ * DP4];
     __shared__ float sw[kTJ];
@@ -270,6 +267,7 @@ k_direct_rowsum(const DirectParams p) {
             }
         }
     }
+    grid_go();
 }
 
 // Finishes the row tiles that a cut falls into.  Block = (32 rows of a row tile, 8 columns), 8 groups of shares read in parallel (a row
