@@ -158,10 +158,13 @@ k_direct(const DirectParams p) {
 #pragma unroll
         for (int r = 0; r < R; ++r)
 #pragma unroll
-            for (int c = 0; c < BT; ++c) {
-                sum[r][c] = acc.get(r, c);
-                if (flushed) sum[r][c] += mine[c * kRowsT + (kRowsT / R) * r];
-            }
+            for (int c = 0; c < BT; ++c) sum[r][c] = acc.get(r, c);
+        if (flushed) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int c = 0; c < BT; ++c) sum[r][c] += mine[c * kRowsT + (kRowsT / R) * r];
+        }
         if (H == 2) {
             // the second half hands its sums to the first
             if (part == 1) {
