@@ -400,8 +400,8 @@ fd_status launch(fd_ctx* c, Kernel kernel, int smem, int per_sm, int BT, NearPar
     ctas = std::max<long long>(1, std::min<long long>(ctas, (long long)(c->L.part_floats / (2 * kWarps * slot_floats))));
     const int warps = (int)ctas * kWarps;
     if (smem > 48 * 1024) FD_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    // (not behind the kernel before: its CTAs would be spread unevenly over the SMs, and the ranges are equal)
-    kernel<<<(unsigned)ctas, kThr, smem, c->stream>>>(p);
+    // (behind the packing: N = 16384, D = 4, b = 16: 69.8 -> 68.0 us a product, launched after it and behind it)
+    FD_CUDA(c, launch_behind(c->stream, dim3((unsigned)ctas), dim3(kThr), smem, kernel, p));
     FD_LAUNCH_CHECK(c, "k_near");
     FD_CUDA(c, launch_behind(c->stream, dim3((unsigned)p.groups * (kRowsG / 32), BT > 0 ? (unsigned)ceil_div(p.b, kFixCols) : 1u), dim3(256), 0,
                              BT > 0 ? k_near_fix<false> : k_near_fix<true>, p, BT, warps));
