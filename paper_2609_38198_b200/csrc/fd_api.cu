@@ -243,9 +243,8 @@ fd_status fd_beta0(fd_ctx* c, double* beta0_host) {
     return FD_OK;
 }
 
-fd_status fd_degree(fd_ctx* c, double beta, double alpha, fd_precision prec, float* q_dev, float* d_dev,
-                    float* s_dev, double* S_off_host, double* S_off_2beta_host) {
-    if (!c) return FD_ERR_INVALID;
+static fd_status degree_passes(fd_ctx* c, double beta, double alpha, fd_precision prec, float* q_dev, float* d_dev,
+                               float* s_dev, double* S_off_host, double* S_off_2beta_host) {
     if (!(beta > 0) || !(beta < 1e30) || !(alpha >= 0) || alpha > 4) return fail(c, FD_ERR_INVALID, "beta or alpha out of range");
     if (prec != FD_PREC_FP32 && prec != FD_PREC_FAST) return fail(c, FD_ERR_INVALID, "bad precision");
     const int64_t N = c->L.N;
@@ -301,6 +300,19 @@ fd_status fd_degree(fd_ctx* c, double beta, double alpha, fd_precision prec, flo
     if (S_off_2beta_host) *S_off_2beta_host = sum_sq - (double)N;
     c->beta = beta; c->alpha = alpha; c->have_s = true;
     return FD_OK;
+}
+
+fd_status fd_degree(fd_ctx* c, double beta, double alpha, fd_precision prec, float* q_dev, float* d_dev,
+                    float* s_dev, double* S_off_host, double* S_off_2beta_host) {
+    if (!c) return FD_ERR_INVALID;
+    const fd_status st = degree_passes(c, beta, alpha, prec, q_dev, d_dev, s_dev, S_off_host, S_off_2beta_host);
+    if (st != FD_OK && c->near_unproven) {
+        // a pass that ran into a bounded wait has not seen every tile: its notes and the lists made from them hold for nothing
+        c->near_beta = -1.0;
+        for (auto& l : c->listed) l.kind = -1;
+    }
+    c->near_unproven = false;
+    return st;
 }
 
 fd_status fd_apply_general(fd_ctx* c, double beta, const float* left_dev, const float* right_dev,

@@ -484,7 +484,7 @@ fd_status apply_direct_listed(fd_ctx* c, const ApplyArgs& a, int kind) {
         if (DP4 == 1) FD_TRY(launch_dp<1>(c, BT, p));
         else FD_TRY(launch_dp<2>(c, BT, p));
     }
-    if (p.near) { c->near_beta = a.beta; c->near_direct = true; }
+    if (p.near) { c->near_beta = a.beta; c->near_direct = true; c->near_unproven = true; }
     return FD_OK;
 }
 

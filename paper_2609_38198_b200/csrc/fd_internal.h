@@ -84,6 +84,7 @@ struct fd_ctx {
     // replay lists by what they say.
     double near_beta = -1.0;
     bool near_direct = false;        // (by a direct-difference pass)
+    bool near_unproven = false;      // the pass that took them has not been seen to finish: a pass that gives up leaves tiles unnoted
     // options
     int opt_path = FD_PATH_AUTO;
     int opt_splits = 0;

@@ -563,7 +563,7 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
         const bool note_near = ordered && a.rowsq && a.decide && !c->captured && (c->near_beta != a.beta || c->near_direct);
         if (note_near) c->near_beta = -1.0;
         FD_TRY(launch_sym_rowsum(c, mr, mc, p.weights, a.left, a.Y, a.rowsq, row_perm, use_lists, note_near));
-        if (note_near) { c->near_beta = a.beta; c->near_direct = false; }
+        if (note_near) { c->near_beta = a.beta; c->near_direct = false; c->near_unproven = true; }
     } else if (rowsum) {
         p.q = a.Y; p.rowsq = a.rowsq; p.b = 1;
         if (p.rowsq) FD_TRY((launch_tc<16>(c, mr, mc, p, grid)));

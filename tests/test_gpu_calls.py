@@ -184,6 +184,62 @@ def test_calls_without_lists_do_not_depend_on_the_order_of_the_points(fd, dev, k
     ctx.close()
 
 
+def _notes(ctx, kind):
+    """The part of the workspace with a degree pass's notes: a byte per tile, 1 for every tile that holds a point's kernel value with itself."""
+    ws, N = ctx._ws[-ctx._ws.data_ptr() % 256:], ctx.N
+    if kind == "direct":
+        first, step, size = 1, N // 16 + 4, (N // 64) * (N // 16)        # groups of 64 rows, entries of 16 points: entry 4 g + 1 is one of group g's own
+    else:
+        first, step, size = 0, N // 128 + 1, 2 * (N // 128) ** 2         # tiles of 128: two planes
+    at = torch.arange(0, ws.numel() - size, 256, device=ws.device)
+    for k in range((N // 64) if kind == "direct" else N // 128):
+        at = at[ws[at + (first + k * step)] == 1]
+    found = [int(a) for a in at.cpu() if int(ws[a:a + size].max()) == 1]
+    assert len(found) == 1, found
+    return ws[found[0]:found[0] + size]
+
+
+@pytest.mark.parametrize("kind", ["direct", "gram"])
+def test_a_failed_degree_pass_leaves_no_notes(fd, dev, kind):
+    """fd_degree reports a bounded wait that ran out (of the self-test here; a pass that gives up in one has not noted the tiles after it).
+    What was noted is not used again: neither by products recorded afterwards nor by the next degree pass, whose results are those of a new
+    context."""
+    stream = torch.cuda.Stream()
+    ctx, X, beta = _listed(fd, dev, kind)
+    V = fd.to_colmajor(workloads.block(X.shape[0], 8, seed=3), dev)
+    torch.cuda.synchronize()
+    s = ctx.degree(beta, 1.0)[2]
+    want = ctx.apply(V)
+    ctx.close()
+
+    def failed(stream=None):
+        c = fd.Context(torch.from_numpy(X).to(dev), b_max=8, stream=stream)
+        c.set_option("path", fd.FD_PATH_SIMT if kind == "direct" else fd.FD_PATH_TC)
+        c.set_option("tc_max_mag", 1e4)
+        c.set_option("wait_selftest", 2.0e6)
+        with pytest.raises(fd.FdError) as e:
+            c.degree(beta, 1.0)
+        assert e.value.status == fd.FD_ERR_TIMEOUT
+        torch.cuda.synchronize()
+        _notes(c, kind).zero_()                                # the pass that gave up noted nothing
+        torch.cuda.synchronize()
+        return c
+
+    ctx = failed()
+    assert torch.equal(ctx.degree(beta, 1.0)[2], s) and torch.equal(ctx.apply(V), want)
+    ctx.close()
+    ctx, Y = failed(stream), torch.zeros_like(want)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream):                   # (lists for itself)
+        ctx.apply_general(beta, V, left=s, right=s, out=Y)
+    torch.cuda.synchronize()
+    g.replay()
+    torch.cuda.synchronize()
+    assert ((Y - want).norm() / want.norm()).item() <= 2e-6    # two orders of fp32 sums
+    ctx.close()
+
+
 # ------------------------------------------------------------------ products recorded into CUDA graphs
 @pytest.mark.parametrize("kind,prec", [("direct", 0), ("gram", 0), ("gram", 1)])
 def test_recorded_products_do_not_depend_on_calls_in_between(fd, dev, kind, prec):
