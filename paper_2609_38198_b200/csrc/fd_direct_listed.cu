@@ -29,7 +29,7 @@ constexpr int kRing = 3;         // entries in a warp's ring
 constexpr int kMaxCtasPerSm = 8;     // (fewer where the room for the shares of cut row groups says so)
 
 struct NearParams {
-    const float4* x;             // ordered points, DP4 float4 each, padded to whole entries with points 1e18 away
+    const float4* x;             // ordered points, DP4 float4 each, padded to whole entries with points whose kernel values are 0
     const float* w;              // ordered right block, BT floats a point (row sums: one weight a point, or null)
     const float* left;           // may be null
     float* Y; int64_t ldy; int b;

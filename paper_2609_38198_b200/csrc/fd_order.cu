@@ -281,13 +281,14 @@ k_scatter(const unsigned short* __restrict__ leaf, int64_t n, const unsigned int
     if (i < n) perm[base[l] + counts[(size_t)l * gridDim.x + blockIdx.x] + rank] = (int)i;
 }
 
-// The points in their order, padded with points 1e18 away (kernel value 0).
+// The points in their order, padded with points whose squared distance from any other overflows (kernel value 0: lists are used only where
+// |x|^2 beta is a normal number).  Points 1e18 away are among those of a data set of that scale, and row sums count what they see.
 __global__ void __launch_bounds__(256)
 k_order_points(const float4* __restrict__ xs, int DP4, int64_t n, int64_t np, const int* __restrict__ perm, float4* __restrict__ out) {
     const int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (p >= np) return;
     const int64_t i = p < n ? perm[p] : -1;
-    for (int k = 0; k < DP4; ++k) out[p * DP4 + k] = i >= 0 ? xs[i * DP4 + k] : make_float4(1e18f, 1e18f, 1e18f, 1e18f);
+    for (int k = 0; k < DP4; ++k) out[p * DP4 + k] = i >= 0 ? xs[i * DP4 + k] : make_float4(3e38f, 3e38f, 3e38f, 3e38f);
 }
 
 // Bounding box of each tile of 16 consecutive positions, for up to 8 coordinates: 16 lanes a tile.

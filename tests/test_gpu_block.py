@@ -281,3 +281,25 @@ def test_far_tiles_are_left_out_of_direct_passes(N, kind, b):
     Zo = _gpu_kernel_rows(Xd, rows, 0.7 * beta) @ V.double()
     assert ((Z - Zo).norm() / Zo.norm()).item() <= 1e-6
     ctx.close()
+
+
+@pytest.mark.parametrize("N", [16385, 16397, 33000])
+def test_listed_passes_at_any_scale_of_the_data(N):
+    """Coordinates of the order of 1e18: scaled by a power of two (and beta by its inverse square), every result is that of the data of
+    order one, bit for bit; the points that fill up the last tile count nowhere."""
+    import __graft_entry__ as g
+    g.build()
+    import paper_2609_38198_b200 as fd
+    dev = torch.device("cuda:0")
+    X = 1.2 * torch.from_numpy(workloads.torus2(N, seed=5)).to(dev)      # (1e18 = 0.867 * 2^60: inside the data)
+    V = fd.to_colmajor(workloads.block(N, 5, seed=2), dev)
+    got = []
+    for p in (0, 60):
+        ctx = fd.Context(X * 2.0 ** p, b_max=8)
+        ctx.set_option("path", fd.FD_PATH_SIMT)
+        out = ctx.degree(40.0 * 2.0 ** (-2 * p), 1.0)
+        got.append((*out, ctx.apply(V)))
+        assert ctx.get_option("tile_share") < 0.8
+        ctx.close()
+    for a, b in zip(*got):
+        assert torch.equal(a, b) if torch.is_tensor(a) else a == b
