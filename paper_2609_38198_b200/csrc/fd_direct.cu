@@ -95,6 +95,12 @@ __device__ __forceinline__ void load_rows(const DirectParams& p, int64_t row0, i
     }
 }
 
+template <bool COPY, int R, int BT, class S>
+__device__ __forceinline__ float (&after_loop(float (&copy)[R][BT], S& acc))[R][BT] {
+    if constexpr (COPY) return copy;
+    else return acc.v;
+}
+
 // Block mode: Y[i, c] = left_i sum_j K_ij right_j V[j, c] for c < b <= BT.
 // (resident CTAs asked for: four, three or two, by the registers that the rows and sums of a thread need)
 constexpr int min_ctas(int regs) { return regs + 40 <= 128 ? 4 : regs + 40 <= 168 ? 3 : 2; }
@@ -116,6 +122,12 @@ k_direct(const DirectParams p) {
         float4 xi[R][DP4];
         load_rows<DP4, R>(p, row0, lane_row, xi);
         Sums<R, BT, (BT > 48 && DP4 != 5 && DP4 != 6)> acc;              // (packed, 17 to 24 coordinates spill 72 and 236 bytes a thread)
+        // After the loop the sums are worked on where they are, or in a copy: where the loop's are packed, and where the compiler spills less with a
+        // copy (up to 4 coordinates, 32 columns: 0 instead of 44 bytes a thread, 1 to 3 % faster; up to 12, 48: 44 instead of 68, 4 %).  In the
+        // other shapes a copy, or add() instead of the plain loop below, costs up to 7 % (N = 12000, b = 12 and 16: D = 4 179 and 181 instead of
+        // 166 and 171 us, D = 12 267 and 274 instead of 262 and 270; b = 8, D = 4: 120 instead of 115).
+        constexpr bool kCopy = (BT > 48 && DP4 != 5 && DP4 != 6) || (DP4 == 1 && BT == 32) || (DP4 == 3 && BT == 48);
+        float copy[R][BT];
         acc.clear();
         // a thread's own slots of sacc: row r, column c at mine[c * 256 + (256 / R) * r]
         float* mine = sacc + part * BT * kRowsT + lane_row;
@@ -139,7 +151,20 @@ k_direct(const DirectParams p) {
             for (int jj = part * (tj / H); jj < (part + 1) * (tj / H); ++jj) {
                 float kij[R];
                 kernel_values<DP4, R>(sx, jj, xi, p.nbeta2, kij);
-                acc.add(kij, reinterpret_cast<const float4*>(&sw[jj * BP]));
+                if constexpr (kCopy) acc.add(kij, reinterpret_cast<const float4*>(&sw[jj * BP]));
+                else {
+#pragma unroll
+                    for (int c4 = 0; c4 < BT / 4; ++c4) {
+                        const float4 w = *reinterpret_cast<const float4*>(&sw[jj * BP + 4 * c4]);
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            acc.v[r][4 * c4 + 0] = fmaf(kij[r], w.x, acc.v[r][4 * c4 + 0]);
+                            acc.v[r][4 * c4 + 1] = fmaf(kij[r], w.y, acc.v[r][4 * c4 + 1]);
+                            acc.v[r][4 * c4 + 2] = fmaf(kij[r], w.z, acc.v[r][4 * c4 + 2]);
+                            acc.v[r][4 * c4 + 3] = fmaf(kij[r], w.w, acc.v[r][4 * c4 + 3]);
+                        }
+                    }
+                }
             }
             if (((t + 1) & (kFlushCols / tj - 1)) == 0 && t + 1 < n) {
                 // two-level summation keeps the rounding error of long column ranges at the 1e-7 level
@@ -154,11 +179,13 @@ k_direct(const DirectParams p) {
                 flushed = true;
             }
         }
-        float sum[R][BT];
+        if (kCopy) {
 #pragma unroll
-        for (int r = 0; r < R; ++r)
+            for (int r = 0; r < R; ++r)
 #pragma unroll
-            for (int c = 0; c < BT; ++c) sum[r][c] = acc.get(r, c);
+                for (int c = 0; c < BT; ++c) copy[r][c] = acc.get(r, c);
+        }
+        float (&sum)[R][BT] = after_loop<kCopy>(copy, acc);
         if (flushed) {
 #pragma unroll
             for (int r = 0; r < R; ++r)
