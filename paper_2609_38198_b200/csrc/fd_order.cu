@@ -43,21 +43,36 @@ namespace {
 
 constexpr int kSamples = 4096;
 
-// Counts pairs of 512 sampled points farther apart than limit2 (squared distance).
+// Counts pairs of 512 sampled points farther apart than limit2 (squared distance), and those within a quarter of that distance.
 __global__ void __launch_bounds__(256)
 k_far_pairs(const float* __restrict__ xs, int DP, int64_t n, float limit2, unsigned int* __restrict__ count) {
     const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;      // one sampled row per warp
     const float* xi = xs + (n * i / 512) * DP;
-    unsigned int far = 0;
+    unsigned int far = 0, close = 0;
     for (int j = lane; j < 512; j += 32) {
         const float* xj = xs + (n * j / 512) * DP;
         float d2 = 0.f;
         for (int k = 0; k < DP; ++k) { const float d = xi[k] - xj[k]; d2 = fmaf(d, d, d2); }
         far += d2 > limit2;
+        close += d2 <= 0.0625f * limit2;
     }
 #pragma unroll
-    for (int m = 16; m >= 1; m >>= 1) far += __shfl_xor_sync(0xffffffffu, far, m);
-    if (lane == 0) atomicAdd(count, far);
+    for (int m = 16; m >= 1; m >>= 1) { far += __shfl_xor_sync(0xffffffffu, far, m); close += __shfl_xor_sync(0xffffffffu, close, m); }
+    if (lane == 0) { atomicAdd(count, far); atomicAdd(count + 1, close); }
+}
+
+// Whether lists by the boxes are expected to leave out enough, from the sampled pairs: `far` of 512 x 512 beyond the limit, `close` within a quarter
+// of its distance r.  The two counts give the data's dimension d at that scale (near pairs within a distance grow with its d-th power), this
+// the radius of the tiles, and tiles count as near up to r and their two radii (twice these where tiles are of 128 points and boxes larger).
+// 19 data sets (circles, tori, spheres, boxes, normal clouds, clusters and lines in 2 to 8 coordinates), N = 16384 .. 32000: direct differences:
+// lists that were used were predicted at up to 0.75 of the tiles, those refused from 0.78 on (one: 0.68); Gram form 0.91 and 1.05.
+bool lists_expected(unsigned int far, unsigned int close, int64_t N, bool direct) {
+    constexpr double kPairs = 512.0 * 512.0;
+    const double near = std::max(1.0 - far / kPairs - 1.0 / 512.0, 1.0 / kPairs), mid = std::max((double)close - 512.0, 1.0) / kPairs;   // (without the points themselves)
+    const double d = std::max(std::log(near / mid) / std::log(4.0), 0.05);
+    auto radius = [&](double points) { return std::pow(points / ((double)N * near), 1.0 / d); };
+    const double reach = direct ? radius(64.0) + radius(16.0) : 2.0 * (radius(256.0) + radius(128.0));
+    return near * std::pow(1.0 + reach, d) < (direct ? 0.77 : 0.97);
 }
 
 // part[block][k * DP + l] = sum over this block's 128 samples of (x_k - mu_k) (x_l - mu_l).
@@ -432,15 +447,18 @@ fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide) {
         // (an order that left out too little at some bandwidth would leave out less at a smaller one: in units of the degree passes' limit)
         if (scaled_beta <= c->refused_beta * 1.2) return FD_OK;
         fresh = true;
-        FD_CUDA(c, cudaMemsetAsync(small, 0, 4, c->stream));
+        FD_CUDA(c, cudaMemsetAsync(small, 0, 8, c->stream));
         k_far_pairs<<<64, 256, 0, c->stream>>>(c->xs(), L.DP, N, limit2, small);
         FD_LAUNCH_CHECK(c, "k_far_pairs");
-        unsigned int far = 0;
-        FD_CUDA(c, cudaMemcpyAsync(&far, small, 4, cudaMemcpyDeviceToHost, c->stream));
+        unsigned int count[2] = {0, 0};
+        FD_CUDA(c, cudaMemcpyAsync(count, small, 8, cudaMemcpyDeviceToHost, c->stream));
         FD_CUDA(c, cudaStreamSynchronize(c->stream));
-        // (Share of far pairs from which an order is worth making: 0.4, where tiles are small against the data's extent; 0.8 for fewer than
-        // 32768 points.  2-torus, beta = 30, 0.70 of the pairs far: 0.53 of the tiles remain at N = 80000, 0.8 at N = 16384.)
-        if ((double)far < 0.4 * 512.0 * 512.0) return FD_OK;
+        // Share of far pairs from which an order is tried: 0.4.  Below 32768 points it costs as much as the pass itself (190 to 450 us), so that between
+        // 0.4 and 0.8 it is made only where it is expected to stay: first degree pass, N = 20000: 6-dimensional data 1120 -> 720 us, 2-torus at
+        // beta = 20 834 -> 520.  Where it stays, two to five products at the bandwidth pay for it (2-torus, N = 16384, beta = 30: 100 us for 153
+        // a product of 16 columns; circle, Gram form, beta = 20: 177 us for 36).
+        if ((double)count[0] < 0.4 * 512.0 * 512.0) return FD_OK;
+        if (N < 32768 && (double)count[0] < 0.8 * 512.0 * 512.0 && !lists_expected(count[0], count[1], N, direct)) return FD_OK;
         // scratch: the operand buffers (re-packed in the new order afterwards); at least 64 bytes per point each
         int depth = 0;
         while (((int64_t)(L.direct_lists ? 16 : 128) << depth) < N && depth < 12) ++depth;

@@ -82,6 +82,27 @@ def test_products_over_noted_tiles(fd, dev, kind, N):
     ctx.close(); plain.close()
 
 
+@pytest.mark.parametrize("D,N,beta,kind,listed", [(4, 16384, 30.0, "direct", True), (4, 20000, 20.0, "direct", False), (6, 16384, 20.0, "direct", False),
+                                                  (4, 32767, 22.0, "direct", True), (4, 32767, 10.0, "gram", True), (4, 16384, 10.0, "gram", False)])
+def test_an_order_that_would_not_stay_is_not_made(fd, dev, D, N, beta, kind, listed):
+    """Below 32768 points, with 0.4 to 0.8 of the pairs far: the points of flat tori are ordered where lists come out of it; else the first degree pass
+    launches what one without far pairs does, and the sampling of the pairs."""
+    a = np.random.default_rng(7).random((N, D // 2)) * 2 * np.pi
+    X = torch.from_numpy(np.concatenate([np.cos(a), np.sin(a)], 1).astype(np.float32)).to(dev)
+    launches = []
+    for bt in (0.01 * beta, beta):
+        ctx = fd.Context(X, b_max=8)
+        ctx.set_option("path", fd.FD_PATH_SIMT if kind == "direct" else fd.FD_PATH_TC)
+        ctx.set_option("tc_max_mag", 1e4)
+        n = fd.fd_launch_count()
+        ctx.degree(bt, 1.0)
+        launches.append(fd.fd_launch_count() - n)
+        share = ctx.get_option("tile_share")
+        ctx.close()
+    assert (share < 0.9) == listed
+    assert listed or launches[1] <= launches[0] + (1 if kind == "direct" else 2)       # (Gram form: sampled for the product's limit and for the sums')
+
+
 @pytest.mark.parametrize("N,k,b,m_max", [(24, 5, 7, 24), (65, 12, 16, 65), (300, 20, 1, 64), (300, 9, 33, 96), (700, 30, 64, 224), (900, 20, 70, 210),
                                          (512, 8, 16, 59)])
 def test_solves_with_blocks_of_many_widths(fd, dev, N, k, b, m_max):
