@@ -65,14 +65,15 @@ k_far_pairs(const float* __restrict__ xs, int DP, int64_t n, float limit2, unsig
 // of its distance r.  The two counts give the data's dimension d at that scale (near pairs within a distance grow with its d-th power), this
 // the radius of the tiles, and tiles count as near up to r and their two radii (twice these where tiles are of 128 points and boxes larger).
 // 19 data sets (circles, tori, spheres, boxes, normal clouds, clusters and lines in 2 to 8 coordinates), N = 16384 .. 32000: direct differences:
-// lists that were used were predicted at up to 0.75 of the tiles, those refused from 0.78 on (one: 0.68); Gram form 0.91 and 1.05.
+// lists that were used were predicted at up to 0.75 of the tiles, those refused from 0.76 on (two: 0.67, 0.68); Gram form up to 1.00 and, most of
+// them, from 1.05 on (eight: 0.88 to 0.99).
 bool lists_expected(unsigned int far, unsigned int close, int64_t N, bool direct) {
     constexpr double kPairs = 512.0 * 512.0;
     const double near = std::max(1.0 - far / kPairs - 1.0 / 512.0, 1.0 / kPairs), mid = std::max((double)close - 512.0, 1.0) / kPairs;   // (without the points themselves)
     const double d = std::max(std::log(near / mid) / std::log(4.0), 0.05);
     auto radius = [&](double points) { return std::pow(points / ((double)N * near), 1.0 / d); };
     const double reach = direct ? radius(64.0) + radius(16.0) : 2.0 * (radius(256.0) + radius(128.0));
-    return near * std::pow(1.0 + reach, d) < (direct ? 0.77 : 0.97);
+    return near * std::pow(1.0 + reach, d) < (direct ? 0.77 : 1.04);
 }
 
 // part[block][k * DP + l] = sum over this block's 128 samples of (x_k - mu_k) (x_l - mu_l).

@@ -83,12 +83,15 @@ def test_products_over_noted_tiles(fd, dev, kind, N):
 
 
 @pytest.mark.parametrize("D,N,beta,kind,listed", [(4, 16384, 30.0, "direct", True), (4, 20000, 20.0, "direct", False), (6, 16384, 20.0, "direct", False),
-                                                  (4, 32767, 22.0, "direct", True), (4, 32767, 10.0, "gram", True), (4, 16384, 10.0, "gram", False)])
+                                                  (4, 32767, 22.0, "direct", True), (4, 32767, 10.0, "gram", True), (4, 16384, 10.0, "gram", False),
+                                                  (3, 24000, 17.0, "gram", True), (3, 16384, 24.0, "gram", True)])
 def test_an_order_that_would_not_stay_is_not_made(fd, dev, D, N, beta, kind, listed):
-    """Below 32768 points, with 0.4 to 0.8 of the pairs far: the points of flat tori are ordered where lists come out of it; else the first degree pass
+    """Below 32768 points, with 0.4 to 0.8 of the pairs far: the points of flat tori and of a sphere are ordered where lists come out of it; else the first degree pass
     launches what one without far pairs does, and the sampling of the pairs."""
-    a = np.random.default_rng(7).random((N, D // 2)) * 2 * np.pi
-    X = torch.from_numpy(np.concatenate([np.cos(a), np.sin(a)], 1).astype(np.float32)).to(dev)
+    rng = np.random.default_rng(7)
+    a, z = rng.random((N, D // 2)) * 2 * np.pi, rng.standard_normal((N, 3))
+    X = z / np.linalg.norm(z, axis=1, keepdims=True) if D == 3 else np.concatenate([np.cos(a), np.sin(a)], 1)
+    X = torch.from_numpy(X.astype(np.float32)).to(dev)
     launches = []
     for bt in (0.01 * beta, beta):
         ctx = fd.Context(X, b_max=8)
