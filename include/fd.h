@@ -81,8 +81,10 @@ enum { FD_PATH_AUTO = 0, FD_PATH_SIMT = 1, FD_PATH_TC = 2 };
  * max|x - mu|^2 >= "tc_max_mag", then returns FD_ERR_UNSUPPORTED).  fd_create refuses D > FD_MAX_D. */
 #define FD_MAX_D 60
 
-/* Bytes of device workspace fd_create needs.  O(N (D + b_max + m_max)); beside that, up to 2^19 points, tile lists and notes of N^2 / 4096 bytes
- * (N^2 / 200 with up to 8 coordinates and 2^17 points).
+/* Bytes of device workspace fd_create asks for.  O(N (D + b_max + m_max)); beside that, up to 2^19 points, tile lists and notes of
+ * 5 N^2 / 16384 bytes (5 N^2 / 1024 with up to 8 coordinates and 2^17 points).  fd_create also takes a workspace with room for
+ * N^2 / 16384 (N^2 / 2048) bytes of them: Gram-form passes then list tiles by bounding boxes alone, direct-difference passes take every
+ * tile.  Anything smaller is refused.
  * b_max: widest block passed to fd_apply / fd_apply_general (1..256).
  * m_max: basis capacity for fd_eigs (columns); 0 if fd_eigs will not be called. */
 size_t fd_workspace_bytes(int64_t N, int32_t D, int32_t b_max, int32_t m_max);

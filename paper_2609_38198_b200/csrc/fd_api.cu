@@ -34,7 +34,7 @@ static size_t carve(size_t& cur, size_t bytes) {
     return off;
 }
 
-Layout make_layout(int64_t N, int32_t D, int32_t b_max, int32_t m_max) {
+Layout make_layout(int64_t N, int32_t D, int32_t b_max, int32_t m_max, bool notes) {
     Layout L;
     L.N = N; L.D = D; L.b_max = b_max; L.m_max = m_max;
     L.DP = (int32_t)round_up(D, 4);
@@ -69,23 +69,29 @@ Layout make_layout(int64_t N, int32_t D, int32_t b_max, int32_t m_max) {
     L.status = carve(cur, 512);      // status word, cycles, sums (64), counts (128); notes of the direct-difference products (256)
     L.symsum = carve(cur, (size_t)N * 8);
     L.weights = carve(cur, (size_t)L.NP * 4);
-    // tile lists: N^2 / 16384 bytes, 17 MB at 2^19 points; larger sets run over all tiles (as do small ones, where nothing is gained)
+    // tile lists and notes: 5 N^2 / 16384 bytes, 84 MB at 2^19 points; larger sets run over all tiles (as do small ones, where nothing is gained)
     if (N >= (L.DP <= 8 ? 16384 : 32768) && N <= (int64_t)1 << 19) {
         const size_t tiles = (size_t)(L.NP / 128), pairs = tiles / 2;
         L.perm = carve(cur, (size_t)N * 4);
-        // (direct-difference kernels: 64 rows x 16 points; up to 8 coordinates and 2^17 points, 33 MB of lists)
-        L.direct_lists = L.DP <= 8 && N <= (int64_t)1 << 17;
-        const size_t groups = L.direct_lists ? 2 * tiles : pairs, col_tiles = L.direct_lists ? 8 * tiles : tiles;
+        // (direct-difference kernels: 64 rows x 16 points; up to 8 coordinates and 2^17 points: 5 N^2 / 1024 bytes, 84 MB there)
+        const bool fine = L.DP <= 8 && N <= (int64_t)1 << 17;
+        L.direct_lists = fine && notes;
+        const size_t groups = L.direct_lists ? 2 * tiles : pairs, col_tiles = fine ? 8 * tiles : tiles;
         L.boxes = carve(cur, col_tiles * 2 * 8 * 4);
         if (L.DP > 8) L.zproj = carve(cur, (size_t)N * 8 * 4);
-        for (int i = 0; i < 2; ++i) {
-            L.lists[i] = carve(cur, groups * col_tiles * 2);
-            L.list_counts[i] = carve(cur, (4 * groups + 2) * 4);
+        L.lists[0] = carve(cur, groups * col_tiles * 2);
+        L.list_counts[0] = carve(cur, (4 * groups + 2) * 4);
+        if (notes) {
+            L.lists[1] = carve(cur, groups * col_tiles * 2);
+            L.list_counts[1] = carve(cur, (4 * groups + 2) * 4);
+            L.lists[2] = carve(cur, pairs * tiles * 2);
+            L.list_counts[2] = carve(cur, (4 * pairs + 2) * 4);
+            L.near = carve(cur, std::max(2 * tiles * tiles, L.direct_lists ? groups * col_tiles : 0));
+            if (L.direct_lists) L.xord = carve(cur, (size_t)L.NP * L.DP * 4);
+        } else {
+            L.lists[1] = L.lists[2] = L.lists[0];
+            L.list_counts[1] = L.list_counts[2] = L.list_counts[0];
         }
-        L.lists[2] = carve(cur, pairs * tiles * 2);
-        L.list_counts[2] = carve(cur, (4 * pairs + 2) * 4);
-        L.near = carve(cur, std::max(2 * tiles * tiles, L.direct_lists ? groups * col_tiles : 0));
-        if (L.direct_lists) L.xord = carve(cur, (size_t)L.NP * L.DP * 4);
     }
     if (m_max > 0) {
         L.eig_q = carve(cur, (size_t)N * m_max * 4);
@@ -145,6 +151,7 @@ fd_status fd_create(fd_ctx** out, const float* X_dev, int64_t N, int32_t D, int6
     if (N > ((int64_t)1 << 31) - 1024) return FD_ERR_UNSUPPORTED;
     if ((reinterpret_cast<uintptr_t>(ws_dev) & 255) != 0) return FD_ERR_INVALID;
     Layout L = make_layout(N, D, b_max, m_max);
+    if (ws_bytes < L.total) L = make_layout(N, D, b_max, m_max, false);       // (what a workspace was before there were notes)
     if (ws_bytes < L.total) return FD_ERR_WORKSPACE;
     fd_ctx* c = new (std::nothrow) fd_ctx();
     if (!c) return FD_ERR_INVALID;

@@ -30,7 +30,8 @@ struct Layout {
     size_t wp = 0;                   // N x BP block of scratch (numerators and denominator of the out-of-sample extension)
     size_t part = 0, part_floats = 0;
     size_t xp_col = 0, xp_row = 0, wt_hi = 0, wt_lo = 0, colscale = 0, status = 0;
-    // order of the points and tile lists of the Gram-form kernels (fd_order.cu); 0: not provisioned for this N
+    // order of the points and tile lists of the Gram-form kernels (fd_order.cu); 0: not provisioned for this N (near: for this workspace; all
+    // lists then share one buffer)
     size_t perm = 0, boxes = 0, zproj = 0, lists[3] = {0, 0, 0}, list_counts[3] = {0, 0, 0}, near = 0, xord = 0;
     bool direct_lists = false;       // provisioned for the direct-difference kernels as well
     size_t weights = 0;              // NP right weights of a Gram-form row sum
@@ -38,7 +39,9 @@ struct Layout {
     size_t eig_q = 0, eig_w = 0, eig_x = 0, eig_r = 0, eig_small = 0, eig_small_doubles = 0;
     size_t total = 0;
 };
-Layout make_layout(int64_t N, int32_t D, int32_t b_max, int32_t m_max);
+// notes: with the degree passes' notes, a list buffer for every kind of pass and lists of the direct-difference kernels; else one buffer for
+// lists by the boxes (Gram form only).
+Layout make_layout(int64_t N, int32_t D, int32_t b_max, int32_t m_max, bool notes = true);
 
 // Coordinates the kernels work on (keep[0 .. kept)) and those left out because all points share them, with the shared values.
 struct Coords {

@@ -419,7 +419,8 @@ fd_status tile_lists(fd_ctx* c, double beta, int kind, bool decide) {
     if (L.perm == 0 || c->order_state < 0) return FD_OK;
     const bool direct = kind == 2 || kind == 4;
     const bool noted = c->near_beta == beta && c->near_direct == direct && kind != 1 && kind != 2;
-    const int buf = kind == 0 || kind == 4 ? 0 : kind == 3 ? 2 : 1;
+    if (kind == 3 && L.near == 0) kind = 1;                        // (one buffer for all, by the boxes: the first degree pass's lists serve the second)
+    const int buf = L.near == 0 || kind == 0 || kind == 4 ? 0 : kind == 3 ? 2 : 1;
     auto& listed = c->listed[buf];
     const int held = noted ? 8 + kind : kind;                      // what the buffer would hold
     if (st.beta == beta && (!st.on || (!c->captured && listed.kind == held && listed.beta == beta))) return FD_OK;

@@ -560,7 +560,7 @@ fd_status apply_tc(fd_ctx* c, const ApplyArgs& a) {
     }
     if (rowsum && sym) {
         // the pass with squares notes which tiles hold values that count, for the lists of the pass and the products after it
-        const bool note_near = ordered && a.rowsq && a.decide && !c->captured && (c->near_beta != a.beta || c->near_direct);
+        const bool note_near = L.near != 0 && ordered && a.rowsq && a.decide && !c->captured && (c->near_beta != a.beta || c->near_direct);
         if (note_near) c->near_beta = -1.0;
         FD_TRY(launch_sym_rowsum(c, mr, mc, p.weights, a.left, a.Y, a.rowsq, row_perm, use_lists, note_near));
         if (note_near) { c->near_beta = a.beta; c->near_direct = false; c->near_unproven = true; }

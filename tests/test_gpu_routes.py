@@ -132,3 +132,51 @@ def test_solves_with_blocks_of_many_widths(fd, dev, N, k, b, m_max):
         assert (M @ Ud - Ud * torch.tensor(ev, device=dev)).norm(dim=0).max().item() <= 5e-6 * lam[0]
         Q0 = U
     ctx.close()
+
+
+@pytest.mark.parametrize("kind,N", [("gram", 33023), ("direct", 16384), ("direct", 33000)])
+def test_a_workspace_without_room_for_notes(fd, dev, kind, N, monkeypatch):
+    """The smallest workspace that fd_create takes is smaller than what fd_workspace_bytes asks for where that has room for notes.  Gram form: tiles by
+    the boxes, direct differences: every tile; the same results as with notes (to the rounding of another order of the sums), degrees and products
+    in either precision, after a change of bandwidth too, and nothing beyond the workspace's end is touched."""
+    from paper_2609_38198_b200 import binding
+    if kind == "direct":
+        X, beta, path = workloads.torus2(N, seed=1), 60.0, fd.FD_PATH_SIMT
+    else:
+        X, beta, path = workloads.latent_torus(N, seed=42), 3.0, fd.FD_PATH_TC
+    Xt = torch.from_numpy(X).to(dev)
+    V = fd.to_colmajor(workloads.block(N, 20, seed=3), dev)
+    asked = fd.fd_workspace_bytes(N, X.shape[1], 20, 0)
+
+    def context(size):
+        monkeypatch.setattr(binding, "fd_workspace_bytes", lambda *a: size)
+        ctx = fd.Context(Xt, b_max=20)
+        ctx.set_option("path", path)
+        ctx.set_option("tc_max_mag", 1e4)
+        return ctx
+
+    refused, taken = asked // 2, asked
+    while taken - refused > 256:
+        size = (refused + taken) // 512 * 256
+        try:
+            context(size).close()
+            taken = size
+        except fd.FdError as e:
+            assert e.status == fd.FD_ERR_WORKSPACE
+            refused = size
+    assert taken < asked - N * N // 32768
+    small, full = context(taken), context(asked)
+    end = small._ws[-small._ws.data_ptr() % 256 + taken:]
+    end.fill_(0x5A)
+    for bt in (beta, 0.4 * beta, beta):
+        (q, d, s, so, so2), (qf, df, sf, sof, so2f) = small.degree(bt, 1.0), full.degree(bt, 1.0)
+        assert max(((a - b).abs() / b).max().item() for a, b in ((q, qf), (d, df), (s, sf))) <= 2e-6
+        assert abs(so - sof) <= 1e-6 * sof and abs(so2 - so2f) <= 1e-6 * so2f
+        Y, Z = small.apply(V), full.apply(V)
+        assert ((Y - Z).norm() / Z.norm()).item() <= 2e-6 and torch.equal(small.apply(V), Y)
+        Y, Z = small.apply(V, prec=fd.FD_PREC_FAST), full.apply(V, prec=fd.FD_PREC_FAST)
+        assert ((Y - Z).norm() / Z.norm()).item() <= 2e-5
+    share, noted = small.get_option("tile_share"), full.get_option("tile_share")
+    assert noted < 0.8 and (share == 1.0 if kind == "direct" else noted < share < 0.9)
+    assert bool((end == 0x5A).all())
+    small.close(); full.close()
