@@ -31,7 +31,8 @@ def _kernel_rows(Zd, Xd, beta):
                                    (2048, 3, 16), (2049, 4, 16), (3071, 2, 1), (3072, 4, 8), (3073, 4, 8)])
 def test_small_narrow_products(fd, dev, N, D, b):
     """Up to 3072 points with up to 8 coordinates and 8 columns (2048 and 16): one launch, sums inside a cluster.  Square products with scalings on both sides, a
-    right block and an output with a pitch of their own, external rows, a replay from a graph.  Gate 1e-6 of the direct-difference family."""
+    right block and an output with a pitch of their own, external rows, a replay from a graph with another right block in the same buffer (the bits of
+    the eager call).  Gate 1e-6 of the direct-difference family."""
     rng = np.random.default_rng(N + 7 * b)
     X = torch.from_numpy(rng.standard_normal((N, D)).astype(np.float32)).to(dev)
     beta, ld = 0.7, N + 5
@@ -51,13 +52,29 @@ def test_small_narrow_products(fd, dev, N, D, b):
         Ro = _kernel_rows(Z.double(), Xd, beta) @ Vd
         assert ((R.double() - Ro).norm() / Ro.norm()).item() <= 1e-6
     ctx.close()
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    ctx = fd.Context(X, b_max=b, stream=stream)
+    ctx.apply_general(beta, V, left=left, right=right, out=Y)
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=stream):
+        ctx.apply_general(beta, V, left=left, right=right, out=Y)
+    V.mul_(-0.7).add_(0.2)
+    torch.cuda.synchronize()
+    want = ctx.apply_general(beta, V, left=left, right=right)
+    Y.zero_()
+    torch.cuda.synchronize()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(Y, want)
+    ctx.close()
 
 
 @pytest.mark.parametrize("kind", ["direct", "gram"])
 @pytest.mark.parametrize("N", [16384, 33023])
 def test_products_over_noted_tiles(fd, dev, kind, N):
-    """The tiles that a degree pass noted: the product with them is that over all tiles (to the rounding of another order of the sums), and never
-    over more of them than the boxes leave."""
+    """The tiles that a degree pass noted: the product with them is that over all tiles (to the rounding of another order of the sums), and over
+    clearly fewer than the boxes leave.  (A context in which a product has been recorded into a graph takes no notes: it lists by the boxes.)"""
     if kind == "direct":
         X, beta, path = workloads.torus2(N, seed=1), 60.0, fd.FD_PATH_SIMT
     else:
@@ -66,20 +83,33 @@ def test_products_over_noted_tiles(fd, dev, kind, N):
         X, beta, path = workloads.latent_torus(N, seed=42), 3.0, fd.FD_PATH_TC
     Xt = torch.from_numpy(X).to(dev)
     V = fd.to_colmajor(workloads.block(N, 20, seed=3), dev)
-    ctx, plain = (fd.Context(Xt, b_max=20) for _ in range(2))
-    for c in (ctx, plain):
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    ctx, plain, boxes = fd.Context(Xt, b_max=20), fd.Context(Xt, b_max=20), fd.Context(Xt, b_max=20, stream=stream)
+    for c in (ctx, plain, boxes):
         c.set_option("path", path)
         c.set_option("tc_max_mag", 1e4)
     s = ctx.degree(beta, 1.0)[2]
     share = ctx.get_option("tile_share")
-    assert share < 0.8
     Y = ctx.apply_general(beta, V, left=s, right=s)
     Z = plain.apply_general(beta, V, left=s, right=s)            # (no degree pass: every tile)
     assert ((Y - Z).norm() / Z.norm()).item() <= 2e-6
+    torch.cuda.synchronize()
+    B = boxes.apply_general(0.01 * beta, V)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        boxes.apply_general(0.01 * beta, V, out=B)
+    torch.cuda.synchronize()
+    boxes.degree(beta, 1.0)
+    B = boxes.apply_general(beta, V, left=s, right=s)
+    torch.cuda.synchronize()
+    assert ((B - Z).norm() / Z.norm()).item() <= 2e-6
+    assert share < 0.9 * boxes.get_option("tile_share") and boxes.get_option("tile_share") < 0.9
     ctx.degree(0.5 * beta, 1.0)
     assert torch.equal(ctx.degree(beta, 1.0)[2], s) and ctx.get_option("tile_share") == share
     assert torch.equal(ctx.apply_general(beta, V, left=s, right=s), Y)
-    ctx.close(); plain.close()
+    ctx.close(); plain.close(); boxes.close()
 
 
 @pytest.mark.parametrize("D,N,beta,kind,listed", [(4, 16384, 30.0, "direct", True), (4, 20000, 20.0, "direct", False), (6, 16384, 20.0, "direct", False),
