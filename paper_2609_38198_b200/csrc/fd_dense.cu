@@ -42,7 +42,6 @@ __device__ __forceinline__ void copy4(uint32_t dst, const float* src, int valid)
 template <int UI, int UJ, bool ALIGNED>
 __global__ void __launch_bounds__(128)
 k_tn_partial(const Panel A, const Panel B, int64_t N, int64_t rows_per_chunk, double* __restrict__ part) {
-    grid_wait();
     grid_go();
     extern __shared__ __align__(16) float sm[];
     constexpr int TI = 16 * UI, TJ = 8 * UJ, kStage = (TI + TJ) * kTnPitch;

@@ -11,11 +11,11 @@
 // results are bit-reproducible run to run.  (Letting the CTA that comes last add them needs no second launch but puts one
 // CTA's chain of dependent reads at the end: 183 us instead of 8 at N = 2048.)
 //
-// What bounds it: instruction issue and the latency between dependent instructions, 2 D + b + 2 FMA-pipe operations per pair (N = 16384, listed:
-// two of three issue slots taken, FMA pipe 54 %, 1.6 eligible warps a scheduler).  A thread owns two or four rows (four: the two halves of the
+// What bounds it: instruction issue and the latency between dependent instructions, 2 D + b + 2 FMA-pipe operations per pair (N = 12000,
+// D = 4, b = 16: 74 % of the issue slots taken, FMA pipe 62 %, 2.0 eligible warps a scheduler).  A thread owns two or four rows (four: the two halves of the
 // CTA take half the columns of a tile each), which share the broadcast reads of x_j and w_j from shared memory; with one row per
 // thread these cost as many slots as a fifth of the FMAs.  (Two rows per packed instruction, add / fma.rn.f32x2, halve
-// the instruction count but ran at half the FMA rate: 5 to 15 % slower in every shape.)  Right-hand columns are read from V
+// the instruction count but ran at half the FMA rate: 5 to 15 % slower in every shape; two columns per packed instruction gain for 64 columns, fd_direct.h.)  Right-hand columns are read from V
 // as it is (column-major) and scaled on the way into shared memory: no packing pass.
 // N = 16384, D = 4, b = 16: 412 -> 309 us a product; N = 12000, D = 12, b = 48: 944 -> 639 us; N = 6000, D = 2, both degree passes:
 // 136 -> 109 us (one row per thread, separate packing pass, one CTA more or less per SM at the end).
@@ -33,7 +33,6 @@ namespace {
 
 using namespace direct;
 
-constexpr int kThr = 128;        // threads per CTA
 constexpr int kRowsT = 256;      // rows per row tile
 constexpr int kTJ = 64;          // points per column tile, at most (DirectParams::tj_log2)
 constexpr int kFlushCols = 2048; // columns between flushes of the fp32 tile accumulators
@@ -497,13 +496,6 @@ fd_status launch(fd_ctx* c, Kernel kernel, int smem, int per_sm, int BT, DirectP
     }
     return FD_OK;
 }
-template <class Kernel>
-int resident(Kernel kernel, int smem) {              // a property of the compiled kernel: asked once
-    int n = 0;
-    if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kThr, smem) != cudaSuccess || n < 1) n = 1;
-    return std::min(n, kMaxCtasPerSm);
-}
 
 // Largest set that goes to the cluster kernel.  Against the ranges above: N = 1000, b = 8: 18.0 -> 8.8 us; 2048: 15.5 -> 11.3; 4096: 25.5 -> 25.3; b = 16,
 // N = 2048: 19.4 -> 11.7, 4096: 34.7 -> 36.5.
@@ -519,7 +511,7 @@ fd_status launch_block(fd_ctx* c, const DirectParams& p) {
         }
     constexpr int R = 4 * DP4 + BT <= 32 ? 4 : 2, H = R * kThr / kRowsT;
     constexpr int smem = (kTJ * DP4 * 4 + kTJ * (BT + 4) + H * BT * kRowsT) * 4;
-    static const int per_sm = resident(k_direct<DP4, BT, R>, smem);
+    static const int per_sm = resident(k_direct<DP4, BT, R>, smem, kMaxCtasPerSm);
     return launch(c, k_direct<DP4, BT, R>, smem, per_sm, BT, p);
 }
 
@@ -527,7 +519,7 @@ template <int DP4>
 fd_status launch_dp(fd_ctx* c, int BT, const DirectParams& p) {
     switch (BT) {
         case 0: {
-            static const int per_sm = resident(k_direct_rowsum<DP4>, 0);
+            static const int per_sm = resident(k_direct_rowsum<DP4>, 0, kMaxCtasPerSm);
             return launch(c, k_direct_rowsum<DP4>, 0, per_sm, 0, p);
         }
         case 4: return launch_block<DP4, 4>(c, p);

@@ -10,6 +10,16 @@ fd_status apply_direct_listed(fd_ctx* c, const ApplyArgs& a, int kind);
 
 namespace direct {
 
+constexpr int kThr = 128;        // threads per CTA
+
+template <class Kernel>
+int resident(Kernel kernel, int smem, int most) {    // CTAs per SM, a property of the compiled kernel: asked once
+    int n = 0;
+    if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kThr, smem) != cudaSuccess || n < 1) n = 1;
+    return n < most ? n : most;
+}
+
 inline int pick_bt(int bc) { return bc <= 4 ? 4 : bc <= 8 ? 8 : bc <= 16 ? 16 : bc <= 24 ? 24 : bc <= 32 ? 32 : bc <= 48 ? 48 : 64; }
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -42,7 +52,8 @@ __device__ __forceinline__ void kernel_values(const float4* sx, int jj, const fl
 }
 
 // Sums of BT columns for R rows.  add(): sum[r][c] += kij[r] w[c].  64 columns use packed arithmetic (two columns an instruction: half the issue
-// slots, the same time on the FMA pipe): N = 12000, D = 4: 744 -> 627 us a product.  Narrower blocks are 2 to 8 % slower with it.
+// slots, the same time on the FMA pipe): N = 12000, D = 4: 744 -> 627 us a product, D = 32: 988 -> 930 (below 4500 points 2 to 4 % slower there).
+// Narrower blocks are 2 to 8 % slower with it.
 template <int R, int BT, bool PACKED = (BT > 48)>
 struct Sums;
 template <int R, int BT>

@@ -21,7 +21,7 @@ namespace {
 
 using namespace direct;
 
-constexpr int kThr = 128, kWarps = kThr / 32;
+constexpr int kWarps = kThr / 32;
 constexpr int kRowsG = 64;       // rows of a group: two per lane
 constexpr int kRows = 2;
 constexpr int kEntry = 16;       // points of a list entry
@@ -408,25 +408,18 @@ fd_status launch(fd_ctx* c, Kernel kernel, int smem, int per_sm, int BT, NearPar
     FD_LAUNCH_CHECK(c, "k_near_fix");
     return FD_OK;
 }
-template <class Kernel>
-int resident(Kernel kernel, int smem) {              // a property of the compiled kernel: asked once
-    int n = 0;
-    if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kThr, smem) != cudaSuccess || n < 1) n = 1;
-    return std::min(n, kMaxCtasPerSm);
-}
 
 template <int DP4, int BT>
 fd_status launch_block(fd_ctx* c, const NearParams& p) {
     constexpr int smem = kWarps * kRing * kEntry * (DP4 + BT / 4) * 16;
-    static const int per_sm = resident(k_near<DP4, BT>, smem);
+    static const int per_sm = resident(k_near<DP4, BT>, smem, kMaxCtasPerSm);
     return launch(c, k_near<DP4, BT>, smem, per_sm, BT, p);
 }
 template <int DP4>
 fd_status launch_dp(fd_ctx* c, int BT, const NearParams& p) {
     switch (BT) {
         case 0: {
-            static const int plain = resident(k_near_rowsum<DP4, false>, 0), weighted = resident(k_near_rowsum<DP4, true>, 0);
+            static const int plain = resident(k_near_rowsum<DP4, false>, 0, kMaxCtasPerSm), weighted = resident(k_near_rowsum<DP4, true>, 0, kMaxCtasPerSm);
             if (p.w) return launch(c, k_near_rowsum<DP4, true>, 0, weighted, 0, p);
             return launch(c, k_near_rowsum<DP4, false>, 0, plain, 0, p);
         }

@@ -74,7 +74,7 @@ struct fd_ctx {
     bool packed_ordered = false, packed_row_ordered = false;     // they hold the points in the order of L.perm
     int order_state = 0;             // 1: L.perm holds an order of the points; -1: none will be made
     // tile lists, for Gram-form block products (0) and degree passes (1) and all passes of the direct-difference kernels (2): bandwidth they were decided for, whether
-    // they leave out enough to be used, entries in all; which of the three the workspace holds, and for which bandwidth
+    // they leave out enough to be used, entries in all (products: of the list they go by)
     struct { double beta = -1.0; bool on = false; int64_t total = 0; } lists[3];
     // A pass of this context was recorded into a CUDA graph (set by note_capture, for good).  What the workspace holds is then known to nobody
     // on the host: recording runs nothing, and a replay packs and lists again.  Every pass packs and lists for itself from then on.

@@ -73,7 +73,8 @@ constexpr int smem_total(int K16) { return 1024 + kStages * K16 * kXChunk + 2 * 
 // Steps before resident pair r: pair r has the streamed tiles 2 r .. num_jt - 1.
 __host__ __device__ __forceinline__ long long steps_before(long long r, long long num_jt) { return r * num_jt - r * (r - 1); }
 // A CTA's range, item by item.  One type without lists and one with them: the exponential warps of the weighted instantiation
-// have no register to spare (one type with a run-time choice spilled 176 B a thread instead of 28: N = 2^18, both passes 21.7 -> 23.0 ms).
+// have no register to spare (scalar sums: one type with a run-time choice spilled 176 B a thread instead of 28: N = 2^18, both passes 21.7 ->
+// 23.0 ms; with packed sums the weighted instantiations spill 36 and, with lists, 44 B, those with squares 12).
 template <bool LISTED> struct Item;
 template <> struct Item<false> {
     int pair, j0, n;             // streamed tiles j0 ..
