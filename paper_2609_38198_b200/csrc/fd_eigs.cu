@@ -60,6 +60,7 @@ struct Solver {
     int m = 0;
     int applies = 0, restarts = 0;
     double t_apply = 0.0;
+    bool clean = true;              // the latest block was far from dependent: one orthogonalisation was enough
     bool timing = false;            // the events around the latest products are not read yet
 
     Panel own(const float* p, int cols) const { return panel(p + r0, cols, N); }
@@ -327,7 +328,8 @@ struct Solver {
             dst = src == other ? target : other;
             FD_TRY(subtract_and_mix(src, p, h, ld, F.data(), rank, dst));
             p = rank;
-            if (pass == 0 && lam_min > 1e-2 && cmax < 1e-2) break;
+            clean = pass == 0 && lam_min > 1e-2 && cmax < 1e-2;
+            if (clean) break;
         }
         if (dst == other) FD_TRY(copy_cols(c, other + r0, N, target + r0, N, p, n));
         return FD_OK;
@@ -429,10 +431,16 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
     // The block after the last one before a Rayleigh-Ritz step is made, and M applied to it, while the host solves the projected
     // eigenproblem: the residuals of all Ritz vectors lie in its span, so it is the next expansion whatever that step decides.  It
     // waits in R and its image in the extension's scratch: the basis may be full.  Only while the blocks are a Krylov sequence (cold starts,
-    // no direction dropped), and while the residuals are expected to stay well above the tolerance: a solve's last steps take
-    // explicit residuals, which also see what the stored images have lost to rounding.  6-torus, N = 2^17, k = 64: 323 -> 293 ms, N = 86893, k = 40:
-    // 185 -> 152; R^30, N = 65536, k = 32: 38 -> 32; 2-torus, N = 16384, k = 32: 29.1 -> 26.3 (as many products but for one or two).
-    constexpr double kAhead = 100.0;
+    // from the first step on), and while the residuals are expected to stay well above the tolerance (kAhead): a solve's last steps take
+    // explicit residuals, which also see what the stored images have lost to rounding.
+    // What the sequence has lost to rounding it never finds again.  A nearly dependent block is mostly rounding in its weak directions, so
+    // it ends the sequence (an explicit residual block nearly always is one: smallest eigenvalue 1e-3 to 3e-5 where Krylov blocks have 0.1), and
+    // so does a wanted residual of which a part as large as kLost of the worst one lies outside the block's span: that block is still taken,
+    // the next one is of explicit residuals.  Without these two, solves stalled at 1e-4 until max_applies (6-torus, N = 2000, k = 23, capacity
+    // 328: 120 products and 1 pair where 49 had given 24) or took up to twice the products.
+    // 6-torus, N = 2^17, k = 64, capacity 259: 323 -> 293 ms, N = 86893, k = 40: 185 -> 152; R^30, N = 65536, k = 32: 38 -> 32; 2-torus, N = 16384,
+    // k = 32: 29.1 -> 26.3.
+    constexpr double kAhead = 100.0, kLost = 0.1;
     bool krylov = !Q0_dev && !small_basis;
     float* const ahead_image = c->at<float>(L.wp);
     int ahead = 0;
@@ -490,6 +498,7 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
         const double thr = tol * std::fabs(theta[0]);
         bool all = false;
         int first = 0;                                             // X[:, i - first] holds the residual of pair i >= first
+        double outside = 0.0;                                      // largest squared part of a wanted residual that the block ahead does not span
         for (int pass = 0; pass < 2; ++pass) {
             first = std::min(nlock, nsel);
             const int w = nsel - first;
@@ -506,8 +515,15 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
                 FD_TRY(S.send_slot(cnt));
                 FD_TRY(nn_product(c, S.own(S.W, m, S.Q, m), S.d_S, 2 * m, w, S.X + r0, N, n));
                 FD_TRY(col_sqnorms(c, S.X + r0, N, w, n, S.h));
-                FD_TRY(S.fetch(w));
+                if (ahead > 0) FD_TRY(tn_product(c, S.own(S.R, ahead), S.own(S.X, w), n, S.h + w, S.d_scr, S.scr_n));
+                FD_TRY(S.fetch(w + (int64_t)ahead * w));
                 for (int jj = 0; jj < w; ++jj) resid[first + jj] = std::sqrt(std::max(0.0, S.h[jj]));
+                outside = 0.0;
+                for (int jj = 0; jj < w && first + jj < nwant && ahead > 0; ++jj) {
+                    double rest = S.h[jj];
+                    for (int i = 0; i < ahead; ++i) { const double z = S.h[w + i + (size_t)jj * ahead]; rest -= z * z; }
+                    outside = std::max(outside, rest);
+                }
             }
             nconv = 0;
             while (nconv < std::min(nwant, nsel) && resid[nconv] <= thr) ++nconv;
@@ -537,6 +553,7 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
                     last_rate = std::log(last_worst / worst) / std::max(1, S.applies - last_applies);
                     blocks = std::max(1, std::min(kMaxBlocks, (int)std::ceil(std::log(worst / thr) / last_rate)));
                 }
+                if (outside > kLost * kLost * worst * worst) krylov = false;
                 last_worst = worst;
                 last_applies = S.applies;
             }
@@ -615,7 +632,7 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
                 FD_TRY(copy_cols(c, ahead_image + r0, N, S.W + (int64_t)S.m * N + r0, N, p, n));
                 ahead = 0;
             } else FD_TRY(S.expand(B, p, z, ldz));
-            krylov = krylov && p == b;
+            krylov = krylov && p == b && (have_image || S.clean);
             if (p == 0) {
                 if (blk > 0) break;                                // the continuation added nothing: back to the Ritz pairs
                 // the residuals lie (numerically) inside the basis: try a random direction, give up after a few
@@ -640,12 +657,12 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
         }
         if (stuck) break;
         // ---- the next block, ahead of the step that decides ----------------------------------------
-        if (krylov && p == b && nsel >= nwant && S.m + b <= N && S.applies + 1 < max_applies &&
-            last_worst * std::exp(-last_rate * (S.applies - last_applies)) > kAhead * tol * std::fabs(theta[0])) {
+        if (krylov && p == b && S.m + b <= N && S.applies + 1 < max_applies &&
+            (nsel < nwant || last_worst * std::exp(-last_rate * (S.applies - last_applies)) > kAhead * tol * std::fabs(theta[0]))) {
             ldz = S.m + p;
             zkeep.assign(S.h + (size_t)p * ldz, S.h + (size_t)2 * p * ldz);
             FD_TRY(S.expand(S.W + (int64_t)(S.m - p) * N, p, zkeep.data(), ldz, S.R, S.X));
-            krylov = p == b;
+            krylov = p == b && S.clean;
             if (p > 0) FD_TRY(S.apply_block(S.R, ahead_image, p, b));
             ahead = p;
         }

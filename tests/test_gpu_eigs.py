@@ -179,6 +179,25 @@ def test_warm_start_matches_cold_and_saves_applies(fd, dev):
     ctx.close()
 
 
+def _flat_torus(N, d, seed):
+    a = np.random.default_rng(seed).random((N, d)) * 2 * np.pi
+    return np.concatenate([np.cos(a), np.sin(a)], 1).astype(np.float32)
+
+
+@pytest.mark.parametrize("N,beta,k,b,m_max,seed,most", [(2000, 1.4099127106205451, 23, 32, 328, 107, 65), (4096, 1.4175922193559278, 15, 24, 192, 630, 65),
+                                                        (2000, 0.17829840581920364, 40, 32, 219, 859, 16), (8192, 0.19180206907114164, 31, 24, 176, 206, 17)])
+def test_blocks_made_ahead_lose_no_direction(fd, dev, N, beta, k, b, m_max, seed, most):
+    """Solves on 6-tori whose residual blocks are nearly dependent: every pair converges within the products that a solver with an explicit residual
+    block at every step takes (49, 48, 10 and 13), and a third."""
+    ctx = fd.Context(torch.from_numpy(_flat_torus(N, 6, seed)).to(dev), b_max=b, m_max=m_max)
+    ctx.degree(beta, 1.0)
+    lam, U, info = ctx.eigs(k, b, max_applies=2 * most)
+    V = ctx.apply(U) if b >= k + 1 else torch.cat([ctx.apply(U[:, i:i + b]) for i in range(0, k + 1, b)], 1)
+    assert info.converged == k + 1 and info.applies <= most, info.applies
+    assert (V - U * torch.from_numpy(lam).to(dev).float()).norm(dim=0).max().item() <= 5e-6
+    ctx.close()
+
+
 def test_eigs_argument_errors(fd, dev):
     X = workloads.torus2(256, seed=1)
     ctx = fd.Context(torch.from_numpy(X).to(dev), b_max=8, m_max=16)
