@@ -422,10 +422,14 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
     const bool small_basis = m_cap < 3 * nwant && m_cap < N;
     const int kMaxBlocks = small_basis ? 1 : 4;
     const bool wanted_first = !small_basis;
-    // Ritz vectors kept at a restart: three fifths of the basis or, where twice the wanted pairs are less, as many above that as leave room for whole
-    // blocks: a group of blocks more between two restarts for as many products in all (6-torus, N = 2^17, k = 64: 11 -> 8 restarts, 293 -> 282 ms;
-    // N = 86893, k = 40: 19 -> 12, 153 -> 133 ms; 2-torus, N = 16384, k = 25: 20 -> 12, 28.5 -> 23.5 ms).
-    const int restart_keep = small_basis || 2 * nwant > (m_cap * 3) / 5 ? (m_cap * 3) / 5 : m_cap - (m_cap - 2 * nwant) / b * b;
+    // Ritz vectors kept at a restart: three fifths of the basis and the room that no whole block fits in.  Fewer, down to twice the wanted pairs, where that
+    // leaves the gap between the last wanted Ritz value and the first one not kept: a block or more beyond the next restart for about as
+    // many products (6-torus, N = 2^17, k = 64: 11 -> 8 restarts, 293 -> 282 ms; N = 86893, k = 40: 19 -> 12, 153 -> 133 ms; 2-torus, N = 16384,
+    // k = 25: 20 -> 12, 28.5 -> 23.5 ms).  Fewer in a cluster that the wanted pairs belong to closes the gap: 6-torus, N = 20000, k = 3, capacity 28:
+    // 29 -> 81 products, N = 16384, k = 32, capacity 163: 27 -> 45 (now 31 and 26).  kGap: 0.15 still cuts clusters (32 products), 0.5 and 0.8 keep
+    // more than they need (2-torus, k = 32: 25.6 -> 25.8 ms; R^30: 31.0 -> 32.0 at 0.5).
+    constexpr double kGap = 0.3;
+    const int most_kept = small_basis ? (m_cap * 3) / 5 : m_cap - (m_cap - (m_cap * 3) / 5) / b * b;
     double last_worst = 0.0, last_rate = 0.0;
     int last_applies = 0;
     // The block after the last one before a Rayleigh-Ritz step is made, and M applied to it, while the host solves the projected
@@ -474,7 +478,7 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
         auto tp1 = clk::now();
         // eigenvectors: the leading Ritz vectors on every step; the larger kept set only when this step may restart
         const int nvec_ritz = std::min(nsel_max, m);
-        const int nvec = (m + b > m_cap) ? std::max(nvec_ritz, std::min(m - 1, restart_keep)) : nvec_ritz;
+        const int nvec = (m + b > m_cap) ? std::max(nvec_ritz, std::min(m - 1, most_kept)) : nvec_ritz;
         if (!sym_eig(Tc.data(), m, lam, U, nvec)) return fail(c, FD_ERR_NOT_CONVERGED, "projected eigenproblem failed");
         auto tp2 = clk::now();
         t_rr += secs(tp0, tp1); t_eig += secs(tp1, tp2);
@@ -586,7 +590,13 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
 
         // ---- thick restart when the new block would not fit ----------------------------------------
         if (m + p > m_cap) {
-            int keep = std::max(nsel, std::min(m - 1, restart_keep));
+            int keep = std::min(m - 1, most_kept);
+            if (!small_basis && m >= nwant) {
+                const double last = lam[m - nwant], gap = last - lam[m - 1 - keep];
+                for (int fewer = m_cap - (m_cap - 2 * nwant) / b * b; fewer < keep; fewer += b)
+                    if (last - lam[m - 1 - fewer] >= kGap * gap) { keep = fewer; break; }
+            }
+            keep = std::max(nsel, keep);
             keep = std::min(keep, m_cap - p);
             keep = std::min(keep, m);
             // Ritz vectors for the kept block (beyond nsel use the uncorrected eigenvectors)

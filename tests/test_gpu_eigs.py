@@ -198,6 +198,19 @@ def test_blocks_made_ahead_lose_no_direction(fd, dev, N, beta, k, b, m_max, seed
     ctx.close()
 
 
+@pytest.mark.parametrize("N,beta,k,b,m_max,most", [(20000, 1.0, 3, 8, 28, 42), (16384, 1.0, 32, 32, 163, 34), (40000, 1.0, 3, 8, 48, 29), (8192, 0.3, 20, 16, 95, 32)])
+@pytest.mark.parametrize("seed", [0, 1])
+def test_restarts_keep_the_cluster_of_the_wanted_pairs(fd, dev, N, beta, k, b, m_max, most, seed):
+    """6-tori, whose eigenvalues come in clusters of 12, 60, ..: a restart that cuts the cluster of the last wanted pair takes two to three times the
+    products (81, 45, 34 at the first three).  `most`: the products of restarts that keep three fifths of the basis (29 to 35, 27, 22, 26 over
+    the seeds), and a fifth."""
+    ctx = fd.Context(torch.from_numpy(_flat_torus(N, 6, seed)).to(dev), b_max=b, m_max=m_max)
+    ctx.degree(beta, 1.0)
+    lam, U, info = ctx.eigs(k, b, max_applies=2 * most)
+    assert info.converged == k + 1 and info.applies <= most, info.applies
+    ctx.close()
+
+
 def test_eigs_argument_errors(fd, dev):
     X = workloads.torus2(256, seed=1)
     ctx = fd.Context(torch.from_numpy(X).to(dev), b_max=8, m_max=16)
