@@ -1,5 +1,6 @@
 // Tall-skinny dense helpers (fd_dense.cu) and the host symmetric eigensolver (fd_symeig.cpp).
 #pragma once
+#include <functional>
 #include <vector>
 
 #include "fd_internal.h"
@@ -33,7 +34,9 @@ double host_dot(const double* x, const double* y, int n);
 // Eigen-decomposition of a dense symmetric n x n matrix (column-major, only read).  On return evals ascending (all n) and
 // evecs n x n column-major with orthonormal columns; with 0 <= nvec < n only the columns of the nvec LARGEST eigenvalues
 // (columns n - nvec .. n - 1) are computed, the others are zero.  Householder tridiagonalisation followed by implicit
-// symmetric QR.  Returns false if the iteration fails to converge.
-bool sym_eig(const double* A, int n, std::vector<double>& evals, std::vector<double>& evecs, int nvec = -1);
+// symmetric QR.  Returns false if the iteration fails to converge.  needed, if given, says how many of the nvec columns are needed
+// once the (ascending) eigenvalues are known.
+bool sym_eig(const double* A, int n, std::vector<double>& evals, std::vector<double>& evecs, int nvec = -1,
+             const std::function<int(const double*)>& needed = nullptr);
 
 }  // namespace fd

@@ -430,6 +430,14 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
     // more than they need (2-torus, k = 32: 25.6 -> 25.8 ms; R^30: 31.0 -> 32.0 at 0.5).
     constexpr double kGap = 0.3;
     const int most_kept = small_basis ? (m_cap * 3) / 5 : m_cap - (m_cap - (m_cap * 3) / 5) / b * b;
+    const auto kept_at = [&](const double* ritz, int m) {          // ascending Ritz values of m columns
+        const int most = std::min(m - 1, most_kept);
+        if (small_basis || m < nwant) return most;
+        const double last = ritz[m - nwant], gap = last - ritz[m - 1 - most];
+        for (int fewer = m_cap - (m_cap - 2 * nwant) / b * b; fewer < most; fewer += b)
+            if (last - ritz[m - 1 - fewer] >= kGap * gap) return fewer;
+        return most;
+    };
     double last_worst = 0.0, last_rate = 0.0;
     int last_applies = 0;
     // The block after the last one before a Rayleigh-Ritz step is made, and M applied to it, while the host solves the projected
@@ -478,8 +486,10 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
         auto tp1 = clk::now();
         // eigenvectors: the leading Ritz vectors on every step; the larger kept set only when this step may restart
         const int nvec_ritz = std::min(nsel_max, m);
-        const int nvec = (m + b > m_cap) ? std::max(nvec_ritz, std::min(m - 1, most_kept)) : nvec_ritz;
-        if (!sym_eig(Tc.data(), m, lam, U, nvec)) return fail(c, FD_ERR_NOT_CONVERGED, "projected eigenproblem failed");
+        const bool may_restart = m + b > m_cap;
+        const int nvec = may_restart ? std::max(nvec_ritz, std::min(m - 1, most_kept)) : nvec_ritz;
+        const auto needed = [&](const double* l) { return may_restart ? std::max(nvec_ritz, kept_at(l, m)) : nvec; };
+        if (!sym_eig(Tc.data(), m, lam, U, nvec, needed)) return fail(c, FD_ERR_NOT_CONVERGED, "projected eigenproblem failed");
         auto tp2 = clk::now();
         t_rr += secs(tp0, tp1); t_eig += secs(tp1, tp2);
         nsel = std::min(nsel_max, m);
@@ -590,13 +600,7 @@ extern "C" fd_status fd_eigs(fd_ctx* c, int32_t k, int32_t b, double tol, int32_
 
         // ---- thick restart when the new block would not fit ----------------------------------------
         if (m + p > m_cap) {
-            int keep = std::min(m - 1, most_kept);
-            if (!small_basis && m >= nwant) {
-                const double last = lam[m - nwant], gap = last - lam[m - 1 - keep];
-                for (int fewer = m_cap - (m_cap - 2 * nwant) / b * b; fewer < keep; fewer += b)
-                    if (last - lam[m - 1 - fewer] >= kGap * gap) { keep = fewer; break; }
-            }
-            keep = std::max(nsel, keep);
+            int keep = std::max(nsel, kept_at(lam.data(), m));
             keep = std::min(keep, m_cap - p);
             keep = std::min(keep, m);
             // Ritz vectors for the kept block (beyond nsel use the uncorrected eigenvectors)

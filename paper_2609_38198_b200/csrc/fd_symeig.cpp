@@ -292,7 +292,7 @@ FD_HOST_CLONES void apply_rotations_reversed(double* w, int cw, const std::vecto
 
 }  // namespace
 
-bool sym_eig(const double* A, int n, std::vector<double>& evals, std::vector<double>& evecs, int nvec) {
+bool sym_eig(const double* A, int n, std::vector<double>& evals, std::vector<double>& evecs, int nvec, const std::function<int(const double*)>& needed) {
     evals.assign(n, 0.0);
     evecs.assign((size_t)n * n, 0.0);
     if (n == 0) return true;
@@ -313,6 +313,7 @@ bool sym_eig(const double* A, int n, std::vector<double>& evals, std::vector<dou
         if (!tridiagonal_qr(diag, e, n, nullptr, 0, rots, true)) return false;
         std::sort(order.begin(), order.end(), [&](int a, int b) { return diag[a] < diag[b]; });
         for (int c = 0; c < n; ++c) evals[c] = diag[order[c]];
+        if (needed) nvec = std::min(nvec, needed(evals.data()));
         // The nvec largest eigenvalues sit at ascending positions n - nvec .. n - 1.  Their vectors are independent of one
         // another from here on: each thread takes a slice of them in a buffer of its own (no cache line is shared between
         // threads), starts from the unit vectors that select them, undoes the rotations and then the reflectors.
