@@ -3,7 +3,7 @@
 //
 // Everything here is in the points' order: an ordered copy of the points (made with the order) and an ordered, scaled copy of the right
 // block (made per product, two microseconds), so that the 16 points of a list entry and their right rows are one contiguous piece each.
-// A WARP owns 64 rows, two a lane, and takes its entries through a ring of its own in shared memory (cp.async), without any
+// A WARP owns 64 rows, two a lane (up to 4 columns: four), and takes its entries through a ring of its own in shared memory (cp.async), without any
 // barrier of the block: neighbouring warps need not agree on which tiles are near.  The flat sequence of (64 rows, entry) steps is cut
 // into equal ranges, one per warp; shares of row groups that a cut falls into are added by k_near_fix in the order of the warps.
 //
@@ -22,8 +22,7 @@ namespace {
 using namespace direct;
 
 constexpr int kWarps = kThr / 32;
-constexpr int kRowsG = 64;       // rows of a group: two per lane
-constexpr int kRows = 2;
+constexpr int kRowsG = 64;       // rows of a group: two per lane, or four with the points of an entry shared by the two halves of the warp
 constexpr int kEntry = 16;       // points of a list entry
 constexpr int kRing = 3;         // entries in a warp's ring
 constexpr int kMaxCtasPerSm = 8;     // (fewer where the room for the shares of cut row groups says so)
@@ -97,12 +96,18 @@ __device__ __forceinline__ void load_entry(const NearParams& p, int e, float4* s
     }
 }
 
-template <int DP4>
-__device__ __forceinline__ void load_rows(const NearParams& p, int grp, int lane, float4 (&xi)[kRows][DP4]) {
+// Row r of a lane: row + step r of the group.
+template <int R> struct Rows {
+    static constexpr int kHalves = R / 2, kStep = kRowsG / R, kPoints = kEntry / kHalves;
+    int row, half;                                       // first row; which part of an entry's points
+    __device__ __forceinline__ Rows(int lane) : row(lane % kStep), half(lane / kStep) {}
+};
+template <int DP4, int R>
+__device__ __forceinline__ void load_rows(const NearParams& p, int grp, const Rows<R>& rows, float4 (&xi)[R][DP4]) {
 #pragma unroll
-    for (int r = 0; r < kRows; ++r)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int k = 0; k < DP4; ++k) xi[r][k] = p.x[((size_t)grp * kRowsG + lane + 32 * r) * DP4 + k];
+        for (int k = 0; k < DP4; ++k) xi[r][k] = p.x[((size_t)grp * kRowsG + rows.row + rows.kStep * r) * DP4 + k];
 }
 
 // Runs body(entry, slot) over the entries of a range's part, with kRing - 1 of them in flight.
@@ -133,55 +138,66 @@ __device__ __forceinline__ void for_entries(const NearParams& p, const Range& ra
     __syncwarp();
 }
 
-// (resident CTAs asked for, by the registers that the rows and sums of a thread need)
-constexpr int near_ctas(int DP4, int BT) { return BT <= 8 ? (4 * DP4 + BT <= 8 ? 8 : 6) : BT <= 24 ? 4 : BT <= 32 ? 3 : 2; }
+// Rows per lane: four up to 4 columns, where the reads of x_j and w_j from shared memory are a quarter of the instructions: sets on which boxes are as
+// good as notes were slower than a step of 256 rows x 64 points by a whole block without it (N = 100000, b = 1: circle 1763 us there, 1900 with
+// two rows, 1673 with four; a line in R^7 4339, 4657 and 4313).
+constexpr int near_rows(int BT) { return BT <= 4 ? 4 : 2; }
+// (resident CTAs asked for, by the registers that the rows and sums of a thread need; 4 columns: four CTAs with all eight points of a turn unrolled, six
+// with four of them 1857 us)
+constexpr int near_ctas(int BT) { return BT <= 4 ? 4 : BT <= 8 ? 6 : BT <= 24 ? 4 : BT <= 48 ? 3 : 2; }
+// Points per turn of the inner loop: as many as leave the sums in registers.  48 columns: two, with three resident CTAs, instead of four with two (N = 100000,
+// b = 40: line in R^7 17.4 -> 15.2 ms, circle 9.36 -> 8.79); 5 to 8 coordinates, 8 columns: 5.88 -> 5.55 ms.
+constexpr int near_unroll(int DP4, int BT) { return BT <= 4 ? 8 : BT == 48 || (DP4 == 2 && (BT == 8 || BT == 16)) ? 2 : 4; }
 
 // Y[i, c] = left_i sum_j K_ij w[j, c] for c < b <= BT.
 template <int DP4, int BT>
-__global__ void __launch_bounds__(kThr, near_ctas(DP4, BT))
+__global__ void __launch_bounds__(kThr, near_ctas(BT))
 k_near(const NearParams p) {
     grid_wait();
     grid_go();
-    constexpr int WF4 = BT / 4, kSlot = kEntry * (DP4 + WF4);
+    constexpr int R = near_rows(BT), WF4 = BT / 4, kSlot = kEntry * (DP4 + WF4);
     extern __shared__ __align__(16) float4 smem_near[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, warp = (int)blockIdx.x * kWarps + wib, warps = (int)gridDim.x * kWarps;
     float4* ring = smem_near + wib * kRing * kSlot;
+    const Rows<R> rows(lane);
     Range range(p, warp, warps);
     while (range.next(p, lane)) {
-        float4 xi[kRows][DP4];
-        load_rows<DP4>(p, range.grp, lane, xi);
-        Sums<kRows, BT> acc;
+        float4 xi[R][DP4];
+        load_rows<DP4, R>(p, range.grp, rows, xi);
+        Sums<R, BT> acc;
         acc.clear();
         // Two-level sums: the points are in their order, so one long fp32 sum would add the far points' small values to the near ones' large sum and
         // drop them, always with the same sign.  Up to 16 columns the second level is in registers, for wider blocks in the warp's slot.
         constexpr bool kInRegs = BT <= 16;
-        constexpr int kFlush = kInRegs ? 2 : 8;                    // entries between flushes (4 to memory: 1046 -> 1127 us at N = 65536, b = 32)
-        float sum[kRows][kInRegs ? BT : 1];
+        static_assert(kInRegs || R == 2, "four rows a lane: sums in registers only");
+        constexpr int kFlush = kInRegs ? 2 * rows.kHalves : 8;     // entries between flushes: 32 points (64 to memory: 1046 -> 1127 us at N = 65536, b = 32)
+        float sum[R][kInRegs ? BT : 1];
         if (kInRegs) {
 #pragma unroll
-            for (int r = 0; r < kRows; ++r)
+            for (int r = 0; r < R; ++r)
 #pragma unroll
                 for (int c = 0; c < (kInRegs ? BT : 1); ++c) sum[r][c] = 0.f;
         }
         // the warp's slot for a share of this kind; sums that restart on the way wait there too
-        float* slot_out = static_cast<float*>(p.part) + (size_t)(2 * warp + (range.c0 == 0 ? 1 : 0)) * BT * kRowsG + lane;
+        float* slot_out = static_cast<float*>(p.part) + (size_t)(2 * warp + (range.c0 == 0 ? 1 : 0)) * BT * kRowsG + rows.row;
         bool flushed = false;
         for_entries<DP4, WF4>(p, range, ring, lane, [&](int t, const float4* slot) {
-            const float4* sw = slot + kEntry * DP4;
-#pragma unroll 4
-            for (int jj = 0; jj < kEntry; ++jj) {
-                float kij[kRows];
-                kernel_values<DP4, kRows>(slot, jj, xi, p.nbeta2, kij);
+            const float4* sx = slot + rows.half * rows.kPoints * DP4;
+            const float4* sw = slot + kEntry * DP4 + rows.half * rows.kPoints * WF4;
+#pragma unroll near_unroll(DP4, BT)
+            for (int jj = 0; jj < rows.kPoints; ++jj) {
+                float kij[R];
+                kernel_values<DP4, R>(sx, jj, xi, p.nbeta2, kij);
                 acc.add(kij, sw + jj * WF4);
             }
             if ((t + 1) % kFlush == 0 && t + 1 < range.n) {
 #pragma unroll
-                for (int r = 0; r < kRows; ++r)
+                for (int r = 0; r < R; ++r)
 #pragma unroll
                     for (int c = 0; c < BT; ++c) {
                         if constexpr (kInRegs) sum[r][c] += acc.get(r, c);
                         else {
-                            float* s = slot_out + c * kRowsG + 32 * r;
+                            float* s = slot_out + c * kRowsG + rows.kStep * r;
                             *s = flushed ? *s + acc.get(r, c) : acc.get(r, c);
                         }
                     }
@@ -191,18 +207,26 @@ k_near(const NearParams p) {
         });
         const bool whole = range.n == range.full;
 #pragma unroll
-        for (int r = 0; r < kRows; ++r) {
-            const int64_t pos = (int64_t)range.grp * kRowsG + lane + 32 * r;
+        for (int u = 0; u < 2; ++u) {
+            // (four rows a lane: each half of the warp finishes two of them, and gets its share of these from the other)
+            const int r = R == 2 ? u : u + 2 * rows.half;
+            const int64_t pos = (int64_t)range.grp * kRowsG + rows.row + rows.kStep * r;
             const bool valid = pos < p.N;
             const int64_t i = valid ? p.perm[pos] : 0;
             const float l = whole && p.left ? p.left[i] : 1.0f;
 #pragma unroll
             for (int c = 0; c < BT; ++c)
                 if (c < p.b) {
-                    float a = acc.get(r, c);
-                    if constexpr (kInRegs) a += sum[r][c];
-                    else if (flushed) a += slot_out[c * kRowsG + 32 * r];
-                    if (!whole) slot_out[c * kRowsG + 32 * r] = a;
+                    float a;
+                    if constexpr (R == 4) {
+                        const float lo = acc.get(u, c) + sum[u][c], hi = acc.get(u + 2, c) + sum[u + 2][c];
+                        a = (rows.half ? hi : lo) + __shfl_xor_sync(0xffffffffu, rows.half ? lo : hi, 16);
+                    } else {
+                        a = acc.get(u, c);
+                        if constexpr (kInRegs) a += sum[u][c];
+                        else if (flushed) a += slot_out[c * kRowsG + rows.kStep * r];
+                    }
+                    if (!whole) slot_out[c * kRowsG + rows.kStep * r] = a;
                     else if (valid) p.Y[i + (int64_t)c * p.ldy] = a * l;
                 }
         }
@@ -217,12 +241,13 @@ k_near_rowsum(const NearParams p) {
     grid_go();
     constexpr int kSlot = kEntry * DP4;
     __shared__ float4 ring_store[kWarps * kRing * kSlot];
+    constexpr int kRows = 2;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, warp = (int)blockIdx.x * kWarps + wib, warps = (int)gridDim.x * kWarps;
     float4* ring = ring_store + wib * kRing * kSlot;
     Range range(p, warp, warps);
     while (range.next(p, lane)) {
         float4 xi[kRows][DP4];
-        load_rows<DP4>(p, range.grp, lane, xi);
+        load_rows<DP4, kRows>(p, range.grp, Rows<kRows>(lane), xi);
         double dsum[kRows], dsq[kRows];
 #pragma unroll
         for (int r = 0; r < kRows; ++r) { dsum[r] = 0.0; dsq[r] = 0.0; }

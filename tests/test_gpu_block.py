@@ -250,7 +250,8 @@ def test_far_tiles_are_left_out(N, kind):
 @pytest.mark.parametrize("N,kind,b", [(16384, "torus2", 16), (16385, "circle", 5), (17001, "clusters7", 40), (33001, "duplicates", 24),
                                       (20011, "torus2", 70), (40000, "line", 3), (16400, "torus2", 1), (17000, "clusters7", 8), (16385, "clusters7", 16),
                                       (19999, "torus2", 24), (18001, "torus2", 32), (16640, "clusters7", 32), (17920, "torus2", 48), (16386, "torus2", 64),
-                                      (17003, "clusters7", 64)])
+                                      (17003, "clusters7", 64), (17100, "clusters7", 3),
+                                      (16777, "circle", 4)])
 def test_far_tiles_are_left_out_of_direct_passes(N, kind, b):
     """Direct-difference passes without the tiles whose kernel values are exactly zero: degrees, sums and products against float64 sums
     (gate 1e-6 of that family), bit-identical repeats, bandwidths with and without lists, and a product at a bandwidth that no
