@@ -168,9 +168,9 @@ typedef struct {
  * implicitly restarted Lanczos and gives no further detail; Sec. 2.3).  b = block size,
  * tol = residual tolerance relative to theta_0, Q0_dev = optional warm-start basis (N x q0_cols,
  * need not be orthonormal).  evals_host: k + 1 doubles, descending.  evecs_dev: N x (k + 1)
- * column-major, orthonormal.  Needs m_max >= 2 (k + 1) + b at fd_create; the thick restart keeps up to 3/5 of m_max, so a
+ * column-major, orthonormal.  Needs m_max >= 2 (k + 1) + b at fd_create; the thick restart keeps about 3/5 of m_max or less, so a
  * capacity near 3 (k + 1) + 2 b keeps room for the rest of an eigenvalue cluster that the request cuts (on the
- * 6-torus, k = 128 cuts a 160-fold cluster: 129 of 129 pairs converge in 43 block products with m_max = 576, 384
+ * 6-torus, k = 128 cuts a 160-fold cluster: 129 of 129 pairs converge in 44 block products with m_max = 576, 384
  * stalls above tol).  Below 3 (k + 1) every block is a residual block, with a projected eigenproblem after each product, and a
  * solve that stalls just above tol is reported as it is; from there on M is applied to the basis again first.
  * info->converged counts the LEADING pairs below tol.  Residuals (tol, max_residual) are formed from the basis's stored images
