@@ -488,7 +488,9 @@ k_block(const __grid_constant__ CUtensorMap map_xrow, const __grid_constant__ CU
     }
 }
 
-// Finishes the row pairs that a cut falls into: adds the CTAs' shares in the order of the CTAs.  Block = (row pair, 8 columns).
+// Finishes the row pairs that a cut falls into: adds the CTAs' shares in the order of the CTAs.  Block = (row pair, 8 columns).  A product of few rows is
+// cut into up to 37 shares a pair: eight are read ahead of their additions (one after the other, with a 64-bit division each: 50 us of
+// the 100 of a product of 1000 rows, 16384 points and 16 columns; 26 of 74 so).
 template <int BT>
 __global__ void __launch_bounds__(256)
 k_block_fix(const BlockParams p, int ctas) {
@@ -499,9 +501,9 @@ k_block_fix(const BlockParams p, int ctas) {
     const long long g0 = p.list ? (long long)p.offs[pair] : (long long)pair * p.num_jt;
     const long long g1 = p.list ? (long long)p.offs[pair + 1] : g0 + p.num_jt;
     ctas = range_count(total, ctas);
-    // the last CTA whose range begins at or before step g0
-    int cta = (int)(((g0 + 1) * ctas - 1) / total);
-    if (range_begin(total, cta + 1, ctas) >= g1) return;               // not cut: the CTA stored it
+    // the last CTA whose range begins at or before step g0, and the last one whose range begins before g1
+    const int first = (int)(((g0 + 1) * ctas - 1) / total), last = (int)((g1 * ctas - 1) / total);
+    if (first == last) return;                                         // not cut: the CTA stored it
     int64_t row = (int64_t)pair * 256 + threadIdx.x;
     if (row >= p.Nrow) return;
     if (p.perm) row = p.perm[row];
@@ -509,11 +511,10 @@ k_block_fix(const BlockParams p, int ctas) {
     float acc[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) acc[c] = 0.f;
-    for (; cta < ctas; ++cta) {
-        const long long b = range_begin(total, cta, ctas);
-        if (b >= g1) break;
+#pragma unroll 8
+    for (int cta = first; cta <= last; ++cta) {
         // the share whose item starts the row pair sits in slot 1 of its CTA, every later one in slot 0
-        const float* o = p.part + (size_t)(2 * cta + (b <= g0 ? 1 : 0)) * BT * 256 + threadIdx.x;
+        const float* o = p.part + (size_t)(2 * cta + (cta == first ? 1 : 0)) * BT * 256 + threadIdx.x;
 #pragma unroll
         for (int c = 0; c < 8; ++c)
             if (c0 + c < p.b) acc[c] += o[(c0 + c) * 256];
